@@ -109,58 +109,60 @@ __device__ __forceinline__ bool decide(float r2, float H2, float band, int gi, i
 }
 
 // =========================================================================== density
+struct Box3 {
+  float3 lo, hi;
+};
+
+// Per warp: the constants of a task and the candidate clusters of the current
+// scan.  Read back with broadcast loads where they are needed, which costs less
+// than the registers they would hold through the batches.
+struct __align__(16) TaskShared {
+  float4 blo;            // box of the own cluster's particles to find partners for (leaf frame); w: their largest H
+  float4 bhi;            // ... w: culling slack
+  float4 sh;             // frame offset of the partner cell's clusters; w: 1 / L
+  float4 win;            // x: sorted window offset (projection of the cell offset minus the drift and the own upper
+                         //   end), y: the partner cell's largest H, z: length scale of the position rounding,
+                         //   w: the own cluster's largest H
+  float4 clo, chi;       // later passes: box of the whole own cluster
+  unsigned int sb, ntj, tb0;   // the partner cell's sorted list (SORT_NONE: its clusters in their own order)
+  int box;
+  float4 co[32];         // candidates: frame offset, first particle (bits)
+  unsigned int cn[32];   //   size
+};
+
+// The lane's own particle of a density task: lo and hi bound the guard band around
+// H^2 (r^2 below lo is inside, above hi outside, between them decided in FP64).
 struct DensI {
   float3 p;
-  float H, invH, H2, band, Hphys, m;
+  float H, invH, lo, hi, Hphys, m;
   int g;
   bool valid, act;
 };
 
-// The raw loads of one particle, issued ahead of their use (see the pair kernel).
-struct DensRaw {
-  float4 p, c;
-  unsigned char a;
-};
-
-__device__ __forceinline__ DensRaw fetch_dens(bool valid, unsigned int gidx, const float4* pos4, const float4* cen4,
-                                              const unsigned char* act) {
-  DensRaw r;
-  if (valid) {
-    r.p = pos4[gidx];
-    r.c = cen4[gidx];
-    r.a = act ? act[gidx] : 1;      // no activity array: every particle iterates
-  } else {
-    r.p = make_float4(0.f, 0.f, 0.f, 0.f);
-    r.c = r.p;
-    r.a = 0;
-  }
-  return r;
-}
-
-__device__ __forceinline__ DensI make_dens(bool valid, unsigned int gidx, const DensRaw& raw, float3 shift,
-                                           float invL, float e) {
+// (in the frame of its leaf: its offset as stored)
+__device__ __forceinline__ DensI load_dens(bool valid, unsigned int gidx, const float4* pos4, const float4* cen4,
+                                           const unsigned char* act, float invL, float e) {
   DensI r;
   r.valid = valid;
   if (valid) {
-    const float4 p = raw.p;
-    const float4 c = raw.c;
-    // the cell offsets (c + shift) are exact dyadic values: add them first, round once
-    r.p = make_float3(p.x + (c.x + shift.x), p.y + (c.y + shift.y), p.z + (c.z + shift.z));
+    const float4 p = pos4[gidx];
+    r.p = make_float3(p.x, p.y, p.z);
     const float H = p.w * invL;
+    const float H2 = H * H, band = BAND_REL * H * (e + H);
     r.H = H;
     r.invH = __fdividef(1.0f, H);   // 2 ulp: enters the kernel's argument only
-    r.H2 = H * H;
-    r.band = BAND_REL * H * (e + H);
+    r.lo = H2 - band;
+    r.hi = H2 + band;
     r.Hphys = p.w;
-    r.m = c.w;
+    r.m = cen4[gidx].w;
     r.g = (int)gidx;
-    r.act = raw.a != 0;
+    r.act = act ? act[gidx] != 0 : true;   // no activity array: every particle iterates
   } else {
     r.p = make_float3(1e30f, 1e30f, 1e30f);
     r.H = 0.0f;
     r.invH = 0.0f;
-    r.H2 = -1.0f;
-    r.band = 0.0f;
+    r.lo = -1.0f;
+    r.hi = -1.0f;
     r.Hphys = 0.0f;
     r.m = 0.0f;
     r.g = -1;
@@ -169,18 +171,22 @@ __device__ __forceinline__ DensI make_dens(bool valid, unsigned int gidx, const 
   return r;
 }
 
-__device__ __forceinline__ DensI load_dens(bool valid, unsigned int gidx, float3 shift, const float4* pos4,
-                                           const float4* cen4, const unsigned char* act, float invL, float e) {
-  return make_dens(valid, gidx, fetch_dens(valid, gidx, pos4, cen4, act), shift, invL, e);
-}
-
-// Per warp: the staged partners (p, a, g, act) and the warp's own cluster (ip).
-struct DensShared {
-  float4 p[32];     // partner position, H^2 (units of L; H^2 = -1 marks an empty slot)
-  float4 a[32];     // partner 1/H, band, m, H (physical)
+// Per warp: the staged partners, the warp's own cluster (ip), and what the task
+// keeps out of registers (tk, and one entry per candidate cluster of the current
+// scan).  The coordinates are kept apart so that the mask phase reads four slots of
+// one coordinate with one 16-byte load, as two packed FP32 pairs.  A partner is
+// staged with its position, H and index only; what follows from them is computed
+// once per batch, by the slot's lane, and its mass is loaded then.
+struct __align__(16) DensShared {
+  float x[32], y[32], z[32];
+  float hi[32];     // H^2 + guard band (units of L^2); -1 marks an empty slot
+  float H[32];      // H (physical)
+  float m[32];
   int g[32];
-  unsigned char act[32];
   float4 ip[32];    // own cluster: position, m
+  int ig[32];       //   index
+  TaskShared tk;
+  unsigned char act[32];
   // pair records (first pass): the current task's first batch, batch count and
   // record slot, and 0 once one of its batches was lost (lane 0 keeps them)
   unsigned int rc_first, rc_nb, rc_slot, rc_ok;
@@ -192,15 +198,13 @@ struct RecW {
   unsigned int pos = 0;
 };
 
-__device__ __forceinline__ void dens_put(DensShared& S, int lane, const DensI& j) {
-  S.p[lane] = make_float4(j.p.x, j.p.y, j.p.z, j.H2);
-  S.a[lane] = make_float4(j.invH, j.band, j.m, j.Hphys);
-  S.g[lane] = j.g;
-  S.act[lane] = j.act ? 1 : 0;
-}
-
-__device__ __forceinline__ void dens_stage_own(DensShared& S, int lane, const DensI& i) {
-  S.ip[lane] = make_float4(i.p.x, i.p.y, i.p.z, i.m);
+__device__ __forceinline__ void dens_put(DensShared& S, int slot, float3 p, float Hphys, unsigned int g, bool act) {
+  S.x[slot] = p.x;
+  S.y[slot] = p.y;
+  S.z[slot] = p.z;
+  S.H[slot] = Hphys;
+  S.g[slot] = (int)g;
+  S.act[slot] = act ? 1 : 0;
 }
 
 struct Counters {
@@ -455,6 +459,84 @@ __device__ __forceinline__ void pair_masks(const float3 ip, float iH2, float iba
   mJ &= allow;
 }
 
+// Two FP32 values in one 64-bit register, added and multiplied by one instruction
+// (rounded as the scalar ones, element by element).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, unsigned int& a, unsigned int& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// r^2 of a pair, in the order of operations of the mask phase (the sign of the
+// separation does not matter: both phases then take the same value).
+__device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
+  return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+}
+
+// Mask phase over the first n staged partners (n a multiple of 4): the slots not
+// surely outside, r^2 <= hi of the own particle (mI) and of the partner (mJ).  Four
+// slots take four 16-byte loads and, two slots per instruction, six operations for
+// r^2 and one per threshold; each decision is the sign of hi - r^2, shifted into
+// its mask (slots taken from the last, so that slot s lands in bit s).  The few
+// slots inside the band are told apart in the sweeps, which have r^2 again: testing
+// them here as well took 17 instructions per slot instead of 7.  With this phase, one
+// copy of the task code for pair and self tasks and the partners' values derived
+// once per batch, the density passes of a 33.5M clustered step took 55.4 ms instead
+// of 63.7 and issued a sixth fewer instructions (issue slots are what bounds them:
+// 74 % busy, DRAM at 3 %).  Unrolled further, the loops cost registers: 256 bytes
+// spilled, 100 ms.  Empty slots and empty lanes (1e30, hi = -1) pass neither test.
+template <bool BOTH>
+__device__ __forceinline__ void near_masks(float3 ip, float ihi, const float* X, const float* Y, const float* Z,
+                                           const float* W, int n, unsigned int& mI, unsigned int& mJ) {
+  const f32x2 nx = pack2(-ip.x, -ip.x), ny = pack2(-ip.y, -ip.y), nz = pack2(-ip.z, -ip.z);
+  const f32x2 hi = pack2(ihi, ihi), neg = pack2(-1.0f, -1.0f);
+  unsigned int oI = 0, oJ = 0;     // surely outside
+#pragma unroll 1
+  for (int s0 = n - 4; s0 >= 0; s0 -= 4) {
+    const ulonglong2 xx = *reinterpret_cast<const ulonglong2*>(X + s0);
+    const ulonglong2 yy = *reinterpret_cast<const ulonglong2*>(Y + s0);
+    const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(Z + s0);
+    ulonglong2 ww = make_ulonglong2(0, 0);
+    if (BOTH) ww = *reinterpret_cast<const ulonglong2*>(W + s0);
+#pragma unroll
+    for (int k = 1; k >= 0; --k) {
+      const f32x2 dx = add2(k ? xx.y : xx.x, nx), dy = add2(k ? yy.y : yy.x, ny), dz = add2(k ? zz.y : zz.x, nz);
+      const f32x2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+      unsigned int a0, a1;
+      unpack2(fma2(r2, neg, hi), a0, a1);
+      oI = __funnelshift_l(a1, oI, 1);
+      oI = __funnelshift_l(a0, oI, 1);
+      if (BOTH) {
+        unsigned int b0, b1;
+        unpack2(fma2(r2, neg, k ? ww.y : ww.x), b0, b1);
+        oJ = __funnelshift_l(b1, oJ, 1);
+        oJ = __funnelshift_l(b0, oJ, 1);
+      }
+    }
+  }
+  mI = ~oI;
+  mJ = ~oJ;
+}
+
 // lane s receives the lanes whose mask has bit s: the 32 x 32 bit matrix (row =
 // lane) transposed by recursive exchange of its off-diagonal blocks, 16 x 16
 // down to 1 x 1, one shuffle per level.
@@ -503,65 +585,167 @@ struct DensAcc {
 };
 
 // r from r^2 by the fast reciprocal square root (its rounding enters the kernel's
-// argument only; the neighbour decision is taken on r^2)
-__device__ __forceinline__ float pair_r(float r2) { return r2 > 0.0f ? r2 * rsqrtf(r2) : 0.0f; }
+// argument only; the neighbour decision is taken on r^2).  The floor keeps r = 0
+// at 0 without a test; it is below any r^2 of distinct positions that matters to W
+// (r = 1e-19 L).
+__device__ __forceinline__ float pair_r(float r2) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(r2, 1.2e-38f)));
+  return r2 * y;
+}
 
 // One density contribution: w and q w'(q) at q = r / H, weighted by m.
 template <bool KAHAN>
-__device__ __forceinline__ void dens_add(float r, float invH, float m, DensAcc<KAHAN>& acc, unsigned int& cnt) {
+__device__ __forceinline__ void dens_add(float r, float invH, float m, DensAcc<KAHAN>& acc) {
   float w, dw;
   const float q = r * invH;
   spline_w_dw(q, w, dw);
   const float gg = q * dw;                 // q w'(q) = r dW/dr in units of W
   acc.add(m, w, gg);
-  cnt++;
 }
 
-// Density batch: own side for r < H_i (active i), partner side for r < H_j
-// (active j) unless own_only.  cmask selects the bits the counters count (the
-// upper triangle inside one cluster, where every pair appears in both rows).
-template <bool COUNT, bool KAHAN>
-__device__ __forceinline__ void dens_tile(const DensI& I, DensShared& S, unsigned int allow, unsigned int jvalid,
-                                          unsigned int jact, float bandJ, int n, bool own_only, unsigned int cmask,
-                                          DensAcc<KAHAN>& acc, unsigned int& cnt, const unsigned int* perm,
-                                          const double* x, const ItemGeom& g, float4* dacc, unsigned int* dcnt,
-                                          Counters& C, bool rec, const PairRec& R, RecW& W) {
+// The pairs of a sweep inside the guard band, decided in FP64 and added to the
+// particle's sums in global memory (about one batch in ten has one).  Out of line,
+// with everything read back from memory, so that the sweeps keep their registers.
+// column: this lane's staged partner against own lanes (bits of unc); else this
+// lane's own particle against staged partners.
+__device__ __noinline__ void dens_band(const DensShared& S, unsigned int unc, bool column,
+                                       const unsigned int* __restrict__ perm, const double* __restrict__ x,
+                                       const float4* __restrict__ pos4, const BoxDesc* __restrict__ box,
+                                       float4* dacc, unsigned int* dcnt) {
   const int lane = threadIdx.x & 31;
-  unsigned int mI, mJ, rc = 0;
-  pair_masks(I.p, I.H2, I.band, I.g, I.Hphys, S, bandJ, allow, n, perm, x, box_exact(g), mI, mJ, rc);
+  const BoxDesc& bd = box[S.tk.box];
+  const int gme = column ? S.g[lane] : S.ig[lane];
+  const float Hp = pos4[gme].w;
+  const float invH = __fdividef(1.0f, Hp * (float)bd.invL);
+  const float4 me = column ? make_float4(S.x[lane], S.y[lane], S.z[lane], 0.0f) : S.ip[lane];
+  for (; unc; unc &= unc - 1) {
+    const int k = __ffs(unc) - 1;
+    const int go = column ? S.ig[k] : S.g[k];
+    if (!exact_less(gme, go, Hp, perm, x, bd.L, 0.5 * bd.L, bd.periodic)) continue;
+    const float4 o = column ? S.ip[k] : make_float4(S.x[k], S.y[k], S.z[k], S.m[k]);
+    DensAcc<false> a;
+    dens_add(pair_r(pair_r2(me.x - o.x, me.y - o.y, me.z - o.z)), invH, o.w, a);
+    flush_dens(gme, a.total(), 1u, dacc, dcnt);
+  }
+}
+
+// Own side of a density batch: the lane walks its mask of staged partners.
+template <bool KAHAN>
+__device__ __forceinline__ void dens_row(const DensI& I, const DensShared& S, unsigned int ui, DensAcc<KAHAN>& acc,
+                                         unsigned int& cnt, const unsigned int* perm, const double* x,
+                                         const float4* pos4, const BoxDesc* box, float4* dacc, unsigned int* dcnt) {
+  unsigned int unc = 0;
+#pragma unroll 1
+  for (unsigned int m = ui; m; m &= m - 1) {
+    const int sj = __ffs(m) - 1;
+    const float r2 = pair_r2(I.p.x - S.x[sj], I.p.y - S.y[sj], I.p.z - S.z[sj]);
+    if (r2 >= I.lo) {
+      unc |= m & (0u - m);
+      continue;
+    }
+    dens_add(pair_r(r2), I.invH, S.m[sj], acc);
+  }
+  cnt += __popc(ui & ~unc);
+  if (unc) dens_band(S, unc, false, perm, x, pos4, box, dacc, dcnt);
+}
+
+// The masks as exact decisions (counting and recording passes, which need them
+// before the sweeps): both decisions of a slot inside either band, in FP64.
+__device__ __noinline__ void resolve_masks(const DensShared& S, float ilo, float jlo, unsigned int& mI,
+                                           unsigned int& mJ, unsigned int& rc, const unsigned int* perm,
+                                           const double* x, const float4* pos4, const BoxDesc* box) {
+  const int lane = threadIdx.x & 31;
+  const BoxDesc& bd = box[S.tk.box];
+  const float4 P = S.ip[lane];
+  for (int s = 0; s < 32; ++s) {
+    const float lo = __shfl_sync(0xffffffffu, jlo, s);     // the slot's lane holds its lower bound
+    const unsigned int bit = 1u << s;
+    if (!((mI | mJ) & bit)) continue;
+    const float r2 = pair_r2(P.x - S.x[s], P.y - S.y[s], P.z - S.z[s]);
+    if (((mI & bit) && r2 >= ilo) || ((mJ & bit) && r2 >= lo)) {
+      rc += 2;
+      const int gi = S.ig[lane];
+      mI = exact_less(gi, S.g[s], pos4[gi].w, perm, x, bd.L, 0.5 * bd.L, bd.periodic) ? (mI | bit) : (mI & ~bit);
+      mJ = exact_less(gi, S.g[s], S.H[s], perm, x, bd.L, 0.5 * bd.L, bd.periodic) ? (mJ | bit) : (mJ & ~bit);
+    }
+  }
+}
+
+// One density batch of q <= 32 staged partners (slots 0..q-1) against the warp's
+// cluster: the slots' derived values and masses by their lanes, the masks over the
+// first q rounded up to 4, then the two sweeps: own side for r < H_i (active i),
+// partner side for r < H_j (active j).  own_only: the partners are the warp's own
+// cluster (each lane leaves itself out and updates its own side only; the
+// counters count the upper triangle, since every pair appears in both rows).
+template <bool COUNT, bool PART, bool KAHAN, bool REC>
+__device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsigned int q, bool own_only,
+                                           DensAcc<KAHAN>& acc, unsigned int& cnt, const unsigned int* perm,
+                                           const double* x, const float4* __restrict__ pos4,
+                                           const BoxDesc* __restrict__ box, const float4* __restrict__ cen4,
+                                           float4* dacc, unsigned int* dcnt, Counters& C, const PairRec& R,
+                                           RecW& W) {
+  const int lane = threadIdx.x & 31;
+  const bool v = (unsigned int)lane < q;
+  __syncwarp();
+  float jm = 0.0f, jlo = -1.0f, jinvH = 0.0f;
+  if (v) {
+    jm = cen4[S.g[lane]].w;       // needed after the masks
+    const float H = S.H[lane] * S.tk.sh.w;
+    const float H2 = H * H, band = BAND_REL * H * (S.tk.win.z + H);
+    jinvH = __fdividef(1.0f, H);
+    jlo = H2 - band;
+    S.hi[lane] = H2 + band;
+  } else {
+    S.x[lane] = 1e30f;
+    S.y[lane] = 1e30f;
+    S.z[lane] = 1e30f;
+    S.hi[lane] = -1.0f;
+  }
+  const unsigned int jvalid = __ballot_sync(0xffffffffu, v);
+  const unsigned int jact = PART ? __ballot_sync(0xffffffffu, v && S.act[lane]) : jvalid;
+  __syncwarp();
+  const unsigned int allow = own_only ? jvalid & ~(1u << lane) : jvalid;
+  unsigned int mI, mJ;
+  near_masks<true>(I.p, I.hi, S.x, S.y, S.z, S.hi, (int)((q + 3u) & ~3u), mI, mJ);
+  mI &= allow;
+  mJ &= allow;
+  unsigned int rc = 0;
+  if (COUNT || (REC && !PART)) resolve_masks(S, I.lo, jlo, mI, mJ, rc, perm, x, pos4, box);
   // the pairs for the force pass: each unordered pair once (inside one cluster,
   // the partners above the lane)
-  if (rec) rec_batch(R, W, S, jvalid, (mI | mJ) & (own_only ? upper_mask(lane) : 0xffffffffu));
+  if (REC && !PART) rec_batch(R, W, S, jvalid, (mI | mJ) & (own_only ? upper_mask(lane) : 0xffffffffu));
   const unsigned int ui = I.act ? mI : 0u, uj = own_only ? 0u : (mJ & jact);
   if (COUNT) {
+    const unsigned int cmask = own_only ? upper_mask(lane) : 0xffffffffu;
     C.cand += I.valid ? __popc(allow & jvalid & cmask) : 0u;
     C.rechecks += rc;
     C.pairs += __popc((ui | (mJ & jact)) & cmask);
     C.sides += __popc(ui) + __popc(uj);
   }
-  // row sweep: own side
-  for (unsigned int m = ui; m; m &= m - 1) {
-    const int sj = __ffs(m) - 1;
-    const float4 J = S.p[sj];
-    const float dx = I.p.x - J.x, dy = I.p.y - J.y, dz = I.p.z - J.z;
-    dens_add(pair_r(fmaf(dz, dz, fmaf(dy, dy, dx * dx))), I.invH, S.a[sj].z, acc, cnt);
-  }
-  if (own_only) return;
+  S.m[lane] = jm;
+  __syncwarp();
+  dens_row(I, S, ui, acc, cnt, perm, x, pos4, box, dacc, dcnt);
   // column sweep: partner side, staged partner = lane
-  unsigned int col = transpose_bits(uj);
+  const unsigned int col = own_only ? 0u : transpose_bits(uj);
   if (col) {
-    const float4 J = S.p[lane];
-    const float jinvH = S.a[lane].x;
+    const float3 J = make_float3(S.x[lane], S.y[lane], S.z[lane]);
     DensAcc<KAHAN> pacc;
-    unsigned int pcnt = 0;
-    for (; col; col &= col - 1) {
-      const int li = __ffs(col) - 1;
-      const float4 P = S.ip[li];
-      const float dx = P.x - J.x, dy = P.y - J.y, dz = P.z - J.z;
-      dens_add(pair_r(fmaf(dz, dz, fmaf(dy, dy, dx * dx))), jinvH, P.w, pacc, pcnt);
+    unsigned int unc = 0;
+#pragma unroll 1
+    for (unsigned int m = col; m; m &= m - 1) {
+      const float4 P = S.ip[__ffs(m) - 1];
+      const float r2 = pair_r2(P.x - J.x, P.y - J.y, P.z - J.z);
+      if (r2 >= jlo) {
+        unc |= m & (0u - m);
+        continue;
+      }
+      dens_add(pair_r(r2), jinvH, P.w, pacc);
     }
-    flush_dens(S.g[lane], pacc.total(), pcnt, dacc, dcnt);
+    flush_dens(S.g[lane], pacc.total(), __popc(col & ~unc), dacc, dcnt);
+    if (unc) dens_band(S, unc, true, perm, x, pos4, box, dacc, dcnt);
   }
+  __syncwarp();
 }
 
 // What one side of a force pair needs of a particle: position, velocity, rho,
@@ -803,29 +987,6 @@ __device__ __forceinline__ void force_tile(ForceShared& S, unsigned int allow, u
   force_rounds<COUNT>(S, m, own_only, alpha, fcnt);
 }
 
-// One batch of q <= 32 staged partners (slots 0..q-1) against the warp's
-// cluster: empty the slots past the batch and run both phases over the first
-// q rounded up to 4.  own_only: the partners are the warp's own cluster (each
-// lane excludes itself and updates its own side only).
-template <bool COUNT, bool PART, bool KAHAN, bool REC>
-__device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsigned int q, bool own_only,
-                                           DensAcc<KAHAN>& acc, unsigned int& cnt, const unsigned int* perm,
-                                           const double* x, const ItemGeom& g, float4* dacc, unsigned int* dcnt,
-                                           Counters& C, const PairRec& R, RecW& W) {
-  const int lane = threadIdx.x & 31;
-  const bool v = (unsigned int)lane < q;
-  __syncwarp();
-  if (!v) S.p[lane] = make_float4(1e30f, 1e30f, 1e30f, -1.0f);
-  const unsigned int jvalid = __ballot_sync(0xffffffffu, v);
-  const unsigned int jact = PART ? __ballot_sync(0xffffffffu, v && S.act[lane]) : jvalid;
-  const float bandJ = warp_max(v ? S.a[lane].y : 0.0f);
-  __syncwarp();
-  const unsigned int allow = own_only ? jvalid & ~(1u << lane) : jvalid;
-  dens_tile<COUNT, KAHAN>(I, S, allow, jvalid, jact, bandJ, (int)((q + 3u) & ~3u), own_only,
-                   own_only ? upper_mask(lane) : 0xffffffffu, acc, cnt, perm, x, g, dacc, dcnt, C, REC && !PART, R, W);
-  __syncwarp();
-}
-
 // Not inlined: the pair and self tasks share one copy of the batch code, which
 // keeps the force kernel's instructions within the instruction cache (inlined
 // twice, instruction fetch was the largest stall of the kernel).  Everything is
@@ -887,10 +1048,6 @@ __device__ __forceinline__ float3 axis_unit_f(int a) {
   const float s = n2 == 1 ? 1.0f : (n2 == 2 ? 0.70710678118654752f : 0.57735026918962576f);
   return make_float3(dx * s, dy * s, dz * s);
 }
-
-struct Box3 {
-  float3 lo, hi;
-};
 
 // box of cluster t in the frame whose origin sits at -off from the leaf frame:
 // box + (leaf centre + off), the offset being exact (dyadic)
@@ -1020,16 +1177,204 @@ __device__ __forceinline__ LeafFrame leaf_frame(const Tiles& TL, const Tree& T, 
   return F;
 }
 
+// The geometry of one task (cluster ti of A against the clusters of B; self: B = A
+// and the clusters after the own one), in the frame of the own cluster's leaf: the
+// constants go to shared memory.  A final self interaction's cell is a leaf, so
+// that both kinds use the leaf's frame.
+__device__ __forceinline__ void task_geom(TaskShared& K, bool self, int item, unsigned int ti, const Lists& Lq,
+                                          const Tree& T, const Tiles& TL, const BoxDesc* box) {
+  const int A = self ? Lq.self_a[item] : Lq.pair_a[item];
+  const int B = self ? A : Lq.pair_b[item];
+  const int ax = self ? 0 : Lq.pair_axis[item];
+  ItemGeom g = item_geom(T, box, A, ax);
+  if (self) g.offB = make_float3(0.f, 0.f, 0.f);
+  const float4 cA = T.cen[A], cB = T.cen[B], cl = TL.cen[ti];
+  const float3 d = make_float3(cl.x - cA.x, cl.y - cA.y, cl.z - cA.z);   // the leaf centre in A's frame, exact
+  const float4 blo = TL.lo[ti], bhi = TL.hi[ti];
+  const Box3 bil{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)};
+  const float HmB = T.hmax[B] * g.invL, Hi = blo.w * g.invL;
+  const float slack = g.e * 1.52587890625e-05f + g.es + 1e-6f * fmaxf(HmB, T.hmax[A] * g.invL);   // 2^-16 e
+  const unsigned int t0 = T.tile0[B], nt = T.ntile[B];
+  unsigned int sb = SORT_NONE;
+  if (!self) {
+    const unsigned int sbB = T.sortbase[B];
+    if (sbB != SORT_NONE) sb = sbB + (unsigned int)__popc(T.axes[B] & ((1u << ax) - 1u)) * nt;
+  }
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    K.blo = make_float4(blo.x, blo.y, blo.z, Hi);
+    K.bhi = make_float4(bhi.x, bhi.y, bhi.z, slack);
+    K.sh = make_float4((g.offB.x - cB.x) - d.x, (g.offB.y - cB.y) - d.y, (g.offB.z - cB.z) - d.z, g.invL);
+    // sort keys are the projections at the build; a cluster's projection has
+    // since moved by at most the drift
+    K.win = make_float4(g.offBp - g.drift - box_rhi(box_shift(bil, d), axis_unit_f(ax)), HmB, g.eb, Hi);
+    K.sb = sb;
+    K.ntj = self ? t0 + nt - (ti + 1u) : nt;
+    K.tb0 = self ? ti + 1u : t0;
+    K.box = T.box[A];
+  }
+  __syncwarp();
+}
+
+// Lane-parallel scan of the partner cell's cluster list from entry e0 on: the
+// clusters in reach (sorted window, then box distance) as a ballot, with their size,
+// first particle and exact frame offset in K.cn, K.co.  e0 advances past the
+// entries scanned, to the end of the list once the sorted window has passed every
+// cluster.  PART: the clusters that hold neighbours of the particles that iterate
+// (box blo, bhi), and those that iterate near any particle of the own cluster (all:
+// every particle iterates, the first test covers the second).
+template <bool PART>
+__device__ __forceinline__ unsigned int scan_clusters(TaskShared& K, const Tiles& TL,
+                                                      const float* __restrict__ sort_r,
+                                                      const unsigned int* __restrict__ sort_i, unsigned int& e0,
+                                                      bool any, bool all) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int sb = K.sb, ntj = K.ntj, e = e0 + lane;
+  const bool sorted = sb != SORT_NONE;
+  const float4 win = K.win;
+  const float slack = K.bhi.w;
+  if (sorted && sort_r[sb + e0] + win.x > fmaxf(win.w, win.y) + slack) {
+    e0 = ntj;          // the sorted list only moves further away
+    return 0u;
+  }
+  e0 += 32;
+  bool pass = false;
+  if (e < ntj) {
+    const unsigned int t = sorted ? sort_i[sb + e] : K.tb0 + e;
+    const float4 lo = TL.lo[t], sh = K.sh;
+    const float Hj = lo.w * sh.w;
+    if (!sorted || sort_r[sb + e] + win.x <= fmaxf(win.w, Hj) + slack) {
+      const float4 lc = TL.cen[t], hi = TL.hi[t];
+      const float3 o = make_float3(lc.x + sh.x, lc.y + sh.y, lc.z + sh.z);
+      const Box3 bj{make_float3(lo.x + o.x, lo.y + o.y, lo.z + o.z), make_float3(hi.x + o.x, hi.y + o.y, hi.z + o.z)};
+      const float4 blo = K.blo, bhi = K.bhi;
+      const Box3 b{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)};
+      pass = (!PART || any) && box_near(b, bj, fmaxf(blo.w, Hj) + slack);
+      if (PART && !pass && !all && TL.active[t]) {
+        const float4 clo = K.clo, chi = K.chi;
+        pass = box_near(Box3{make_float3(clo.x, clo.y, clo.z), make_float3(chi.x, chi.y, chi.z)}, bj, Hj + slack);
+      }
+      if (pass) {
+        K.co[lane] = make_float4(o.x, o.y, o.z, __uint_as_float(TL.start[t]));
+        K.cn[lane] = TL.n[t];
+      }
+    }
+  }
+  const unsigned int mask = __ballot_sync(0xffffffffu, pass);
+  __syncwarp();
+  return mask;
+}
+
+// One density task: cluster ti of cell A against the clusters of cell B, or (self)
+// against itself and the later clusters of its cell.  One copy of the code serves
+// both kinds, with one copy of the batch.
+template <bool COUNT, bool PART, bool KAHAN, bool REC>
+__device__ __forceinline__ void density_task(bool self, int item, unsigned int ti, const Lists& Lq, const Tree& T,
+    const Tiles& TL, const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
+    const float4* __restrict__ cen4, const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
+    const unsigned char* __restrict__ act, const unsigned int* __restrict__ perm, const double* __restrict__ x,
+    float4* dacc, unsigned int* dcnt, DensShared& S, Counters& C, const PairRec& R, RecW& W) {
+  const int lane = threadIdx.x & 31;
+  TaskShared& K = S.tk;
+  task_geom(K, self, item, ti, Lq, T, TL, box);
+  if (REC) rec_task_begin(S, self ? Lq.s_toff[item] + (ti - T.tile0[Lq.self_a[item]])
+                                  : Lq.p_toff[item] + (ti - T.tile0[Lq.pair_a[item]]));
+  const unsigned int ni = TL.n[ti], own0 = TL.start[ti];
+  const unsigned char* actp = PART ? act : nullptr;
+  const DensI I = load_dens((unsigned int)lane < ni, own0 + lane, pos4, cen4, actp, K.sh.w, K.win.z);
+  S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
+  S.ig[lane] = I.g;
+  bool any = true, all = true;
+  if (PART) {
+    const float4 blo = K.blo, bhi = K.bhi;
+    const ActiveBox AB = active_box(I, Box3{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)}, blo.w);
+    any = AB.any;
+    all = AB.all;
+    __syncwarp();
+    if (lane == 0) {
+      K.clo = blo;
+      K.chi = bhi;
+      K.blo = make_float4(AB.b.lo.x, AB.b.lo.y, AB.b.lo.z, AB.H);
+      K.bhi = make_float4(AB.b.hi.x, AB.b.hi.y, AB.b.hi.z, bhi.w);
+    }
+    __syncwarp();
+  }
+  DensAcc<KAHAN> acc;
+  unsigned int cnt = 0, q = 0;
+  bool own_only = self;      // inside the cluster itself first
+  if (self) {
+    if (I.valid) dens_put(S, lane, I.p, I.Hphys, own0 + lane, I.act);
+    q = ni;
+  }
+  // mask: candidates of the scan; k: the one whose particles nr holds (-1: none),
+  // loaded one candidate ahead, so that the load overlaps the work on the one before
+  unsigned int e0 = 0, mask = 0;
+  int k = -1;
+  float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (;;) {
+    if (k < 0) {
+      while (!mask && e0 < K.ntj) mask = scan_clusters<PART>(K, TL, sort_r, sort_i, e0, any, all);
+      if (mask) {
+        k = __ffs(mask) - 1;
+        mask &= mask - 1;
+        if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
+      }
+    }
+    const bool last = k < 0;
+    unsigned int bal = 0, gj = 0;
+    float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool pass = false, aj = true;
+    if (!last) {
+      const float4 o = K.co[k];
+      const bool vj = (unsigned int)lane < K.cn[k];
+      gj = __float_as_uint(o.w) + lane;
+      pj = make_float4(nr.x + o.x, nr.y + o.y, nr.z + o.z, nr.w);
+      if (PART) aj = vj && actp[gj] != 0;
+      k = -1;
+      if (mask) {
+        k = __ffs(mask) - 1;
+        mask &= mask - 1;
+        if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
+      }
+      // stage only the partners within reach: of the particles that iterate (own
+      // side), or, when the partner iterates, of any particle of the cluster
+      const float4 blo = K.blo, bhi = K.bhi;
+      const float Hj = pj.w * K.sh.w;
+      const float3 p3 = make_float3(pj.x, pj.y, pj.z);
+      pass = vj && (!PART || any) &&
+             near_box(p3, Box3{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)},
+                      fmaxf(blo.w, Hj) + bhi.w);
+      if (PART && !pass && !all && aj) {
+        const float4 clo = K.clo, chi = K.chi;
+        pass = near_box(p3, Box3{make_float3(clo.x, clo.y, clo.z), make_float3(chi.x, chi.y, chi.z)}, Hj + bhi.w);
+      }
+      bal = __ballot_sync(0xffffffffu, pass);
+    }
+    if (own_only || last || q + __popc(bal) > 32u) {
+      if (q)
+        dens_batch<COUNT, PART, KAHAN, REC>(I, S, q, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt, C, R,
+                                            W);
+      q = 0;
+      own_only = false;
+    }
+    if (last) break;
+    if (pass)
+      dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), make_float3(pj.x, pj.y, pj.z), pj.w, gj, aj);
+    q += __popc(bal);
+  }
+  flush_dens(I.g, acc.total(), cnt, dacc, dcnt);
+  if (REC) rec_task_end(self ? R.stask : R.ptask, S);
+}
+
 // Lane-parallel scan of B's sorted cluster list for the i cluster (box bi,
 // largest support Hi): returns in *jt, *jn, *js the lane's candidate cluster,
 // its size and first particle, and a ballot of the lanes whose cluster is in
 // reach (sorted window, then box distance).
 // *stop is set when the sorted window has passed every cluster of B.
-template <bool DENS>
-__device__ __forceinline__ unsigned int scan_clusters(const PairSetup& P, const Tree& T, const Tiles& TL,
+__device__ __forceinline__ unsigned int scan_clusters_force(const PairSetup& P, const Tree& T, const Tiles& TL,
                                                       const float* __restrict__ sort_r,
                                                       const unsigned int* __restrict__ sort_i, unsigned int e0,
-                                                      const Box3& bi, float rhi_i, float Hi, const ActiveBox& A,
+                                                      const Box3& bi, float rhi_i, float Hi,
                                                       unsigned int* jt, unsigned int* jn, unsigned int* js,
                                                       bool* stop) {
   const int lane = threadIdx.x & 31;
@@ -1053,154 +1398,13 @@ __device__ __forceinline__ unsigned int scan_clusters(const PairSetup& P, const 
     const bool window = !sorted || sort_r[P.sb + e] + P.g.offBp - P.g.drift - rhi_i <= reach;
     if (window) {
       const Box3 bj = tile_box3(TL, T, t, P.tshB);
-      if (DENS) {
-        // the neighbours of the particles that iterate, and the clusters that
-        // iterate near any particle of this one
-        // (with every particle iterating, the first test covers the second)
-        pass = (A.any && box_near(A.b, bj, fmaxf(A.H, Hj) + P.slack)) ||
-               (!A.all && TL.active[t] && box_near(bi, bj, Hj + P.slack));
-      } else {
-        pass = box_near(bi, bj, reach);
-      }
+      pass = box_near(bi, bj, reach);
     }
   }
   *jt = t;
   *jn = pass ? TL.n[t] : 0u;
   *js = pass ? TL.start[t] : 0u;
   return __ballot_sync(0xffffffffu, pass);
-}
-
-// One pair task: cluster ti of cell A against the sorted clusters of cell B.
-template <bool COUNT, bool PART, bool KAHAN, bool REC>
-__device__ __forceinline__ void density_pair_task(int item, unsigned int ti, const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box,
-    const float4* __restrict__ pos4, const float4* __restrict__ cen4, const float* __restrict__ sort_r,
-    const unsigned int* __restrict__ sort_i, const unsigned char* __restrict__ act,
-    const unsigned int* __restrict__ perm, const double* __restrict__ x, float4* dacc, unsigned int* dcnt, DensShared& S,
-    Counters& C, const PairRec& R, RecW& W) {
-  const int lane = threadIdx.x & 31;
-  const PairSetup P = pair_setup(Lq, T, box, item);
-  if (REC) rec_task_begin(S, Lq.p_toff[item] + (ti - T.tile0[P.A]));
-  const LeafFrame F = leaf_frame(TL, T, ti, P);
-  const Box3 bi = tile_box3(TL, T, ti, P.tshA);          // the cluster in A's frame (the sorted sweep)
-  const Box3 bil = tile_box3(TL, T, ti, F.sh_own);       // ... and in its leaf's frame (the particles)
-  const float Hi = TL.lo[ti].w * P.g.invL;
-  const float rhi_i = box_rhi(bi, P.u);
-  const unsigned int ni = TL.n[ti];
-  const bool vi = (unsigned int)lane < ni;
-  const unsigned char* actp = PART ? act : nullptr;
-  const DensI I = load_dens(vi, TL.start[ti] + lane, F.sh_own, pos4, cen4, actp, P.g.invL, P.g.eb);
-  dens_stage_own(S, lane, I);
-  const ActiveBox AB = PART ? active_box(I, bil, Hi) : ActiveBox{bil, Hi, true, true};
-  const ActiveBox ABc{box_shift(AB.b, F.d), AB.H, AB.any, AB.all};   // in A's frame
-  DensAcc<KAHAN> acc;
-  unsigned int cnt = 0, q = 0;
-  for (unsigned int e0 = 0; e0 < P.ntj; e0 += 32) {
-    unsigned int jt, jn, js;
-    bool stop;
-    unsigned int mask =
-        scan_clusters<true>(P, T, TL, sort_r, sort_i, e0, bi, rhi_i, Hi, ABc, &jt, &jn, &js, &stop);
-    if (stop) break;
-    // the loads of the next candidate cluster are issued before the current
-    // one is tested, so that their latency overlaps that work
-    bool nv = false;
-    unsigned int ng = 0;
-    DensRaw nr;
-    if (mask) {
-      const int k = __ffs(mask) - 1;
-      nv = (unsigned int)lane < __shfl_sync(0xffffffffu, jn, k);
-      ng = __shfl_sync(0xffffffffu, js, k) + lane;
-      nr = fetch_dens(nv, ng, pos4, cen4, actp);
-    }
-    while (mask) {
-      mask &= mask - 1;
-      const bool vj = nv;
-      const unsigned int gj = ng;
-      const DensRaw cr = nr;
-      if (mask) {
-        const int k = __ffs(mask) - 1;
-        nv = (unsigned int)lane < __shfl_sync(0xffffffffu, jn, k);
-        ng = __shfl_sync(0xffffffffu, js, k) + lane;
-        nr = fetch_dens(nv, ng, pos4, cen4, actp);
-      }
-      const DensI J = make_dens(vj, gj, cr, F.sh_part, P.g.invL, P.g.eb);
-      // stage only the partners within reach: of the particles that iterate (own
-      // side), or, when the partner iterates, of any particle of the cluster
-      const bool pass = vj && ((AB.any && near_box(J.p, AB.b, fmaxf(AB.H, J.H) + P.slack)) ||
-                               (!AB.all && J.act && near_box(J.p, bil, J.H + P.slack)));
-      const unsigned int bal = __ballot_sync(0xffffffffu, pass);
-      const unsigned int np = __popc(bal);
-      if (q + np > 32u) {
-        dens_batch<COUNT, PART, KAHAN, REC>(I, S, q, false, acc, cnt, perm, x, P.g, dacc, dcnt, C, R, W);
-        q = 0;
-      }
-      if (pass) dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), J);
-      q += np;
-    }
-  }
-  if (q) dens_batch<COUNT, PART, KAHAN, REC>(I, S, q, false, acc, cnt, perm, x, P.g, dacc, dcnt, C, R, W);
-  flush_dens(I.g, acc.total(), cnt, dacc, dcnt);
-  if (REC) rec_task_end(R.ptask, S);
-}
-
-// One self task: cluster ti against itself and the later clusters of its cell.
-template <bool COUNT, bool PART, bool KAHAN, bool REC>
-__device__ __forceinline__ void density_self_task(int item, unsigned int ti, const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box,
-    const float4* __restrict__ pos4, const float4* __restrict__ cen4, const float* __restrict__ sort_r,
-    const unsigned int* __restrict__ sort_i, const unsigned char* __restrict__ act,
-    const unsigned int* __restrict__ perm, const double* __restrict__ x, float4* dacc, unsigned int* dcnt, DensShared& S,
-    Counters& C, const PairRec& R, RecW& W) {
-  const int lane = threadIdx.x & 31;
-  const int A = Lq.self_a[item];
-  if (REC) rec_task_begin(S, Lq.s_toff[item] + (ti - T.tile0[A]));
-  const ItemGeom g = item_geom(T, box, A, 0);
-  const float4 cA = T.cen[A];
-  const float3 sh = make_float3(-cA.x, -cA.y, -cA.z);
-  const float slack = g.e * 1.52587890625e-05f + g.es + 1e-6f * T.hmax[A] * g.invL;
-  const unsigned int t0 = T.tile0[A], nt = T.ntile[A];
-  const Box3 bi = tile_box3(TL, T, ti, sh);
-  const float Hi = TL.lo[ti].w * g.invL;
-  const bool vi = (unsigned int)lane < TL.n[ti];
-  const unsigned char* actp = PART ? act : nullptr;
-  const DensI I = load_dens(vi, TL.start[ti] + lane, sh, pos4, cen4, actp, g.invL, g.eb);
-  dens_stage_own(S, lane, I);
-  const ActiveBox AB = PART ? active_box(I, bi, Hi) : ActiveBox{bi, Hi, true, true};
-  DensAcc<KAHAN> acc;
-  unsigned int cnt = 0, q = 0;
-  // inside the cluster itself each unordered pair once: partners above the lane
-  if (vi) dens_put(S, lane, I);
-  dens_batch<COUNT, PART, KAHAN, REC>(I, S, TL.n[ti], true, acc, cnt, perm, x, g, dacc, dcnt, C, R, W);
-  // the later clusters of the cell, 32 box tests at a time
-  for (unsigned int b0 = ti + 1; b0 < t0 + nt; b0 += 32) {
-    const unsigned int tl = b0 + lane;
-    bool ok = false;
-    if (tl < t0 + nt) {
-      const Box3 bj = tile_box3(TL, T, tl, sh);
-      const float Hj = TL.lo[tl].w * g.invL;
-      ok = (AB.any && box_near(AB.b, bj, fmaxf(AB.H, Hj) + slack)) ||
-           (!AB.all && TL.active[tl] && box_near(bi, bj, Hj + slack));
-    }
-    unsigned int mask = __ballot_sync(0xffffffffu, ok);
-    while (mask) {
-      const int k = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const unsigned int tj = b0 + (unsigned int)k;
-      const bool vj = (unsigned int)lane < TL.n[tj];
-      const DensI J = load_dens(vj, TL.start[tj] + lane, sh, pos4, cen4, actp, g.invL, g.eb);
-      const bool pass = vj && ((AB.any && near_box(J.p, AB.b, fmaxf(AB.H, J.H) + slack)) ||
-                               (!AB.all && J.act && near_box(J.p, bi, J.H + slack)));
-      const unsigned int bal = __ballot_sync(0xffffffffu, pass);
-      const unsigned int np = __popc(bal);
-      if (q + np > 32u) {
-        dens_batch<COUNT, PART, KAHAN, REC>(I, S, q, false, acc, cnt, perm, x, g, dacc, dcnt, C, R, W);
-        q = 0;
-      }
-      if (pass) dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), J);
-      q += np;
-    }
-  }
-  if (q) dens_batch<COUNT, PART, KAHAN, REC>(I, S, q, false, acc, cnt, perm, x, g, dacc, dcnt, C, R, W);
-  flush_dens(I.g, acc.total(), cnt, dacc, dcnt);
-  if (REC) rec_task_end(R.stask, S);
 }
 
 template <bool COUNT>
@@ -1224,8 +1428,7 @@ __device__ __forceinline__ void force_pair_task(int item, unsigned int ti, const
     unsigned int jt, jn, js;
     bool stop;
     unsigned int mask =
-        scan_clusters<false>(P, T, TL, sort_r, sort_i, e0, bi, rhi_i, Hi, ActiveBox{bi, Hi, true, true}, &jt, &jn, &js,
-                             &stop);
+        scan_clusters_force(P, T, TL, sort_r, sort_i, e0, bi, rhi_i, Hi, &jt, &jn, &js, &stop);
     if (stop) break;
     while (mask) {
       const int k = __ffs(mask) - 1;
@@ -1430,12 +1633,9 @@ __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_B
     for (unsigned int t = base; t < tend; ++t) {
       const uint2 lt = Lq.p_live[t];
       const int item = (int)(lt.x & 0x7fffffffu);
-      if (lt.x >> 31)
-        density_self_task<COUNT, PART, KAHAN, REC && !PART>(item, lt.y, Lq, T, TL, box, pos4, cen4, sort_r, sort_i, act,
-                                                       perm, x, dacc, dcnt, S, Cs, Rec, W);
-      else
-        density_pair_task<COUNT, PART, KAHAN, REC && !PART>(item, lt.y, Lq, T, TL, box, pos4, cen4, sort_r, sort_i, act,
-                                                       perm, x, dacc, dcnt, S, Cp, Rec, W);
+      const bool self = (lt.x >> 31) != 0u;
+      density_task<COUNT, PART, KAHAN, REC && !PART>(self, item, lt.y, Lq, T, TL, box, pos4, cen4, sort_r, sort_i, act,
+                                                     perm, x, dacc, dcnt, S, COUNT && self ? Cs : Cp, Rec, W);
     }
     if (few && lane == 0) raw = atomicAdd(task_ctr, chunk);
   }
@@ -1727,53 +1927,36 @@ __global__ void k_gather_tasks(Lists Lq, Tree T, long long npair, long long nsel
   }
 }
 
-// r < H_i over the first n staged partners (n a multiple of 4), exact: the FP32
-// test outside the guard band, FP64 inside (as pair_masks, the own radius only).
-__device__ __forceinline__ unsigned int own_mask(const DensI& I, const DensShared& S, unsigned int allow, int n,
-                                                 const unsigned int* perm, const double* x, const BoxExact g) {
-  const float iLo = I.H2 - I.band, iHi = I.H2 + I.band;
-  unsigned int m = 0, sure = 0;
-  for (int s0 = n - 4; s0 >= 0; s0 -= 4) {
-#pragma unroll
-    for (int k = 3; k >= 0; --k) {
-      const float4 J = S.p[s0 + k];
-      const float dx = I.p.x - J.x, dy = I.p.y - J.y, dz = I.p.z - J.z;
-      const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-      const unsigned int ai = __float_as_uint(r2 - iLo), bi = __float_as_uint(iHi - r2);   // sign: in / out
-      m = __funnelshift_l(ai, m, 1);
-      sure = __funnelshift_l(ai | bi, sure, 1);
-    }
-  }
-  unsigned int u = ~sure & allow;
-  while (u) {
-    const int s = __ffs(u) - 1;
-    u &= u - 1;
-    const unsigned int bit = 1u << s;
-    m = exact_less(I.g, S.g[s], I.Hphys, perm, x, g.L, g.halfL, g.periodic) ? (m | bit) : (m & ~bit);
-  }
-  return m & allow;
-}
-
 // One batch of q <= 32 staged partners, the own side only; in a self interaction
 // the particle itself (staged with its cell) is left out.
 template <bool KAHAN>
 __device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsigned int q, bool self,
-                                             DensAcc<KAHAN>& acc, unsigned int& cnt, const unsigned int* perm,
-                                             const double* x, const BoxExact g) {
+                                             const float4* __restrict__ cen4, DensAcc<KAHAN>& acc, unsigned int& cnt,
+                                             const unsigned int* perm, const double* x,
+                                             const float4* __restrict__ pos4, const BoxDesc* __restrict__ box,
+                                             float4* dacc, unsigned int* dcnt) {
   const int lane = threadIdx.x & 31;
   const bool v = (unsigned int)lane < q;
   __syncwarp();
-  if (!v) S.p[lane] = make_float4(1e30f, 1e30f, 1e30f, -1.0f);
+  float jm = 0.0f;
+  if (v) {
+    jm = cen4[S.g[lane]].w;       // needed after the mask
+  } else {
+    S.x[lane] = 1e30f;
+    S.y[lane] = 1e30f;
+    S.z[lane] = 1e30f;
+  }
   const unsigned int jvalid = __ballot_sync(0xffffffffu, v);
   __syncwarp();
-  const unsigned int m = I.valid ? own_mask(I, S, jvalid, (int)((q + 3u) & ~3u), perm, x, g) : 0u;
-  for (unsigned int b = m; b; b &= b - 1) {
-    const int sj = __ffs(b) - 1;
-    if (self && S.g[sj] == I.g) continue;
-    const float4 J = S.p[sj];
-    const float dx = I.p.x - J.x, dy = I.p.y - J.y, dz = I.p.z - J.z;
-    dens_add(pair_r(fmaf(dz, dz, fmaf(dy, dy, dx * dx))), I.invH, S.a[sj].z, acc, cnt);
-  }
+  unsigned int m, none;
+  near_masks<false>(I.p, I.hi, S.x, S.y, S.z, nullptr, (int)((q + 3u) & ~3u), m, none);
+  m &= I.valid ? jvalid : 0u;
+  S.m[lane] = jm;
+  __syncwarp();
+  if (self)
+    for (unsigned int b = m; b; b &= b - 1)
+      if (S.g[__ffs(b) - 1] == I.g) m &= ~(b & (0u - b));
+  dens_row(I, S, m, acc, cnt, perm, x, pos4, box, dacc, dcnt);
   __syncwarp();
 }
 
@@ -1811,9 +1994,13 @@ __device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tre
   const float3 shX = make_float3(offX.x - cX.x, offX.y - cX.y, offX.z - cX.z);
   const float3 d = make_float3(cl.x - cO.x, cl.y - cO.y, cl.z - cO.z);
   const float3 sh_part = make_float3(shX.x - d.x, shX.y - d.y, shX.z - d.z);
-  const float3 sh_own = make_float3(-cl.x, -cl.y, -cl.z);
   const bool vi = (unsigned int)lane < n;
-  const DensI I = load_dens(vi, vi ? pk_idx[info.x + lane] : 0u, sh_own, pos4, cen4, nullptr, g.invL, g.eb);
+  const DensI I = load_dens(vi, vi ? pk_idx[info.x + lane] : 0u, pos4, cen4, nullptr, g.invL, g.eb);
+  __syncwarp();
+  S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
+  S.ig[lane] = I.g;
+  if (lane == 0) S.tk.box = T.box[O];
+  __syncwarp();
   // the packed particles' box and largest H: the own side reaches no further
   Box3 bo;
   bo.lo = make_float3(warp_min(vi ? I.p.x : 1e30f), warp_min(vi ? I.p.y : 1e30f), warp_min(vi ? I.p.z : 1e30f));
@@ -1839,21 +2026,22 @@ __device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tre
     while (mask) {
       const int k = __ffs(mask) - 1;
       mask &= mask - 1;
-      const unsigned int tj = t0 + b0 + (unsigned int)k;
+      const unsigned int tj = t0 + b0 + (unsigned int)k, gj = TL.start[tj] + lane;
       const bool vj = (unsigned int)lane < TL.n[tj];
-      const DensI J = load_dens(vj, TL.start[tj] + lane, sh_part, pos4, cen4, nullptr, g.invL, g.eb);
-      const bool pass = vj && near_box(J.p, bo, reach);
+      const float4 c = TL.cen[tj], r = vj ? pos4[gj] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float3 pj = make_float3(r.x + (c.x + sh_part.x), r.y + (c.y + sh_part.y), r.z + (c.z + sh_part.z));
+      const bool pass = vj && near_box(pj, bo, reach);
       const unsigned int bal = __ballot_sync(0xffffffffu, pass);
       const unsigned int np = __popc(bal);
       if (q + np > 32u) {
-        gather_batch<KAHAN>(I, S, q, self, acc, cnt, perm, x, box_exact(g));
+        gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt);
         q = 0;
       }
-      if (pass) dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), J);
+      if (pass) dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), pj, r.w, gj, true);
       q += np;
     }
   }
-  if (q) gather_batch<KAHAN>(I, S, q, self, acc, cnt, perm, x, box_exact(g));
+  if (q) gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt);
   flush_dens(I.g, acc.total(), cnt, dacc, dcnt);
 }
 
