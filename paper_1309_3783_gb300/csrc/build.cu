@@ -684,6 +684,7 @@ __device__ __forceinline__ void tree_node_finish(Tree& T, int id, int d, const B
     T.child[id] = (sp && fits) ? c0 : -1;
     T.nchild[id] = (sp && fits) ? nch : 0;
     T.axes[id] = 0;
+    T.pmask[id] = 0;
     // limit the top grid sets on every particle: H < edge_k - margin
     T.hlim[id] = (T.parent[id] < 0) ? __dsub_rn(ldexp(bd.L, -d), bd.margin) : 1e300;
     unsigned int cx, cy, cz;
@@ -1237,14 +1238,36 @@ __global__ void k_cell_tiles(Tree T, int nnodes, const unsigned int* __restrict_
 // Section II-C keeps, per cell, the particles sorted along each of the 13
 // cell-pair axes.  Here the sorted entries are the cell's clusters, keyed by the
 // lower end of the projection of their box on the axis.
+// Beside the axes, every cell A notes the axes of its pairs (A, B, axis): a cell has
+// at most one pair per axis with itself first.  k_sort_alloc hands out their storage
+// and k_pair_csr fills it, in the order of the axes, so that a unit of work takes its
+// partners in the same order every time.
 __global__ void k_mark_axes(Lists Lq, int cap_pair, Tree T) {
   pdl_wait();
   const int n = min(Lq.counts[1], cap_pair);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const unsigned int bit = 1u << Lq.pair_axis[i];
-    atomicOr(&T.axes[Lq.pair_a[i]], bit);
+    const int A = Lq.pair_a[i];
+    atomicOr(&T.axes[A], bit);
     atomicOr(&T.axes[Lq.pair_b[i]], bit);
+    atomicOr(&T.pmask[A], bit);
   }
+}
+
+// The pairs by their first cell, and the number of (pair, cluster of the first cell)
+// tasks, which bounds the gathered passes' task list.
+__global__ void k_pair_csr(Lists Lq, int cap_pair, Tree T) {
+  pdl_wait();
+  const int n = min(Lq.counts[1], cap_pair);
+  unsigned int tasks = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int A = Lq.pair_a[i];
+    const int ax = Lq.pair_axis[i];
+    Lq.csr[T.pstart[A] + (unsigned int)__popc(T.pmask[A] & ((1u << ax) - 1u))] = make_uint2((unsigned int)Lq.pair_b[i], (unsigned int)ax);
+    tasks += T.ntile[A];
+  }
+  tasks = __reduce_add_sync(0xffffffffu, tasks);
+  if ((threadIdx.x & 31) == 0 && tasks) atomicAdd(&Lq.counts[6], (int)tasks);
 }
 
 // Storage for the sorted lists: every (cell, needed axis) gets ntile entries.
@@ -1265,6 +1288,8 @@ __global__ void k_sort_alloc(Tree T, int nnodes, Lists Lq, int* __restrict__ big
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nnodes; id += gridDim.x * blockDim.x) {
     const unsigned int ax = T.axes[id];
     if (!ax) continue;
+    const unsigned int npr = (unsigned int)__popc(T.pmask[id]);
+    if (npr) T.pstart[id] = (unsigned int)atomicAdd(&Lq.counts[8], (int)npr);
     const unsigned int c = T.ntile[id];
     if (c <= 32u) {
       T.sortbase[id] = SORT_NONE;

@@ -40,6 +40,7 @@ __global__ void k_particle_limits(long long, Tree, const unsigned int*, float*);
 __global__ void k_shift(long long, int, const unsigned long long*, const unsigned int*, const unsigned int*, Tree,
                         const BoxDesc*, const double*, const float*, const float*, float4*, float4*);
 __global__ void k_mark_axes(Lists, int, Tree);
+__global__ void k_pair_csr(Lists, int, Tree);
 __global__ void k_sort_alloc(Tree, int, Lists, int*, int*, unsigned int*, unsigned long long*, int, uint4*,
                              unsigned int*, unsigned int, unsigned int, unsigned int*);
 __global__ void k_sort_small(const uint4*, const unsigned int*, Tree, Tiles, float*, unsigned int*);
@@ -81,6 +82,7 @@ void launch_set_active(Engine& E);
 void launch_mark_active_cells(Engine& E);
 void launch_count_unconverged(Engine& E, int* out);
 void launch_task_offsets(Engine& E);
+void launch_unit_list(Engine& E);
 void launch_task_items(Engine& E);
 void launch_bracket_reset(Engine& E);
 void launch_reduce(Engine& E);
@@ -384,6 +386,7 @@ sph_status Engine::ensure_particle_capacity() {
   CK(err_all.reserve(4));
   CK(pc.reserve(16));
   CK(task_ctr.reserve(4));
+  CK(n_units.reserve(1));
   CK(pk_cnt.reserve(n + 1));
   CK(pk_v.reserve(n + 1));
   CK(pk_idx.reserve(n));
@@ -412,6 +415,8 @@ sph_status Engine::ensure_tree_capacity(int nodes) {
   CK(t_nsmall.reserve(n));
   CK(t_axes.reserve(n));
   CK(t_sortbase.reserve(n));
+  CK(t_pmask.reserve(n));
+  CK(t_pstart.reserve(n));
   CK(t_key.reserve(n));
   CK(t_level.reserve(n));
   CK(t_box.reserve(n));
@@ -446,6 +451,8 @@ sph_status Engine::ensure_tree_capacity(int nodes) {
   T.cen = t_cen.p;
   T.axes = t_axes.p;
   T.sortbase = t_sortbase.p;
+  T.pmask = t_pmask.p;
+  T.pstart = t_pstart.p;
   T.active = t_active.p;
   T.changed = t_changed.p;
   T.alo = t_alo.p;
@@ -471,6 +478,7 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
     CK(l_pb.reserve(pairs));
     CK(l_pax.reserve(pairs));
     CK(l_ptoff.reserve(pairs + 1));
+    CK(l_csr.reserve(pairs));
   }
   CK(scan_tmp.reserve((size_t)std::max(cap_pair, cap_self) / 2048 + 64));
   if (queue > cap_queue || !q_kind[0].p) {
@@ -482,7 +490,7 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
       CK(q_ax[k].reserve(queue));
     }
   }
-  CK(l_counts.reserve(8));
+  CK(l_counts.reserve(12));
   Lq.self_a = l_self.p;
   Lq.pair_a = l_pa.p;
   Lq.pair_b = l_pb.p;
@@ -494,6 +502,7 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
     Lq.q_axis[k] = q_ax[k].p;
   }
   Lq.p_toff = l_ptoff.p;
+  Lq.csr = l_csr.p;
   Lq.s_toff = l_stoff.p;
   Lq.counts = l_counts.p;
   return SPH_OK;
@@ -659,7 +668,7 @@ sph_status Engine::build_once(bool* retry) {
   CK(cudaEventRecord(ev_fork, st));
   CK(cudaStreamWaitEvent(st_side, ev_fork, 0));
   ev = prof_begin(PH_LISTS, &l0);
-  CK(cudaMemsetAsync(l_counts.p, 0, 8 * sizeof(int), st));
+  CK(cudaMemsetAsync(l_counts.p, 0, 12 * sizeof(int), st));
   launch_pdl(k_items_top, grid(13ll * n_top), 256, st, n_top, T, box.p, key.p, top_at.p, dcap, box_shift, Lq, cap_queue,
                                                   err_all.p); count_launch();
   for (int r = 0; r < rounds; ++r) {
@@ -712,7 +721,8 @@ sph_status Engine::build_once(bool* retry) {
   launch_pdl(k_mark_axes, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
   launch_pdl(k_sort_alloc, grid(n_nodes), 256, st, T, n_nodes, Lq, big_node.p, big_axis.p, big_off.p, big_count.p,
              cap_big, mid_seg.p, mid_count.p, 0xffffffffu, 0xffffffffu, err_all.p); count_launch();
-  launch_task_offsets(*this);
+  launch_pdl(k_pair_csr, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
+  if (prm.pair_cache) launch_task_offsets(*this);
   prof_end(PH_AXIS_SORT, ev, l0);
   CK(cudaGetLastError());
   int lc[8];
@@ -747,18 +757,25 @@ sph_status Engine::build_once(bool* retry) {
   n_entries = (unsigned int)lc[5];
   n_big = (int)bc[0];
   n_big_entries = bc[1];
-  CK(l_ptask.reserve(std::max(lc[6], 1)));
-  CK(l_stask.reserve(std::max(lc[7], 1)));
-  CK(l_plive.reserve(std::max(lc[6] + lc[7], 1)));
-  CK(g_live.reserve(l_plive.n));
-  CK(l_nlive.reserve(1));
   n_ptasks = lc[6];
-  n_stasks = lc[7];
+  n_stasks = ntl;           // the self interactions are the leaves': one task per cluster
+  CK(g_live.reserve(std::max<size_t>((size_t)(n_ptasks + n_stasks), 1)));
+  if (prm.pair_cache) {     // the passes list their tasks, for their pair records
+    CK(l_ptask.reserve(std::max<size_t>((size_t)n_ptasks, 1)));
+    CK(l_stask.reserve(std::max<size_t>((size_t)n_stasks, 1)));
+    CK(l_plive.reserve(std::max<size_t>((size_t)(n_ptasks + n_stasks), 1)));
+  }
+  CK(l_nlive.reserve(1));
   Lq.p_task = l_ptask.p;
   Lq.s_task = l_stask.p;
   Lq.p_live = l_plive.p;
   Lq.n_live = l_nlive.p;
-  launch_task_items(*this);
+  // (see k_unit_list for the bounds: about a cluster per warp of the device, and
+  // enough that the longest unit does not matter)
+  unit_list = n_tiles >= nsm * 28 && n_tiles < (long long)nsm * 28 * 512;
+  if (unit_list) CK(units.reserve((size_t)n_tiles * 2 + 65536));
+  launch_unit_list(*this);
+  if (prm.pair_cache) launch_task_items(*this);
   CK(sort_r.reserve(std::max<long long>(n_entries, 1)));
   CK(sort_i.reserve(std::max<long long>(n_entries, 1)));
   ev = prof_begin(PH_AXIS_SORT, &l0);
@@ -1483,7 +1500,7 @@ sph_status Engine::enqueue_captured_build() {
   CKB(cudaEventRecord(ev_fork, st));
   CKB(cudaStreamWaitEvent(st_side, ev_fork, 0));
   ev = prof_begin(PH_LISTS, &l0);
-  CKB(cudaMemsetAsync(l_counts.p, 0, 8 * sizeof(int), st));
+  CKB(cudaMemsetAsync(l_counts.p, 0, 12 * sizeof(int), st));
   launch_pdl(k_items_top, grid(13ll * std::min<long long>(N, cap_nodes)), 256, st, cap_nodes, T, box.p, key.p,
              top_at.p, dcap, box_shift, Lq, cap_queue, err_all.p); count_launch();
   for (int r = 0; r < rounds; ++r) {
@@ -1523,8 +1540,12 @@ sph_status Engine::enqueue_captured_build() {
   launch_pdl(k_sort_alloc, grid(cap_nodes), 256, st, T, cap_nodes, Lq, big_node.p, big_axis.p, big_off.p, big_count.p,
              cap_big, mid_seg.p, mid_count.p, (unsigned int)sort_r.n, (unsigned int)ckey.n, err_all.p);
   count_launch();
-  launch_task_offsets(*this);
-  launch_task_items(*this);
+  launch_pdl(k_pair_csr, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
+  launch_unit_list(*this);
+  if (prm.pair_cache) {
+    launch_task_offsets(*this);
+    launch_task_items(*this);
+  }
   if (prm.sort_merge)
     launch_pdl(k_sort_merge, nsm * 8, 256, st, mid_seg.p, mid_count.p, T, TL, sort_r.p, sort_i.p);
   else
@@ -1549,10 +1570,12 @@ sph_status Engine::capture_build_graph() {
   // capacities with room to grow: a count past one makes the build not hold, and
   // the host completes that step with a build of its own
   const size_t cp = (size_t)(n_ptasks + n_ptasks / 4 + 1024), cs = (size_t)(n_stasks + n_stasks / 4 + 1024);
-  CK(l_ptask.reserve(cp));
-  CK(l_stask.reserve(cs));
-  CK(l_plive.reserve(cp + cs));
-  CK(g_live.reserve(l_plive.n));
+  CK(g_live.reserve(cp + cs));
+  if (prm.pair_cache) {
+    CK(l_ptask.reserve(cp));
+    CK(l_stask.reserve(cs));
+    CK(l_plive.reserve(cp + cs));
+  }
   CK(l_nlive.reserve(1));
   Lq.p_task = l_ptask.p;
   Lq.s_task = l_stask.p;
@@ -1609,7 +1632,8 @@ sph_status Engine::capture_build_graph() {
     if (s != SPH_OK) return s;
   }
   launch_pdl(k_check_build, 1, 1, st, ok, err_all.p, t_n.p, cap_nodes, l_counts.p, cap_self, cap_pair, gb_last_q,
-             (unsigned int)l_ptask.n, (unsigned int)l_stask.n, big_count.p, cap_big, gstat.p); count_launch();
+             prm.pair_cache ? (unsigned int)l_ptask.n : 0xffffffffu,
+             prm.pair_cache ? (unsigned int)l_stask.n : 0xffffffffu, big_count.p, cap_big, gstat.p); count_launch();
   CKB(cudaStreamEndCapture(st, &g1));
   gb_build = launch_count() - c0;
   cudaGraphNode_t n1, n2, n3, n4;
@@ -1798,7 +1822,7 @@ sph_status Engine::build_step_graph() {
     n_segments = lc[4];
     n_entries = (unsigned int)lc[5];
     n_ptasks = lc[6];
-    n_stasks = lc[7];
+    n_stasks = ntl;
     n_tiles = ntl;
     n_big = (int)(bcw >> 40);
     n_big_entries = (long long)(bcw & ((1ull << 40) - 1ull));

@@ -62,16 +62,9 @@ struct BoxExact {
 
 __device__ __forceinline__ BoxExact box_exact(const ItemGeom& g) { return BoxExact{g.L, g.halfL, g.periodic}; }
 
-// Tasks are handed out in chunks from a counter in device memory (zeroed before
-// every launch): the cost of a task varies by orders of magnitude, so a static
-// split leaves most SMs idle behind the longest ones.
-// Consecutive tasks of a list mostly share their interaction (the clusters of one
-// cell against the same partner cell), so a warp that takes several in a row finds
-// the partners' data in its L1: the density pass, light per pair, gains from 8
-// (33.5M: first pass 65.0 -> 62.7 ms); the force pass, heavy per pair, balances
-// better with 2 (8 took it from 67.9 to 69.7 ms).
-constexpr unsigned int TASK_CHUNK_DENSITY = 8;
-constexpr unsigned int TASK_CHUNK_FORCE = 2;
+// Units of work are handed out from a counter in device memory (zeroed before every
+// launch): their cost varies by orders of magnitude, so a static split leaves most
+// SMs idle behind the longest ones.
 
 // blocks per SM of the recording first density pass (5, with a few registers
 // spilled for the record state, measured faster than 4 blocks without spills), of
@@ -113,47 +106,54 @@ struct Box3 {
   float3 lo, hi;
 };
 
-// Per warp: the constants of a task and the candidate clusters of the current
-// scan.  Read back with broadcast loads where they are needed, which costs less
-// than the registers they would hold through the batches.
-struct __align__(16) TaskShared {
+// Per warp: what a unit of work (one cluster against the clusters of its cell's
+// interactions) keeps out of registers: its constants, the current group of
+// interactions, and the candidate clusters of the current scan.  Read back with
+// broadcast loads where they are needed, which costs less than the registers they
+// would hold through the batches.
+constexpr int GROUP = 14;      // interactions whose geometry is set up at once, one per lane (a leaf's self and 13 pairs)
+
+struct __align__(16) UnitShared {
   float4 blo;            // box of the own cluster's particles to find partners for (leaf frame); w: their largest H
-  float4 bhi;            // ... w: culling slack
-  float4 sh;             // frame offset of the partner cell's clusters; w: 1 / L
-  float4 win;            // x: sorted window offset (projection of the cell offset minus the drift and the own upper
-                         //   end), y: the partner cell's largest H, z: length scale of the position rounding,
-                         //   w: the own cluster's largest H
-  float4 clo, chi;       // later passes: box of the whole own cluster
-  unsigned int sb, ntj, tb0;   // the partner cell's sorted list (SORT_NONE: its clusters in their own order)
-  int box;
+  float4 bhi;            // ... w: 1 / L
+  float4 clo, chi;       // box of the whole own cluster; w of clo: its largest H
+  float4 cl;             // its leaf's centre
+  float eb;              // length scale of the position rounding: the cell edge, or 1 (L) for plain FP32 positions
+  float es, L32, drift;
+  int box, cell;         // the cell whose interactions come next (-1: none left)
+  unsigned int ti, at, idx;    // own cluster; position in the cell's list; interactions seen so far
+  unsigned int part, parts;    // the unit's share of the cluster's work
+  unsigned int gidx;           // interactions seen before the current group
+  int selfit;                  // the group's self interaction (-1: none)
+  // per interaction of the group: frame offset of the partner cell's clusters (exact) and culling slack; sorted
+  // window offset (projection of the cell offset minus the drift and the own upper end), the partner cell's
+  // largest H, its sorted list (SORT_NONE: clusters tb, tb + 1, ... in their own order) and length
+  float4 gsh[GROUP];
+  float4 gwin[GROUP];
+  unsigned int gtb[GROUP];
   float4 co[32];         // candidates: frame offset, first particle (bits)
-  unsigned int cn[32];   //   size
-  float4 jlo[32], jhi[32];     // ... box in the task's frame; w of jlo: largest H (fine candidates only)
+  unsigned char cn[32];  //   size
 };
 
-// The lane's own particle of a density task: lo and hi bound the guard band around
-// H^2 (r^2 below lo is inside, above hi outside, between them decided in FP64).
+// The lane's own particle of a density unit.
 struct DensI {
   float3 p;
-  float H, invH, lo, hi, Hphys, m;
+  float H, invH, Hphys, m;
   int g;
   bool valid, act;
 };
 
 // (in the frame of its leaf: its offset as stored)
 __device__ __forceinline__ DensI load_dens(bool valid, unsigned int gidx, const float4* pos4, const float4* cen4,
-                                           const unsigned char* act, float invL, float e) {
+                                           const unsigned char* act, float invL) {
   DensI r;
   r.valid = valid;
   if (valid) {
     const float4 p = pos4[gidx];
     r.p = make_float3(p.x, p.y, p.z);
     const float H = p.w * invL;
-    const float H2 = H * H, band = BAND_REL * H * (e + H);
     r.H = H;
     r.invH = __fdividef(1.0f, H);   // 2 ulp: enters the kernel's argument only
-    r.lo = H2 - band;
-    r.hi = H2 + band;
     r.Hphys = p.w;
     r.m = cen4[gidx].w;
     r.g = (int)gidx;
@@ -162,8 +162,6 @@ __device__ __forceinline__ DensI load_dens(bool valid, unsigned int gidx, const 
     r.p = make_float3(1e30f, 1e30f, 1e30f);
     r.H = 0.0f;
     r.invH = 0.0f;
-    r.lo = -1.0f;
-    r.hi = -1.0f;
     r.Hphys = 0.0f;
     r.m = 0.0f;
     r.g = -1;
@@ -172,9 +170,8 @@ __device__ __forceinline__ DensI load_dens(bool valid, unsigned int gidx, const 
   return r;
 }
 
-// Per warp: the staged partners, the warp's own cluster (ip), and what the task
-// keeps out of registers (tk, and one entry per candidate cluster of the current
-// scan).  The coordinates are kept apart so that the mask phase reads four slots of
+// Per warp: the staged partners, the warp's own cluster (ip), and what the unit of
+// work keeps out of registers.  The coordinates are kept apart so that the mask phase reads four slots of
 // one coordinate with one 16-byte load, as two packed FP32 pairs.  A partner is
 // staged with its position, H and index only; what follows from them is computed
 // once per batch, by the slot's lane, and its mass is loaded then.
@@ -185,8 +182,10 @@ struct __align__(16) DensShared {
   float m[32];
   int g[32];
   float4 ip[32];    // own cluster: position, m
+  float4 is[32];    //   sums over the interactions done
   int ig[32];       //   index
-  TaskShared tk;
+  UnitShared tk;
+  float4 jlo[32], jhi[32];   // the scan's fine candidates: box in the unit's frame, largest H (w of jlo)
   unsigned char act[32];
   // pair records (first pass): the current task's first batch, batch count and
   // record slot, and 0 once one of its batches was lost (lane 0 keeps them)
@@ -300,98 +299,78 @@ __device__ __forceinline__ void rec_task_end(uint2* slots, const DensShared& S) 
 }
 
 // =========================================================================== force
-struct ForceI {
-  float3 p;
-  float H, invH, H2, band, Hphys, m;
-  float3 v;
-  float rho, F, c, K4;
-  int g;
-  bool valid;
-};
-
-__device__ __forceinline__ ForceI load_force(bool valid, unsigned int gidx, float3 shift, const float4* pos4,
-                                             const float4* cen4, const float4* vel4, const float4* ghost4,
-                                             float invL, float L, float e) {
-  ForceI r;
-  r.valid = valid;
-  if (valid) {
-    const float4 p = pos4[gidx];
-    const float4 c = cen4[gidx];
-    const float4 vv = vel4[gidx];
-    const float4 gh = ghost4[gidx];
-    // the cell offsets (c + shift) are exact dyadic values: add them first, round once
-    r.p = make_float3(p.x + (c.x + shift.x), p.y + (c.y + shift.y), p.z + (c.z + shift.z));
-    const float H = p.w * invL;
-    r.H = H;
-    r.invH = gh.w * L;                // 1 / H in units of L
-    r.H2 = H * H;
-    r.band = BAND_REL * H * (e + H);
-    r.Hphys = p.w;
-    r.m = c.w;
-    r.v = make_float3(vv.x, vv.y, vv.z);
-    r.rho = gh.x;
-    r.F = gh.y;
-    r.c = gh.z;
-    const float ih = gh.w;            // 1 / H (physical), from the ghost pass
-    r.K4 = SPH_KNORM * (ih * ih) * (ih * ih);
-    r.g = (int)gidx;
-  } else {
-    r.p = make_float3(1e30f, 1e30f, 1e30f);
-    r.H = 0.f;
-    r.invH = 0.f;
-    r.H2 = -1.f;
-    r.band = 0.f;
-    r.Hphys = 0.f;
-    r.m = 0.f;
-    r.v = make_float3(0.f, 0.f, 0.f);
-    r.rho = 1.f;
-    r.F = 0.f;
-    r.c = 0.f;
-    r.K4 = 0.f;
-    r.g = -1;
-  }
-  return r;
-}
-
-// Per warp: the staged partners (p, a, v, f, g) and the warp's own cluster
-// (ip, iv, if_).  The pair list holds 768 of a batch's up to 1024 pairs, so that
-// 8 blocks of 4 warps fit an SM's shared memory (the register cap's occupancy; with
-// a full list shared memory held the kernel at 7 blocks, 3.5 % slower on the 33.5M
-// box); a batch with more pairs runs as two halves of the own lanes.
-constexpr int PLIST_CAP = 768;
-struct ForceShared {
-  float4 p[32];    // partner position, H^2
-  float4 a[32];    // partner 1/H, band, m, H (physical)
-  float4 v[32];    // partner velocity, rho
-  float4 f[32];    // partner f P / rho^2, c, K/H^4, -
-  float4 jacc[32]; // partner sums of the batch: acceleration (3), du/dt (their largest
-                   //   signal velocity in f[].w)
+// Per warp: the staged partners and the warp's own cluster.  A partner is staged
+// with its position, H and index (as in the density pass); its velocity and ghost
+// quantities are loaded once per batch by the slot's lane, before the masks, and
+// written after them.  8 blocks of 4 warps fit an SM's shared memory.
+struct __align__(16) ForceShared {
+  float x[32], y[32], z[32];
+  float hi[32], lo[32];  // H^2 +- guard band (units of L^2); hi = -1 marks an empty slot
+  float H[32];           // staged: H (physical); in a batch: 1 / H (units of L)
   int g[32];
+  float4 v[32];    // partner velocity, m; between batches the boxes of the scan's
+  float4 f[32];    // partner rho, f P / rho^2, c, K/H^4;   fine candidates (lo, hi)
+  float4 jacc[32]; // partner sums of the batch: acceleration (3), du/dt
+  float jvs[32];   //   and largest signal velocity
   float4 ip[32];   // own cluster: position, m
   float4 iv[32];   // own cluster: velocity, rho
   float4 if_[32];  // own cluster: 1/H, f P / rho^2, c, K/H^4
-  float4 ih[32];   // own cluster: H^2 (-1: no particle), band, H (physical), index (bits)
+  float ilo[32];   // own cluster: H^2 - guard band
   float4 iacc[32]; // own cluster sums over the task
   float ivs[32];
-  unsigned short plist[PLIST_CAP]; // the batch's pairs: own lane | slot << 5
+  UnitShared tk;
+  float4 cb[32];         // partner-side terms of one round, by lane
+  float cv[32];          //   signal velocities
+  unsigned short plist[32];   // the round's pairs: own lane | slot << 5
+  unsigned int own0;     // the own cluster's first particle
 };
 
-__device__ __forceinline__ void force_put(ForceShared& S, int lane, const ForceI& j) {
-  S.p[lane] = make_float4(j.p.x, j.p.y, j.p.z, j.H2);
-  S.a[lane] = make_float4(j.invH, j.band, j.m, j.Hphys);
-  S.v[lane] = make_float4(j.v.x, j.v.y, j.v.z, j.rho);
-  S.f[lane] = make_float4(j.F, j.c, j.K4, 0.f);   // w: the partner's largest v_sig of the batch
-  S.jacc[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-  S.g[lane] = j.g;
-}
-
-__device__ __forceinline__ void force_stage_own(ForceShared& S, int lane, const ForceI& i) {
-  S.ip[lane] = make_float4(i.p.x, i.p.y, i.p.z, i.m);
-  S.iv[lane] = make_float4(i.v.x, i.v.y, i.v.z, i.rho);
-  S.if_[lane] = make_float4(i.invH, i.F, i.c, i.K4);
-  S.ih[lane] = make_float4(i.valid ? i.H2 : -1.0f, i.band, i.Hphys, __int_as_float(i.g));
+// The lane's own particle (p.w: H in units of L; 1e30 and H = 0 on an empty lane).
+__device__ __forceinline__ float4 force_stage_own(ForceShared& S, int lane, bool valid, unsigned int gidx,
+                                                  const float4* pos4, const float4* cen4, const float4* vel4,
+                                                  const float4* ghost4) {
+  float4 p = make_float4(1e30f, 1e30f, 1e30f, 0.0f);
+  float4 v = make_float4(0.f, 0.f, 0.f, 1.f), f = make_float4(0.f, 0.f, 0.f, 0.f);
+  float m = 0.0f;
+  if (valid) {
+    p = pos4[gidx];
+    const float4 vv = vel4[gidx], gh = ghost4[gidx];
+    m = cen4[gidx].w;
+    const float H = p.w * S.tk.bhi.w;
+    p.w = H;
+    v = make_float4(vv.x, vv.y, vv.z, gh.x);
+    f = make_float4(gh.w * S.tk.L32, gh.y, gh.z, SPH_KNORM * (gh.w * gh.w) * (gh.w * gh.w));   // gh.w = 1 / H
+  }
+  S.ip[lane] = make_float4(p.x, p.y, p.z, m);
+  S.iv[lane] = v;
+  S.if_[lane] = f;
   S.iacc[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
   S.ivs[lane] = 0.f;
+  return p;
+}
+
+__device__ __forceinline__ void force_put(ForceShared& S, int slot, float3 p, float Hphys, unsigned int g) {
+  S.x[slot] = p.x;
+  S.y[slot] = p.y;
+  S.z[slot] = p.z;
+  S.H[slot] = Hphys;
+  S.g[slot] = (int)g;
+}
+
+// The loads of a staged partner, and what the pair rounds read of it.
+struct ForceRaw {
+  float4 v, gh;
+  float m;
+};
+
+__device__ __forceinline__ void force_derive(ForceShared& S, int lane, bool v, const ForceRaw& r) {
+  if (v) {
+    S.H[lane] = r.gh.w * S.tk.L32;                 // 1 / H in units of L
+    S.v[lane] = make_float4(r.v.x, r.v.y, r.v.z, r.m);
+    S.f[lane] = make_float4(r.gh.x, r.gh.y, r.gh.z, SPH_KNORM * (r.gh.w * r.gh.w) * (r.gh.w * r.gh.w));
+  }
+  S.jacc[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  S.jvs[lane] = 0.f;
 }
 
 __device__ __forceinline__ void flush_force(int gidx, float4 acc, float vs, float4* facc, float* fvsig) {
@@ -414,51 +393,6 @@ __device__ __forceinline__ void flush_force(int gidx, float4 acc, float vs, floa
 // own side, which keeps the lanes balanced: each pair's two sides are then
 // computed by the two lanes concerned.  Invalid lanes sit at 1e30 with
 // H^2 = -1, so they never pass a test.
-
-// Phase 1: exact bitmasks of r < H_i (mI) and r < H_j (mJ) over the first n
-// staged partners (n a multiple of 4; slots past the batch hold empty entries).
-// The FP32 test decides outside a guard band around H^2; bandJ bounds every
-// partner's band; the few uncertain bits are decided in FP64 afterwards.
-template <class SH>
-__device__ __forceinline__ void pair_masks(const float3 ip, float iH2, float iband, int ig, float iHphys,
-                                           const SH& S, float bandJ, unsigned int allow, int n,
-                                           const unsigned int* perm, const double* x, const BoxExact g,
-                                           unsigned int& mI, unsigned int& mJ, unsigned int& rc) {
-  // Per slot, r^2 against H^2 - band (sure inside) and H^2 + band (sure outside),
-  // for both radii: each test is the sign of one difference, shifted into its mask
-  // (slots taken from the last, so that slot s lands in bit s).  u: slots where
-  // either decision is not sure; both are then taken again in FP64 (the exact
-  // decision equals the FP32 one where that was sure).
-  const float iLo = iH2 - iband, iHi = iH2 + iband;
-  unsigned int sure = 0;   // slots where both decisions are sure
-  mI = 0;
-  mJ = 0;
-  for (int s0 = n - 4; s0 >= 0; s0 -= 4) {
-#pragma unroll
-    for (int k = 3; k >= 0; --k) {
-      const int s = s0 + k;
-      const float4 J = S.p[s];
-      const float dx = ip.x - J.x, dy = ip.y - J.y, dz = ip.z - J.z;
-      const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-      const unsigned int ai = __float_as_uint(r2 - iLo), bi = __float_as_uint(iHi - r2);   // sign: in / out
-      const unsigned int aj = __float_as_uint(r2 - (J.w - bandJ)), bj = __float_as_uint((J.w + bandJ) - r2);
-      mI = __funnelshift_l(ai, mI, 1);
-      mJ = __funnelshift_l(aj, mJ, 1);
-      sure = __funnelshift_l((ai | bi) & (aj | bj), sure, 1);
-    }
-  }
-  unsigned int u = ~sure & allow;
-  while (u) {
-    const int s = __ffs(u) - 1;
-    u &= u - 1;
-    rc += 2;
-    const unsigned int bit = 1u << s;
-    mI = exact_less(ig, S.g[s], iHphys, perm, x, g.L, g.halfL, g.periodic) ? (mI | bit) : (mI & ~bit);
-    mJ = exact_less(ig, S.g[s], S.a[s].w, perm, x, g.L, g.halfL, g.periodic) ? (mJ | bit) : (mJ & ~bit);
-  }
-  mI &= allow;
-  mJ &= allow;
-}
 
 // Two FP32 values in one 64-bit register, added and multiplied by one instruction
 // (rounded as the scalar ones, element by element).
@@ -633,7 +567,8 @@ __device__ __noinline__ void dens_band(const DensShared& S, unsigned int unc, bo
 
 // Own side of a density batch: the lane walks its mask of staged partners.
 template <bool KAHAN>
-__device__ __forceinline__ void dens_row(const DensI& I, const DensShared& S, unsigned int ui, DensAcc<KAHAN>& acc,
+__device__ __forceinline__ void dens_row(const DensI& I, float ilo, const DensShared& S, unsigned int ui,
+                                         DensAcc<KAHAN>& acc,
                                          unsigned int& cnt, const unsigned int* perm, const double* x,
                                          const float4* pos4, const BoxDesc* box, float4* dacc, unsigned int* dcnt) {
   unsigned int unc = 0;
@@ -641,7 +576,7 @@ __device__ __forceinline__ void dens_row(const DensI& I, const DensShared& S, un
   for (unsigned int m = ui; m; m &= m - 1) {
     const int sj = __ffs(m) - 1;
     const float r2 = pair_r2(I.p.x - S.x[sj], I.p.y - S.y[sj], I.p.z - S.z[sj]);
-    if (r2 >= I.lo) {
+    if (r2 >= ilo) {
       unc |= m & (0u - m);
       continue;
     }
@@ -692,8 +627,8 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   float jm = 0.0f, jlo = -1.0f, jinvH = 0.0f;
   if (v) {
     jm = cen4[S.g[lane]].w;       // needed after the masks
-    const float H = S.H[lane] * S.tk.sh.w;
-    const float H2 = H * H, band = BAND_REL * H * (S.tk.win.z + H);
+    const float H = S.H[lane] * S.tk.bhi.w;
+    const float H2 = H * H, band = BAND_REL * H * (S.tk.eb + H);
     jinvH = __fdividef(1.0f, H);
     jlo = H2 - band;
     S.hi[lane] = H2 + band;
@@ -708,11 +643,15 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   __syncwarp();
   const unsigned int allow = own_only ? jvalid & ~(1u << lane) : jvalid;
   unsigned int mI, mJ;
-  near_masks<true>(I.p, I.hi, S.x, S.y, S.z, S.hi, (int)((q + 3u) & ~3u), mI, mJ);
+  // the own guard band: r^2 below ilo is inside, above ihi outside, between them
+  // decided in FP64
+  const float iband = BAND_REL * I.H * (S.tk.eb + I.H), ilo = I.H * I.H - iband;
+  const float ihi = I.valid ? I.H * I.H + iband : -1.0f;
+  near_masks<true>(I.p, ihi, S.x, S.y, S.z, S.hi, (int)((q + 3u) & ~3u), mI, mJ);
   mI &= allow;
   mJ &= allow;
   unsigned int rc = 0;
-  if (COUNT || (REC && !PART)) resolve_masks(S, I.lo, jlo, mI, mJ, rc, perm, x, pos4, box);
+  if (COUNT || (REC && !PART)) resolve_masks(S, ilo, jlo, mI, mJ, rc, perm, x, pos4, box);
   // the pairs for the force pass: each unordered pair once (inside one cluster,
   // the partners above the lane)
   if (REC && !PART) rec_batch(R, W, S, jvalid, (mI | mJ) & (own_only ? upper_mask(lane) : 0xffffffffu));
@@ -726,7 +665,7 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   }
   S.m[lane] = jm;
   __syncwarp();
-  dens_row(I, S, ui, acc, cnt, perm, x, pos4, box, dacc, dcnt);
+  dens_row(I, ilo, S, ui, acc, cnt, perm, x, pos4, box, dacc, dcnt);
   // column sweep: partner side, staged partner = lane
   const unsigned int col = own_only ? 0u : transpose_bits(uj);
   if (col) {
@@ -752,7 +691,7 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
 // What one side of a force pair needs of a particle: position, velocity, rho,
 // f P / rho^2, sound speed, K/H^4, 1/H and mass.
 struct ForceSide {
-  float3 p, v;
+  float3 v;
   float rho, F, c, K4, invH, m;
 };
 
@@ -762,10 +701,8 @@ struct ForceSide {
 // is taken inside its support (q < 1) and is zero outside; at q = 1 it is zero
 // too, so the FP32 test agrees with the exact one to within the gradient's size
 // there, about 6 (1 - q)^2 for q within rounding of 1.
-__device__ __forceinline__ void force_pair_terms(const ForceSide& a, const ForceSide& b,
-                                                 float alpha, float4& ca, float4& cb, float& vsig) {
-  const float dx = a.p.x - b.p.x, dy = a.p.y - b.p.y, dz = a.p.z - b.p.z;
-  const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+__device__ __forceinline__ void force_pair_terms(const ForceSide& a, const ForceSide& b, float dx, float dy, float dz,
+                                                 float r2, float alpha, float4& ca, float4& cb, float& vsig) {
   ca = make_float4(0.f, 0.f, 0.f, 0.f);
   cb = ca;
   vsig = 0.0f;
@@ -792,12 +729,13 @@ __device__ __forceinline__ void force_pair_terms(const ForceSide& a, const Force
   cb = make_float4(kb * dx, kb * dy, kb * dz, a.m * fmaf(b.F, Wb, hv) * wv);
 }
 
-// Sums over runs of adjacent lanes with the same key; true on the first lane of
-// each run, which then holds the run's total (sum of v, max of m).
-__device__ __forceinline__ bool run_sum_max(int key, float4& v, float& m) {
+// Sums (v) and maxima (m) over runs of adjacent lanes with the same key, no run
+// longer than maxrun; true on the first lane of each run, which then holds them.
+__device__ __forceinline__ bool run_sum_max(int key, unsigned int maxrun, float4& v, float& m) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
+  for (unsigned int off = 1; off < 32; off <<= 1) {
+    if (off >= maxrun) break;            // the same in every lane
     const int k2 = __shfl_down_sync(0xffffffffu, key, off);
     const float x = __shfl_down_sync(0xffffffffu, v.x, off), y = __shfl_down_sync(0xffffffffu, v.y, off);
     const float z = __shfl_down_sync(0xffffffffu, v.z, off), w = __shfl_down_sync(0xffffffffu, v.w, off);
@@ -814,230 +752,215 @@ __device__ __forceinline__ bool run_sum_max(int key, float4& v, float& m) {
   return lane == 0 || prev != key;
 }
 
-__device__ __forceinline__ ForceSide side_of(const ForceI& I) {
-  ForceSide s;
-  s.p = I.p;
-  s.v = I.v;
-  s.rho = I.rho;
-  s.F = I.F;
-  s.c = I.c;
-  s.K4 = I.K4;
-  s.invH = I.invH;
-  s.m = I.m;
-  return s;
+// A pair inside the guard band of both radii (or in one band and outside the other
+// radius): r < max(H_i, H_j) in FP64.
+__device__ __noinline__ bool force_band(const ForceShared& S, int li, int sj, const unsigned int* __restrict__ perm,
+                                        const double* __restrict__ x, const float4* __restrict__ pos4,
+                                        const BoxDesc* __restrict__ box) {
+  const BoxDesc& bd = box[S.tk.box];
+  const int gi = (int)S.own0 + li, gj = S.g[sj];
+  const float Hm = fmaxf(pos4[gi].w, pos4[gj].w);      // r < H_i or r < H_j
+  return exact_less(gi, gj, Hm, perm, x, bd.L, 0.5 * bd.L, bd.periodic);
 }
 
-__device__ __forceinline__ ForceSide staged_side(const ForceShared& S, int k) {
-  const float4 P = S.p[k], A = S.a[k], V = S.v[k], F = S.f[k];
-  ForceSide s;
-  s.p = make_float3(P.x, P.y, P.z);
-  s.v = make_float3(V.x, V.y, V.z);
-  s.rho = V.w;
-  s.F = F.x;
-  s.c = F.y;
-  s.K4 = F.z;
-  s.invH = A.x;
-  s.m = A.z;
-  return s;
-}
-
-__device__ __forceinline__ ForceSide own_side(const ForceShared& S, int k) {
-  const float4 P = S.ip[k], V = S.iv[k], F = S.if_[k];
-  ForceSide s;
-  s.p = make_float3(P.x, P.y, P.z);
-  s.v = make_float3(V.x, V.y, V.z);
-  s.rho = V.w;
-  s.invH = F.x;
-  s.F = F.y;
-  s.c = F.z;
-  s.K4 = F.w;
-  s.m = P.w;
-  return s;
-}
+// What the rounds need besides the staged data.
+struct ForceArgs {
+  const unsigned int* perm;
+  const double* x;
+  const float4* pos4;
+  const BoxDesc* box;
+  unsigned int* fcnt;
+  float alpha;
+};
 
 // The pairs of one batch (mask m of the lane's own particle over the staged
-// slots), each evaluated once for both sides.  The pairs go into a list in shared
-// memory (own lane major), which the warp then takes 32 at a time: one pair per
-// lane, so that all lanes work however unevenly the pairs fall on the rows.  The
-// own side is summed by a segmented warp reduction (a particle's pairs are
-// adjacent in the list) into its task sums; the partner side goes to the
-// partner's batch sums (or, inside one cluster, to that particle's task sums).
-template <bool COUNT>
-__device__ __forceinline__ void force_rounds_list(ForceShared& S, unsigned int m, bool own_only, float alpha,
-                                                  unsigned int* fcnt, unsigned int cnt, unsigned int incl,
-                                                  unsigned int total);
-
-// A batch with more pairs than the list holds (rare: dense clusters): two halves
-// of the own lanes, at most 16 x 32 pairs each, out of line so that the common
-// path keeps its registers.
-template <bool COUNT>
-__device__ __noinline__ void force_rounds_halves(ForceShared& S, unsigned int m, bool own_only, float alpha,
-                                                 unsigned int* fcnt) {
+// slots), each evaluated once for both sides.  The pairs form a list, own lane
+// major, which the warp takes 32 at a time, one pair per lane, so that all lanes
+// work however unevenly the pairs fall on the rows (each lane taking its own next
+// pair while most have one left, the own side in registers, measured 5 % slower).
+// The own side is summed by a segmented warp reduction (a particle's pairs are
+// adjacent in the list); the partner side's terms go through shared memory, where
+// the first of each partner's lanes adds them up, to the partner's batch sums (or,
+// inside one cluster, to that particle's task sums).  Shared-memory float atomics
+// are slow, the more so where lanes collide.
+// EXACT: the mask holds exact decisions; else those of slots inside the guard band
+// are taken here, where r^2 is at hand.
+template <bool COUNT, bool EXACT>
+__device__ __forceinline__ void force_rounds(ForceShared& S, unsigned int m, bool own_only, const ForceArgs& A,
+                                             Counters* C) {
   const int lane = threadIdx.x & 31;
-  for (int half = 0; half < 2; ++half) {
-    const unsigned int mh = (lane >> 4) == half ? m : 0u;
-    const unsigned int ch = __popc(mh);
-    unsigned int ih = ch;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int y = __shfl_up_sync(0xffffffffu, ih, o);
-      if (lane >= o) ih += y;
-    }
-    force_rounds_list<COUNT>(S, mh, own_only, alpha, fcnt, ch, ih, __shfl_sync(0xffffffffu, ih, 31));
-  }
-}
-
-template <bool COUNT>
-__device__ __forceinline__ void force_rounds(ForceShared& S, unsigned int m, bool own_only, float alpha,
-                                             unsigned int* fcnt) {
-  const int lane = threadIdx.x & 31;
-  // list the pairs, own lane major (in two halves of the own lanes when they do
-  // not fit the list: at most 16 x 32 pairs each)
+  const unsigned int lt = (1u << lane) - 1u;
   const unsigned int cnt = __popc(m);
-  unsigned int incl = cnt;
+  unsigned int k = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
+    const unsigned int y = __shfl_up_sync(0xffffffffu, k, o);
+    if (lane >= o) k += y;
   }
-  const unsigned int total = __shfl_sync(0xffffffffu, incl, 31);
-  if (total <= (unsigned int)PLIST_CAP) force_rounds_list<COUNT>(S, m, own_only, alpha, fcnt, cnt, incl, total);
-  else force_rounds_halves<COUNT>(S, m, own_only, alpha, fcnt);
-}
-
-// The rounds over one list: cnt pairs of the lane (mask m), incl their inclusive
-// prefix over the lanes, total all of them (<= PLIST_CAP).
-template <bool COUNT>
-__device__ __forceinline__ void force_rounds_list(ForceShared& S, unsigned int m, bool own_only, float alpha,
-                                                  unsigned int* fcnt, unsigned int cnt, unsigned int incl,
-                                                  unsigned int total) {
-  const int lane = threadIdx.x & 31;
+  const unsigned int total = __shfl_sync(0xffffffffu, k, 31);
+  k -= cnt;      // the place of the lane's next pair in the list
+  // the longest run bounds the levels of the segmented sums
+  const unsigned int maxrun = __reduce_max_sync(0xffffffffu, cnt);
   __syncwarp();
-  unsigned int k = incl - cnt;
-  for (unsigned int mm = m; mm; mm &= mm - 1) {
-    const unsigned int sj = __ffs(mm) - 1;
-    S.plist[k++] = (unsigned short)(lane | (sj << 5));
-  }
-  __syncwarp();
-  const unsigned int lt = (1u << lane) - 1u;
+#pragma unroll 1
   for (unsigned int r0 = 0; r0 < total; r0 += 32) {
-    const unsigned int e = r0 + lane;
-    int li = 32 + lane;     // a key no other lane has
+    // the next 32 pairs of the list
+#pragma unroll 1
+    for (; m && k < r0 + 32u; m &= m - 1, ++k) S.plist[k - r0] = (unsigned short)(lane | ((__ffs(m) - 1) << 5));
+    __syncwarp();
+    const bool a = r0 + lane < total;
+    int li = 32 + lane, sj = 64 + lane;     // (keys no other lane has)
+    if (a) {
+      const unsigned int w = S.plist[lane];
+      li = (int)(w & 31u);
+      sj = (int)(w >> 5);
+    }
     float4 ci = make_float4(0.f, 0.f, 0.f, 0.f), cj = ci;
     float vs = 0.0f;
-    int sj = 64 + lane;     // likewise
-    if (e < total) {
-      const unsigned int w = S.plist[e];
-      li = (int)(w & 31u);
-      sj = (int)((w >> 5) & 31u);
-      force_pair_terms(own_side(S, li), staged_side(S, sj), alpha, ci, cj, vs);
-      if (COUNT) {
-        // force partners of both particles (the pair set, checked per particle)
-        atomicAdd(&fcnt[__float_as_int(S.ih[li].w)], 1u);
-        atomicAdd(&fcnt[S.g[sj]], 1u);
+    if (a) {
+      const float4 P = S.ip[li];
+      const float dx = P.x - S.x[sj], dy = P.y - S.y[sj], dz = P.z - S.z[sj];
+      const float r2 = pair_r2(dx, dy, dz);
+      bool in = true;
+      if (!EXACT && r2 >= S.ilo[li] && r2 >= S.lo[sj]) {
+        in = force_band(S, li, sj, A.perm, A.x, A.pos4, A.box);
+        if (COUNT) C->rechecks += 2;
+      }
+      if (in) {
+        const float4 V = S.iv[li], F = S.if_[li], VJ = S.v[sj], FJ = S.f[sj];
+        ForceSide sa, sb;
+        sa.v = make_float3(V.x, V.y, V.z);
+        sa.rho = V.w;
+        sa.invH = F.x;
+        sa.F = F.y;
+        sa.c = F.z;
+        sa.K4 = F.w;
+        sa.m = P.w;
+        sb.v = make_float3(VJ.x, VJ.y, VJ.z);
+        sb.m = VJ.w;
+        sb.rho = FJ.x;
+        sb.F = FJ.y;
+        sb.c = FJ.z;
+        sb.K4 = FJ.w;
+        sb.invH = S.H[sj];
+        force_pair_terms(sa, sb, dx, dy, dz, r2, A.alpha, ci, cj, vs);
+        if (COUNT) {
+          // force partners of both particles (the pair set, checked per particle)
+          atomicAdd(&A.fcnt[S.own0 + li], 1u);
+          atomicAdd(&A.fcnt[S.g[sj]], 1u);
+          C->pairs += 1;
+        }
       }
     }
-    // Shared-memory float atomics are slow, the more so where lanes collide, so
-    // the sums are written plainly in steps that touch each particle once.  Own
-    // side: one head lane per row of the round holds the row's total.
-    float vmax = vs;
-    if (run_sum_max(li, ci, vmax) && li < 32) {
+    const unsigned int peers = __match_any_sync(0xffffffffu, sj);
+    S.cb[lane] = cj;
+    S.cv[lane] = vs;
+    const float vj = vs;
+    if (run_sum_max(li, maxrun, ci, vs) && li < 32) {
+      // the head lane of each row of the round holds the row's total
       float4 t = S.iacc[li];
       t.x += ci.x; t.y += ci.y; t.z += ci.z; t.w += ci.w;
       S.iacc[li] = t;
-      atomicMax(reinterpret_cast<unsigned int*>(&S.ivs[li]), __float_as_uint(vmax));
+      S.ivs[li] = fmaxf(S.ivs[li], vs);
     }
     __syncwarp();
-    // partner side: the lanes of one partner take turns by their rank among them
-    const unsigned int peers = __match_any_sync(0xffffffffu, sj);
-    const unsigned int rank = __popc(peers & lt);
-    const unsigned int nturn = __reduce_max_sync(0xffffffffu, e < total ? rank : 0u);
-    float4* dst = own_only ? S.iacc : S.jacc;
-    for (unsigned int r = 0; r <= nturn; ++r) {
-      if (e < total && rank == r) {
-        float4 t = dst[sj];
-        t.x += cj.x; t.y += cj.y; t.z += cj.z; t.w += cj.w;
-        dst[sj] = t;
+    if (a && (peers & lt) == 0u) {
+      float4* dst = own_only ? &S.iacc[sj] : &S.jacc[sj];
+      float* dv = own_only ? &S.ivs[sj] : &S.jvs[sj];
+      float mv = fmaxf(*dv, vj);
+#pragma unroll 1
+      for (unsigned int b = peers & (peers - 1); b; b &= b - 1) {
+        const int l = __ffs(b) - 1;
+        const float4 t = S.cb[l];
+        cj.x += t.x; cj.y += t.y; cj.z += t.z; cj.w += t.w;
+        mv = fmaxf(mv, S.cv[l]);
       }
-      __syncwarp();
+      float4 t = *dst;
+      t.x += cj.x; t.y += cj.y; t.z += cj.z; t.w += cj.w;
+      *dst = t;
+      *dv = mv;
     }
-    if (e < total) atomicMax(reinterpret_cast<unsigned int*>(own_only ? &S.ivs[sj] : &S.f[sj].w), __float_as_uint(vs));
     __syncwarp();
   }
 }
 
-// Force batch: every pair with r < max(H_i, H_j) among the staged partners,
-// decided exactly (phase 1), then evaluated for both sides.
+// One force batch of q staged partners: every pair with r < max(H_i, H_j), found by
+// the mask phase and evaluated for both sides.  The partners' velocities and ghost
+// quantities are loaded before the masks and used after them (loaded with the
+// position, for every particle of a candidate cluster, they were three quarters of
+// the bytes and two fifths of them were used).
 template <bool COUNT>
-__device__ __forceinline__ void force_tile(ForceShared& S, unsigned int allow, unsigned int jvalid,
-                                           float bandJ, int n, bool own_only, unsigned int cmask,
-                                           const unsigned int* perm, const double* x, const BoxExact g,
-                                           float alpha, unsigned int* fcnt, Counters* C) {
-  // the lane's own particle, read back from the staged cluster
-  const float4 ip = S.ip[threadIdx.x & 31], ih = S.ih[threadIdx.x & 31];
-  const bool ivalid = ih.x >= 0.0f;
-  unsigned int mI, mJ, rc = 0;
-  pair_masks(make_float3(ip.x, ip.y, ip.z), ih.x, ih.y, __float_as_int(ih.w), ih.z, S, bandJ, allow, n, perm, x, g,
-             mI, mJ, rc);
-  const unsigned int m = mI | mJ;
-  if (COUNT) {
-    C->cand += ivalid ? __popc(allow & jvalid & cmask) : 0u;
-    C->rechecks += rc;
-    C->pairs += __popc(m & cmask);
-  }
-  force_rounds<COUNT>(S, m, own_only, alpha, fcnt);
-}
-
-// Not inlined: the pair and self tasks share one copy of the batch code, which
-// keeps the force kernel's instructions within the instruction cache (inlined
-// twice, instruction fetch was the largest stall of the kernel).  Everything is
-// passed by value or by pointer, so that a call stores nothing to local memory.
-template <bool COUNT>
-__device__ __noinline__ void force_batch(ForceShared& S, unsigned int q, bool own_only,
-                                            const unsigned int* perm, const double* x, const BoxExact g,
-                                            float alpha, float4* facc, float* fvsig, unsigned int* fcnt,
-                                            Counters* C) {
+__device__ __forceinline__ void force_batch(ForceShared& S, float3 ip, float iH, unsigned int q, bool own_only,
+                                            const ForceArgs& A, const float4* __restrict__ cen4,
+                                            const float4* __restrict__ vel4, const float4* __restrict__ ghost4,
+                                            float4* facc, float* fvsig, Counters* C) {
   const int lane = threadIdx.x & 31;
   const bool v = (unsigned int)lane < q;
   __syncwarp();
-  if (!v) S.p[lane] = make_float4(1e30f, 1e30f, 1e30f, -1.0f);
+  ForceRaw r;
+  if (v) {
+    const unsigned int g = (unsigned int)S.g[lane];
+    r.v = vel4[g];
+    r.gh = ghost4[g];
+    r.m = cen4[g].w;
+    const float H = S.H[lane] * S.tk.bhi.w;
+    const float H2 = H * H, band = BAND_REL * H * (S.tk.eb + H);
+    S.hi[lane] = H2 + band;
+    S.lo[lane] = H2 - band;
+  } else {
+    S.x[lane] = 1e30f;
+    S.y[lane] = 1e30f;
+    S.z[lane] = 1e30f;
+    S.hi[lane] = -1.0f;
+  }
   const unsigned int jvalid = __ballot_sync(0xffffffffu, v);
-  const float bandJ = warp_max(v ? S.a[lane].y : 0.0f);
   __syncwarp();
   // inside one cluster each unordered pair once (partners above the lane)
   const unsigned int allow = own_only ? jvalid & upper_mask(lane) : jvalid;
-  force_tile<COUNT>(S, allow, jvalid, bandJ, (int)((q + 3u) & ~3u), own_only, 0xffffffffu, perm, x, g, alpha,
-                    fcnt, C);
-  __syncwarp();
-  if (v && !own_only) flush_force(S.g[lane], S.jacc[lane], S.f[lane].w, facc, fvsig);
+  unsigned int mI, mJ;
+  const float iband = BAND_REL * iH * (S.tk.eb + iH), ihi = iH > 0.0f ? iH * iH + iband : -1.0f;
+  S.ilo[lane] = iH * iH - iband;      // (read after the masks)
+  near_masks<true>(ip, ihi, S.x, S.y, S.z, S.hi, (int)((q + 3u) & ~3u), mI, mJ);
+  const unsigned int m = (mI | mJ) & allow;
+  if (COUNT) C->cand += ihi >= 0.0f ? __popc(allow) : 0u;
+  if (!__any_sync(0xffffffffu, m != 0u)) return;
+  force_derive(S, lane, v, r);
+  force_rounds<COUNT, false>(S, m, own_only, A, C);
+  if (v && !own_only) flush_force(S.g[lane], S.jacc[lane], S.jvs[lane], facc, fvsig);
   __syncwarp();
 }
 
 // One recorded batch B of the first density pass: the staged partners are read
-// back by index (own_only: the warp's own cluster, already staged), the pairs come
-// from the recorded masks, and phase 2 runs as in force_batch.
+// back by index (own_only: the warp's own cluster), the pairs come from the recorded
+// masks, and the rounds run as in force_batch.
 template <bool COUNT>
 __device__ __noinline__ void force_replay_batch(ForceShared& S, const unsigned int* __restrict__ B, bool own_only,
-                                                float3 sh, float invL, float L32, float eb,
-                                                const float4* __restrict__ pos4, const float4* __restrict__ cen4,
-                                                const float4* __restrict__ vel4, const float4* __restrict__ ghost4,
-                                                float alpha, float4* facc, float* fvsig, unsigned int* fcnt,
-                                                Counters* C) {
+                                                const float4* __restrict__ cen4, const float4* __restrict__ vel4,
+                                                const float4* __restrict__ ghost4, const ForceArgs A, float3 sh,
+                                                float4* facc, float* fvsig, Counters* C) {
   const int lane = threadIdx.x & 31;
   const unsigned int gj = __ldcs(B + lane);     // read once: evict first
   const unsigned int m = __ldcs(B + 32 + lane);
   const bool v = gj != REC_NONE;
   __syncwarp();
-  if (!own_only) force_put(S, lane, load_force(v, gj, sh, pos4, cen4, vel4, ghost4, invL, L32, eb));
+  ForceRaw r;
+  if (v) {
+    const float4 p = A.pos4[gj], c = cen4[gj];
+    r.v = vel4[gj];
+    r.gh = ghost4[gj];
+    r.m = c.w;
+    // the cell offsets (c + sh) are exact dyadic values: add them first, round once
+    force_put(S, lane, make_float3(p.x + (c.x + sh.x), p.y + (c.y + sh.y), p.z + (c.z + sh.z)), p.w, gj);
+  }
+  force_derive(S, lane, v, r);
   __syncwarp();
   if (COUNT) {
     const unsigned int jvalid = __ballot_sync(0xffffffffu, v);
-    C->cand += S.ih[lane].x >= 0.0f ? __popc(jvalid & (own_only ? upper_mask(lane) : 0xffffffffu)) : 0u;
-    C->pairs += __popc(m);
+    C->cand += S.if_[lane].x > 0.0f ? __popc(jvalid & (own_only ? upper_mask(lane) : 0xffffffffu)) : 0u;
   }
-  force_rounds<COUNT>(S, m, own_only, alpha, fcnt);
+  force_rounds<COUNT, true>(S, m, own_only, A, C);
   __syncwarp();
-  if (v && !own_only) flush_force(S.g[lane], S.jacc[lane], S.f[lane].w, facc, fvsig);
+  if (v && !own_only) flush_force(S.g[lane], S.jacc[lane], S.jvs[lane], facc, fvsig);
   __syncwarp();
 }
 
@@ -1178,50 +1101,189 @@ __device__ __forceinline__ LeafFrame leaf_frame(const Tiles& TL, const Tree& T, 
   return F;
 }
 
-// The geometry of one task (cluster ti of A against the clusters of B; self: B = A
-// and the clusters after the own one), in the frame of the own cluster's leaf: the
-// constants go to shared memory.  A final self interaction's cell is a leaf, so
-// that both kinds use the leaf's frame.
-__device__ __forceinline__ void task_geom(TaskShared& K, bool self, int item, unsigned int ti, const Lists& Lq,
-                                          const Tree& T, const Tiles& TL, const BoxDesc* box) {
+// ------------------------------------------------------------- units of work
+// A unit is one cluster against the partner clusters of its interactions: the self
+// interaction of its leaf and the pairs (A, B, axis) of every cell A on its chain
+// (Section II-B: an interaction of a cell is one of all its particles).  The
+// geometry of up to GROUP interactions is set up at once, one per lane, and the
+// partners of all of them share the staged batches: with a task per (interaction,
+// cluster) a fifth of both passes went into setting the tasks up (2 to 3 staged
+// partners per own particle and task in a uniform box), and most batches were
+// partly filled.  Where a box has few clusters, a unit is split into parts (every
+// parts-th interaction), so that every warp has several.
+// (One unit per warp in the smallest boxes, two where a cluster per warp would leave a
+// partial wave: lattices of 25^3 and 30^3 lose 10 % with twice the parts, of 42^3 and a
+// 40k Plummer box gain 10-40 %.)
+__device__ __forceinline__ unsigned int unit_parts(unsigned int ntile) {
+  const unsigned int warps = gridDim.x * (blockDim.x >> 5);
+  const unsigned int want = 5u * ntile >= 2u * warps ? 2u * warps : warps;
+  return min(16u, max(1u, want / max(ntile, 1u)));
+}
+
+__device__ __forceinline__ void unit_begin(UnitShared& K, unsigned int ti, const Tree& T, const Tiles& TL,
+                                           const BoxDesc* __restrict__ box,
+                                           unsigned int part, unsigned int parts) {
+  const float4 blo = TL.lo[ti], bhi = TL.hi[ti], cl = TL.cen[ti];
+  const int leaf = (int)TL.leaf[ti], b = T.box[leaf];
+  const float invL = (float)box[b].invL;
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    K.blo = make_float4(blo.x, blo.y, blo.z, blo.w * invL);
+    K.bhi = make_float4(bhi.x, bhi.y, bhi.z, invL);
+    K.clo = K.blo;
+    K.chi = K.bhi;
+    K.cl = cl;
+    K.es = box[b].global32 ? 9.5367431640625e-07f : 0.0f;   // 2^-20 L: the 2^-25 rounding of both positions
+    K.L32 = (float)box[b].L;
+    K.drift = box[b].drift_u;
+    K.eb = box[b].global32 ? 1.0f : ldexpf(1.0f, -T.level[leaf]);
+    K.box = b;
+    K.cell = leaf;
+    K.ti = ti;
+    K.part = part;
+    K.parts = parts;
+    K.at = 0;
+    K.idx = 0;
+  }
+  __syncwarp();
+}
+
+// The first run of 32 clusters of an interaction's list that belongs to the unit: its
+// part of the parts takes the runs r with (interaction + r) % parts == part.
+__device__ __forceinline__ unsigned int unit_first_of(const UnitShared& K, unsigned int interaction) {
+  const unsigned int P = K.parts;
+  return P == 1u ? 0u : (K.part + P - interaction % P) % P;
+}
+__device__ __forceinline__ unsigned int unit_first(const UnitShared& K, int it) {
+  return unit_first_of(K, K.gidx + (unsigned int)it);
+}
+
+// The next group of the unit's interactions: one per lane, from the cell's list (the
+// leaf's self interaction first), then from its parent's.  Returns a ballot of the
+// lanes whose interaction has work: its partner cell lies within reach of the own
+// box and, in a later pass (PART; iact: the own cluster holds iterating particles),
+// iterates itself or meets the own cluster's.  K.cell is -1 past the last group.
+// The cell edge sets the guard band (K.eb; it grows along the chain).
+template <bool PART>
+__device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T, const uint2* __restrict__ csr,
+                                                   bool iact) {
+  const int lane = threadIdx.x & 31;
+  const int A = K.cell;
+  const unsigned int at = K.at, idx = K.idx;
+  const int d = T.level[A];
+  const bool leaf = T.child[A] < 0;
+  const unsigned int n = (unsigned int)__popc(T.pmask[A]) + (leaf ? 1u : 0u);     // a leaf's list starts with its self interaction
+  const unsigned int mine = at + lane;
+  const bool valid = lane < GROUP && mine < n;
+  bool live = false;
+  const float e = ldexpf(1.0f, -d);
+  if (valid) {
+    const bool self = leaf && mine == 0u;
+    int B = A, ax = 0;
+    if (!self) {
+      const uint2 pr = csr[T.pstart[A] + mine - (leaf ? 1u : 0u)];
+      B = (int)pr.x;
+      ax = (int)pr.y;
+    }
+    int dx, dy, dz;
+    axis_vec(ax, dx, dy, dz);
+    const float3 off = self ? make_float3(0.f, 0.f, 0.f) : make_float3(e * dx, e * dy, e * dz);   // exact
+    const float4 cA = T.cen[A], cB = T.cen[B], cl = K.cl;
+    const float3 dl = make_float3(cl.x - cA.x, cl.y - cA.y, cl.z - cA.z);   // the leaf centre in A's frame, exact
+    const float4 clo = K.clo, chi = K.chi;
+    const Box3 bil{make_float3(clo.x, clo.y, clo.z), make_float3(chi.x, chi.y, chi.z)};
+    const float invL = chi.w, HmB = T.hmax[B] * invL;
+    const float slack = e * 1.52587890625e-05f + K.es + 1e-6f * fmaxf(HmB, T.hmax[A] * invL);   // 2^-16 e
+    const unsigned int t0 = T.tile0[B], nt = T.ntile[B];
+    unsigned int sb = SORT_NONE;
+    if (!self) {
+      const unsigned int sbB = T.sortbase[B];
+      if (sbB != SORT_NONE) sb = sbB + (unsigned int)__popc(T.axes[B] & ((1u << ax) - 1u)) * nt;
+    }
+    const int n2 = dx * dx + dy * dy + dz * dz;
+    const float offBp = e * (n2 == 1 ? 1.0f : (n2 == 2 ? 1.41421356237f : 1.73205080757f));
+    // sort keys are the projections at the build; a cluster's projection has
+    // since moved by at most the drift
+    const float win = offBp - K.drift - box_rhi(box_shift(bil, dl), axis_unit_f(ax));
+    K.gsh[lane] = make_float4((off.x - cB.x) - dl.x, (off.y - cB.y) - dl.y, (off.z - cB.z) - dl.z, slack);
+    K.gwin[lane] = make_float4(win, HmB, __uint_as_float(sb), __uint_as_float(self ? t0 + nt - (K.ti + 1u) : nt));
+    K.gtb[lane] = self ? K.ti + 1u : t0;
+    // the partner cell, widened by the drift of particles kept in it since the build
+    const float h = 0.5f * e + K.drift;
+    const float3 cb = make_float3(off.x - dl.x, off.y - dl.y, off.z - dl.z);
+    live = self || box_near(bil, Box3{make_float3(cb.x - h, cb.y - h, cb.z - h), make_float3(cb.x + h, cb.y + h, cb.z + h)},
+                            fmaxf(clo.w, HmB) + slack);
+    if (PART && live && !iact) {
+      // only the partner cell's iterating particles need this cluster
+      live = T.active[B] != 0;
+      if (live && !self) {
+        Box3 ba;
+        ba.lo = make_float3(key_float(T.alo[3 * B]) + cb.x, key_float(T.alo[3 * B + 1]) + cb.y,
+                            key_float(T.alo[3 * B + 2]) + cb.z);
+        ba.hi = make_float3(key_float(T.ahi[3 * B]) + cb.x, key_float(T.ahi[3 * B + 1]) + cb.y,
+                            key_float(T.ahi[3 * B + 2]) + cb.z);
+        live = box_near(bil, ba, HmB + slack);
+      }
+    }
+  }
+  if (live && K.parts > 1u)    // the unit's share has a run of this list
+    live = 32u * unit_first_of(K, idx + lane) < __float_as_uint(K.gwin[lane].w);
+  const unsigned int bal = __ballot_sync(0xffffffffu, live);
+  const int up = T.parent[A];
+  __syncwarp();
+  if (lane == 0) {
+    const bool more = at + GROUP < n;
+    K.at = more ? at + GROUP : 0u;
+    K.idx = idx + min((unsigned int)GROUP, n - at);
+    K.cell = more ? A : up;
+    K.selfit = leaf && at == 0u ? 0 : -1;
+    K.gidx = idx;
+    if (K.es == 0.0f) K.eb = e;
+  }
+  __syncwarp();
+  return bal;
+}
+
+// One interaction as a unit's only one (a listed task, params.pair_cache).
+__device__ __forceinline__ void unit_single(UnitShared& K, bool self, int item, const Lists& Lq, const Tree& T) {
   const int A = self ? Lq.self_a[item] : Lq.pair_a[item];
-  const int B = self ? A : Lq.pair_b[item];
-  const int ax = self ? 0 : Lq.pair_axis[item];
-  ItemGeom g = item_geom(T, box, A, ax);
-  if (self) g.offB = make_float3(0.f, 0.f, 0.f);
-  const float4 cA = T.cen[A], cB = T.cen[B], cl = TL.cen[ti];
-  const float3 d = make_float3(cl.x - cA.x, cl.y - cA.y, cl.z - cA.z);   // the leaf centre in A's frame, exact
-  const float4 blo = TL.lo[ti], bhi = TL.hi[ti];
-  const Box3 bil{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)};
-  const float HmB = T.hmax[B] * g.invL, Hi = blo.w * g.invL;
-  const float slack = g.e * 1.52587890625e-05f + g.es + 1e-6f * fmaxf(HmB, T.hmax[A] * g.invL);   // 2^-16 e
+  const int B = self ? A : Lq.pair_b[item], ax = self ? 0 : Lq.pair_axis[item];
+  int dx, dy, dz;
+  axis_vec(ax, dx, dy, dz);
+  const float e = ldexpf(1.0f, -T.level[A]);
+  const float3 off = self ? make_float3(0.f, 0.f, 0.f) : make_float3(e * dx, e * dy, e * dz);
+  const float4 cA = T.cen[A], cB = T.cen[B], cl = K.cl, clo = K.clo, chi = K.chi;
+  const float3 dl = make_float3(cl.x - cA.x, cl.y - cA.y, cl.z - cA.z);
+  const Box3 bil{make_float3(clo.x, clo.y, clo.z), make_float3(chi.x, chi.y, chi.z)};
+  const float invL = chi.w, HmB = T.hmax[B] * invL;
+  const float slack = e * 1.52587890625e-05f + K.es + 1e-6f * fmaxf(HmB, T.hmax[A] * invL);
   const unsigned int t0 = T.tile0[B], nt = T.ntile[B];
   unsigned int sb = SORT_NONE;
   if (!self) {
     const unsigned int sbB = T.sortbase[B];
     if (sbB != SORT_NONE) sb = sbB + (unsigned int)__popc(T.axes[B] & ((1u << ax) - 1u)) * nt;
   }
+  const int n2 = dx * dx + dy * dy + dz * dz;
+  const float offBp = e * (n2 == 1 ? 1.0f : (n2 == 2 ? 1.41421356237f : 1.73205080757f));
   __syncwarp();
   if ((threadIdx.x & 31) == 0) {
-    K.blo = make_float4(blo.x, blo.y, blo.z, Hi);
-    K.bhi = make_float4(bhi.x, bhi.y, bhi.z, slack);
-    K.sh = make_float4((g.offB.x - cB.x) - d.x, (g.offB.y - cB.y) - d.y, (g.offB.z - cB.z) - d.z, g.invL);
-    // sort keys are the projections at the build; a cluster's projection has
-    // since moved by at most the drift
-    K.win = make_float4(g.offBp - g.drift - box_rhi(box_shift(bil, d), axis_unit_f(ax)), HmB, g.eb, Hi);
-    K.sb = sb;
-    K.ntj = self ? t0 + nt - (ti + 1u) : nt;
-    K.tb0 = self ? ti + 1u : t0;
-    K.box = T.box[A];
+    K.gsh[0] = make_float4((off.x - cB.x) - dl.x, (off.y - cB.y) - dl.y, (off.z - cB.z) - dl.z, slack);
+    K.gwin[0] = make_float4(offBp - K.drift - box_rhi(box_shift(bil, dl), axis_unit_f(ax)), HmB, __uint_as_float(sb),
+                            __uint_as_float(self ? t0 + nt - (K.ti + 1u) : nt));
+    K.gtb[0] = self ? K.ti + 1u : t0;
+    if (K.es == 0.0f) K.eb = e;
+    K.cell = -1;
+    K.gidx = 0;
+    K.selfit = self ? 0 : -1;
   }
   __syncwarp();
 }
 
-// Lane-parallel scan of the partner cell's cluster list from entry e0 on: the
-// clusters in reach (sorted window, then box distance) as a ballot, with their size,
-// first particle and exact frame offset in K.cn, K.co.  e0 advances past the
-// entries scanned, to the end of the list once the sorted window has passed every
-// cluster.  PART: the clusters that hold neighbours of the particles that iterate
+// Lane-parallel scan of the cluster list of interaction it of the group, from entry
+// e0 on: the clusters in reach (sorted window, then box distance) as a ballot, with
+// their size, first particle and exact frame offset in K.cn, K.co (entries up to nt).  e0 advances past
+// the entries scanned (and the other parts' runs), to nt once the sorted window has
+// passed every cluster.  PART: the clusters that hold neighbours of the particles that iterate
 // (box blo, bhi), and those that iterate near any particle of the own cluster (all:
 // every particle iterates, the first test covers the second).
 //
@@ -1239,30 +1301,30 @@ __device__ __forceinline__ void task_geom(TaskShared& K, bool self, int item, un
 constexpr float FINE_H = 0.7f;
 
 template <bool PART>
-__device__ __forceinline__ unsigned int scan_clusters(TaskShared& K, const Tiles& TL,
+__device__ __forceinline__ unsigned int scan_clusters(UnitShared& K, float4* jlo, float4* jhi, const Tiles& TL,
                                                       const float* __restrict__ sort_r,
-                                                      const unsigned int* __restrict__ sort_i, unsigned int& e0,
-                                                      bool any, bool all, float3 ip, float iH) {
+                                                      const unsigned int* __restrict__ sort_i, int it,
+                                                      unsigned int& e0, unsigned int nt, bool any, bool all, float3 ip,
+                                                      float iH) {
   const int lane = threadIdx.x & 31;
-  const unsigned int sb = K.sb, ntj = K.ntj, e = e0 + lane;
+  const float4 win = K.gwin[it], sh = K.gsh[it], blo = K.blo, bhi = K.bhi;
+  const unsigned int sb = __float_as_uint(win.z), e = e0 + lane;
   const bool sorted = sb != SORT_NONE;
-  const float4 win = K.win;
-  const float slack = K.bhi.w;
-  if (sorted && sort_r[sb + e0] + win.x > fmaxf(win.w, win.y) + slack) {
-    e0 = ntj;          // the sorted list only moves further away
+  const float slack = sh.w, invL = bhi.w, Hi = K.clo.w;
+  if (sorted && sort_r[sb + e0] + win.x > fmaxf(Hi, win.y) + slack) {
+    e0 = nt;           // the sorted list only moves further away
     return 0u;
   }
-  e0 += 32;
+  e0 += 32u * K.parts;
   bool pass = false, fine = false;
-  if (e < ntj) {
-    const unsigned int t = sorted ? sort_i[sb + e] : K.tb0 + e;
-    const float4 lo = TL.lo[t], sh = K.sh;
-    const float Hj = lo.w * sh.w;
-    if (!sorted || sort_r[sb + e] + win.x <= fmaxf(win.w, Hj) + slack) {
+  if (e < nt) {
+    const unsigned int t = sorted ? sort_i[sb + e] : K.gtb[it] + e;
+    const float4 lo = TL.lo[t];
+    const float Hj = lo.w * invL;
+    if (!sorted || sort_r[sb + e] + win.x <= fmaxf(Hi, Hj) + slack) {
       const float4 lc = TL.cen[t], hi = TL.hi[t];
       const float3 o = make_float3(lc.x + sh.x, lc.y + sh.y, lc.z + sh.z);
       const Box3 bj{make_float3(lo.x + o.x, lo.y + o.y, lo.z + o.z), make_float3(hi.x + o.x, hi.y + o.y, hi.z + o.z)};
-      const float4 blo = K.blo, bhi = K.bhi;
       const Box3 b{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)};
       pass = (!PART || any) && box_near(b, bj, fmaxf(blo.w, Hj) + slack);
       if (PART && !pass && !all && TL.active[t]) {
@@ -1271,11 +1333,11 @@ __device__ __forceinline__ unsigned int scan_clusters(TaskShared& K, const Tiles
       }
       if (pass) {
         K.co[lane] = make_float4(o.x, o.y, o.z, __uint_as_float(TL.start[t]));
-        K.cn[lane] = TL.n[t];
-        fine = Hj < FINE_H * win.w;
+        K.cn[lane] = (unsigned char)TL.n[t];
+        fine = Hj < FINE_H * Hi;
         if (fine) {
-          K.jlo[lane] = make_float4(bj.lo.x, bj.lo.y, bj.lo.z, Hj);
-          K.jhi[lane] = make_float4(bj.hi.x, bj.hi.y, bj.hi.z, 0.0f);
+          jlo[lane] = make_float4(bj.lo.x, bj.lo.y, bj.lo.z, Hj);
+          jhi[lane] = make_float4(bj.hi.x, bj.hi.y, bj.hi.z, 0.0f);
         }
       }
     }
@@ -1285,7 +1347,7 @@ __device__ __forceinline__ unsigned int scan_clusters(TaskShared& K, const Tiles
   __syncwarp();
   for (; todo; todo &= todo - 1) {
     const int k = __ffs(todo) - 1;
-    const float4 lo = K.jlo[k], hi = K.jhi[k];
+    const float4 lo = jlo[k], hi = jhi[k];
     const bool hit = near_box(ip, Box3{make_float3(lo.x, lo.y, lo.z), make_float3(hi.x, hi.y, hi.z)},
                               fmaxf(iH, lo.w) + slack);
     if (!__any_sync(0xffffffffu, hit)) mask &= ~(1u << k);
@@ -1293,25 +1355,58 @@ __device__ __forceinline__ unsigned int scan_clusters(TaskShared& K, const Tiles
   return mask;
 }
 
-// One density task: cluster ti of cell A against the clusters of cell B, or (self)
-// against itself and the later clusters of its cell.  One copy of the code serves
-// both kinds, with one copy of the batch.
-template <bool COUNT, bool PART, bool KAHAN, bool REC>
-__device__ __forceinline__ void density_task(bool self, int item, unsigned int ti, const Lists& Lq, const Tree& T,
-    const Tiles& TL, const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
+// ------------------------------------------------------------- walking a unit
+// Where a unit stands, the same in every lane: the interactions of the group with
+// work (live), the one whose clusters are scanned (it) from e0 to nt, the candidates
+// of the scan (mask).
+struct Walk {
+  unsigned int live = 0, e0 = 0, nt = 0, mask = 0;
+  int it = 0;
+};
+
+// The next candidates (W.mask, non-zero) of the unit; false at its end.
+template <bool PART>
+__device__ __forceinline__ bool unit_next(UnitShared& K, Walk& W, float4* jlo, float4* jhi, const Lists& Lq,
+                                          const Tree& T, const Tiles& TL, const float* __restrict__ sort_r,
+                                          const unsigned int* __restrict__ sort_i, bool any, bool all, float3 ip, float iH) {
+  while (!W.mask) {
+    if (W.e0 < W.nt) {
+      W.mask = scan_clusters<PART>(K, jlo, jhi, TL, sort_r, sort_i, W.it, W.e0, W.nt, any, all, ip, iH);
+    } else if (W.live) {
+      W.it = __ffs(W.live) - 1;
+      W.live &= W.live - 1;
+      W.nt = __float_as_uint(K.gwin[W.it].w);
+      // with parts, every parts-th run of 32 clusters, from one that depends on the interaction
+      W.e0 = 32u * unit_first(K, W.it);
+    } else if (K.cell >= 0) {
+      W.live = unit_group<PART>(K, T, Lq.csr, any);
+    } else {
+      return false;
+    }
+  }
+  return true;
+}
+
+// The density interactions of one unit (cluster ti, part of parts), or of one listed
+// task (LISTED: interaction `item` only, its pairs recorded).  One copy of the batch
+// serves the own cluster (the self interaction's first batch) and all partners.
+template <bool COUNT, bool PART, bool KAHAN, bool LISTED>
+__device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part, unsigned int parts, bool self, int item,
+    const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
     const float4* __restrict__ cen4, const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
     const unsigned char* __restrict__ act, const unsigned int* __restrict__ perm, const double* __restrict__ x,
-    float4* dacc, unsigned int* dcnt, DensShared& S, Counters& C, const PairRec& R, RecW& W) {
+    float4* dacc, unsigned int* dcnt, DensShared& S, Counters& Cp, Counters& Cs, const PairRec& R, RecW& W) {
   const int lane = threadIdx.x & 31;
-  TaskShared& K = S.tk;
-  task_geom(K, self, item, ti, Lq, T, TL, box);
-  if (REC) rec_task_begin(S, self ? Lq.s_toff[item] + (ti - T.tile0[Lq.self_a[item]])
-                                  : Lq.p_toff[item] + (ti - T.tile0[Lq.pair_a[item]]));
+  UnitShared& K = S.tk;
+  unit_begin(K, ti, T, TL, box, part, parts);
+  if (LISTED) {
+    rec_task_begin(S, self ? Lq.s_toff[item] + (ti - T.tile0[Lq.self_a[item]])
+                           : Lq.p_toff[item] + (ti - T.tile0[Lq.pair_a[item]]));
+    unit_single(K, self, item, Lq, T);
+  }
   const unsigned int ni = TL.n[ti], own0 = TL.start[ti];
   const unsigned char* actp = PART ? act : nullptr;
-  const DensI I = load_dens((unsigned int)lane < ni, own0 + lane, pos4, cen4, actp, K.sh.w, K.win.z);
-  S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
-  S.ig[lane] = I.g;
+  DensI I = load_dens((unsigned int)lane < ni, own0 + lane, pos4, cen4, actp, K.bhi.w);
   bool any = true, all = true;
   if (PART) {
     const float4 blo = K.blo, bhi = K.bhi;
@@ -1320,34 +1415,36 @@ __device__ __forceinline__ void density_task(bool self, int item, unsigned int t
     all = AB.all;
     __syncwarp();
     if (lane == 0) {
-      K.clo = blo;
-      K.chi = bhi;
       K.blo = make_float4(AB.b.lo.x, AB.b.lo.y, AB.b.lo.z, AB.H);
       K.bhi = make_float4(AB.b.hi.x, AB.b.hi.y, AB.b.hi.z, bhi.w);
     }
     __syncwarp();
   }
+  S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
+  S.ig[lane] = I.g;
   DensAcc<KAHAN> acc;
-  unsigned int cnt = 0, q = 0;
-  bool own_only = self;      // inside the cluster itself first
-  if (self) {
+  unsigned int cnt = 0, q = 0, done = 0xffffffffu;
+  S.is[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  // inside the cluster itself first (the self interaction is a unit's first)
+  Walk Wk;
+  bool own_only = LISTED ? self : part == 0u && (!PART || any || T.active[TL.leaf[ti]]);
+  if (LISTED) Wk.live = 1u;
+
+  if (own_only) {
     if (I.valid) dens_put(S, lane, I.p, I.Hphys, own0 + lane, I.act);
     q = ni;
   }
-  // mask: candidates of the scan; k: the one whose particles nr holds (-1: none),
-  // loaded one candidate ahead, so that the load overlaps the work on the one before
-  unsigned int e0 = 0, mask = 0;
+  bool in_self = own_only;     // the batch's pairs are counted as those of the self interaction
+  // k: the candidate whose particles nr holds (-1: none), loaded one candidate ahead,
+  // so that the load overlaps the work on the one before
   int k = -1;
   float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
   for (;;) {
-    if (k < 0) {
-      while (!mask && e0 < K.ntj) mask = scan_clusters<PART>(K, TL, sort_r, sort_i, e0, any, all, I.p,
-                                                                      I.act ? I.H : 0.0f);
-      if (mask) {
-        k = __ffs(mask) - 1;
-        mask &= mask - 1;
-        if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
-      }
+    if (k < 0 && unit_next<PART>(K, Wk, S.jlo, S.jhi, Lq, T, TL, sort_r, sort_i, any, all, I.p,
+                                 I.act ? I.H : 0.0f)) {
+      k = __ffs(Wk.mask) - 1;
+      Wk.mask &= Wk.mask - 1;
+      if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
     }
     const bool last = k < 0;
     unsigned int bal = 0, gj = 0;
@@ -1360,177 +1457,125 @@ __device__ __forceinline__ void density_task(bool self, int item, unsigned int t
       pj = make_float4(nr.x + o.x, nr.y + o.y, nr.z + o.z, nr.w);
       if (PART) aj = vj && actp[gj] != 0;
       k = -1;
-      if (mask) {
-        k = __ffs(mask) - 1;
-        mask &= mask - 1;
+      if (Wk.mask) {
+        k = __ffs(Wk.mask) - 1;
+        Wk.mask &= Wk.mask - 1;
         if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
       }
       // stage only the partners within reach: of the particles that iterate (own
       // side), or, when the partner iterates, of any particle of the cluster
       const float4 blo = K.blo, bhi = K.bhi;
-      const float Hj = pj.w * K.sh.w;
+      const float Hj = pj.w * bhi.w, slack = K.gsh[Wk.it].w;
       const float3 p3 = make_float3(pj.x, pj.y, pj.z);
       pass = vj && (!PART || any) &&
              near_box(p3, Box3{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)},
-                      fmaxf(blo.w, Hj) + bhi.w);
+                      fmaxf(blo.w, Hj) + slack);
       if (PART && !pass && !all && aj) {
         const float4 clo = K.clo, chi = K.chi;
-        pass = near_box(p3, Box3{make_float3(clo.x, clo.y, clo.z), make_float3(chi.x, chi.y, chi.z)}, Hj + bhi.w);
+        pass = near_box(p3, Box3{make_float3(clo.x, clo.y, clo.z), make_float3(chi.x, chi.y, chi.z)}, Hj + slack);
       }
       bal = __ballot_sync(0xffffffffu, pass);
     }
-    if (own_only || last || q + __popc(bal) > 32u) {
+    if (own_only || last || q + __popc(bal) > 32u || (COUNT && in_self != (Wk.it == K.selfit))) {
       if (q)
-        dens_batch<COUNT, PART, KAHAN, REC>(I, S, q, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt, C, R,
-                                            W);
+        dens_batch<COUNT, PART, KAHAN, LISTED>(I, S, q, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt,
+                                               COUNT && in_self ? Cs : Cp, R, W);
       q = 0;
       own_only = false;
+      in_self = Wk.it == K.selfit;
+      // plain sums are kept per interaction: one chain over all of a unit's partners
+      // would round more than the sums of separate interactions
+      const unsigned int now = K.gidx + (unsigned int)Wk.it;
+      if (!KAHAN && now != done) {
+        const float4 t = S.is[lane];
+        S.is[lane] = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
+        acc = DensAcc<KAHAN>();
+        done = now;
+      }
     }
     if (last) break;
     if (pass)
       dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), make_float3(pj.x, pj.y, pj.z), pj.w, gj, aj);
     q += __popc(bal);
   }
-  flush_dens(I.g, acc.total(), cnt, dacc, dcnt);
-  if (REC) rec_task_end(self ? R.stask : R.ptask, S);
+  float4 sum = acc.total();
+  if (!KAHAN) {
+    const float4 t = S.is[lane];
+    sum = make_float4(t.x + sum.x, t.y + sum.y, t.z + sum.z, t.w + sum.w);
+  }
+  flush_dens(I.g, sum, cnt, dacc, dcnt);
+  if (LISTED) rec_task_end(self ? R.stask : R.ptask, S);
 }
 
-// Lane-parallel scan of B's sorted cluster list for the i cluster (box bi,
-// largest support Hi): returns in *jt, *jn, *js the lane's candidate cluster,
-// its size and first particle, and a ballot of the lanes whose cluster is in
-// reach (sorted window, then box distance).
-// *stop is set when the sorted window has passed every cluster of B.
-__device__ __forceinline__ unsigned int scan_clusters_force(const PairSetup& P, const Tree& T, const Tiles& TL,
-                                                      const float* __restrict__ sort_r,
-                                                      const unsigned int* __restrict__ sort_i, unsigned int e0,
-                                                      const Box3& bi, float rhi_i, float Hi,
-                                                      unsigned int* jt, unsigned int* jn, unsigned int* js,
-                                                      bool* stop) {
+// The force interactions of one unit, as density_unit.
+template <bool COUNT, bool LISTED>
+__device__ __forceinline__ void force_unit(unsigned int ti, unsigned int part, unsigned int parts, bool self, int item,
+    const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box, const float4* __restrict__ cen4,
+    const float4* __restrict__ vel4, const float4* __restrict__ ghost4, const float* __restrict__ sort_r,
+    const unsigned int* __restrict__ sort_i, const ForceArgs& A, float4* facc, float* fvsig, ForceShared& S,
+    Counters& Cp, Counters& Cs) {
   const int lane = threadIdx.x & 31;
-  const bool sorted = P.sb != SORT_NONE;
-  if (sorted) {
-    // sort keys are the projections at the build; a cluster's projection has
-    // since moved by at most the drift
-    const float r0 = sort_r[P.sb + e0] + P.g.offBp - P.g.drift;
-    *stop = r0 - rhi_i > fmaxf(Hi, P.HmB) + P.slack;     // the sorted list only moves further away
-    if (*stop) return 0u;
-  } else {
-    *stop = false;
-  }
-  const unsigned int e = e0 + lane;
-  bool pass = false;
-  unsigned int t = 0;
-  if (e < P.ntj) {
-    t = sorted ? sort_i[P.sb + e] : P.tb0 + e;
-    const float Hj = TL.lo[t].w * P.g.invL;
-    const float reach = fmaxf(Hi, Hj) + P.slack;
-    const bool window = !sorted || sort_r[P.sb + e] + P.g.offBp - P.g.drift - rhi_i <= reach;
-    if (window) {
-      const Box3 bj = tile_box3(TL, T, t, P.tshB);
-      pass = box_near(bi, bj, reach);
-    }
-  }
-  *jt = t;
-  *jn = pass ? TL.n[t] : 0u;
-  *js = pass ? TL.start[t] : 0u;
-  return __ballot_sync(0xffffffffu, pass);
-}
-
-template <bool COUNT>
-__device__ __forceinline__ void force_pair_task(int item, unsigned int ti, const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box,
-    const float4* __restrict__ pos4, const float4* __restrict__ cen4, const float4* __restrict__ vel4,
-    const float4* __restrict__ ghost4, const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
-    const unsigned int* __restrict__ perm, const double* __restrict__ x, float alpha, float4* facc, float* fvsig,
-    unsigned int* fcnt, ForceShared& S, Counters* C) {
-  const int lane = threadIdx.x & 31;
-  const PairSetup P = pair_setup(Lq, T, box, item);
-  const LeafFrame F = leaf_frame(TL, T, ti, P);
-  const Box3 bi = tile_box3(TL, T, ti, P.tshA);          // the cluster in A's frame (the sorted sweep)
-  const Box3 bil = tile_box3(TL, T, ti, F.sh_own);       // ... and in its leaf's frame (the particles)
-  const float Hi = TL.lo[ti].w * P.g.invL;
-  const float rhi_i = box_rhi(bi, P.u);
-  const bool vi = (unsigned int)lane < TL.n[ti];
-  const ForceI I = load_force(vi, TL.start[ti] + lane, F.sh_own, pos4, cen4, vel4, ghost4, P.g.invL, P.g.L32, P.g.eb);
-  force_stage_own(S, lane, I);
+  UnitShared& K = S.tk;
+  unit_begin(K, ti, T, TL, box, part, parts);
+  if (LISTED) unit_single(K, self, item, Lq, T);
+  const unsigned int ni = TL.n[ti], own0 = TL.start[ti];
+  const bool vi = (unsigned int)lane < ni;
+  if (lane == 0) S.own0 = own0;
+  const float4 P = force_stage_own(S, lane, vi, own0 + lane, A.pos4, cen4, vel4, ghost4);
+  const float3 ip = make_float3(P.x, P.y, P.z);
   unsigned int q = 0;
-  for (unsigned int e0 = 0; e0 < P.ntj; e0 += 32) {
-    unsigned int jt, jn, js;
-    bool stop;
-    unsigned int mask =
-        scan_clusters_force(P, T, TL, sort_r, sort_i, e0, bi, rhi_i, Hi, &jt, &jn, &js, &stop);
-    if (stop) break;
-    while (mask) {
-      const int k = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const bool vj = (unsigned int)lane < __shfl_sync(0xffffffffu, jn, k);
-      const ForceI J = load_force(vj, __shfl_sync(0xffffffffu, js, k) + lane, F.sh_part, pos4, cen4, vel4, ghost4,
-                                  P.g.invL, P.g.L32, P.g.eb);
-      const bool pass = vj && near_box(J.p, bil, fmaxf(Hi, J.H) + P.slack);
-      const unsigned int bal = __ballot_sync(0xffffffffu, pass);
-      const unsigned int np = __popc(bal);
-      if (q + np > 32u) {
-        force_batch<COUNT>(S, q, false, perm, x, box_exact(P.g), alpha, facc, fvsig, fcnt, C);
-        q = 0;
-      }
-      if (pass) force_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), J);
-      q += np;
-    }
-  }
-  if (q) force_batch<COUNT>(S, q, false, perm, x, box_exact(P.g), alpha, facc, fvsig, fcnt, C);
-  __syncwarp();
-  flush_force(__float_as_int(S.ih[lane].w), S.iacc[lane], S.ivs[lane], facc, fvsig);
-}
+  Walk Wk;
+  bool own_only = LISTED ? self : part == 0u;      // inside the cluster itself first: each unordered pair once
+  if (LISTED) Wk.live = 1u;
 
-template <bool COUNT>
-__device__ __forceinline__ void force_self_task(int item, unsigned int ti, const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box,
-    const float4* __restrict__ pos4, const float4* __restrict__ cen4, const float4* __restrict__ vel4,
-    const float4* __restrict__ ghost4, const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
-    const unsigned int* __restrict__ perm, const double* __restrict__ x, float alpha, float4* facc, float* fvsig,
-    unsigned int* fcnt, ForceShared& S, Counters* C) {
-  const int lane = threadIdx.x & 31;
-  const int A = Lq.self_a[item];
-  const ItemGeom g = item_geom(T, box, A, 0);
-  const float4 cA = T.cen[A];
-  const float3 sh = make_float3(-cA.x, -cA.y, -cA.z);
-  const float slack = g.e * 1.52587890625e-05f + g.es + 1e-6f * T.hmax[A] * g.invL;
-  const unsigned int t0 = T.tile0[A], nt = T.ntile[A];
-  const Box3 bi = tile_box3(TL, T, ti, sh);
-  const float Hi = TL.lo[ti].w * g.invL;
-  const bool vi = (unsigned int)lane < TL.n[ti];
-  const ForceI I = load_force(vi, TL.start[ti] + lane, sh, pos4, cen4, vel4, ghost4, g.invL, g.L32, g.eb);
-  force_stage_own(S, lane, I);
-  unsigned int q = 0;
-  // inside the cluster itself each unordered pair once: partners above the lane
-  if (vi) force_put(S, lane, I);
-  force_batch<COUNT>(S, TL.n[ti], true, perm, x, box_exact(g), alpha, facc, fvsig, fcnt, C);
-  for (unsigned int b0 = ti + 1; b0 < t0 + nt; b0 += 32) {
-    const unsigned int tl = b0 + lane;
-    bool ok = false;
-    if (tl < t0 + nt) {
-      const Box3 bj = tile_box3(TL, T, tl, sh);
-      ok = box_near(bi, bj, fmaxf(Hi, TL.lo[tl].w * g.invL) + slack);
-    }
-    unsigned int mask = __ballot_sync(0xffffffffu, ok);
-    while (mask) {
-      const int k = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const unsigned int tj = b0 + (unsigned int)k;
-      const bool vj = (unsigned int)lane < TL.n[tj];
-      const ForceI J = load_force(vj, TL.start[tj] + lane, sh, pos4, cen4, vel4, ghost4, g.invL, g.L32, g.eb);
-      const bool pass = vj && near_box(J.p, bi, fmaxf(Hi, J.H) + slack);
-      const unsigned int bal = __ballot_sync(0xffffffffu, pass);
-      const unsigned int np = __popc(bal);
-      if (q + np > 32u) {
-        force_batch<COUNT>(S, q, false, perm, x, box_exact(g), alpha, facc, fvsig, fcnt, C);
-        q = 0;
-      }
-      if (pass) force_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), J);
-      q += np;
-    }
+  if (own_only) {
+    if (vi) force_put(S, lane, ip, A.pos4[own0 + lane].w, own0 + lane);
+    q = ni;
   }
-  if (q) force_batch<COUNT>(S, q, false, perm, x, box_exact(g), alpha, facc, fvsig, fcnt, C);
+  bool in_self = own_only;
+  int k = -1;
+  float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (;;) {
+    if (k < 0 && unit_next<false>(K, Wk, S.v, S.f, Lq, T, TL, sort_r, sort_i, true, true, ip, P.w)) {
+      k = __ffs(Wk.mask) - 1;
+      Wk.mask &= Wk.mask - 1;
+      if ((unsigned int)lane < K.cn[k]) nr = A.pos4[__float_as_uint(K.co[k].w) + lane];
+    }
+    const bool last = k < 0;
+    unsigned int bal = 0, gj = 0;
+    float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool pass = false;
+    if (!last) {
+      const float4 o = K.co[k];
+      const bool vj = (unsigned int)lane < K.cn[k];
+      gj = __float_as_uint(o.w) + lane;
+      pj = make_float4(nr.x + o.x, nr.y + o.y, nr.z + o.z, nr.w);
+      k = -1;
+      if (Wk.mask) {
+        k = __ffs(Wk.mask) - 1;
+        Wk.mask &= Wk.mask - 1;
+        if ((unsigned int)lane < K.cn[k]) nr = A.pos4[__float_as_uint(K.co[k].w) + lane];
+      }
+      const float4 blo = K.blo, bhi = K.bhi;
+      pass = vj && near_box(make_float3(pj.x, pj.y, pj.z),
+                            Box3{make_float3(blo.x, blo.y, blo.z), make_float3(bhi.x, bhi.y, bhi.z)},
+                            fmaxf(blo.w, pj.w * bhi.w) + K.gsh[Wk.it].w);
+      bal = __ballot_sync(0xffffffffu, pass);
+    }
+    if (own_only || last || q + __popc(bal) > 32u || (COUNT && in_self != (Wk.it == K.selfit))) {
+      if (q)
+        force_batch<COUNT>(S, ip, P.w, q, own_only, A, cen4, vel4, ghost4, facc, fvsig,
+                           COUNT ? (in_self ? &Cs : &Cp) : nullptr);
+      q = 0;
+      own_only = false;
+      in_self = Wk.it == K.selfit;
+    }
+    if (last) break;
+    if (pass) force_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), make_float3(pj.x, pj.y, pj.z), pj.w, gj);
+    q += __popc(bal);
+  }
   __syncwarp();
-  flush_force(__float_as_int(S.ih[lane].w), S.iacc[lane], S.ivs[lane], facc, fvsig);
+  if (vi) flush_force((int)(own0 + lane), S.iacc[lane], S.ivs[lane], facc, fvsig);
 }
 
 // Whether a task's records still hold when its partner cell (the own cell for a
@@ -1576,44 +1621,24 @@ __device__ __forceinline__ bool changed_out_of_reach(bool self, int item, unsign
 template <bool COUNT>
 __device__ __forceinline__ void force_replay_task(bool self, int item, unsigned int ti, uint2 rec, const PairRec& R,
     const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box,
-    const float4* __restrict__ pos4, const float4* __restrict__ cen4, const float4* __restrict__ vel4,
-    const float4* __restrict__ ghost4, float alpha, float4* facc, float* fvsig, unsigned int* fcnt, ForceShared& S,
-    Counters* C) {
+    const float4* __restrict__ cen4, const float4* __restrict__ vel4, const float4* __restrict__ ghost4,
+    const ForceArgs& A, float4* facc, float* fvsig, ForceShared& S, Counters* C) {
   const int lane = threadIdx.x & 31;
-  ItemGeom g;
-  float3 sh_own, sh_part;
-  if (self) {
-    const int A = Lq.self_a[item];
-    g = item_geom(T, box, A, 0);
-    const float4 cA = T.cen[A];
-    sh_own = make_float3(-cA.x, -cA.y, -cA.z);
-    sh_part = sh_own;
-  } else {
-    // as pair_setup and leaf_frame
-    const int A = Lq.pair_a[item], Bc = Lq.pair_b[item];
-    g = item_geom(T, box, A, Lq.pair_axis[item]);
-    const float4 cA = T.cen[A], cB = T.cen[Bc], cl = TL.cen[ti];
-    const float3 shB = make_float3(g.offB.x - cB.x, g.offB.y - cB.y, g.offB.z - cB.z);
-    const float3 d = make_float3(cl.x - cA.x, cl.y - cA.y, cl.z - cA.z);
-    sh_own = make_float3(-cl.x, -cl.y, -cl.z);
-    sh_part = make_float3(shB.x - d.x, shB.y - d.y, shB.z - d.z);
-  }
+  unit_begin(S.tk, ti, T, TL, box, 0u, 1u);
+  unit_single(S.tk, self, item, Lq, T);
+  const unsigned int own0 = TL.start[ti];
   const bool vi = (unsigned int)lane < TL.n[ti];
-  const ForceI I = load_force(vi, TL.start[ti] + lane, sh_own, pos4, cen4, vel4, ghost4, g.invL, g.L32, g.eb);
-  force_stage_own(S, lane, I);
+  if (lane == 0) S.own0 = own0;
+  force_stage_own(S, lane, vi, own0 + lane, A.pos4, cen4, vel4, ghost4);
+  const float4 sh4 = S.tk.gsh[0];
+  const float3 sh = make_float3(sh4.x, sh4.y, sh4.z);
   unsigned int b = rec.x;
   for (unsigned int k = 0; k < rec.y; ++k, ++b) {
     if (k > 0 && b % REC_CHUNK == 0u) b = R.next[b / REC_CHUNK - 1u] * REC_CHUNK;   // the chunk is full: next one
-    const bool own_only = self && k == 0;
-    if (own_only) {
-      __syncwarp();
-      if (vi) force_put(S, lane, I);
-    }
-    force_replay_batch<COUNT>(S, R.pool + 64ull * b, own_only, sh_part, g.invL, g.L32, g.eb, pos4, cen4, vel4,
-                              ghost4, alpha, facc, fvsig, fcnt, C);
+    force_replay_batch<COUNT>(S, R.pool + 64ull * b, self && k == 0, cen4, vel4, ghost4, A, sh, facc, fvsig, C);
   }
   __syncwarp();
-  flush_force(__float_as_int(S.ih[lane].w), S.iacc[lane], S.ivs[lane], facc, fvsig);
+  if (vi) flush_force((int)(own0 + lane), S.iacc[lane], S.ivs[lane], facc, fvsig);
 }
 
 // Density interactions of one pass: the live pair and self tasks in one queue.
@@ -1638,46 +1663,53 @@ __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_B
                                                          unsigned int* __restrict__ task_ctr, int partial_host,
                                                          const int* __restrict__ it_dev, const int* __restrict__ gflag,
                                                          const unsigned int* __restrict__ g_n, unsigned int cap_g,
+                                                         unsigned int ntcap, const unsigned int* __restrict__ ntile_dev,
+                                                         const uint2* __restrict__ units,
+                                                         const unsigned int* __restrict__ n_units, unsigned int cap_units,
                                                          const __grid_constant__ PairRec Rec) {
   pdl_wait();
   const int partial = it_dev ? (*it_dev > 1 ? 1 : 0) : partial_host;
   if ((partial != 0) != PART) return;
+  if (it_dev && it_dev[2] != 0) return;                        // the iteration has stopped
   if (PART && gflag && gather_on(gflag, g_n, cap_g)) return;   // the pass gathers
   __shared__ DensShared SH[SPH_WARPS_PER_CTA];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   DensShared& S = SH[wl];
   RecW W;
   Counters Cp, Cs;
-  const unsigned int ntask = *Lq.n_live;
-  // few tasks (the later passes of the h iteration): one task per fetch and no
-  // fetch ahead, so that no warp queues several while others idle
-  const bool few = ntask < 4u * gridDim.x * (blockDim.x >> 5);
-  // (8 at a time only where every warp gets many: smaller passes keep their balance)
-  const unsigned int chunk = few ? 1u : (ntask >= 64u * gridDim.x * (blockDim.x >> 5) ? TASK_CHUNK_DENSITY : 2u);
+  // units of work (REC: the listed tasks, whose pairs are recorded one by one)
+  const unsigned int nt = ntile_dev ? min(ntcap, *ntile_dev) : ntcap;
+  const bool listed = !REC && units && *n_units <= cap_units;
+  const unsigned int parts = REC ? 1u : unit_parts(nt);
+  const unsigned int nunit = REC ? *Lq.n_live : (listed ? *n_units : nt * parts);
+  // the next unit is fetched while the current one runs, unless there are so few that
+  // a warp would hold one back from an idle warp
+  const bool few = nunit < 4u * gridDim.x * (blockDim.x >> 5);
   unsigned int raw = 0;
-  if (lane == 0) raw = atomicAdd(task_ctr, chunk);
-  for (unsigned int base = __shfl_sync(0xffffffffu, raw, 0); base < ntask; base = __shfl_sync(0xffffffffu, raw, 0)) {
-    if (!few && lane == 0) raw = atomicAdd(task_ctr, chunk);    // the next chunk, fetched while this one runs
-    const unsigned int tend = min(base + chunk, ntask);
-    for (unsigned int t = base; t < tend; ++t) {
-      const uint2 lt = Lq.p_live[t];
-      const int item = (int)(lt.x & 0x7fffffffu);
-      const bool self = (lt.x >> 31) != 0u;
-      density_task<COUNT, PART, KAHAN, REC && !PART>(self, item, lt.y, Lq, T, TL, box, pos4, cen4, sort_r, sort_i, act,
-                                                     perm, x, dacc, dcnt, S, COUNT && self ? Cs : Cp, Rec, W);
-    }
-    if (few && lane == 0) raw = atomicAdd(task_ctr, chunk);
+  if (lane == 0) raw = atomicAdd(task_ctr, 1u);
+  for (unsigned int u = __shfl_sync(0xffffffffu, raw, 0); u < nunit; u = __shfl_sync(0xffffffffu, raw, 0)) {
+    if (!few && lane == 0) raw = atomicAdd(task_ctr, 1u);
+    // (REC: interaction and cluster; else cluster, part and parts)
+    uint2 un = make_uint2(0u, 0u);
+    if (REC) un = Lq.p_live[u];
+    else un = listed ? units[u] : make_uint2(u / parts, (u % parts) | (parts << 16));
+    const bool self = REC && (un.x >> 31) != 0u;
+    density_unit<COUNT, PART, KAHAN, REC>(REC ? un.y : un.x, REC ? 0u : un.y & 0xffffu, REC ? 1u : un.y >> 16, self,
+                                          (int)(un.x & 0x7fffffffu), Lq, T, TL, box, pos4, cen4, sort_r, sort_i, act,
+                                          perm, x, dacc, dcnt, S, Cp, Cs, Rec, W);
+    if (few && lane == 0) raw = atomicAdd(task_ctr, 1u);
   }
   commit_counters<COUNT>(Cp, pc, 0);
   commit_counters<COUNT>(Cs, pc, 1);
 }
 
-// Force interactions of one pass: the pair and self tasks in one queue.
+// Force interactions of one pass: one queue of units, or (REC) of the listed tasks,
+// whose pairs the first density pass recorded.
 // Registers capped at 64 per thread (8 blocks of 128 threads, whose shared memory
-// fits an SM with the 768-entry pair list): more warps in flight to hide the
-// partner loads outweigh the few spilled values (33.5M: 6, 5 and 4 blocks took 74,
-// 84 and 98 ms against 65 ms).
-template <bool COUNT>
+// fits an SM): more warps in flight to hide the partner loads outweigh the few
+// spilled values (33.5M, an earlier form of the kernel: 6, 5 and 4 blocks took 74, 84
+// and 98 ms against 65 ms).
+template <bool COUNT, bool REC>
 __global__ void __launch_bounds__(SPH_THREADS, 8) k_force(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box,
                                                        const float4* __restrict__ pos4,
                                                        const float4* __restrict__ cen4,
@@ -1688,55 +1720,108 @@ __global__ void __launch_bounds__(SPH_THREADS, 8) k_force(Lists Lq, Tree T, Tile
                                                        const unsigned int* __restrict__ perm,
                                                        const double* __restrict__ x, float alpha, float4* facc,
                                                        float* fvsig, unsigned int* fcnt, unsigned long long* pc,
-                                                       unsigned int* __restrict__ task_ctr,
+                                                       unsigned int* __restrict__ task_ctr, unsigned int ntcap,
+                                                       const unsigned int* __restrict__ ntile_dev,
+                                                       const uint2* __restrict__ units,
+                                                       const unsigned int* __restrict__ n_units, unsigned int cap_units,
                                                        const __grid_constant__ PairRec R) {
   pdl_wait();
   __shared__ ForceShared SH[SPH_WARPS_PER_CTA];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   ForceShared& S = SH[wl];
   Counters Cp, Cs;
-  const unsigned int ntask = *Lq.n_live;
-  // few tasks (the later passes of the h iteration): one task per fetch and no
-  // fetch ahead, so that no warp queues several while others idle
-  const bool few = ntask < 4u * gridDim.x * (blockDim.x >> 5);
-  const unsigned int chunk = few ? 1u : TASK_CHUNK_FORCE;
+  const ForceArgs A{perm, x, pos4, box, fcnt, alpha};
+  const unsigned int nt = ntile_dev ? min(ntcap, *ntile_dev) : ntcap;
+  const bool listed = !REC && units && *n_units <= cap_units;
+  const unsigned int parts = REC ? 1u : unit_parts(nt);
+  const unsigned int nunit = REC ? *Lq.n_live : (listed ? *n_units : nt * parts);
+  // as in k_density
+  const bool few = nunit < 4u * gridDim.x * (blockDim.x >> 5);
   unsigned int raw = 0;
-  if (lane == 0) raw = atomicAdd(task_ctr, chunk);
-  for (unsigned int base = __shfl_sync(0xffffffffu, raw, 0); base < ntask; base = __shfl_sync(0xffffffffu, raw, 0)) {
-    if (!few && lane == 0) raw = atomicAdd(task_ctr, chunk);    // the next chunk, fetched while this one runs
-    const unsigned int tend = min(base + chunk, ntask);
-    for (unsigned int t = base; t < tend; ++t) {
-      const uint2 lt = Lq.p_live[t];
+  if (lane == 0) raw = atomicAdd(task_ctr, 1u);
+  for (unsigned int u = __shfl_sync(0xffffffffu, raw, 0); u < nunit; u = __shfl_sync(0xffffffffu, raw, 0)) {
+    if (!few && lane == 0) raw = atomicAdd(task_ctr, 1u);
+    if (!REC) {
+      if (COUNT && lane == 0) atomicAdd(&pc[12], 1ull);
+      const uint2 un = listed ? units[u] : make_uint2(u / parts, (u % parts) | (parts << 16));
+      force_unit<COUNT, false>(un.x, un.y & 0xffffu, un.y >> 16, false, 0, Lq, T, TL, box, cen4, vel4, ghost4, sort_r,
+                               sort_i, A, facc, fvsig, S, Cp, Cs);
+    } else {
+      const uint2 lt = Lq.p_live[u];
       const int item = (int)(lt.x & 0x7fffffffu);
       const bool self = (lt.x >> 31) != 0u;
       // the records of the first density pass, where they hold
       uint2 rec = make_uint2(REC_NONE, 0u);
-      if (R.pool && !TL.changed[lt.y]) {
-        const int A = self ? Lq.self_a[item] : Lq.pair_a[item];
-        const int C = self ? A : Lq.pair_b[item];
-        if (!T.changed[C] || changed_out_of_reach(self, item, lt.y, Lq, T, TL, box))
-          rec = self ? R.stask[Lq.s_toff[item] + (lt.y - T.tile0[A])] : R.ptask[Lq.p_toff[item] + (lt.y - T.tile0[A])];
+      if (!TL.changed[lt.y]) {
+        const int a = self ? Lq.self_a[item] : Lq.pair_a[item];
+        const int c = self ? a : Lq.pair_b[item];
+        if (!T.changed[c] || changed_out_of_reach(self, item, lt.y, Lq, T, TL, box))
+          rec = self ? R.stask[Lq.s_toff[item] + (lt.y - T.tile0[a])] : R.ptask[Lq.p_toff[item] + (lt.y - T.tile0[a])];
       }
       if (COUNT && lane == 0) atomicAdd(&pc[rec.x != REC_NONE ? 11 : 12], 1ull);
       if (rec.x != REC_NONE)
-        force_replay_task<COUNT>(self, item, lt.y, rec, R, Lq, T, TL, box, pos4, cen4, vel4, ghost4, alpha, facc,
-                                 fvsig, fcnt, S, COUNT ? (self ? &Cs : &Cp) : nullptr);
-      else if (self)
-        force_self_task<COUNT>(item, lt.y, Lq, T, TL, box, pos4, cen4, vel4, ghost4, sort_r, sort_i, perm, x, alpha,
-                               facc, fvsig, fcnt, S, COUNT ? &Cs : nullptr);
+        force_replay_task<COUNT>(self, item, lt.y, rec, R, Lq, T, TL, box, cen4, vel4, ghost4, A, facc, fvsig, S,
+                                 COUNT ? (self ? &Cs : &Cp) : nullptr);
       else
-        force_pair_task<COUNT>(item, lt.y, Lq, T, TL, box, pos4, cen4, vel4, ghost4, sort_r, sort_i, perm, x, alpha,
-                               facc, fvsig, fcnt, S, COUNT ? &Cp : nullptr);
+        force_unit<COUNT, true>(lt.y, 0u, 1u, self, item, Lq, T, TL, box, cen4, vel4, ghost4, sort_r, sort_i, A, facc,
+                                fvsig, S, Cp, Cs);
     }
-    if (few && lane == 0) raw = atomicAdd(task_ctr, chunk);
+    if (few && lane == 0) raw = atomicAdd(task_ctr, 1u);
   }
   commit_counters<COUNT>(Cp, pc, 2);
   commit_counters<COUNT>(Cs, pc, 3);
 }
 
+// The units of a decomposition whose clusters are neither few (all are then split the
+// same way) nor so many that the longest does not matter: a cluster's expected
+// partners, from the share of each partner cell within reach of its box, and one unit
+// per UNIT_PARTNERS of them.  A sparse cluster beside a dense cell (the rim of a
+// clump, or a first guess of h far from its root) has thousands: as one unit, one
+// warp held the force pass of a 636k-particle log-normal box at its first guess for
+// as long again as all the others took.  One warp per cluster.
+constexpr float UNIT_PARTNERS = 2048.0f;
 
-
-
+__global__ void k_unit_list(unsigned int ntcap, const unsigned int* __restrict__ ntile_dev, Lists Lq, Tree T, Tiles TL,
+                            const BoxDesc* __restrict__ box, uint2* __restrict__ units,
+                            unsigned int* __restrict__ n_units, unsigned int cap) {
+  pdl_wait();
+  const unsigned int nt = ntile_dev ? min(ntcap, *ntile_dev) : ntcap;
+  const int lane = threadIdx.x & 31;
+  const unsigned int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (unsigned int t = warp; t < nt; t += nwarps) {
+    const int leaf = (int)TL.leaf[t];
+    const float4 lo = TL.lo[t], hi = TL.hi[t], cl = TL.cen[t];
+    const float H = lo.w * (float)box[T.box[leaf]].invL;
+    float est = 0.0f;
+    for (int A = leaf; A >= 0; A = T.parent[A]) {
+      const unsigned int n = (unsigned int)__popc(T.pmask[A]) + (A == leaf ? 1u : 0u);
+      const float e = ldexpf(1.0f, -T.level[A]);
+      for (unsigned int k = lane; k < n; k += 32) {
+        int B = A, dx = 0, dy = 0, dz = 0;
+        if (A != leaf || k > 0u) {
+          const uint2 pr = Lq.csr[T.pstart[A] + k - (A == leaf ? 1u : 0u)];
+          B = (int)pr.x;
+          axis_vec((int)pr.y, dx, dy, dz);
+        }
+        const float4 cA = T.cen[A];
+        // the partner cell's centre in the frame of the own leaf; the part of each of
+        // its edges within H of the own box
+        const float bx = e * dx - (cl.x - cA.x), by = e * dy - (cl.y - cA.y), bz = e * dz - (cl.z - cA.z);
+        const float fx = fminf(hi.x + H, bx + 0.5f * e) - fmaxf(lo.x - H, bx - 0.5f * e);
+        const float fy = fminf(hi.y + H, by + 0.5f * e) - fmaxf(lo.y - H, by - 0.5f * e);
+        const float fz = fminf(hi.z + H, bz + 0.5f * e) - fmaxf(lo.z - H, bz - 0.5f * e);
+        const float ie = 1.0f / e;
+        est += fmaxf(fx, 0.0f) * ie * (fmaxf(fy, 0.0f) * ie) * (fmaxf(fz, 0.0f) * ie) * (float)T.count[B];
+      }
+    }
+    est = warp_sum(est);
+    const unsigned int parts = (unsigned int)fminf(32.0f, fmaxf(1.0f, ceilf(est * (1.0f / UNIT_PARTNERS))));
+    unsigned int at = 0;
+    if (lane == 0) at = atomicAdd(n_units, parts);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if ((unsigned int)lane < parts && at + lane < cap) units[at + lane] = make_uint2(t, (unsigned int)lane | (parts << 16));
+  }
+}
 
 // Tasks of one pass that have work, as (interaction, cluster); bit 31 of the
 // interaction marks a self task.  Pair tasks: in a density pass those whose
@@ -1978,14 +2063,15 @@ __device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsi
   const unsigned int jvalid = __ballot_sync(0xffffffffu, v);
   __syncwarp();
   unsigned int m, none;
-  near_masks<false>(I.p, I.hi, S.x, S.y, S.z, nullptr, (int)((q + 3u) & ~3u), m, none);
+  const float iband = BAND_REL * I.H * (S.tk.eb + I.H), ilo = I.H * I.H - iband;
+  near_masks<false>(I.p, I.H * I.H + iband, S.x, S.y, S.z, nullptr, (int)((q + 3u) & ~3u), m, none);
   m &= I.valid ? jvalid : 0u;
   S.m[lane] = jm;
   __syncwarp();
   if (self)
     for (unsigned int b = m; b; b &= b - 1)
       if (S.g[__ffs(b) - 1] == I.g) m &= ~(b & (0u - b));
-  dens_row(I, S, m, acc, cnt, perm, x, pos4, box, dacc, dcnt);
+  dens_row(I, ilo, S, m, acc, cnt, perm, x, pos4, box, dacc, dcnt);
   __syncwarp();
 }
 
@@ -2024,11 +2110,14 @@ __device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tre
   const float3 d = make_float3(cl.x - cO.x, cl.y - cO.y, cl.z - cO.z);
   const float3 sh_part = make_float3(shX.x - d.x, shX.y - d.y, shX.z - d.z);
   const bool vi = (unsigned int)lane < n;
-  const DensI I = load_dens(vi, vi ? pk_idx[info.x + lane] : 0u, pos4, cen4, nullptr, g.invL, g.eb);
+  const DensI I = load_dens(vi, vi ? pk_idx[info.x + lane] : 0u, pos4, cen4, nullptr, g.invL);
   __syncwarp();
   S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
   S.ig[lane] = I.g;
-  if (lane == 0) S.tk.box = T.box[O];
+  if (lane == 0) {
+    S.tk.box = T.box[O];
+    S.tk.eb = g.eb;
+  }
   __syncwarp();
   // the packed particles' box and largest H: the own side reaches no further
   Box3 bo;
@@ -2605,7 +2694,7 @@ __global__ void k_get_field(long long off, long long n, int field, const unsigne
 // may run in several host threads)
 static int resident_ctas(const void* fn) {
   static std::mutex mu;
-  static const void* fns[24] = {nullptr};   // the 12 density, 2 gathered density and 2 force instances
+  static const void* fns[24] = {nullptr};   // the 12 density, 2 gathered density and 4 force instances
   static int val[24] = {0};
   std::lock_guard<std::mutex> lock(mu);
   for (int k = 0; k < 24; ++k) {
@@ -2622,6 +2711,7 @@ static int resident_ctas(const void* fn) {
 }
 
 void launch_live_tasks(Engine& E, bool dens, const int* it_dev) {
+  if (!E.rec_for_force().pool) return;     // the passes walk their clusters' interactions (with pair records they list their tasks)
   cudaMemsetAsync(E.Lq.n_live, 0, sizeof(unsigned int), E.st);
   // a captured rebuild step sizes the launch by the task capacity and the kernel
   // reads the counts of the build from the device
@@ -2644,7 +2734,7 @@ void launch_live_tasks(Engine& E, bool dens, const int* it_dev) {
 // the caller knows the pass needs (-1: both, as in a captured step, where the
 // one that does not match the counter returns at once).
 void launch_density(Engine& E, const int* it_dev, int only) {
-  cudaMemsetAsync(E.task_ctr.p + 0, 0, sizeof(unsigned int), E.st);
+  cudaMemsetAsync(E.task_ctr.p, 0, 2 * sizeof(unsigned int), E.st);
   for (int part = 0; part < 2; ++part) {
     if (!it_dev && part != (E.partial_pass ? 1 : 0)) continue;
     if (it_dev && only >= 0 && part != only) continue;
@@ -2665,8 +2755,10 @@ void launch_density(Engine& E, const int* it_dev, int only) {
                                 : (rec ? k_density<false, false, false, true> : k_density<false, false, false, false>));
     launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st,
         E.Lq, E.T, E.TL, E.box.p, E.pos4.p, E.cen4.p, E.sort_r.p, E.sort_i.p, E.act.p, E.perm.p, E.x.p, E.dacc.p,
-        E.dcnt.p, E.pc.p, E.task_ctr.p + 0, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr, E.g_n.p,
-        (unsigned int)E.g_live.n, E.rec_for_force());
+        E.dcnt.p, E.pc.p, E.task_ctr.p + part, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr, E.g_n.p,
+        (unsigned int)E.g_live.n, (unsigned int)(E.gcap ? E.N : E.n_tiles),
+        E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr,
+        E.unit_list ? E.units.p : nullptr, E.n_units.p, (unsigned int)E.units.n, E.rec_for_force());
     count_launch();
   }
 }
@@ -2699,32 +2791,35 @@ void launch_gather_prep(Engine& E, const int* it_dev) {
 void launch_density_gather(Engine& E) {
   const bool kahan = E.prm.compensated > 0 || (E.prm.compensated < 0 && E.prm.n_ngb >= 100.0f);
   const auto k = kahan ? k_density_gather<true> : k_density_gather<false>;
-  cudaMemsetAsync(E.task_ctr.p + 2, 0, sizeof(unsigned int), E.st);
+  cudaMemsetAsync(E.task_ctr.p + 3, 0, sizeof(unsigned int), E.st);
   launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st, E.Lq, E.T, E.TL, E.box.p, E.pos4.p,
              E.cen4.p, E.perm.p, E.x.p, E.dacc.p, E.dcnt.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n,
-             E.gflag.p, E.pk_info.p, E.pk_n.p, E.pk_idx.p, E.task_ctr.p + 2);
+             E.gflag.p, E.pk_info.p, E.pk_n.p, E.pk_idx.p, E.task_ctr.p + 3);
   count_launch();
 }
 
-#ifndef FORCE_BLOCKS
-#define FORCE_BLOCKS 0
-#endif
 void launch_force(Engine& E) {
-  const auto k = E.count_pairs ? k_force<true> : k_force<false>;
-  cudaMemsetAsync(E.task_ctr.p + 1, 0, sizeof(unsigned int), E.st);
-  int nb = resident_ctas((const void*)k);
-  if (FORCE_BLOCKS > 0) {
-    static bool set[2] = {false, false};
-    if (!set[E.count_pairs ? 1 : 0]) {
-      const int pct = (int)std::ceil(100.0 * FORCE_BLOCKS * (sizeof(ForceShared) * SPH_WARPS_PER_CTA + 1024) / (228.0 * 1024));
-      cudaFuncSetAttribute((const void*)k, cudaFuncAttributePreferredSharedMemoryCarveout, std::min(pct, 100));
-      set[E.count_pairs ? 1 : 0] = true;
-    }
-    nb = std::min(nb, FORCE_BLOCKS);
-  }
-  launch_pdl(k, E.nsm * nb, SPH_THREADS, E.st,
+  const bool rec = E.rec_for_force().pool != nullptr;
+  const auto k = E.count_pairs ? (rec ? k_force<true, true> : k_force<true, false>)
+                               : (rec ? k_force<false, true> : k_force<false, false>);
+  cudaMemsetAsync(E.task_ctr.p + 2, 0, sizeof(unsigned int), E.st);
+  launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st,
       E.Lq, E.T, E.TL, E.box.p, E.pos4.p, E.cen4.p, E.vel4.p, E.ghost4.p, E.sort_r.p, E.sort_i.p, E.perm.p, E.x.p,
-      E.prm.alpha_visc, E.facc.p, E.fvsig.p, E.fcnt.p, E.pc.p, E.task_ctr.p + 1, E.rec_for_force());
+      E.prm.alpha_visc, E.facc.p, E.fvsig.p, E.fcnt.p, E.pc.p, E.task_ctr.p + 2,
+      (unsigned int)(E.gcap ? E.N : E.n_tiles),
+      E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr,
+      E.unit_list ? E.units.p : nullptr, E.n_units.p, (unsigned int)E.units.n, E.rec_for_force());
+  count_launch();
+}
+
+// The unit list of a decomposition (built with it; see k_unit_list).
+void launch_unit_list(Engine& E) {
+  if (!E.unit_list) return;
+  cudaMemsetAsync(E.n_units.p, 0, sizeof(unsigned int), E.st);
+  const long long nt = E.gcap ? E.N : E.n_tiles;
+  launch_pdl(k_unit_list, E.grid(32 * nt), 256, E.st, (unsigned int)nt,
+             E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr, E.Lq, E.T, E.TL, E.box.p,
+             E.units.p, E.n_units.p, (unsigned int)E.units.n);
   count_launch();
 }
 

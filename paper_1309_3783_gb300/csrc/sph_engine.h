@@ -175,7 +175,7 @@ class Engine {
 
   // cell tree
   int cap_nodes = 0;
-  DBuf<unsigned int> t_start, t_count, t_nsmall, t_axes, t_sortbase;
+  DBuf<unsigned int> t_start, t_count, t_nsmall, t_axes, t_sortbase, t_pmask, t_pstart;
   DBuf<unsigned long long> t_key;
   DBuf<int> t_level, t_box, t_child, t_nchild, t_parent, t_split, t_n;
   DBuf<float> t_hmax;
@@ -191,6 +191,7 @@ class Engine {
   // interaction lists
   int cap_self = 0, cap_pair = 0, cap_queue = 0;
   DBuf<int> l_self, l_pa, l_pb, l_pax, l_counts;
+  DBuf<uint2> l_csr;
   DBuf<unsigned int> l_ptoff, l_stoff, scan_tmp, l_ptask, l_stask, l_nlive;
   DBuf<uint2> l_plive;
   // gathered later passes of the h iteration: per cluster the particles still
@@ -241,7 +242,12 @@ class Engine {
   DBuf<double> red;               // 8 per box
   DBuf<unsigned int> err_all;     // global error bits
   DBuf<unsigned long long> pc;    // pair counters per kernel (see commit_counters)
-  DBuf<unsigned int> task_ctr;    // task counters of the four interaction kernels
+  DBuf<unsigned int> task_ctr;    // unit counters of the interaction kernels
+  // units of work of the passes, (cluster, part | parts << 16), and their number; in use
+  // when unit_list
+  DBuf<uint2> units;
+  DBuf<unsigned int> n_units;
+  bool unit_list = false;
   DBuf<int> dev_counters;         // [0] particles still active after a ghost pass
   DBuf<unsigned char> staging;    // output staging (input order)
   DBuf<unsigned char> staging_many;   // one region per field of a multi-field read

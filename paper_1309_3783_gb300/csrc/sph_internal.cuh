@@ -227,6 +227,9 @@ struct Tree {
   float4* cen;              // centre minus its top cell's centre (units of L), exact
   unsigned int* axes;       // bit a: a sorted list along axis a is needed
   unsigned int* sortbase;   // offset of the first sorted list of this cell
+  unsigned int* pmask;      // bit a: a pair-interaction (A, B, a) with A this cell (one B per axis); the first of
+                            //   them in Lists::csr, by axis
+  unsigned int* pstart;
   unsigned char* active;    // 1 when a particle inside still iterates h
   unsigned char* changed;   // 1 when a particle inside took a new h after the first density pass
   unsigned int* clo;        // box of those particles, relative to the cell centre (units of L),
@@ -281,6 +284,7 @@ struct Lists {
   int* q_a[2];
   int* q_b[2];
   int* q_axis[2];
+  uint2* csr;               // the pairs by their first cell: (B, axis)
   unsigned int* p_toff;     // per pair: first task (i-tile) number, exclusive prefix
   unsigned int* s_toff;     // per self: first task number
   unsigned int* p_task;     // per pair task: its pair
@@ -288,7 +292,7 @@ struct Lists {
   uint2* p_live;            // pair tasks of the current pass that have work: (pair, cluster)
   unsigned int* n_live;     // their number
   int* counts;              // [0] selfs, [1] pairs, [2] queue 0 size, [3] queue 1 size, [4] sort segments,
-                            // [5] sort entries, [6] pair tasks, [7] self tasks
+                            // [5] sort entries, [6] pair tasks, [7] self tasks, [8] entries of csr
 };
 
 // Per-box counters kept by the pair kernels when counting is on.
