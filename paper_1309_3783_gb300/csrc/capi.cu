@@ -377,6 +377,7 @@ sph_status Engine::ensure_particle_capacity() {
   TL.active = tl_active.p;
   TL.changed = tl_changed.p;
   CK(dacc.reserve(n));
+  if (kahan()) CK(dcomp.reserve(n));
   CK(dcnt.reserve(n));
   CK(ghost4.reserve(n));
   CK(facc.reserve(n));

@@ -217,12 +217,6 @@ __device__ __forceinline__ bool gather_on(const int* gflag, const unsigned int* 
   return gflag[0] != 0 && *g_n <= cap_g;
 }
 
-__device__ __forceinline__ void flush_dens(int gidx, float4 acc, unsigned int cnt, float4* dacc, unsigned int* dcnt) {
-  if (gidx < 0 || cnt == 0) return;
-  atomicAdd(&dacc[gidx], acc);
-  atomicAdd(&dcnt[gidx], cnt);
-}
-
 template <bool COUNT>
 __device__ __forceinline__ void commit_counters(const Counters& C, unsigned long long* pc, int which) {
   if (!COUNT) return;
@@ -402,6 +396,9 @@ __device__ __forceinline__ f32x2 pack2(float a, float b) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
   return r;
 }
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
 __device__ __forceinline__ void unpack2(f32x2 v, unsigned int& a, unsigned int& b) {
   asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
 }
@@ -514,20 +511,45 @@ struct DensAcc {
       s.w += gg;
     }
   }
-  __device__ __forceinline__ float4 total() const {
-    return KAHAN ? make_float4(s.x + c.x, s.y + c.y, s.z + c.z, s.w + c.w) : s;
-  }
+  __device__ __forceinline__ float4 total() const { return make_float4(s.x + c.x, s.y + c.y, s.z + c.z, s.w + c.w); }
 };
+
+// A particle's sums added to its sums in global memory (dacc), its neighbours to
+// dcnt.  Compensated sums (dcomp given) carry the rounding of the additions in memory
+// too: an atomic addition returns what it found, so that its rounding error is known
+// exactly and is added to dcomp, which the ghost pass joins to the sums.
+__device__ __forceinline__ float two_sum_err(float a, float b) {
+  const float t = a + b, bb = t - a;
+  return (a - (t - bb)) + (b - bb);
+}
+
+template <bool KAHAN>
+__device__ __forceinline__ void flush_dens(int gidx, const DensAcc<KAHAN>& acc, unsigned int cnt, float4* dacc,
+                                           unsigned int* dcnt, float4* dcomp) {
+  if (gidx < 0 || cnt == 0) return;
+  if (KAHAN) {
+    const float4 x = acc.total();
+    const float4 o = atomicAdd(&dacc[gidx], x);
+    atomicAdd(&dcomp[gidx], make_float4(((acc.s.x - x.x) + acc.c.x) + two_sum_err(o.x, x.x),
+                                        ((acc.s.y - x.y) + acc.c.y) + two_sum_err(o.y, x.y),
+                                        ((acc.s.z - x.z) + acc.c.z) + two_sum_err(o.z, x.z),
+                                        ((acc.s.w - x.w) + acc.c.w) + two_sum_err(o.w, x.w)));
+  } else {
+    atomicAdd(&dacc[gidx], acc.s);
+  }
+  atomicAdd(&dcnt[gidx], cnt);
+}
 
 // r from r^2 by the fast reciprocal square root (its rounding enters the kernel's
 // argument only; the neighbour decision is taken on r^2).  The floor keeps r = 0
 // at 0 without a test; it is below any r^2 of distinct positions that matters to W
 // (r = 1e-19 L).
-__device__ __forceinline__ float pair_r(float r2) {
+__device__ __forceinline__ float rsqrt_floor(float r2) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(r2, 1.2e-38f)));
-  return r2 * y;
+  return y;
 }
+__device__ __forceinline__ float pair_r(float r2) { return r2 * rsqrt_floor(r2); }
 
 // One density contribution: w and q w'(q) at q = r / H, weighted by m.
 template <bool KAHAN>
@@ -544,10 +566,11 @@ __device__ __forceinline__ void dens_add(float r, float invH, float m, DensAcc<K
 // with everything read back from memory, so that the sweeps keep their registers.
 // column: this lane's staged partner against own lanes (bits of unc); else this
 // lane's own particle against staged partners.
+template <bool KAHAN>
 __device__ __noinline__ void dens_band(const DensShared& S, unsigned int unc, bool column,
                                        const unsigned int* __restrict__ perm, const double* __restrict__ x,
                                        const float4* __restrict__ pos4, const BoxDesc* __restrict__ box,
-                                       float4* dacc, unsigned int* dcnt) {
+                                       float4* dacc, unsigned int* dcnt, float4* dcomp) {
   const int lane = threadIdx.x & 31;
   const BoxDesc& bd = box[S.tk.box];
   const int gme = column ? S.g[lane] : S.ig[lane];
@@ -559,10 +582,80 @@ __device__ __noinline__ void dens_band(const DensShared& S, unsigned int unc, bo
     const int go = column ? S.ig[k] : S.g[k];
     if (!exact_less(gme, go, Hp, perm, x, bd.L, 0.5 * bd.L, bd.periodic)) continue;
     const float4 o = column ? S.ip[k] : make_float4(S.x[k], S.y[k], S.z[k], S.m[k]);
-    DensAcc<false> a;
+    DensAcc<KAHAN> a;
     dens_add(pair_r(pair_r2(me.x - o.x, me.y - o.y, me.z - o.z)), invH, o.w, a);
-    flush_dens(gme, a.total(), 1u, dacc, dcnt);
+    flush_dens(gme, a, 1u, dacc, dcnt, dcomp);
   }
+}
+
+// One sweep of a density batch: the lane's particle (at me, with 1/H) against the
+// partners of its mask, whose position and mass get(slot) gives.  Two partners per
+// turn, packed, so that most of the arithmetic takes one instruction for both; an odd
+// one's second partner, and those inside the guard band (set aside in unc, decided
+// afterwards), take q = 1, where w and w' vanish.
+template <bool KAHAN, class Get>
+__device__ __forceinline__ unsigned int dens_sweep(unsigned int mask, float3 me, float lo, float invH, Get get,
+                                                   DensAcc<KAHAN>& acc) {
+  const f32x2 nx = pack2(-me.x, -me.x), ny = pack2(-me.y, -me.y), nz = pack2(-me.z, -me.z), ih = pack2(invH, invH);
+  f32x2 s0 = 0, s1 = 0, s2 = 0, s3 = 0;     // (packed +0)
+  unsigned int unc = 0;
+#pragma unroll 1
+  for (unsigned int m = mask; m;) {
+    const int ja = __ffs(m) - 1;
+    m &= m - 1;
+    const bool two = m != 0;
+    const int jb = two ? __ffs(m) - 1 : ja;
+    m &= m - 1;
+    const float4 A = get(ja), B = get(jb);
+    const f32x2 dx = add2(pack2(A.x, B.x), nx), dy = add2(pack2(A.y, B.y), ny), dz = add2(pack2(A.z, B.z), nz);
+    const f32x2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+    float ra, rb;
+    unpack2(r2, ra, rb);
+    const bool ua = ra >= lo, ub = rb >= lo;
+    if (ua) unc |= 1u << ja;
+    if (ub && two) unc |= 1u << jb;
+    float qa, qb;
+    unpack2(mul2(mul2(r2, pack2(rsqrt_floor(ra), rsqrt_floor(rb))), ih), qa, qb);
+    qa = ua ? 1.0f : qa;
+    qb = ub || !two ? 1.0f : qb;
+    // spline_w_dw of both
+    const f32x2 q = pack2(qa, qb), one = pack2(1.0f, 1.0f);
+    const f32x2 om = fma2(q, pack2(-1.0f, -1.0f), one), q2 = mul2(q, q);
+    float wia, wib, wda, wdb, woa, wob, wea, web;
+    unpack2(fma2(mul2(q2, pack2(-6.0f, -6.0f)), om, one), wia, wib);                                   // 1 - 6q^2 + 6q^3
+    unpack2(mul2(q, fma2(q, pack2(18.0f, 18.0f), pack2(-12.0f, -12.0f))), wda, wdb);                   // -12q + 18q^2
+    const f32x2 o2 = mul2(om, om);
+    unpack2(mul2(mul2(o2, om), pack2(2.0f, 2.0f)), woa, wob);                                          // 2(1-q)^3
+    unpack2(mul2(o2, pack2(-6.0f, -6.0f)), wea, web);                                                  // -6(1-q)^2
+    const bool ia = qa < 0.5f, ib = qb < 0.5f;
+    const f32x2 w = pack2(ia ? wia : woa, ib ? wib : wob);
+    const f32x2 g = mul2(q, pack2(ia ? wda : wea, ib ? wdb : web));      // q w'(q) = r dW/dr in units of W
+    if (KAHAN) {
+      float wa, wb, ga, gb;
+      unpack2(w, wa, wb);
+      unpack2(g, ga, gb);
+      acc.add(A.w, wa, ga);
+      acc.add(B.w, wb, gb);
+    } else {
+      const f32x2 mm = pack2(A.w, B.w);
+      s0 = fma2(mm, w, s0);
+      s1 = fma2(mm, g, s1);
+      s2 = add2(s2, w);
+      s3 = add2(s3, g);
+    }
+  }
+  if (!KAHAN) {
+    float a, b;
+    unpack2(s0, a, b);
+    acc.s.x += a + b;
+    unpack2(s1, a, b);
+    acc.s.y += a + b;
+    unpack2(s2, a, b);
+    acc.s.z += a + b;
+    unpack2(s3, a, b);
+    acc.s.w += a + b;
+  }
+  return unc;
 }
 
 // Own side of a density batch: the lane walks its mask of staged partners.
@@ -570,20 +663,12 @@ template <bool KAHAN>
 __device__ __forceinline__ void dens_row(const DensI& I, float ilo, const DensShared& S, unsigned int ui,
                                          DensAcc<KAHAN>& acc,
                                          unsigned int& cnt, const unsigned int* perm, const double* x,
-                                         const float4* pos4, const BoxDesc* box, float4* dacc, unsigned int* dcnt) {
-  unsigned int unc = 0;
-#pragma unroll 1
-  for (unsigned int m = ui; m; m &= m - 1) {
-    const int sj = __ffs(m) - 1;
-    const float r2 = pair_r2(I.p.x - S.x[sj], I.p.y - S.y[sj], I.p.z - S.z[sj]);
-    if (r2 >= ilo) {
-      unc |= m & (0u - m);
-      continue;
-    }
-    dens_add(pair_r(r2), I.invH, S.m[sj], acc);
-  }
+                                         const float4* pos4, const BoxDesc* box, float4* dacc, unsigned int* dcnt,
+                                         float4* dcomp) {
+  const unsigned int unc = dens_sweep(
+      ui, I.p, ilo, I.invH, [&](int s) { return make_float4(S.x[s], S.y[s], S.z[s], S.m[s]); }, acc);
   cnt += __popc(ui & ~unc);
-  if (unc) dens_band(S, unc, false, perm, x, pos4, box, dacc, dcnt);
+  if (unc) dens_band<KAHAN>(S, unc, false, perm, x, pos4, box, dacc, dcnt, dcomp);
 }
 
 // The masks as exact decisions (counting and recording passes, which need them
@@ -619,7 +704,7 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
                                            DensAcc<KAHAN>& acc, unsigned int& cnt, const unsigned int* perm,
                                            const double* x, const float4* __restrict__ pos4,
                                            const BoxDesc* __restrict__ box, const float4* __restrict__ cen4,
-                                           float4* dacc, unsigned int* dcnt, Counters& C, const PairRec& R,
+                                           float4* dacc, unsigned int* dcnt, float4* dcomp, Counters& C, const PairRec& R,
                                            RecW& W) {
   const int lane = threadIdx.x & 31;
   const bool v = (unsigned int)lane < q;
@@ -665,25 +750,16 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   }
   S.m[lane] = jm;
   __syncwarp();
-  dens_row(I, ilo, S, ui, acc, cnt, perm, x, pos4, box, dacc, dcnt);
+  dens_row(I, ilo, S, ui, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
   // column sweep: partner side, staged partner = lane
   const unsigned int col = own_only ? 0u : transpose_bits(uj);
   if (col) {
     const float3 J = make_float3(S.x[lane], S.y[lane], S.z[lane]);
     DensAcc<KAHAN> pacc;
-    unsigned int unc = 0;
-#pragma unroll 1
-    for (unsigned int m = col; m; m &= m - 1) {
-      const float4 P = S.ip[__ffs(m) - 1];
-      const float r2 = pair_r2(P.x - J.x, P.y - J.y, P.z - J.z);
-      if (r2 >= jlo) {
-        unc |= m & (0u - m);
-        continue;
-      }
-      dens_add(pair_r(r2), jinvH, P.w, pacc);
-    }
-    flush_dens(S.g[lane], pacc.total(), __popc(col & ~unc), dacc, dcnt);
-    if (unc) dens_band(S, unc, true, perm, x, pos4, box, dacc, dcnt);
+    const unsigned int unc = dens_sweep(
+        col, J, jlo, jinvH, [&](int s) { return S.ip[s]; }, pacc);
+    flush_dens(S.g[lane], pacc, __popc(col & ~unc), dacc, dcnt, dcomp);
+    if (unc) dens_band<KAHAN>(S, unc, true, perm, x, pos4, box, dacc, dcnt, dcomp);
   }
   __syncwarp();
 }
@@ -1395,7 +1471,7 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
     const Lists& Lq, const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
     const float4* __restrict__ cen4, const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
     const unsigned char* __restrict__ act, const unsigned int* __restrict__ perm, const double* __restrict__ x,
-    float4* dacc, unsigned int* dcnt, DensShared& S, Counters& Cp, Counters& Cs, const PairRec& R, RecW& W) {
+    float4* dacc, unsigned int* dcnt, float4* dcomp, DensShared& S, Counters& Cp, Counters& Cs, const PairRec& R, RecW& W) {
   const int lane = threadIdx.x & 31;
   UnitShared& K = S.tk;
   unit_begin(K, ti, T, TL, box, part, parts);
@@ -1478,7 +1554,7 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
     }
     if (own_only || last || q + __popc(bal) > 32u || (COUNT && in_self != (Wk.it == K.selfit))) {
       if (q)
-        dens_batch<COUNT, PART, KAHAN, LISTED>(I, S, q, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt,
+        dens_batch<COUNT, PART, KAHAN, LISTED>(I, S, q, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt, dcomp,
                                                COUNT && in_self ? Cs : Cp, R, W);
       q = 0;
       own_only = false;
@@ -1498,12 +1574,11 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
       dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), make_float3(pj.x, pj.y, pj.z), pj.w, gj, aj);
     q += __popc(bal);
   }
-  float4 sum = acc.total();
   if (!KAHAN) {
     const float4 t = S.is[lane];
-    sum = make_float4(t.x + sum.x, t.y + sum.y, t.z + sum.z, t.w + sum.w);
+    acc.s = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
   }
-  flush_dens(I.g, sum, cnt, dacc, dcnt);
+  flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
   if (LISTED) rec_task_end(self ? R.stask : R.ptask, S);
 }
 
@@ -1659,7 +1734,8 @@ __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_B
                                                          const unsigned char* __restrict__ act,
                                                          const unsigned int* __restrict__ perm,
                                                          const double* __restrict__ x, float4* dacc,
-                                                         unsigned int* dcnt, unsigned long long* pc,
+                                                         unsigned int* dcnt, float4* dcomp,
+                                                         unsigned long long* pc,
                                                          unsigned int* __restrict__ task_ctr, int partial_host,
                                                          const int* __restrict__ it_dev, const int* __restrict__ gflag,
                                                          const unsigned int* __restrict__ g_n, unsigned int cap_g,
@@ -1696,7 +1772,7 @@ __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_B
     const bool self = REC && (un.x >> 31) != 0u;
     density_unit<COUNT, PART, KAHAN, REC>(REC ? un.y : un.x, REC ? 0u : un.y & 0xffffu, REC ? 1u : un.y >> 16, self,
                                           (int)(un.x & 0x7fffffffu), Lq, T, TL, box, pos4, cen4, sort_r, sort_i, act,
-                                          perm, x, dacc, dcnt, S, Cp, Cs, Rec, W);
+                                          perm, x, dacc, dcnt, dcomp, S, Cp, Cs, Rec, W);
     if (few && lane == 0) raw = atomicAdd(task_ctr, 1u);
   }
   commit_counters<COUNT>(Cp, pc, 0);
@@ -2048,7 +2124,7 @@ __device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsi
                                              const float4* __restrict__ cen4, DensAcc<KAHAN>& acc, unsigned int& cnt,
                                              const unsigned int* perm, const double* x,
                                              const float4* __restrict__ pos4, const BoxDesc* __restrict__ box,
-                                             float4* dacc, unsigned int* dcnt) {
+                                             float4* dacc, unsigned int* dcnt, float4* dcomp) {
   const int lane = threadIdx.x & 31;
   const bool v = (unsigned int)lane < q;
   __syncwarp();
@@ -2071,7 +2147,7 @@ __device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsi
   if (self)
     for (unsigned int b = m; b; b &= b - 1)
       if (S.g[__ffs(b) - 1] == I.g) m &= ~(b & (0u - b));
-  dens_row(I, ilo, S, m, acc, cnt, perm, x, pos4, box, dacc, dcnt);
+  dens_row(I, ilo, S, m, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
   __syncwarp();
 }
 
@@ -2084,7 +2160,7 @@ template <bool KAHAN>
 __device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tree& T, const Tiles& TL,
                                             const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
                                             const float4* __restrict__ cen4, const unsigned int* __restrict__ perm,
-                                            const double* __restrict__ x, float4* dacc, unsigned int* dcnt,
+                                            const double* __restrict__ x, float4* dacc, unsigned int* dcnt, float4* dcomp,
                                             const uint2* __restrict__ pk_info, const unsigned char* __restrict__ pk_n,
                                             const unsigned int* __restrict__ pk_idx, DensShared& S) {
   const int lane = threadIdx.x & 31;
@@ -2152,15 +2228,15 @@ __device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tre
       const unsigned int bal = __ballot_sync(0xffffffffu, pass);
       const unsigned int np = __popc(bal);
       if (q + np > 32u) {
-        gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt);
+        gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
         q = 0;
       }
       if (pass) dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), pj, r.w, gj, true);
       q += np;
     }
   }
-  if (q) gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt);
-  flush_dens(I.g, acc.total(), cnt, dacc, dcnt);
+  if (q) gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
+  flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
 }
 
 #ifndef GATHER_BLOCKS
@@ -2173,7 +2249,7 @@ template <bool KAHAN>
 __global__ void __launch_bounds__(SPH_THREADS, GATHER_BLOCKS) k_density_gather(
     Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
     const float4* __restrict__ cen4, const unsigned int* __restrict__ perm, const double* __restrict__ x,
-    float4* dacc, unsigned int* dcnt, const uint2* __restrict__ tasks, unsigned int* __restrict__ g_n,
+    float4* dacc, unsigned int* dcnt, float4* dcomp, const uint2* __restrict__ tasks, unsigned int* __restrict__ g_n,
     unsigned int cap_g, const int* __restrict__ gflag, const uint2* __restrict__ pk_info,
     const unsigned char* __restrict__ pk_n, const unsigned int* __restrict__ pk_idx,
     unsigned int* __restrict__ task_ctr) {
@@ -2187,7 +2263,7 @@ __global__ void __launch_bounds__(SPH_THREADS, GATHER_BLOCKS) k_density_gather(
   unsigned int t = 0;
   if (lane == 0) t = atomicAdd(task_ctr, 1u);
   for (t = __shfl_sync(0xffffffffu, t, 0); t < ntask; t = __shfl_sync(0xffffffffu, t, 0)) {
-    gather_task<KAHAN>(tasks[t], Lq, T, TL, box, pos4, cen4, perm, x, dacc, dcnt, pk_info, pk_n, pk_idx, S);
+    gather_task<KAHAN>(tasks[t], Lq, T, TL, box, pos4, cen4, perm, x, dacc, dcnt, dcomp, pk_info, pk_n, pk_idx, S);
     if (lane == 0) t = atomicAdd(task_ctr, 1u);
   }
 }
@@ -2200,7 +2276,8 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
                         float gamma_k, float n_ngb, float tol,
                         float gamma_gas, const unsigned int* __restrict__ perm, float* __restrict__ Hs,
                         float4* __restrict__ pos4, const float4* __restrict__ cen4, const float4* __restrict__ vel4,
-                        const float4* __restrict__ dacc, unsigned char* __restrict__ act, float* __restrict__ h,
+                        float4* __restrict__ dacc, const float4* __restrict__ dcomp, unsigned char* __restrict__ act,
+                        float* __restrict__ h,
                         float* __restrict__ hlo, float* __restrict__ hhi, int* __restrict__ conv,
                         const float* __restrict__ hlimp, const unsigned int* __restrict__ leaf_of, Tree T,
                         float4* __restrict__ ghost4, float4* __restrict__ hhist, int* __restrict__ n_active,
@@ -2214,7 +2291,12 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
     const unsigned int i = perm[p];
     const float H = Hs[p];
     const float m = cen4[p].w;
-    const float4 a = dacc[p];
+    float4 a = dacc[p];
+    if (dcomp) {      // compensated sums: the rounding of their additions
+      const float4 c = dcomp[p];
+      a = make_float4(a.x + c.x, a.y + c.y, a.z + c.z, a.w + c.w);
+      dacc[p] = a;
+    }
     const float sw = a.z + 1.0f;          // self term w(0) = 1
     const float Nw = (32.0f / 3.0f) * sw; // (4 pi / 3) H^3 n with n = (8/pi) sum w / H^3
     const float F = Nw - n_ngb;
@@ -2275,12 +2357,13 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
 }
 
 __global__ void k_zero_active(long long N, const unsigned char* __restrict__ act, float4* __restrict__ dacc,
-                              unsigned int* __restrict__ dcnt, int all) {
+                              unsigned int* __restrict__ dcnt, float4* __restrict__ dcomp, int all) {
   pdl_wait();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     if (all || act[p]) {
       dacc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
       dcnt[p] = 0;
+      if (dcomp) dcomp[p] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
 }
@@ -2738,8 +2821,7 @@ void launch_density(Engine& E, const int* it_dev, int only) {
   for (int part = 0; part < 2; ++part) {
     if (!it_dev && part != (E.partial_pass ? 1 : 0)) continue;
     if (it_dev && only >= 0 && part != only) continue;
-    // compensated sums when asked, or (compensated < 0) from 100 neighbours on
-    const bool kahan = E.prm.compensated > 0 || (E.prm.compensated < 0 && E.prm.n_ngb >= 100.0f);
+    const bool kahan = E.kahan();
     // the first pass records its pairs for the force pass when the records are on
     const bool rec = part == 0 && E.rec_valid;
     decltype(&k_density<false, false, false, false>) k;
@@ -2755,7 +2837,7 @@ void launch_density(Engine& E, const int* it_dev, int only) {
                                 : (rec ? k_density<false, false, false, true> : k_density<false, false, false, false>));
     launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st,
         E.Lq, E.T, E.TL, E.box.p, E.pos4.p, E.cen4.p, E.sort_r.p, E.sort_i.p, E.act.p, E.perm.p, E.x.p, E.dacc.p,
-        E.dcnt.p, E.pc.p, E.task_ctr.p + part, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr, E.g_n.p,
+        E.dcnt.p, E.dcomp.p, E.pc.p, E.task_ctr.p + part, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr, E.g_n.p,
         (unsigned int)E.g_live.n, (unsigned int)(E.gcap ? E.N : E.n_tiles),
         E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr,
         E.unit_list ? E.units.p : nullptr, E.n_units.p, (unsigned int)E.units.n, E.rec_for_force());
@@ -2789,11 +2871,11 @@ void launch_gather_prep(Engine& E, const int* it_dev) {
 
 // The gathered density pass; returns at once unless the pass gathers.
 void launch_density_gather(Engine& E) {
-  const bool kahan = E.prm.compensated > 0 || (E.prm.compensated < 0 && E.prm.n_ngb >= 100.0f);
+  const bool kahan = E.kahan();
   const auto k = kahan ? k_density_gather<true> : k_density_gather<false>;
   cudaMemsetAsync(E.task_ctr.p + 3, 0, sizeof(unsigned int), E.st);
   launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st, E.Lq, E.T, E.TL, E.box.p, E.pos4.p,
-             E.cen4.p, E.perm.p, E.x.p, E.dacc.p, E.dcnt.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n,
+             E.cen4.p, E.perm.p, E.x.p, E.dacc.p, E.dcnt.p, E.dcomp.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n,
              E.gflag.p, E.pk_info.p, E.pk_n.p, E.pk_idx.p, E.task_ctr.p + 3);
   count_launch();
 }
@@ -2826,13 +2908,13 @@ void launch_unit_list(Engine& E) {
 void launch_ghost(Engine& E, int mode, int it, const int* it_dev) {
   launch_pdl(k_ghost, E.grid(E.N), 256, E.st, E.N, mode, it, it_dev, E.prm.h_max_iter, E.prm.gamma_kernel, E.prm.n_ngb,
                                           E.prm.h_tol, E.prm.gamma_gas, E.perm.p, E.Hs.p, E.pos4.p, E.cen4.p,
-                                          E.vel4.p, E.dacc.p, E.act.p, E.h.p, E.hlo.p, E.hhi.p, E.conv.p,
+                                          E.vel4.p, E.dacc.p, E.dcomp.p, E.act.p, E.h.p, E.hlo.p, E.hhi.p, E.conv.p,
                                           E.hlimp.p, E.leaf_of.p, E.T, E.ghost4.p, E.hhist.p, E.dev_counters.p,
                                           E.err_all.p); count_launch();
 }
 
 void launch_zero_density(Engine& E, bool all) {
-  launch_pdl(k_zero_active, E.grid(E.N), 256, E.st, E.N, E.act.p, E.dacc.p, E.dcnt.p, all ? 1 : 0); count_launch();
+  launch_pdl(k_zero_active, E.grid(E.N), 256, E.st, E.N, E.act.p, E.dacc.p, E.dcnt.p, E.dcomp.p, all ? 1 : 0); count_launch();
 }
 
 void launch_set_active(Engine& E) {

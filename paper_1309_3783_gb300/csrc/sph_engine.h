@@ -234,6 +234,9 @@ class Engine {
 
   // pass results (sorted order)
   DBuf<float4> dacc;              // sum m w, sum m q w', sum w, sum q w'
+  DBuf<float4> dcomp;             // the rounding errors of their additions (compensated sums)
+  // compensated sums when asked, or (compensated < 0) from 100 neighbours on
+  bool kahan() const { return prm.compensated > 0 || (prm.compensated < 0 && prm.n_ngb >= 100.0f); }
   DBuf<unsigned int> dcnt;
   DBuf<float4> ghost4;            // rho, f P / rho^2, c, f
   DBuf<float4> facc;              // a (3), du/dt
