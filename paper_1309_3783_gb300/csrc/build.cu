@@ -1084,21 +1084,158 @@ __global__ void k_shift(long long N, int box_shift, const unsigned long long* __
 }
 
 // ============================================================== clusters
-// Inside every leaf, put the particles whose H exceeds the leaf edge after the
-// others (stable), so that warp-sized clusters hold particles of similar reach.
-// lsrc[p] = the particle that moves to position p.
-__global__ void k_leaf_partition(Tree T, int nnodes, const BoxDesc* __restrict__ box, const float* __restrict__ Hs,
-                                 unsigned int* __restrict__ lsrc) {
+// Sorts 32 I values, value 32 i + lane in v[i] (bitonic, in registers).
+template <int I>
+__device__ __forceinline__ void warp_sort(unsigned int (&v)[I]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 2; k <= 32 * I; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll
+      for (int i = 0; i < I; ++i) {
+        const bool up = ((32 * i + lane) & k) == 0;
+        if (j >= 32) {
+          const int p = i ^ (j >> 5);
+          if (p > i) {
+            const unsigned int a = min(v[i], v[p]), b = max(v[i], v[p]);
+            v[i] = up ? a : b;
+            v[p] = up ? b : a;
+          }
+        } else {
+          const unsigned int y = __shfl_xor_sync(0xffffffffu, v[i], j);
+          v[i] = ((lane & j) == 0) == up ? min(v[i], y) : max(v[i], y);
+        }
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ int high_bit(unsigned long long v) { return v ? 63 - __clzll((long long)v) : -1; }
+
+// Per warp: the particles of the node being divided -- position relative to the leaf
+// centre (units of L) and source index.
+struct NodeShared {
+  float x[3][128];
+  unsigned int src[128];
+};
+
+// The longest axis of particles id[0 .. n) of the node, and their range along it.
+template <int I>
+__device__ __forceinline__ int node_axis(const NodeShared& S, const unsigned int (&v)[I], int r0, int r1, float& lo,
+                                         float& scale) {
+  const int lane = threadIdx.x & 31;
+  float a[3], b[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    a[k] = FLT_MAX;
+    b[k] = -FLT_MAX;
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+      const int r = 32 * i + lane;
+      if (r < r0 || r >= r1) continue;
+      const float t = S.x[k][v[i] & 127u];
+      a[k] = fminf(a[k], t);
+      b[k] = fmaxf(b[k], t);
+    }
+    a[k] = warp_min(a[k]);
+    b[k] = warp_max(b[k]);
+  }
+  int ax = 0;
+  if (b[1] - a[1] > b[0] - a[0]) ax = 1;
+  if (b[2] - a[2] > b[ax] - a[ax]) ax = 2;
+  lo = a[ax];
+  scale = b[ax] > a[ax] ? 1.0f / (b[ax] - a[ax]) : 0.0f;
+  return ax;
+}
+
+// The order of a node's n particles (n <= 32 I) and its clusters: k = ceil(n / cmax)
+// of them, by halving along the longest axis (a third first when k = 3), each part
+// along its own.  v[i] on return: the particle at place 32 i + lane (low 7 bits).
+template <int I>
+__device__ __forceinline__ void divide_node(const NodeShared& S, int n, int cmax, unsigned int* __restrict__ lsrc,
+                                            unsigned int* __restrict__ flag) {
+  const int lane = threadIdx.x & 31;
+  const int k = (n + cmax - 1) / cmax;
+  unsigned int v[I];
+#pragma unroll
+  for (int i = 0; i < I; ++i) v[i] = (unsigned int)(32 * i + lane);
+  float lo, sc;
+  int ax = node_axis(S, v, 0, n, lo, sc);
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    const int r = 32 * i + lane;
+    v[i] = r < n ? ((unsigned int)((S.x[ax][r] - lo) * sc * 16777215.0f) << 7) | (unsigned int)r : 0xffffffffu;
+  }
+  warp_sort(v);
+  const int nl = k == 3 ? (n + 2) / 3 : (n + 1) / 2;      // the left part
+  int c1 = nl, c2 = n, c3 = n;                            // starts of the clusters after the first
+  if (k > 2) {
+    float lo1, sc1;
+    const int ax0 = node_axis(S, v, 0, nl, lo, sc), ax1 = node_axis(S, v, nl, n, lo1, sc1);
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+      const int r = 32 * i + lane;
+      const unsigned int id = v[i] & 127u;
+      const bool right = r >= nl;
+      if (r < n)
+        v[i] = (right ? 0x80000000u : 0u) |
+               ((unsigned int)((right ? (S.x[ax1][id] - lo1) * sc1 : (S.x[ax0][id] - lo) * sc) * 16777215.0f) << 7) | id;
+      else
+        v[i] = 0xffffffffu;
+    }
+    warp_sort(v);
+    if (k == 3) {
+      c2 = nl + (n - nl + 1) / 2;
+    } else {
+      c1 = (nl + 1) / 2;
+      c2 = nl;
+      c3 = nl + (n - nl + 1) / 2;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    const int r = 32 * i + lane;
+    if (r >= n) continue;
+    lsrc[r] = S.src[v[i] & 127u];
+    flag[r] = r == 0 || r == c1 || r == c2 || r == c3 ? 1u : 0u;
+  }
+}
+
+// The order of every leaf's particles and its clusters (flag[p] = 1 where one
+// starts; lsrc[p] = the particle that moves to position p).  The particles whose H
+// exceeds the leaf edge come after the others, so that clusters hold particles of
+// similar reach.  Each of the two classes is cut along its Morton keys into the
+// largest nodes (the keys that agree from some bit up) of at most 4 cmax particles
+// (cmax: the cluster size, at most 32: a warp's lanes), and a node of more than cmax
+// into as few clusters as hold it, by its particles' positions.  Nodes of at most cmax
+// particles as clusters (boxes as compact, but 21 of 32 lanes filled on average
+// against 27 here) made the interaction passes 10-20 % slower.  Walking a class from
+// its first particle a, the next node is the largest that starts at a and fits: its
+// bit b* is the smallest of the highest bits in which key[a] differs from key[a - 1]
+// (the node must start at a) and from key[a + 4 cmax] (it must end before).  One
+// warp per leaf.
+constexpr int CLUSTER_WARPS = 4;
+
+__global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
+    Tree T, int nnodes, int box_shift, const BoxDesc* __restrict__ box, const float* __restrict__ Hs,
+    const unsigned long long* __restrict__ key, const unsigned int* __restrict__ perm, const double* __restrict__ x,
+    unsigned int* lsrc, unsigned int* __restrict__ flag, int cmax) {
   pdl_wait();
+  __shared__ NodeShared SH[CLUSTER_WARPS];
   nnodes = min(nnodes, T.n_nodes[0]);
   const int lane = threadIdx.x & 31;
+  NodeShared& S = SH[threadIdx.x >> 5];
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   const unsigned int lt = (1u << lane) - 1u;
+  const unsigned int cap = 4u * (unsigned int)cmax;
   for (int id = warp; id < nnodes; id += nwarps) {
     if (T.child[id] >= 0) continue;
     const unsigned int s = T.start[id], c = T.count[id];
-    const float thr = (float)ldexp(box[T.box[id]].L, -T.level[id]);
+    const BoxDesc& bd = box[T.box[id]];
+    const int d = T.level[id];
+    const float thr = (float)ldexp(bd.L, -d);
     unsigned int nsmall = 0;
     for (unsigned int b = 0; b < c; b += 32) {
       const unsigned int q = b + lane;
@@ -1118,6 +1255,51 @@ __global__ void k_leaf_partition(Tree T, int nnodes, const BoxDesc* __restrict__
       os += __popc(bs);
       ol += __popc(bl);
     }
+    __syncwarp();
+    const int lb = box_shift - 3 * d;      // key bits below the leaf's cell
+    unsigned int cx, cy, cz;
+    cell_coords(T.key[id], d, cx, cy, cz);
+    const double inv = ldexp(1.0, -d), iL = bd.invL;
+    const double cen[3] = {((double)cx + 0.5) * inv, ((double)cy + 0.5) * inv, ((double)cz + 0.5) * inv};
+    for (int cls = 0; cls < 2; ++cls) {
+      const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
+      unsigned int a = beg;
+      while (a < end) {
+        const unsigned long long ka = key[lsrc[a]];
+        int bs = lb;
+        if (a > beg) bs = min(bs, high_bit(key[lsrc[a - 1]] ^ ka));
+        if (a + cap < end) bs = min(bs, high_bit(ka ^ key[lsrc[a + cap]]));
+        unsigned int n = min(cap, end - a);   // equal keys (bs < 0): no node starts here, take a chunk
+        if (bs >= 0) {
+          unsigned int m = 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const unsigned int q = 32u * i + lane;
+            m += __popc(__ballot_sync(0xffffffffu, q < n && ((key[lsrc[a + q]] ^ ka) >> bs) == 0ull));
+          }
+          n = m;      // (the node's particles are adjacent)
+        }
+        if (n <= (unsigned int)cmax) {
+          if ((unsigned int)lane < n) flag[a + lane] = lane == 0 ? 1u : 0u;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const unsigned int q = 32u * i + lane;
+            if (q >= n) break;
+            const unsigned int src = lsrc[a + q];
+            const long long p = perm[src];
+            S.src[q] = src;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) S.x[k][q] = (float)(x[3 * p + k] * iL - cen[k]);
+          }
+          __syncwarp();
+          if (n <= 64u) divide_node<2>(S, (int)n, cmax, lsrc + a, flag + a);
+          else divide_node<4>(S, (int)n, cmax, lsrc + a, flag + a);
+          __syncwarp();
+        }
+        a += n;
+      }
+    }
   }
 }
 
@@ -1133,60 +1315,6 @@ __global__ void k_apply_partition(long long N, const unsigned int* __restrict__ 
     key_out[p] = key_in[q];
     H_out[p] = H_in[q];
     vel_out[p] = vel_in[q];
-  }
-}
-
-// flag[p] = 1 where a cluster starts.  Inside each leaf, separately for its two
-// H classes, the clusters are the leaves of a binary split of the class along
-// its Morton keys: a node (the keys that agree on every bit from some bit b up)
-// is halved at bit b - 1 while it holds more than cmax particles (the cluster
-// size, at most 32: a warp's lanes).  Each cluster is then an aligned box of
-// aspect ratio at most 2, much tighter than cmax particles taken in Morton order,
-// which often straddle octants.  Walking a class from its first particle a, the
-// next cluster is the largest node that starts at a and holds at most cmax
-// particles: its bit b* is the smallest of the highest bits in which key[a]
-// differs from key[a - 1] (the node must start at a) and from key[a + cmax] (it
-// must end before a + cmax).  One warp per leaf.
-__device__ __forceinline__ int high_bit(unsigned long long v) { return v ? 63 - __clzll((long long)v) : -1; }
-
-__global__ void k_tile_flags(Tree T, int nnodes, int box_shift, const BoxDesc* __restrict__ box,
-                             const float* __restrict__ Hs, const unsigned long long* __restrict__ key,
-                             unsigned int* __restrict__ flag, int cmax) {
-  pdl_wait();
-  nnodes = min(nnodes, T.n_nodes[0]);
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int id = warp; id < nnodes; id += nwarps) {
-    if (T.child[id] >= 0) continue;
-    const unsigned int s = T.start[id], c = T.count[id];
-    const float thr = (float)ldexp(box[T.box[id]].L, -T.level[id]);
-    unsigned int nsmall = 0;
-    for (unsigned int b = 0; b < c; b += 32) {
-      const unsigned int q = b + lane;
-      nsmall += __popc(__ballot_sync(0xffffffffu, q < c && !(Hs[s + q] > thr)));
-    }
-    const int lb = box_shift - 3 * T.level[id];      // key bits below the leaf's cell
-    for (int cls = 0; cls < 2; ++cls) {
-      const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
-      unsigned int a = beg;
-      while (a < end) {
-        const unsigned long long ka = key[a];
-        int bs = lb;
-        if (a > beg) bs = min(bs, high_bit(key[a - 1] ^ ka));
-        if (a + cmax < end) bs = min(bs, high_bit(ka ^ key[a + cmax]));
-        unsigned int n;
-        if (bs < 0) {
-          n = min((unsigned int)cmax, end - a);   // equal keys: no node starts here, take a chunk
-        } else {
-          const unsigned int q = a + 1 + lane;
-          const bool in = lane < cmax - 1 && q < end && ((key[q] ^ ka) >> bs) == 0ull;
-          n = 1u + __popc(__ballot_sync(0xffffffffu, in));
-        }
-        if ((unsigned int)lane < n) flag[a + lane] = lane == 0 ? 1u : 0u;
-        a += n;
-      }
-    }
   }
 }
 

@@ -49,12 +49,11 @@ __global__ void k_sort_big_keys(int, const int*, const int*, const unsigned int*
                                 unsigned int*, const unsigned long long*, int);
 __global__ void k_sort_big_scatter(int, const int*, const int*, const unsigned int*, Tree, Tiles,
                                    const unsigned int*, float*, unsigned int*, const unsigned long long*, int);
-__global__ void k_leaf_partition(Tree, int, const BoxDesc*, const float*, unsigned int*);
+__global__ void k_leaf_clusters(Tree, int, int, const BoxDesc*, const float*, const unsigned long long*,
+                                const unsigned int*, const double*, unsigned int*, unsigned int*, int);
 __global__ void k_apply_partition(long long, const unsigned int*, const unsigned int*, unsigned int*,
                                   const unsigned long long*, unsigned long long*, const float*, float*,
                                   const float4*, float4*);
-__global__ void k_tile_flags(Tree, int, int, const BoxDesc*, const float*, const unsigned long long*,
-                             unsigned int*, int);
 __global__ void k_tile_table(long long, Tree, const unsigned int*, const unsigned int*, const unsigned int*,
                              const float4*, unsigned int*, Tiles, int);
 __global__ void k_cell_tiles(Tree, int, const unsigned int*);
@@ -682,8 +681,9 @@ sph_status Engine::build_once(bool* retry) {
   cudaStream_t ss = st_side;
   ev = prof_begin(PH_SHIFT, &l0, ss);
   launch_pdl(k_leaves, nsm * 8, 256, ss, T, n_nodes, leaf_of.p); count_launch();
-  // particles of each leaf: the ones with H above the leaf edge last (stable)
-  launch_pdl(k_leaf_partition, nsm * 8, 256, ss, T, n_nodes, box.p, Hs.p, lsrc.p); count_launch();
+  // the order of each leaf's particles and its clusters (at most 32 particles each)
+  launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, n_nodes, box_shift, box.p, Hs.p, key.p, perm.p, x.p, lsrc.p, tflag.p,
+             prm.cluster_max); count_launch();
   launch_pdl(k_apply_partition, grid(N), 256, ss, N, lsrc.p, perm.p, perm_tmp.p, key.p, key_tmp.p, Hs.p, Hs_tmp.p,
              vel4.p, vel4_tmp.p); count_launch();
   perm.swap(perm_tmp);
@@ -692,9 +692,6 @@ sph_status Engine::build_once(bool* retry) {
   vel4.swap(vel4_tmp);
   launch_pdl(k_shift, grid(N), 256, ss, N, box_shift, key.p, perm.p, leaf_of.p, T, box.p, x.p, m.p, Hs.p, pos4.p,
              cen4.p); count_launch();
-  // clusters of at most 32 particles inside each leaf
-  launch_pdl(k_tile_flags, nsm * 8, 256, ss, T, n_nodes, box_shift, box.p, Hs.p, key.p, tflag.p, prm.cluster_max);
-  count_launch();
   exclusive_scan(tflag.p, texcl.p, N, rs_scratch.p, reinterpret_cast<unsigned int*>(dev_counters.p + 4), ss);
   launch_pdl(k_tile_table, grid(N), 256, ss, N, T, leaf_of.p, tflag.p, texcl.p, pos4.p, tile_of.p, TL, prm.cluster_max);
   count_launch();
@@ -1514,7 +1511,8 @@ sph_status Engine::enqueue_captured_build() {
   cudaStream_t ss = st_side;
   ev = prof_begin(PH_SHIFT, &l0, ss);
   launch_pdl(k_leaves, nsm * 8, 256, ss, T, cap_nodes, leaf_of.p); count_launch();
-  launch_pdl(k_leaf_partition, nsm * 8, 256, ss, T, cap_nodes, box.p, Hs.p, lsrc.p); count_launch();
+  launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, cap_nodes, box_shift, box.p, Hs.p, key.p, perm.p, x.p, lsrc.p,
+             tflag.p, prm.cluster_max); count_launch();
   launch_pdl(k_apply_partition, grid(N), 256, ss, N, lsrc.p, perm.p, perm_tmp.p, key.p, key_tmp.p, Hs.p, Hs_tmp.p,
              vel4.p, vel4_tmp.p); count_launch();
   perm.swap(perm_tmp);
@@ -1523,8 +1521,6 @@ sph_status Engine::enqueue_captured_build() {
   vel4.swap(vel4_tmp);
   launch_pdl(k_shift, grid(N), 256, ss, N, box_shift, key.p, perm.p, leaf_of.p, T, box.p, x.p, m.p, Hs.p, pos4.p,
              cen4.p); count_launch();
-  launch_pdl(k_tile_flags, nsm * 8, 256, ss, T, cap_nodes, box_shift, box.p, Hs.p, key.p, tflag.p, prm.cluster_max);
-  count_launch();
   exclusive_scan(tflag.p, texcl.p, N, rs_scratch.p, reinterpret_cast<unsigned int*>(dev_counters.p + 4), ss);
   launch_pdl(k_tile_table, grid(N), 256, ss, N, T, leaf_of.p, tflag.p, texcl.p, pos4.p, tile_of.p, TL,
              prm.cluster_max); count_launch();
