@@ -297,6 +297,7 @@ __device__ __forceinline__ void rec_task_end(uint2* slots, const DensShared& S) 
 // with its position, H and index (as in the density pass); its velocity and ghost
 // quantities are loaded once per batch by the slot's lane, before the masks, and
 // written after them.  8 blocks of 4 warps fit an SM's shared memory.
+constexpr unsigned int PLIST_CAP = 320;    // pairs listed at once (a batch with more runs in several goes)
 struct __align__(16) ForceShared {
   float x[32], y[32], z[32];
   float hi[32], lo[32];  // H^2 +- guard band (units of L^2); hi = -1 marks an empty slot
@@ -315,7 +316,7 @@ struct __align__(16) ForceShared {
   UnitShared tk;
   float4 cb[32];         // partner-side terms of one round, by lane
   float cv[32];          //   signal velocities
-  unsigned short plist[32];   // the round's pairs: own lane | slot << 5
+  unsigned char plist[PLIST_CAP];   // the batch's pairs, own lane major: slot, bit 5: the first of its row
   unsigned int own0;     // the own cluster's first particle
 };
 
@@ -764,45 +765,50 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   __syncwarp();
 }
 
-// What one side of a force pair needs of a particle: position, velocity, rho,
-// f P / rho^2, sound speed, K/H^4, 1/H and mass.
-struct ForceSide {
-  float3 v;
-  float rho, F, c, K4, invH, m;
-};
-
-// Both sides of one force pair, a (own particle) and b (partner), d = x_a - x_b:
-// a gains ca, b gains cb (the antisymmetric acceleration terms and each side's
-// du/dt), both see vsig.  No contribution when r = 0.  A side's kernel gradient
-// is taken inside its support (q < 1) and is zero outside; at q = 1 it is zero
-// too, so the FP32 test agrees with the exact one to within the gradient's size
-// there, about 6 (1 - q)^2 for q within rounding of 1.
-__device__ __forceinline__ void force_pair_terms(const ForceSide& a, const ForceSide& b, float dx, float dy, float dz,
-                                                 float r2, float alpha, float4& ca, float4& cb, float& vsig) {
+// Both sides of one force pair, a (own particle: mass ma, VA = velocity and rho, FA =
+// 1/H, f P / rho^2, c, K/H^4) and b (partner: VB = velocity and mass, FB = rho, f P /
+// rho^2, c, K/H^4, and 1/H), d = x_a - x_b: a gains ca, b gains cb (the antisymmetric
+// acceleration terms and each side's du/dt), both see vsig.  No contribution when r =
+// 0.  A side's kernel gradient is taken inside its support and is zero outside (q
+// clamped to 1, where it is zero too: the FP32 test agrees with the exact one to within
+// the gradient's size there, about 6 (1 - q)^2 for q within rounding of 1).  The two
+// sides' kernels are evaluated packed.
+__device__ __forceinline__ void force_pair_terms(float ma, const float4& VA, const float4& FA, const float4& VB,
+                                                 const float4& FB, float invHb, float dx, float dy, float dz, float r2,
+                                                 float alpha, float4& ca, float4& cb, float& vsig) {
   ca = make_float4(0.f, 0.f, 0.f, 0.f);
   cb = ca;
   vsig = 0.0f;
   if (!(r2 > 0.0f)) return;
   const float rinv = rsqrtf(r2);
   const float r = r2 * rinv;
-  float w, dwa, dwb;
-  const float qa = r * a.invH, qb = r * b.invH;
-  spline_w_dw(qa, w, dwa);
-  spline_w_dw(qb, w, dwb);
-  dwa = qa < 1.0f ? dwa : 0.0f;
-  dwb = qb < 1.0f ? dwb : 0.0f;
-  const float Wa = a.K4 * dwa, Wb = b.K4 * dwb;
-  const float vdx = fmaf(a.v.x - b.v.x, dx, fmaf(a.v.y - b.v.y, dy, (a.v.z - b.v.z) * dz));
+  float qa, qb;
+  unpack2(mul2(pack2(r, r), pack2(FA.x, invHb)), qa, qb);
+  qa = fminf(qa, 1.0f);
+  qb = fminf(qb, 1.0f);
+  const f32x2 q = pack2(qa, qb);
+  const f32x2 om = fma2(q, pack2(-1.0f, -1.0f), pack2(1.0f, 1.0f));
+  float ia, ib, oa, ob;
+  unpack2(mul2(q, fma2(q, pack2(18.0f, 18.0f), pack2(-12.0f, -12.0f))), ia, ib);   // -12q + 18q^2
+  unpack2(mul2(mul2(om, om), pack2(-6.0f, -6.0f)), oa, ob);                         // -6(1-q)^2
+  const f32x2 W = mul2(pack2(FA.w, FB.w), pack2(qa < 0.5f ? ia : oa, qb < 0.5f ? ib : ob));
+  const f32x2 FW = mul2(pack2(FA.y, FB.y), W);
+  float Wa, Wb, FWa, FWb;
+  unpack2(W, Wa, Wb);
+  unpack2(FW, FWa, FWb);
+  const float vdx = fmaf(VA.x - VB.x, dx, fmaf(VA.y - VB.y, dy, (VA.z - VB.z) * dz));
   const float wv = vdx * rinv;
   const float mu = fminf(wv, 0.0f);
-  vsig = a.c + b.c - 3.0f * mu;
-  const float Pi = __fdividef(-alpha * vsig * mu, a.rho + b.rho);
-  const float Wbar = 0.5f * (Wa + Wb);
-  const float coef = fmaf(a.F, Wa, fmaf(b.F, Wb, Pi * Wbar)) * rinv;
-  const float hv = 0.5f * Pi * Wbar;
-  const float ka = -b.m * coef, kb = a.m * coef;
-  ca = make_float4(ka * dx, ka * dy, ka * dz, b.m * fmaf(a.F, Wa, hv) * wv);
-  cb = make_float4(kb * dx, kb * dy, kb * dz, a.m * fmaf(b.F, Wb, hv) * wv);
+  vsig = FA.z + FB.z - 3.0f * mu;
+  const float Pi = __fdividef(-alpha * vsig * mu, VA.w + FB.x);
+  const float PW = Pi * (0.5f * (Wa + Wb));
+  const float coef = ((FWa + FWb) + PW) * rinv;
+  const float hv = 0.5f * PW;
+  const float ka = -VB.w * coef, kb = ma * coef;
+  float ea, eb;
+  unpack2(mul2(mul2(add2(FW, pack2(hv, hv)), pack2(wv, wv)), pack2(VB.w, ma)), ea, eb);
+  ca = make_float4(ka * dx, ka * dy, ka * dz, ea);
+  cb = make_float4(kb * dx, kb * dy, kb * dz, eb);
 }
 
 // Sums (v) and maxima (m) over runs of adjacent lanes with the same key, no run
@@ -851,14 +857,19 @@ struct ForceArgs {
 
 // The pairs of one batch (mask m of the lane's own particle over the staged
 // slots), each evaluated once for both sides.  The pairs form a list, own lane
-// major, which the warp takes 32 at a time, one pair per lane, so that all lanes
-// work however unevenly the pairs fall on the rows (each lane taking its own next
-// pair while most have one left, the own side in registers, measured 5 % slower).
-// The own side is summed by a segmented warp reduction (a particle's pairs are
-// adjacent in the list); the partner side's terms go through shared memory, where
-// the first of each partner's lanes adds them up, to the partner's batch sums (or,
-// inside one cluster, to that particle's task sums).  Shared-memory float atomics
-// are slow, the more so where lanes collide.
+// major, of which every lane takes an equal run, so that all lanes work however
+// unevenly the pairs fall on the rows.  Own side: a lane's run mostly stays in one
+// row, whose terms it sums in registers; where a row ends inside a run, the sum goes
+// to the row's task sums (only one lane sees a row end), and what is left at the end
+// is summed over adjacent lanes (rounds of 32 consecutive pairs, each with a
+// segmented reduction, took 60 instructions more per round; each lane taking its own
+// next pair while most have one left was slower still).  Partner side: the terms go
+// through shared memory, where the first of each partner's lanes adds them up, to the
+// partner's batch sums (or, inside one cluster, to that particle's task sums).
+// Shared-memory float atomics are slow, the more so where lanes collide.
+// With the two sides' kernels packed (force_pair_terms): force pass of 33.5M clustered
+// particles 38.7 -> 36.6 ms (at wide supports 78.9 -> 68.1), of the 1M open lattice
+// 0.85 -> 0.72 ms, of 4096 particles 38 -> 33 us.
 // EXACT: the mask holds exact decisions; else those of slots inside the guard band
 // are taken here, where r^2 is at hand.
 template <bool COUNT, bool EXACT>
@@ -875,86 +886,98 @@ __device__ __forceinline__ void force_rounds(ForceShared& S, unsigned int m, boo
   }
   const unsigned int total = __shfl_sync(0xffffffffu, k, 31);
   k -= cnt;      // the place of the lane's next pair in the list
-  // the longest run bounds the levels of the segmented sums
-  const unsigned int maxrun = __reduce_max_sync(0xffffffffu, cnt);
+  const unsigned int maxrow = __reduce_max_sync(0xffffffffu, cnt);
+  const unsigned int rowmask = __ballot_sync(0xffffffffu, cnt != 0u);
+  const unsigned int incl = k + cnt;
+  bool first = true;       // the lane's next listed pair is its row's first
   __syncwarp();
 #pragma unroll 1
-  for (unsigned int r0 = 0; r0 < total; r0 += 32) {
-    // the next 32 pairs of the list
+  for (unsigned int w0 = 0; w0 < total; w0 += PLIST_CAP) {
+    const unsigned int np = min(PLIST_CAP, total - w0), R = (np + 31u) >> 5;
 #pragma unroll 1
-    for (; m && k < r0 + 32u; m &= m - 1, ++k) S.plist[k - r0] = (unsigned short)(lane | ((__ffs(m) - 1) << 5));
-    __syncwarp();
-    const bool a = r0 + lane < total;
-    int li = 32 + lane, sj = 64 + lane;     // (keys no other lane has)
-    if (a) {
-      const unsigned int w = S.plist[lane];
-      li = (int)(w & 31u);
-      sj = (int)(w >> 5);
+    for (; m && k < w0 + PLIST_CAP; m &= m - 1, ++k) {
+      S.plist[k - w0] = (unsigned char)((__ffs(m) - 1) | (first ? 32 : 0));
+      first = false;
     }
-    float4 ci = make_float4(0.f, 0.f, 0.f, 0.f), cj = ci;
-    float vs = 0.0f;
-    if (a) {
-      const float4 P = S.ip[li];
-      const float dx = P.x - S.x[sj], dy = P.y - S.y[sj], dz = P.z - S.z[sj];
-      const float r2 = pair_r2(dx, dy, dz);
-      bool in = true;
-      if (!EXACT && r2 >= S.ilo[li] && r2 >= S.lo[sj]) {
-        in = force_band(S, li, sj, A.perm, A.x, A.pos4, A.box);
-        if (COUNT) C->rechecks += 2;
-      }
-      if (in) {
-        const float4 V = S.iv[li], F = S.if_[li], VJ = S.v[sj], FJ = S.f[sj];
-        ForceSide sa, sb;
-        sa.v = make_float3(V.x, V.y, V.z);
-        sa.rho = V.w;
-        sa.invH = F.x;
-        sa.F = F.y;
-        sa.c = F.z;
-        sa.K4 = F.w;
-        sa.m = P.w;
-        sb.v = make_float3(VJ.x, VJ.y, VJ.z);
-        sb.m = VJ.w;
-        sb.rho = FJ.x;
-        sb.F = FJ.y;
-        sb.c = FJ.z;
-        sb.K4 = FJ.w;
-        sb.invH = S.H[sj];
-        force_pair_terms(sa, sb, dx, dy, dz, r2, A.alpha, ci, cj, vs);
-        if (COUNT) {
-          // force partners of both particles (the pair set, checked per particle)
-          atomicAdd(&A.fcnt[S.own0 + li], 1u);
-          atomicAdd(&A.fcnt[S.g[sj]], 1u);
-          C->pairs += 1;
+    const unsigned int i0 = lane * R, i1 = min(i0 + R, np);
+    // the row of pair w0 + i0: the first lane whose pairs end behind it
+    int li = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned int e = __shfl_sync(0xffffffffu, incl, li + o - 1);
+      if (e <= w0 + i0) li += o;
+    }
+    if (i0 >= i1) li = 32 + lane;     // (a key no other lane has)
+    float4 oa = make_float4(0.f, 0.f, 0.f, 0.f);
+    float ov = 0.0f;
+    __syncwarp();
+#pragma unroll 1
+    for (unsigned int r = 0; r < R; ++r) {
+      const bool a = i0 + r < i1;
+      int sj = 64 + lane;      // (likewise)
+      float4 cj = make_float4(0.f, 0.f, 0.f, 0.f);
+      float vs = 0.0f;
+      if (a) {
+        const unsigned int w = S.plist[i0 + r];
+        sj = (int)(w & 31u);
+        if (r > 0u && (w & 32u)) {
+          float4 t = S.iacc[li];
+          t.x += oa.x; t.y += oa.y; t.z += oa.z; t.w += oa.w;
+          S.iacc[li] = t;
+          S.ivs[li] = fmaxf(S.ivs[li], ov);
+          oa = make_float4(0.f, 0.f, 0.f, 0.f);
+          ov = 0.0f;
+          li = __ffs(rowmask & (0xfffffffeu << li)) - 1;
+        }
+        const float4 P = S.ip[li];
+        const float dx = P.x - S.x[sj], dy = P.y - S.y[sj], dz = P.z - S.z[sj];
+        const float r2 = pair_r2(dx, dy, dz);
+        bool in = true;
+        if (!EXACT && r2 >= S.ilo[li] && r2 >= S.lo[sj]) {
+          in = force_band(S, li, sj, A.perm, A.x, A.pos4, A.box);
+          if (COUNT) C->rechecks += 2;
+        }
+        if (in) {
+          const float4 V = S.iv[li], F = S.if_[li], VJ = S.v[sj], FJ = S.f[sj];
+          float4 ci;
+          force_pair_terms(P.w, V, F, VJ, FJ, S.H[sj], dx, dy, dz, r2, A.alpha, ci, cj, vs);
+          oa.x += ci.x; oa.y += ci.y; oa.z += ci.z; oa.w += ci.w;
+          ov = fmaxf(ov, vs);
+          if (COUNT) {
+            // force partners of both particles (the pair set, checked per particle)
+            atomicAdd(&A.fcnt[S.own0 + li], 1u);
+            atomicAdd(&A.fcnt[S.g[sj]], 1u);
+            C->pairs += 1;
+          }
         }
       }
-    }
-    const unsigned int peers = __match_any_sync(0xffffffffu, sj);
-    S.cb[lane] = cj;
-    S.cv[lane] = vs;
-    const float vj = vs;
-    if (run_sum_max(li, maxrun, ci, vs) && li < 32) {
-      // the head lane of each row of the round holds the row's total
-      float4 t = S.iacc[li];
-      t.x += ci.x; t.y += ci.y; t.z += ci.z; t.w += ci.w;
-      S.iacc[li] = t;
-      S.ivs[li] = fmaxf(S.ivs[li], vs);
-    }
-    __syncwarp();
-    if (a && (peers & lt) == 0u) {
-      float4* dst = own_only ? &S.iacc[sj] : &S.jacc[sj];
-      float* dv = own_only ? &S.ivs[sj] : &S.jvs[sj];
-      float mv = fmaxf(*dv, vj);
+      const unsigned int peers = __match_any_sync(0xffffffffu, sj);
+      S.cb[lane] = cj;
+      S.cv[lane] = vs;
+      __syncwarp();
+      if (a && (peers & lt) == 0u) {
+        float4* dst = own_only ? &S.iacc[sj] : &S.jacc[sj];
+        float* dv = own_only ? &S.ivs[sj] : &S.jvs[sj];
 #pragma unroll 1
-      for (unsigned int b = peers & (peers - 1); b; b &= b - 1) {
-        const int l = __ffs(b) - 1;
-        const float4 t = S.cb[l];
-        cj.x += t.x; cj.y += t.y; cj.z += t.z; cj.w += t.w;
-        mv = fmaxf(mv, S.cv[l]);
+        for (unsigned int b = peers & (peers - 1); b; b &= b - 1) {
+          const int l = __ffs(b) - 1;
+          const float4 t = S.cb[l];
+          cj.x += t.x; cj.y += t.y; cj.z += t.z; cj.w += t.w;
+          vs = fmaxf(vs, S.cv[l]);
+        }
+        float4 t = *dst;
+        t.x += cj.x; t.y += cj.y; t.z += cj.z; t.w += cj.w;
+        *dst = t;
+        *dv = fmaxf(*dv, vs);
       }
-      float4 t = *dst;
-      t.x += cj.x; t.y += cj.y; t.z += cj.z; t.w += cj.w;
-      *dst = t;
-      *dv = mv;
+      __syncwarp();
+    }
+    // what is left of each lane's last row: a row spans at most maxrow / R + 2 lanes
+    if (run_sum_max(li, R == 1u ? maxrow : (maxrow + R - 1u) / R + 1u, oa, ov) && li < 32) {
+      float4 t = S.iacc[li];
+      t.x += oa.x; t.y += oa.y; t.z += oa.z; t.w += oa.w;
+      S.iacc[li] = t;
+      S.ivs[li] = fmaxf(S.ivs[li], ov);
     }
     __syncwarp();
   }
@@ -1188,11 +1211,11 @@ __device__ __forceinline__ LeafFrame leaf_frame(const Tiles& TL, const Tree& T, 
 // partly filled.  Where a box has few clusters, a unit is split into parts (every
 // parts-th interaction), so that every warp has several.
 // (One unit per warp in the smallest boxes, two where a cluster per warp would leave a
-// partial wave: lattices of 25^3 and 30^3 lose 10 % with twice the parts, of 42^3 and a
-// 40k Plummer box gain 10-40 %.)
+// partial wave: lattices of 25^3 and 30^3 lose 10 % with twice the parts, of 36^3, 42^3
+// and a 40k Plummer box gain 10-40 %; three or five times the warps lose 5-30 % there.)
 __device__ __forceinline__ unsigned int unit_parts(unsigned int ntile) {
   const unsigned int warps = gridDim.x * (blockDim.x >> 5);
-  const unsigned int want = 5u * ntile >= 2u * warps ? 2u * warps : warps;
+  const unsigned int want = 10u * ntile >= 3u * warps ? 2u * warps : warps;
   return min(16u, max(1u, want / max(ntile, 1u)));
 }
 
