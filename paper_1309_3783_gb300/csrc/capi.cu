@@ -76,14 +76,12 @@ void launch_iter_start(Engine& E, cudaGraphConditionalHandle iter);
 void launch_iter_next(Engine& E, cudaGraphConditionalHandle iter, cudaGraphConditionalHandle force);
 void launch_iter_step(Engine& E);
 void launch_set_drift(Engine& E);
-void launch_zero_density(Engine& E, bool all);
-void launch_set_active(Engine& E);
+void launch_pass_setup(Engine& E, bool brackets, bool errors, int it);
 void launch_mark_active_cells(Engine& E);
 void launch_count_unconverged(Engine& E, int* out);
 void launch_task_offsets(Engine& E);
 void launch_unit_list(Engine& E);
 void launch_task_items(Engine& E);
-void launch_bracket_reset(Engine& E);
 void launch_reduce(Engine& E);
 void launch_save_acc(Engine& E);
 void launch_kick(Engine& E);
@@ -880,16 +878,9 @@ void Engine::rec_enqueue_reset() {
   rec_unread = true;
 }
 
-sph_status Engine::set_all_active() {
-  launch_set_active(*this);
-  CK(cudaGetLastError());
-  return SPH_OK;
-}
-
 sph_status Engine::density_pass() {
   {
     Scope sc(this, PH_DENSITY_TASKS);
-    launch_zero_density(*this, false);
     launch_live_tasks(*this, true);
   }
   {
@@ -906,14 +897,12 @@ sph_status Engine::density() {
     if (s != SPH_OK) return s;
   }
   if (count_pairs) CK(cudaMemsetAsync(pc.p, 0, 16 * sizeof(unsigned long long), st));
-  sph_status s = set_all_active();
-  if (s != SPH_OK) return s;
-  s = rec_prepare();
+  launch_pass_setup(*this, false, false, 0);
+  sph_status s = rec_prepare();
   if (s != SPH_OK) return s;
   rec_enqueue_reset();
   s = density_pass();
   if (s != SPH_OK) return s;
-  CK(cudaMemsetAsync(dev_counters.p, 0, 4 * sizeof(int), st));
   {
     Scope sc(this, PH_GHOST);
     launch_ghost(*this, 0, 1);
@@ -933,10 +922,9 @@ sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
     if (s != SPH_OK) return s;
   }
   if (count_pairs) CK(cudaMemsetAsync(pc.p, 0, 16 * sizeof(unsigned long long), st));
-  launch_bracket_reset(*this);
-  sph_status s = set_all_active();
-  if (s != SPH_OK) return s;
-  s = rec_prepare();
+  CK(it_dev.reserve(4));
+  launch_pass_setup(*this, true, true, 1);
+  sph_status s = rec_prepare();
   if (s != SPH_OK) return s;
   rec_enqueue_reset();
   // Iterations run in batches launched without a host round trip: the iteration
@@ -945,23 +933,19 @@ sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
   // synchronisation per batch reads where the iteration stands.
   constexpr int H_BATCH = 2;
   int it = 1, rebuilds = 0;
-  CK(it_dev.reserve(4));
-  CK(cudaMemsetAsync(dev_counters.p, 0, 4 * sizeof(int), st));
-  CK(cudaMemsetAsync(err_all.p, 0, 4 * sizeof(unsigned int), st));
   int itv[3] = {1, 0, 0};
-  CK(cudaMemcpyAsync(it_dev.p, itv, 3 * sizeof(int), cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(g_n.p + 1, 0, sizeof(unsigned int), st));
   unsigned int ngath = 0;
   bool fresh = true;      // all particles marked active (first iteration, or after a rebuild)
   for (;;) {
     const int nb = std::min(H_BATCH, prm.h_max_iter - it + 1);
     for (int k = 0; k < nb; ++k) {
-      if (!fresh) launch_mark_active_cells(*this);
-      fresh = false;
       {
         Scope sc(this, PH_DENSITY_TASKS);
-        launch_zero_density(*this, false);
-        if (it + k > 1) launch_gather_prep(*this, it_dev.p);
+        if (!fresh) {
+          launch_mark_active_cells(*this);
+          launch_gather_prep(*this, it_dev.p);
+        }
+        fresh = false;
         launch_live_tasks(*this, true, it_dev.p);
       }
       {
@@ -995,16 +979,13 @@ sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
     if (itv[2] == 2) {
       s = build();   // the input-order h carries the iteration's state
       if (s != SPH_OK) return s;
-      s = set_all_active();
-      if (s != SPH_OK) return s;
       ++rebuilds;
-      if (it >= prm.h_max_iter) break;
+      if (it >= prm.h_max_iter) {
+        launch_pass_setup(*this, false, false, 0);
+        break;
+      }
       ++it;
-      itv[0] = it;
-      itv[2] = 0;
-      CK(cudaMemcpyAsync(it_dev.p, itv, 3 * sizeof(int), cudaMemcpyHostToDevice, st));
-      CK(cudaMemsetAsync(err_all.p, 0, 4 * sizeof(unsigned int), st));
-      CK(cudaMemsetAsync(dev_counters.p, 0, 4 * sizeof(int), st));
+      launch_pass_setup(*this, false, true, it);
       fresh = true;
       continue;
     }
@@ -1307,10 +1288,7 @@ sph_status Engine::capture_step_graph() {
   CKG(cudaMemsetAsync(t_hmax.p, 0, n_nodes * sizeof(float), st));
   launch_pdl(k_leaf_hmax, nsm * 8, 256, st, T, n_nodes, Hs.p); count_launch();
   launch_pdl(k_tile_boxes, grid(32 * n_tiles), 256, st, n_tiles, TL, pos4.p); count_launch();
-  launch_bracket_reset(*this);
-  launch_set_active(*this);
-  CKG(cudaMemsetAsync(dev_counters.p, 0, 4 * sizeof(int), st));
-  CKG(cudaMemsetAsync(err_all.p, 0, 4 * sizeof(unsigned int), st));
+  launch_pass_setup(*this, true, true, 0);
   rec_enqueue_reset();
   launch_iter_start(*this, iter);
   CKG(cudaStreamEndCapture(st, &body));
@@ -1325,7 +1303,6 @@ sph_status Engine::capture_step_graph() {
   body = cp.conditional.phGraph_out[0];
   c1 = launch_count();
   CKG(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
-  launch_zero_density(*this, false);
   launch_gather_prep(*this, it_dev.p);
   launch_live_tasks(*this, true, it_dev.p);
   launch_density(*this, it_dev.p);
@@ -1646,10 +1623,7 @@ sph_status Engine::capture_build_graph() {
   cudaGraph_t body = cp_.conditional.phGraph_out[0];
   long long c1 = launch_count();
   CKB(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
-  launch_bracket_reset(*this);
-  launch_set_active(*this);
-  CKB(cudaMemsetAsync(dev_counters.p, 0, 4 * sizeof(int), st));
-  CKB(cudaMemsetAsync(err_all.p, 0, 4 * sizeof(unsigned int), st));
+  launch_pass_setup(*this, true, true, 0);
   rec_enqueue_reset();
   launch_iter_start(*this, iter);
   CKB(cudaStreamEndCapture(st, &body));
@@ -1675,7 +1649,6 @@ sph_status Engine::capture_build_graph() {
   prof = false;                      // no per-pass events inside the loop
   prof_into_graph = false;
   CKB(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
-  launch_zero_density(*this, false);
   launch_gather_prep(*this, it_dev.p);
   launch_live_tasks(*this, true, it_dev.p);
   launch_density(*this, it_dev.p);

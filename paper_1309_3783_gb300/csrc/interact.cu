@@ -2011,26 +2011,6 @@ __global__ void k_live_tasks(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restri
 // iteration returns at once, and so does a stopped iteration).
 __device__ __forceinline__ bool later_pass(const int* it_dev) { return it_dev[0] > 1 && it_dev[2] == 0; }
 
-// Particles still iterating per cluster (cnt[t] for the nt clusters of this
-// build, and cnt[nt] = 0); clears the gathered task count.  One warp per cluster.
-__global__ void k_pack_count(long long ntcap, const unsigned int* __restrict__ ntile_dev, const int* __restrict__ it_dev,
-                             Tiles TL, const unsigned char* __restrict__ act, unsigned int* __restrict__ cnt,
-                             unsigned int* __restrict__ g_n) {
-  pdl_wait();
-  if (!later_pass(it_dev)) return;
-  const long long nt = ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap;
-  const int lane = threadIdx.x & 31;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *g_n = 0;
-  const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long t = warp; t <= nt; t += nwarps) {
-    bool a = false;
-    if (t < nt) a = (unsigned int)lane < TL.n[t] && act[TL.start[t] + lane];
-    const unsigned int c = __popc(__ballot_sync(0xffffffffu, a));
-    if (lane == 0) cnt[t] = c;
-  }
-}
-
 // After the scan of the counts (rank[t]: iterating particles before cluster t):
 // the packed clusters of each leaf, at its first cluster (0 elsewhere).
 __global__ void k_pack_leaf(long long ntcap, const unsigned int* __restrict__ ntile_dev, const int* __restrict__ it_dev,
@@ -2053,13 +2033,11 @@ __global__ void k_pack_leaf(long long ntcap, const unsigned int* __restrict__ nt
 // packed cluster of the leaf whose first cluster is t): the sorted indices of the
 // iterating particles by rank (idx), and per packed cluster its first rank and
 // its leaf's first cluster (info) and its size (pn).  One warp per cluster.
-__global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ ntile_dev, const int* __restrict__ it_dev,
-                            Tree T, Tiles TL, const unsigned char* __restrict__ act,
-                            const unsigned int* __restrict__ rank, const unsigned int* __restrict__ pk0,
-                            unsigned int* __restrict__ idx, uint2* __restrict__ info, unsigned char* __restrict__ pn) {
-  pdl_wait();
-  if (!later_pass(it_dev)) return;
-  const long long nt = ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap;
+__device__ __forceinline__ void pack_fill(long long nt, const Tree& T, const Tiles& TL,
+                                          const unsigned char* __restrict__ act,
+                                          const unsigned int* __restrict__ rank, const unsigned int* __restrict__ pk0,
+                                          unsigned int* __restrict__ idx, uint2* __restrict__ info,
+                                          unsigned char* __restrict__ pn) {
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -2081,22 +2059,26 @@ __global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ nt
   }
 }
 
-// The gathered tasks of a later pass, when it gathers: (interaction, packed
-// cluster), bit 31 of the interaction marking a self interaction and bit 30 the
-// direction of a pair (0: the packed clusters of A against B, 1: of B against
-// A).  The pass gathers when it is a later one, the caller allows it and at most
-// an eighth of the particles iterate (gflag[0]); the symmetric path runs instead
-// when the tasks exceed the buffer.  One thread per interaction, self
-// interactions first; warp-aggregated appends.
-__global__ void k_gather_tasks(Lists Lq, Tree T, long long npair, long long nself, int cap_pair, int cap_self,
-                               const int* __restrict__ it_dev, long long N, int allow,
-                               const unsigned int* __restrict__ pk0, const unsigned int* __restrict__ pk_tot,
-                               uint2* __restrict__ tasks, unsigned int* __restrict__ g_n, unsigned int cap_g,
-                               int* __restrict__ gflag) {
+// The packed clusters and the gathered tasks of a later pass, when it gathers:
+// (interaction, packed cluster), bit 31 of the interaction marking a self interaction
+// and bit 30 the direction of a pair (0: the packed clusters of A against B, 1: of B
+// against A).  The pass gathers when it is a later one, the caller allows it and at
+// most an eighth of the particles iterate (gflag[0]); the symmetric path runs instead
+// when the tasks exceed the buffer.  One thread per interaction, self interactions
+// first; warp-aggregated appends.
+__global__ void k_pack_tasks(Lists Lq, Tree T, Tiles TL, long long ntcap, const unsigned int* __restrict__ ntile_dev,
+                             const unsigned char* __restrict__ act, const unsigned int* __restrict__ rank,
+                             unsigned int* __restrict__ idx, uint2* __restrict__ info, unsigned char* __restrict__ pn,
+                             long long npair, long long nself, int cap_pair, int cap_self,
+                             const int* __restrict__ it_dev, long long N,
+                             const unsigned int* __restrict__ pk0, const unsigned int* __restrict__ pk_tot,
+                             uint2* __restrict__ tasks, unsigned int* __restrict__ g_n, unsigned int cap_g,
+                             int* __restrict__ gflag) {
   pdl_wait();
-  const bool on = allow != 0 && later_pass(it_dev) && 8ull * pk_tot[0] <= (unsigned long long)N;
+  const bool on = later_pass(it_dev) && 8ull * pk_tot[0] <= (unsigned long long)N;
   if (blockIdx.x == 0 && threadIdx.x == 0) gflag[0] = on ? 1 : 0;
   if (!on) return;
+  pack_fill(ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap, T, TL, act, rank, pk0, idx, info, pn);
   if (npair < 0) {
     npair = min(Lq.counts[1], cap_pair);
     nself = min(Lq.counts[0], cap_self);
@@ -2266,7 +2248,7 @@ __device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tre
 #define GATHER_BLOCKS 8
 #endif
 // The gathered density pass (a later pass of the h iteration that gathers): the
-// tasks of k_gather_tasks, one per fetch; g_n[1] counts the passes that gathered.
+// tasks of k_pack_tasks, one per fetch; g_n[1] counts the passes that gathered.
 // Returns at once when the pass runs the symmetric tasks instead.
 template <bool KAHAN>
 __global__ void __launch_bounds__(SPH_THREADS, GATHER_BLOCKS) k_density_gather(
@@ -2299,16 +2281,29 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
                         float gamma_k, float n_ngb, float tol,
                         float gamma_gas, const unsigned int* __restrict__ perm, float* __restrict__ Hs,
                         float4* __restrict__ pos4, const float4* __restrict__ cen4, const float4* __restrict__ vel4,
-                        float4* __restrict__ dacc, const float4* __restrict__ dcomp, unsigned char* __restrict__ act,
-                        float* __restrict__ h,
+                        float4* __restrict__ dacc, unsigned int* __restrict__ dcnt, float4* __restrict__ dcomp,
+                        unsigned char* __restrict__ act, float* __restrict__ h,
                         float* __restrict__ hlo, float* __restrict__ hhi, int* __restrict__ conv,
                         const float* __restrict__ hlimp, const unsigned int* __restrict__ leaf_of, Tree T,
                         float4* __restrict__ ghost4, float4* __restrict__ hhist, int* __restrict__ n_active,
-                        unsigned int* __restrict__ err_all) {
+                        unsigned int* __restrict__ err_all, long long nnodes, long long ntile,
+                        unsigned char* __restrict__ t_active, unsigned char* __restrict__ tl_active,
+                        unsigned int* __restrict__ t_alo, unsigned int* __restrict__ t_ahi) {
   pdl_wait();
   // the iteration number: the host's, or in a captured step the device counter
   const int it = it_dev ? *it_dev : it_host;
   if (it_dev && it_dev[2] != 0) return;    // the iteration has stopped (batched iterations)
+  if (mode == 1) {
+    // the marks of this pass's cells and clusters, and the boxes of their iterating
+    // particles (those of the next pass are set anew)
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+    for (long long k = t0; k < 3 * nnodes; k += nth) {
+      t_alo[k] = 0xffffffffu;
+      t_ahi[k] = 0u;
+      if (k < nnodes) t_active[k] = 0;
+    }
+    for (long long k = t0; k < ntile; k += nth) tl_active[k] = 0;
+  }
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     if (mode == 1 && !act[p]) continue;
     const unsigned int i = perm[p];
@@ -2354,6 +2349,10 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
         const unsigned int am = __activemask();
         if ((threadIdx.x & 31) == __ffs(am) - 1) atomicAdd(n_active, __popc(am));
       }
+      // the next pass sums anew
+      dacc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+      dcnt[p] = 0;
+      if (dcomp) dcomp[p] = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
     act[p] = 0;
@@ -2379,35 +2378,32 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
   }
 }
 
-__global__ void k_zero_active(long long N, const unsigned char* __restrict__ act, float4* __restrict__ dacc,
-                              unsigned int* __restrict__ dcnt, float4* __restrict__ dcomp, int all) {
-  pdl_wait();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-    if (all || act[p]) {
-      dacc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-      dcnt[p] = 0;
-      if (dcomp) dcomp[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  }
-}
-
 // Mark every cell that holds a particle still iterating h (and its ancestors).
 // After an h iteration: the clusters and cells that still hold a particle
 // iterating h (a cluster's largest H follows the H its particles took), and for
 // every cell the box of those particles in the cell's
 // frame.  One warp per cluster; the cluster's box of active particles is added
 // to every cell on its chain with ordered-key atomics.
+// Counts the particles still iterating per cluster (cnt[t], and cnt[ntile] = 0) and
+// clears the gathered task count for the packing that follows.
 __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ ntile_dev,
-                              const unsigned char* __restrict__ act, const float4* __restrict__ pos4, Tree T, Tiles TL) {
+                              const unsigned char* __restrict__ act, const float4* __restrict__ pos4, Tree T, Tiles TL,
+                              unsigned int* __restrict__ cnt, unsigned int* __restrict__ g_n) {
   pdl_wait();
   if (ntile_dev) ntile = min(ntile, (long long)*ntile_dev);   // a captured step: this build's clusters
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    cnt[ntile] = 0;
+    *g_n = 0;
+  }
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long t = warp; t < ntile; t += nwarps) {
     const unsigned int n = TL.n[t], s0 = TL.start[t];
     const bool a = (unsigned int)lane < n && act[s0 + lane];
-    if (!__any_sync(0xffffffffu, a)) continue;
+    const unsigned int bal = __ballot_sync(0xffffffffu, a);
+    if (lane == 0) cnt[t] = __popc(bal);
+    if (!bal) continue;
     float3 lo = make_float3(FLT_MAX, FLT_MAX, FLT_MAX), hi = make_float3(-FLT_MAX, -FLT_MAX, -FLT_MAX);
     float hm = 0.0f;
     if (a) {
@@ -2493,19 +2489,47 @@ __global__ void k_count_unconverged(long long N, const int* __restrict__ conv, i
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
-__global__ void k_set_active(long long N, unsigned char* __restrict__ act) {
+// Sets up a first pass: every particle, cell and cluster takes part, with fresh sums;
+// in an h iteration (hlo given) also fresh brackets and flags, and the iteration's state
+// on the device (it > 0: that iteration comes next).
+__global__ void k_pass_setup(long long N, unsigned char* __restrict__ act, float4* __restrict__ dacc,
+                             unsigned int* __restrict__ dcnt, float4* __restrict__ dcomp, float* __restrict__ hlo,
+                             float* __restrict__ hhi, int* __restrict__ conv, long long nnodes,
+                             unsigned char* __restrict__ t_active, long long ntile,
+                             unsigned char* __restrict__ tl_active, unsigned int* __restrict__ task_ctr,
+                             int* __restrict__ dev_counters, unsigned int* __restrict__ err_all,
+                             int* __restrict__ gflag, int* __restrict__ it_dev, int it, unsigned int* __restrict__ g_n) {
   pdl_wait();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x)
-    act[p] = 1;
-}
-
-__global__ void k_h_bracket_reset(long long N, float* __restrict__ hlo, float* __restrict__ hhi, int* __restrict__ conv) {
-  pdl_wait();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-    hlo[p] = 0.0f;
-    hhi[p] = __int_as_float(0x7f800000);
-    conv[p] = 0;
+  const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+  if (t0 < 4) {
+    task_ctr[t0] = 0;
+    dev_counters[t0] = 0;
+    if (err_all) err_all[t0] = 0;
   }
+  if (t0 == 0) {
+    gflag[0] = 0;
+    if (it > 0) {
+      it_dev[0] = it;
+      it_dev[2] = 0;
+      if (it == 1) {
+        it_dev[1] = 0;
+        g_n[1] = 0;
+      }
+    }
+  }
+  for (long long p = t0; p < N; p += nth) {
+    act[p] = 1;
+    dacc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+    dcnt[p] = 0;
+    if (dcomp) dcomp[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (hlo) {
+      hlo[p] = 0.0f;
+      hhi[p] = __int_as_float(0x7f800000);
+      conv[p] = 0;
+    }
+  }
+  for (long long k = t0; k < nnodes; k += nth) t_active[k] = 1;
+  for (long long k = t0; k < ntile; k += nth) tl_active[k] = 1;
 }
 
 // =========================================================================== captured steps
@@ -2529,9 +2553,10 @@ __global__ void k_iter_start(cudaGraphConditionalHandle iter, int* __restrict__ 
 // advance to the next iteration.  Kernels of later iterations launched ahead
 // return at once after a stop.
 __global__ void k_iter_step(int* __restrict__ it_dev, int* __restrict__ n_active,
-                            const unsigned int* __restrict__ err_all, int max_iter) {
+                            const unsigned int* __restrict__ err_all, int max_iter, unsigned int* __restrict__ task_ctr) {
   pdl_wait();
   if (it_dev[2] != 0) return;
+  task_ctr[0] = task_ctr[1] = task_ctr[3] = 0;      // the density passes' queues
   const int na = *n_active;
   if (it_dev[0] == 1) it_dev[1] = na;
   if ((*err_all & ERR_REBUILD) != 0u) it_dev[2] = 2;
@@ -2545,8 +2570,9 @@ __global__ void k_iter_step(int* __restrict__ it_dev, int* __restrict__ n_active
 // needed (the host then takes over).  n_active is cleared for the next iteration.
 __global__ void k_iter_next(cudaGraphConditionalHandle iter, cudaGraphConditionalHandle force, int* __restrict__ it_dev,
                             int* __restrict__ n_active, const unsigned int* __restrict__ err_all, int max_iter,
-                            int* __restrict__ first_active) {
+                            int* __restrict__ first_active, unsigned int* __restrict__ task_ctr) {
   pdl_wait();
+  task_ctr[0] = task_ctr[1] = task_ctr[3] = 0;      // the density passes' queues
   const bool rebuild = (*err_all & ERR_REBUILD) != 0u;
   const int na = *n_active;
   if (*it_dev == 1) *first_active = na;
@@ -2840,7 +2866,6 @@ void launch_live_tasks(Engine& E, bool dens, const int* it_dev) {
 // the caller knows the pass needs (-1: both, as in a captured step, where the
 // one that does not match the counter returns at once).
 void launch_density(Engine& E, const int* it_dev, int only) {
-  cudaMemsetAsync(E.task_ctr.p, 0, 2 * sizeof(unsigned int), E.st);
   for (int part = 0; part < 2; ++part) {
     if (!it_dev && part != (E.partial_pass ? 1 : 0)) continue;
     if (it_dev && only >= 0 && part != only) continue;
@@ -2871,24 +2896,23 @@ void launch_density(Engine& E, const int* it_dev, int only) {
 // The packing and the task list of a gathered later pass (a pass of the h
 // iteration given by it_dev; the kernels decide on the device whether it gathers).
 void launch_gather_prep(Engine& E, const int* it_dev) {
+  if (E.prm.h_gather == 0 || E.count_pairs) return;      // (gflag stays 0: no pass gathers)
   // a captured rebuild step covers the capacities (this build's sizes are on the device)
   const long long nt = E.gcap ? E.N : E.n_tiles;
   const unsigned int* ntd = E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr;
-  launch_pdl(k_pack_count, E.grid(32 * (nt + 1)), 256, E.st, nt, ntd, it_dev, E.TL, E.act.p, E.pk_cnt.p, E.g_n.p);
-  count_launch();
-  exclusive_scan(E.pk_cnt.p, E.pk_cnt.p, nt + 1, E.pk_sums.p, E.pk_tot.p + 0, E.st, ntd, it_dev);
-  launch_pdl(k_pack_leaf, E.grid(nt + 1), 256, E.st, nt, ntd, it_dev, E.T, E.TL, E.pk_cnt.p, E.pk_v.p);
-  count_launch();
-  exclusive_scan(E.pk_v.p, E.pk_v.p, nt + 1, E.pk_sums.p, E.pk_tot.p + 1, E.st, ntd, it_dev);
-  launch_pdl(k_pack_fill, E.grid(32 * nt), 256, E.st, nt, ntd, it_dev, E.T, E.TL, E.act.p, E.pk_cnt.p,
-             E.pk_v.p, E.pk_idx.p, E.pk_info.p, E.pk_n.p);
-  count_launch();
+  if (E.N <= PACK_ONE) {
+    launch_pack_scan(E, nt, ntd, it_dev);
+  } else {
+    exclusive_scan(E.pk_cnt.p, E.pk_cnt.p, nt + 1, E.pk_sums.p, E.pk_tot.p + 0, E.st, ntd, it_dev);
+    launch_pdl(k_pack_leaf, E.grid(nt + 1), 256, E.st, nt, ntd, it_dev, E.T, E.TL, E.pk_cnt.p, E.pk_v.p);
+    count_launch();
+    exclusive_scan(E.pk_v.p, E.pk_v.p, nt + 1, E.pk_sums.p, E.pk_tot.p + 1, E.st, ntd, it_dev);
+  }
   const long long npair = E.gcap ? -1 : E.n_pairs, nself = E.gcap ? -1 : E.n_selfs;
   const long long nitem = E.gcap ? (long long)E.cap_pair + E.cap_self : (long long)E.n_pairs + E.n_selfs;
-  const int allow = E.prm.h_gather != 0 && !E.count_pairs ? 1 : 0;
-  launch_pdl(k_gather_tasks, E.grid(std::max<long long>(nitem, 1)), 256, E.st, E.Lq, E.T, npair, nself,
-             E.cap_pair, E.cap_self, it_dev, (long long)E.N, allow, E.pk_v.p, E.pk_tot.p, E.g_live.p, E.g_n.p,
-             (unsigned int)E.g_live.n, E.gflag.p);
+  launch_pdl(k_pack_tasks, E.grid(std::max<long long>(nitem, 32 * nt)), 256, E.st, E.Lq, E.T, E.TL, nt, ntd, E.act.p,
+             E.pk_cnt.p, E.pk_idx.p, E.pk_info.p, E.pk_n.p, npair, nself, E.cap_pair, E.cap_self, it_dev,
+             (long long)E.N, E.pk_v.p, E.pk_tot.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n, E.gflag.p);
   count_launch();
 }
 
@@ -2896,7 +2920,6 @@ void launch_gather_prep(Engine& E, const int* it_dev) {
 void launch_density_gather(Engine& E) {
   const bool kahan = E.kahan();
   const auto k = kahan ? k_density_gather<true> : k_density_gather<false>;
-  cudaMemsetAsync(E.task_ctr.p + 3, 0, sizeof(unsigned int), E.st);
   launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st, E.Lq, E.T, E.TL, E.box.p, E.pos4.p,
              E.cen4.p, E.perm.p, E.x.p, E.dacc.p, E.dcnt.p, E.dcomp.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n,
              E.gflag.p, E.pk_info.p, E.pk_n.p, E.pk_idx.p, E.task_ctr.p + 3);
@@ -2931,20 +2954,20 @@ void launch_unit_list(Engine& E) {
 void launch_ghost(Engine& E, int mode, int it, const int* it_dev) {
   launch_pdl(k_ghost, E.grid(E.N), 256, E.st, E.N, mode, it, it_dev, E.prm.h_max_iter, E.prm.gamma_kernel, E.prm.n_ngb,
                                           E.prm.h_tol, E.prm.gamma_gas, E.perm.p, E.Hs.p, E.pos4.p, E.cen4.p,
-                                          E.vel4.p, E.dacc.p, E.dcomp.p, E.act.p, E.h.p, E.hlo.p, E.hhi.p, E.conv.p,
+                                          E.vel4.p, E.dacc.p, E.dcnt.p, E.dcomp.p, E.act.p, E.h.p, E.hlo.p, E.hhi.p, E.conv.p,
                                           E.hlimp.p, E.leaf_of.p, E.T, E.ghost4.p, E.hhist.p, E.dev_counters.p,
-                                          E.err_all.p); count_launch();
+                                          E.err_all.p, (long long)(E.gcap ? E.cap_nodes : E.n_nodes),
+                                          (long long)(E.gcap ? E.N : E.n_tiles), E.t_active.p, E.tl_active.p, E.t_alo.p,
+                                          E.t_ahi.p); count_launch();
 }
 
-void launch_zero_density(Engine& E, bool all) {
-  launch_pdl(k_zero_active, E.grid(E.N), 256, E.st, E.N, E.act.p, E.dacc.p, E.dcnt.p, E.dcomp.p, all ? 1 : 0); count_launch();
-}
-
-void launch_set_active(Engine& E) {
+void launch_pass_setup(Engine& E, bool brackets, bool errors, int it) {
   E.partial_pass = 0;
-  launch_pdl(k_set_active, E.grid(E.N), 256, E.st, E.N, E.act.p); count_launch();
-  cudaMemsetAsync(E.t_active.p, 1, E.gcap ? (size_t)E.cap_nodes : (size_t)E.n_nodes, E.st);
-  cudaMemsetAsync(E.tl_active.p, 1, E.gcap ? (size_t)E.N : (size_t)E.n_tiles, E.st);
+  launch_pdl(k_pass_setup, E.grid(E.N), 256, E.st, E.N, E.act.p, E.dacc.p, E.dcnt.p, E.dcomp.p,
+             brackets ? E.hlo.p : nullptr, E.hhi.p, E.conv.p, (long long)(E.gcap ? E.cap_nodes : E.n_nodes),
+             E.t_active.p, (long long)(E.gcap ? E.N : E.n_tiles), E.tl_active.p, E.task_ctr.p, E.dev_counters.p,
+             errors ? E.err_all.p : nullptr, E.gflag.p, E.it_dev.p, it, E.g_n.p);
+  count_launch();
 }
 
 void launch_count_unconverged(Engine& E, int* out) {
@@ -2954,14 +2977,10 @@ void launch_count_unconverged(Engine& E, int* out) {
 void launch_mark_active_cells(Engine& E) {
   E.partial_pass = 1;
   // a captured rebuild step covers the capacities (this build's sizes are on the device)
-  const long long nn = E.gcap ? E.cap_nodes : E.n_nodes, nt = E.gcap ? E.N : E.n_tiles;
-  cudaMemsetAsync(E.t_active.p, 0, nn, E.st);
-  cudaMemsetAsync(E.tl_active.p, 0, nt, E.st);
-  cudaMemsetAsync(E.t_alo.p, 0xff, 3 * (size_t)nn * sizeof(unsigned int), E.st);
-  cudaMemsetAsync(E.t_ahi.p, 0, 3 * (size_t)nn * sizeof(unsigned int), E.st);
+  const long long nt = E.gcap ? E.N : E.n_tiles;
   launch_pdl(k_mark_active, E.grid(32 * nt), 256, E.st, nt,
              E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr, E.act.p, E.pos4.p, E.T,
-             E.TL);
+             E.TL, E.pk_cnt.p, E.g_n.p);
   count_launch();
 }
 
@@ -2977,10 +2996,6 @@ void launch_task_items(Engine& E) {
   launch_pdl(k_task_items, E.nsm * 8, 256, E.st, E.Lq, E.T, E.gcap ? -1 : E.n_pairs, E.gcap ? -1 : E.n_selfs,
              E.cap_pair, E.cap_self, (unsigned int)E.l_ptask.n, (unsigned int)E.l_stask.n);
   count_launch();
-}
-
-void launch_bracket_reset(Engine& E) {
-  launch_pdl(k_h_bracket_reset, E.grid(E.N), 256, E.st, E.N, E.hlo.p, E.hhi.p, E.conv.p); count_launch();
 }
 
 void launch_reduce(Engine& E) {
@@ -3015,12 +3030,13 @@ void launch_iter_start(Engine& E, cudaGraphConditionalHandle iter) {
 }
 
 void launch_iter_step(Engine& E) {
-  launch_pdl(k_iter_step, 1, 1, E.st, E.it_dev.p, E.dev_counters.p, E.err_all.p, E.prm.h_max_iter); count_launch();
+  launch_pdl(k_iter_step, 1, 1, E.st, E.it_dev.p, E.dev_counters.p, E.err_all.p, E.prm.h_max_iter,
+             E.task_ctr.p); count_launch();
 }
 
 void launch_iter_next(Engine& E, cudaGraphConditionalHandle iter, cudaGraphConditionalHandle force) {
   launch_pdl(k_iter_next, 1, 1, E.st, iter, force, E.it_dev.p, E.dev_counters.p, E.err_all.p, E.prm.h_max_iter,
-                                 E.it_dev.p + 1); count_launch();
+                                 E.it_dev.p + 1, E.task_ctr.p); count_launch();
 }
 
 void launch_set_drift(Engine& E) {

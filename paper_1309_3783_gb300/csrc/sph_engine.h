@@ -66,6 +66,11 @@ extern const char* const kPhaseNames[PH_COUNT];
 void exclusive_scan(const unsigned int* in, unsigned int* out, long long n, unsigned int* tile_sums,
                     unsigned int* total, cudaStream_t st, const unsigned int* n_dev = nullptr,
                     const int* gate = nullptr);
+// Up to this many particles one block does both scans of a gathered pass's packing (4096
+// entries of each per microsecond or so, against the 25 us of seven launches; clusters
+// are a sixteenth to a thirtieth of the particles in ordinary boxes).
+constexpr long long PACK_ONE = 1 << 20;
+void launch_pack_scan(struct Engine& E, long long nt, const unsigned int* ntd, const int* it_dev);
 long long radix_scratch_words(long long n);
 void radix_sort(unsigned long long* k0, unsigned int* v0, unsigned long long* k1, unsigned int* v1, long long n,
                 int bits, unsigned int* scratch, cudaStream_t st);
@@ -331,7 +336,6 @@ class Engine {
   sph_status ensure_tree_capacity(int nodes);
   sph_status ensure_list_capacity(int selfs, int pairs, int queue);
   sph_status build_once(bool* retry);
-  sph_status set_all_active();
   sph_status density_pass();
   sph_status ghost_pass(int mode, int it, int* n_active, bool* rebuild);
   sph_status upload_boxes();
