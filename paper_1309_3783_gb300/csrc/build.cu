@@ -33,7 +33,7 @@ __global__ void k_ingest(long long N, const int* __restrict__ bid, BoxDesc* box,
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         const double xk = x[3 * p + k];
-        ok &= (xk >= 0.0) && (xk < L);
+        ok &= in_box(xk, L);
         ok &= isfinite(v[3 * p + k]);
       }
       const float hp = h[p];
@@ -127,24 +127,39 @@ __global__ void k_check_build(cudaGraphConditionalHandle ok, const unsigned int*
 }
 
 // ============================================================== keys
+// floor(u 2^56) of u in [0, 1); 2^56 - 1 above and 0 below (invalid input, which the
+// ingest has flagged).  Exact for u >= 2^-4, else rounded down.
+__device__ __forceinline__ unsigned long long unit_fraction(double u) {
+  const unsigned long long b = dbits(u);
+  const int e = (int)(b >> 52) - 1023;           // (negative numbers: beyond 1023)
+  if (b >> 63 || e < -56) return 0ull;
+  if (e >= 0) return (1ull << 56) - 1ull;
+  const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+  return e >= -4 ? m << (4 + e) : m >> (-4 - e);
+}
+
 // key = box << (3 dcap) | Morton(floor((x / L) 2^dcap)) with the cell index
 // clamped to [0, 2^dcap - 1]; the value is the input index.
+// Bound by memory (40 bytes a particle) once the index is taken from the bits of x / L:
+// with an FP64 scaling, floor and clamp per coordinate 33.5M particles took 1.13 ms.
 __global__ void k_keys(long long N, int dcap, const int* __restrict__ bid, const BoxDesc* __restrict__ box,
                        const double* __restrict__ x, unsigned long long* __restrict__ key,
                        unsigned int* __restrict__ val) {
   pdl_wait();
-  const double scale = ldexp(1.0, dcap);
   const unsigned int qmax = (1u << dcap) - 1u;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     const int b = bid[p];
-    const double L = box[b].L;
+    const bool p2 = box[b].pow2 != 0;
+    const double iL = box[b].invL;
     unsigned int q[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const double uu = box[b].pow2 ? x[3 * p + k] * box[b].invL : __ddiv_rn(x[3 * p + k], L);
-      double f = floor(__dmul_rn(uu, scale));
-      f = fmin(fmax(f, 0.0), (double)qmax);
-      q[k] = (unsigned int)f;
+      // the leading dcap fraction bits of x / L; a product with 1 / L that is not exact
+      // decides it unless they change within its rounding (a few 2^-53)
+      const double xk = x[3 * p + k];
+      unsigned long long f = unit_fraction(xk * iL);
+      if (!p2 && ((f + 32) >> (56 - dcap)) != ((f - 32) >> (56 - dcap))) f = unit_fraction(__ddiv_rn(xk, box[b].L));
+      q[k] = min((unsigned int)(f >> (56 - dcap)), qmax);
     }
     key[p] = ((unsigned long long)b << (3 * dcap)) | morton3(q[0], q[1], q[2]);
     val[p] = (unsigned int)p;
@@ -194,7 +209,7 @@ __global__ void k_relayout(const long long* __restrict__ tab, const double* __re
 // ============================================================== decomposition reuse
 // Largest displacement of every box since its decomposition was built (FP64,
 // periodic minimum image), as the bits of a non-negative double (they order
-// like the values).
+// like the values).  The root of the largest square is taken, once per warp.
 __global__ void k_displacement(long long N, const int* __restrict__ bid, const BoxDesc* __restrict__ box,
                                const double* __restrict__ x, const double* __restrict__ xb,
                                unsigned long long* __restrict__ dmax) {
@@ -215,14 +230,11 @@ __global__ void k_displacement(long long N, const int* __restrict__ bid, const B
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         double t = x[3 * p + k] - xb[3 * p + k];
-        if (per) {
-          if (t > halfL) t -= L;
-          else if (t < -halfL) t += L;
-        }
+        if (per && abs_above(t, halfL)) t += t > 0.0 ? -L : L;
         d2 = fma(t, t, d2);
       }
     }
-    unsigned long long bits = valid ? (unsigned long long)__double_as_longlong(sqrt(d2)) : 0ull;
+    unsigned long long bits = dbits(d2);      // (0 where invalid)
     const int b0 = __shfl_sync(0xffffffffu, b, 0);
     if (__all_sync(0xffffffffu, !valid || b == b0)) {
 #pragma unroll
@@ -232,19 +244,30 @@ __global__ void k_displacement(long long N, const int* __restrict__ bid, const B
       }
       if (b0 >= 0 && __all_sync(0xffffffffu, valid)) {
         if (b0 != rb) {
-          if (rb >= 0 && (threadIdx.x & 31) == 0) atomicMax(&dmax[rb], rbits);
+          if (rb >= 0 && (threadIdx.x & 31) == 0) atomicMax(&dmax[rb], dbits(sqrt(__longlong_as_double((long long)rbits))));
           rb = b0;
           rbits = 0ull;
         }
         rbits = bits > rbits ? bits : rbits;
       } else if ((threadIdx.x & 31) == 0 && b0 >= 0) {
-        atomicMax(&dmax[b0], bits);
+        atomicMax(&dmax[b0], dbits(sqrt(__longlong_as_double((long long)bits))));
       }
     } else if (valid) {
-      atomicMax(&dmax[b], bits);
+      atomicMax(&dmax[b], dbits(sqrt(__longlong_as_double((long long)bits))));
     }
   }
-  if (rb >= 0 && (threadIdx.x & 31) == 0) atomicMax(&dmax[rb], rbits);
+  if (rb >= 0 && (threadIdx.x & 31) == 0) atomicMax(&dmax[rb], dbits(sqrt(__longlong_as_double((long long)rbits))));
+}
+
+// The smallest H limit along a cell's chain (limits order like their bits as signed
+// integers unless two are negative, where any of them stops every H).
+__device__ __forceinline__ double chain_limit(const Tree& T, int id) {
+  long long lim = __double_as_longlong(1e300);
+  while (id >= 0) {
+    lim = min(lim, __double_as_longlong(T.hlim[id]));
+    id = T.parent[id];
+  }
+  return __longlong_as_double(lim);
 }
 
 // The limit every particle's H must stay below with the decomposition kept:
@@ -261,12 +284,8 @@ __global__ void k_reuse_limits(long long N, int box_shift, const unsigned long l
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     const int b = (int)(key[p] >> box_shift);
     int id = (int)leaf_of[p];
-    double lim = 1e300;
-    while (id >= 0) {
-      lim = fmin(lim, T.hlim[id]);
-      id = T.parent[id];
-    }
-    lim -= 2.0 * __longlong_as_double((long long)dmax[b]);
+    const double lim0 = chain_limit(T, id);
+    const double lim = lim0 - 2.0 * __longlong_as_double((long long)dmax[b]);
     const float lf = __double2float_rz(lim);
     hlimp[p] = lf;
     const float H = __fmul_rn(gamma_k, h[perm[p]]);
@@ -617,12 +636,18 @@ __global__ void k_gather_sorted(long long N, const unsigned int* __restrict__ pe
                                 const BoxDesc* __restrict__ box, const float4* __restrict__ a_in, int vpred,
                                 float* __restrict__ Hs, float4* __restrict__ vel4) {
   pdl_wait();
+  int lb = -1;             // (FP64 once per box)
+  float hdt = 0.0f;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     const unsigned int i = perm[p];
     Hs[p] = H_in[i];
     float4 w = make_float4(v[3ll * i], v[3ll * i + 1], v[3ll * i + 2], u[i]);
     if (vpred) {
-      const float hdt = (float)(0.5 * box[bid[i]].dt);
+      const int b = bid[i];
+      if (b != lb) {
+        hdt = (float)(0.5 * box[b].dt);
+        lb = b;
+      }
       if (hdt != 0.0f) {
         const float4 a = a_in[i];
         w.x += a.x * hdt;
@@ -1119,17 +1144,15 @@ __global__ void k_particle_limits(long long N, Tree T, const unsigned int* __res
   pdl_wait();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     int id = (int)leaf_of[p];
-    double lim = 1e300;
-    while (id >= 0) {
-      lim = fmin(lim, T.hlim[id]);
-      id = T.parent[id];
-    }
-    hlimp[p] = __double2float_rz(lim);
+    const double lim0 = chain_limit(T, id);
+    hlimp[p] = __double2float_rz(lim0);
   }
 }
 
 // Particle offsets relative to the centre of their leaf (units of L, FP32) and
-// the leaf centre relative to its top cell's centre (exact), plus the mass.
+// the leaf centre relative to its top cell's centre (exact), plus the mass.  Two FP64
+// operations and a conversion per coordinate (with centres and images in FP64 too, eight,
+// the kernel took 1.96 ms for 33.5M particles).
 __global__ void k_shift(long long N, int box_shift, const unsigned long long* __restrict__ key,
                         const unsigned int* __restrict__ perm, const unsigned int* __restrict__ leaf_of, Tree T,
                         const BoxDesc* __restrict__ box, const double* __restrict__ x, const float* __restrict__ m,
@@ -1143,26 +1166,36 @@ __global__ void k_shift(long long N, int box_shift, const unsigned long long* __
     const int d = T.level[leaf];
     unsigned int cx, cy, cz;
     cell_coords(T.key[leaf], d, cx, cy, cz);
-    const double inv = ldexp(1.0, -d);
+    // cell centres have at most SPH_MAX_DEPTH + 1 bits
+    const float e = ldexpf(1.0f, -d - 1);
+    const double tx = widen((float)(2u * cx + 1u) * e), ty = widen((float)(2u * cy + 1u) * e),
+                 tz = widen((float)(2u * cz + 1u) * e);
     // x / L: a power-of-two L scales exactly, so the FP64 division is needed only otherwise
-    const bool p2 = box[b].pow2 != 0;
     const double iL = box[b].invL;
-    double ux = p2 ? x[3ll * i] * iL : __ddiv_rn(x[3ll * i], L);
-    double uy = p2 ? x[3ll * i + 1] * iL : __ddiv_rn(x[3ll * i + 1], L);
-    double uz = p2 ? x[3ll * i + 2] * iL : __ddiv_rn(x[3ll * i + 2], L);
-    if (box[b].global32) {
-      // plain FP32: the position is held as x / L rounded to FP32 (the offset below
-      // then carries that rounding, up to 2^-25 of L per coordinate)
-      ux = (double)__double2float_rn(ux);
-      uy = (double)__double2float_rn(uy);
-      uz = (double)__double2float_rn(uz);
+    const double x0 = x[3ll * i], x1 = x[3ll * i + 1], x2 = x[3ll * i + 2];
+    double ox, oy, oz;
+    if (box[b].pow2 && !box[b].global32) {
+      ox = fma(x0, iL, -tx);
+      oy = fma(x1, iL, -ty);
+      oz = fma(x2, iL, -tz);
+    } else {
+      double ux = __ddiv_rn(x0, L), uy = __ddiv_rn(x1, L), uz = __ddiv_rn(x2, L);
+      if (box[b].global32) {
+        // plain FP32: the position is held as x / L rounded to FP32 (the offset below
+        // then carries that rounding, up to 2^-25 of L per coordinate)
+        ux = (double)__double2float_rn(ux);
+        uy = (double)__double2float_rn(uy);
+        uz = (double)__double2float_rn(uz);
+      }
+      ox = ux - tx;
+      oy = uy - ty;
+      oz = uz - tz;
     }
-    double ox = ux - ((double)cx + 0.5) * inv, oy = uy - ((double)cy + 0.5) * inv, oz = uz - ((double)cz + 0.5) * inv;
     if (box[b].periodic) {
       // a particle kept in its cell after a drift across the boundary: nearest image
-      ox -= rint(ox);
-      oy -= rint(oy);
-      oz -= rint(oz);
+      if (abs_above(ox, 0.5)) ox -= rint(ox);
+      if (abs_above(oy, 0.5)) oy -= rint(oy);
+      if (abs_above(oz, 0.5)) oz -= rint(oz);
     }
     const float sx = (float)ox, sy = (float)oy, sz = (float)oz;
     pos4[p] = make_float4(sx, sy, sz, Hs[p]);
@@ -1408,45 +1441,53 @@ __global__ void k_apply_partition(long long N, const unsigned int* __restrict__ 
 
 // cluster table from the exclusive prefix of the flags: tile_of[p], start, size,
 // leaf, box (relative to the leaf centre) and largest H
-__global__ void k_tile_table(long long N, Tree T, const unsigned int* __restrict__ leaf_of,
-                             const unsigned int* __restrict__ flag, const unsigned int* __restrict__ excl,
-                             const float4* __restrict__ pos4, unsigned int* __restrict__ tile_of, Tiles TL,
-                             int cmax) {
+__global__ void k_tile_table(long long N, const unsigned int* __restrict__ flag, const unsigned int* __restrict__ excl,
+                             unsigned int* __restrict__ tile_of, Tiles TL) {
   pdl_wait();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-    tile_of[p] = excl[p] + flag[p] - 1u;
-    if (!flag[p]) continue;
-    const unsigned int t = excl[p];
-    const unsigned int leaf = leaf_of[p];
-    const unsigned int end = T.start[leaf] + T.count[leaf];
-    unsigned int n = 1;
-    while ((unsigned int)p + n < end && n < (unsigned int)cmax && !flag[p + n]) ++n;
-    float4 lo = make_float4(FLT_MAX, FLT_MAX, FLT_MAX, 0.0f);
-    float4 hi = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, 0.0f);
-    for (unsigned int q = 0; q < n; ++q) {
-      const float4 a = pos4[p + q];
-      lo.x = fminf(lo.x, a.x); lo.y = fminf(lo.y, a.y); lo.z = fminf(lo.z, a.z);
-      hi.x = fmaxf(hi.x, a.x); hi.y = fmaxf(hi.y, a.y); hi.z = fmaxf(hi.z, a.z);
-      lo.w = fmaxf(lo.w, a.w);
-    }
-    TL.start[t] = (unsigned int)p;
-    TL.n[t] = n;
-    TL.leaf[t] = leaf;
-    TL.lo[t] = lo;
-    TL.hi[t] = hi;
-    TL.cen[t] = T.cen[leaf];
-    TL.active[t] = 1;
+    const unsigned int f = flag[p], t = excl[p];
+    tile_of[p] = t + f - 1u;
+    if (f) TL.start[t] = (unsigned int)p;
   }
 }
 
-__global__ void k_cell_tiles(Tree T, int nnodes, const unsigned int* __restrict__ tile_of) {
+// The clusters (a cluster ends where the next one starts) with their boxes, a warp
+// each, and the cells' ranges of clusters, a thread each.  (A thread per cluster over
+// its particles took 0.97 ms for 33.5M particles, and 10 us for 10^5.)
+__global__ void k_cluster_table(long long N, const unsigned int* __restrict__ ntile_dev, Tree T, int nnodes,
+                                const unsigned int* __restrict__ leaf_of, const float4* __restrict__ pos4,
+                                const unsigned int* __restrict__ tile_of, Tiles TL) {
   pdl_wait();
+  const unsigned int nt = *ntile_dev;
   nnodes = min(nnodes, T.n_nodes[0]);
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nnodes; id += gridDim.x * blockDim.x) {
     const unsigned int s = T.start[id], c = T.count[id];
     const unsigned int t0 = tile_of[s];
     T.tile0[id] = t0;
     T.ntile[id] = tile_of[s + c - 1] - t0 + 1u;
+  }
+  const int lane = threadIdx.x & 31;
+  const unsigned int warp = (unsigned int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+  const unsigned int nwarps = (unsigned int)(((long long)gridDim.x * blockDim.x) >> 5);
+  for (unsigned int t = warp; t < nt; t += nwarps) {
+    const unsigned int s0 = TL.start[t], n = (t + 1u < nt ? TL.start[t + 1u] : (unsigned int)N) - s0;
+    float4 lo = make_float4(FLT_MAX, FLT_MAX, FLT_MAX, 0.0f), hi = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, 0.0f);
+    if ((unsigned int)lane < n) {
+      const float4 a = pos4[s0 + lane];
+      lo = a;
+      hi = make_float4(a.x, a.y, a.z, 0.0f);
+    }
+    lo.x = warp_min(lo.x); lo.y = warp_min(lo.y); lo.z = warp_min(lo.z); lo.w = warp_max(lo.w);
+    hi.x = warp_max(hi.x); hi.y = warp_max(hi.y); hi.z = warp_max(hi.z);
+    if (lane == 0) {
+      const unsigned int leaf = leaf_of[s0];
+      TL.n[t] = n;
+      TL.leaf[t] = leaf;
+      TL.lo[t] = lo;
+      TL.hi[t] = hi;
+      TL.cen[t] = T.cen[leaf];
+      TL.active[t] = 1;
+    }
   }
 }
 

@@ -54,9 +54,9 @@ __global__ void k_leaf_clusters(Tree, int, int, const BoxDesc*, const float*, co
 __global__ void k_apply_partition(long long, const unsigned int*, const unsigned int*, unsigned int*,
                                   const unsigned long long*, unsigned long long*, const float*, float*,
                                   const float4*, float4*);
-__global__ void k_tile_table(long long, Tree, const unsigned int*, const unsigned int*, const unsigned int*,
-                             const float4*, unsigned int*, Tiles, int);
-__global__ void k_cell_tiles(Tree, int, const unsigned int*);
+__global__ void k_tile_table(long long, const unsigned int*, const unsigned int*, unsigned int*, Tiles);
+__global__ void k_cluster_table(long long, const unsigned int*, Tree, int, const unsigned int*, const float4*,
+                                const unsigned int*, Tiles);
 __global__ void k_box_reset(int, BoxDesc*);
 __global__ void k_check_shape(int, const BoxDesc*, int, float, unsigned int*);
 __global__ void k_check_build(cudaGraphConditionalHandle, const unsigned int*, const int*, int, const int*, int, int, int,
@@ -691,9 +691,9 @@ sph_status Engine::build_once(bool* retry) {
   launch_pdl(k_shift, grid(N), 256, ss, N, box_shift, key.p, perm.p, leaf_of.p, T, box.p, x.p, m.p, Hs.p, pos4.p,
              cen4.p); count_launch();
   exclusive_scan(tflag.p, texcl.p, N, rs_scratch.p, reinterpret_cast<unsigned int*>(dev_counters.p + 4), ss);
-  launch_pdl(k_tile_table, grid(N), 256, ss, N, T, leaf_of.p, tflag.p, texcl.p, pos4.p, tile_of.p, TL, prm.cluster_max);
-  count_launch();
-  launch_pdl(k_cell_tiles, grid(n_nodes), 256, ss, T, n_nodes, tile_of.p); count_launch();
+  launch_pdl(k_tile_table, grid(N), 256, ss, N, tflag.p, texcl.p, tile_of.p, TL); count_launch();
+  launch_pdl(k_cluster_table, grid(N), 256, ss, N, reinterpret_cast<const unsigned int*>(dev_counters.p + 4), T,
+             n_nodes, leaf_of.p, pos4.p, tile_of.p, TL); count_launch();
   prof_end(PH_SHIFT, ev, l0, ss);
   CK(cudaEventRecord(ev_join, ss));
   CK(cudaStreamWaitEvent(st, ev_join, 0));
@@ -1499,9 +1499,9 @@ sph_status Engine::enqueue_captured_build() {
   launch_pdl(k_shift, grid(N), 256, ss, N, box_shift, key.p, perm.p, leaf_of.p, T, box.p, x.p, m.p, Hs.p, pos4.p,
              cen4.p); count_launch();
   exclusive_scan(tflag.p, texcl.p, N, rs_scratch.p, reinterpret_cast<unsigned int*>(dev_counters.p + 4), ss);
-  launch_pdl(k_tile_table, grid(N), 256, ss, N, T, leaf_of.p, tflag.p, texcl.p, pos4.p, tile_of.p, TL,
-             prm.cluster_max); count_launch();
-  launch_pdl(k_cell_tiles, grid(cap_nodes), 256, ss, T, cap_nodes, tile_of.p); count_launch();
+  launch_pdl(k_tile_table, grid(N), 256, ss, N, tflag.p, texcl.p, tile_of.p, TL); count_launch();
+  launch_pdl(k_cluster_table, grid(N), 256, ss, N, reinterpret_cast<const unsigned int*>(dev_counters.p + 4), T,
+             cap_nodes, leaf_of.p, pos4.p, tile_of.p, TL); count_launch();
   prof_end(PH_SHIFT, ev, l0, ss);
   CKB(cudaEventRecord(ev_join, ss));
   CKB(cudaStreamWaitEvent(st, ev_join, 0));

@@ -2682,8 +2682,14 @@ void launch_set_acc(Engine& E, long long off, long long n, int which, const floa
 __global__ void k_kick(long long N, const int* __restrict__ bid, const BoxDesc* __restrict__ box,
                        const float4* __restrict__ a_in, float* __restrict__ v, float* __restrict__ u) {
   pdl_wait();
+  int lb = -1;             // (FP64 once per box)
+  float hdt = 0.0f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const float hdt = (float)(0.5 * box[bid[i]].dt);
+    const int b = bid[i];
+    if (b != lb) {
+      hdt = (float)(0.5 * box[b].dt);
+      lb = b;
+    }
     if (hdt == 0.0f) continue;
     const float4 a = a_in[i];
     v[3 * i] += a.x * hdt;
@@ -2729,7 +2735,9 @@ __global__ void k_drift(long long N, const int* __restrict__ bid, const BoxDesc*
     hhist[p] = hh;
     for (int k = 0; k < 3; ++k) {
       double xn = x[3 * p + k] + (double)v[3 * p + k] * bd.dt;
-      if (bd.periodic) {
+      // inside by more than the rounding of x / L: nothing to wrap or clamp
+      if (dbits(xn) + 16 < dbits(bd.L)) {
+      } else if (bd.periodic) {
         xn -= bd.L * floor(xn * bd.invL);
         if (xn >= bd.L) xn -= bd.L;
         if (xn < 0.0 || xn >= bd.L) xn = 0.0;

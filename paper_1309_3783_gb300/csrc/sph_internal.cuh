@@ -181,6 +181,31 @@ __device__ __forceinline__ bool canonical_less(double r2, float H) {
   return r2 < __dmul_rn(h, h);   // exact: the product of two FP32 fits FP64
 }
 
+// ------------------------------------------------------------ FP64 by integer
+// FP64 instructions issue at a 60th of the FP32 rate here (2 lanes per clock and SM):
+// kernels with a few dozen per particle are bound by them, not by memory.  What the bit
+// patterns tell is taken from them instead, with the same results.
+__device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
+
+// x >= 0 and x < L, for a positive finite L (non-negative doubles order like their bits;
+// -0 is 0; NaN is beyond every bound)
+__device__ __forceinline__ bool in_box(double x, double L) {
+  const unsigned long long b = dbits(x);
+  return b < dbits(L) || b == 0x8000000000000000ull;
+}
+
+// |a| > b for a non-negative b
+__device__ __forceinline__ bool abs_above(double a, double b) {
+  return (dbits(a) & 0x7fffffffffffffffull) > dbits(b);
+}
+
+// The FP64 value of a positive normal float.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned int b = __float_as_uint(f);
+  return __longlong_as_double((long long)(((unsigned long long)((b >> 23) + 896u) << 52) |
+                                          ((unsigned long long)(b & 0x7fffffu) << 29)));
+}
+
 // ------------------------------------------------------------ warp helpers
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
