@@ -1512,7 +1512,7 @@ sph_status Engine::enqueue_captured_build() {
   CKB(cudaMemsetAsync(mid_count.p, 0, sizeof(unsigned int), st));
   launch_pdl(k_mark_axes, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
   launch_pdl(k_sort_alloc, grid(cap_nodes), 256, st, T, cap_nodes, Lq, big_node.p, big_axis.p, big_off.p, big_count.p,
-             cap_big, mid_seg.p, mid_count.p, (unsigned int)sort_r.n, (unsigned int)ckey.n, err_all.p);
+             gb_cap_big, mid_seg.p, mid_count.p, (unsigned int)sort_r.n, (unsigned int)ckey.n, err_all.p);
   count_launch();
   launch_pdl(k_pair_csr, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
   launch_unit_list(*this);
@@ -1527,13 +1527,15 @@ sph_status Engine::enqueue_captured_build() {
   count_launch();
   // cells of many clusters: one global sort over the key storage, its unused
   // entries holding the largest key so that they sort last
-  CKB(cudaMemsetAsync(ckey.p, 0xff, ckey.n * sizeof(unsigned long long), st));
-  launch_pdl(k_sort_big_keys, nsm * 8, 256, st, -1, big_node.p, big_axis.p, big_off.p, T, TL, ckey.p, cval.p,
-             big_count.p, cap_big); count_launch();
-  radix_sort(ckey.p, cval.p, ckey_tmp.p, cval_tmp.p, (long long)ckey.n, 32 + ceil_log2((long long)cap_big + 1),
-             rs_scratch.p, st);
-  launch_pdl(k_sort_big_scatter, nsm * 8, 256, st, -1, big_node.p, big_axis.p, big_off.p, T, TL, cval.p, sort_r.p,
-             sort_i.p, big_count.p, cap_big); count_launch();
+  if (gb_cap_big > 0) {
+    CKB(cudaMemsetAsync(ckey.p, 0xff, ckey.n * sizeof(unsigned long long), st));
+    launch_pdl(k_sort_big_keys, nsm * 8, 256, st, -1, big_node.p, big_axis.p, big_off.p, T, TL, ckey.p, cval.p,
+               big_count.p, gb_cap_big); count_launch();
+    radix_sort(ckey.p, cval.p, ckey_tmp.p, cval_tmp.p, (long long)ckey.n, 32 + ceil_log2((long long)gb_cap_big + 1),
+               rs_scratch.p, st);
+    launch_pdl(k_sort_big_scatter, nsm * 8, 256, st, -1, big_node.p, big_axis.p, big_off.p, T, TL, cval.p, sort_r.p,
+               sort_i.p, big_count.p, gb_cap_big); count_launch();
+  }
   prof_end(PH_AXIS_SORT, ev, l0);
   CKB(cudaMemcpyAsync(x_build.p, x.p, 3 * N * sizeof(double), cudaMemcpyDeviceToDevice, st));
   return SPH_OK;
@@ -1557,6 +1559,10 @@ sph_status Engine::capture_build_graph() {
   Lq.n_live = l_nlive.p;
   CK(sort_r.reserve((size_t)(n_entries + n_entries / 4 + 4096)));
   CK(sort_i.reserve(sort_r.n));
+  // a box without cells of many clusters is captured without their sort (20 launches,
+  // 60 us of a small box's step); when one appears, the build does not hold, the host
+  // completes that step, and the next capture has it
+  gb_cap_big = n_big > 0 ? cap_big : 0;
   const size_t nb = (size_t)(n_big_entries + n_big_entries / 4 + 4096);
   CK(ckey.reserve(nb));
   CK(ckey_tmp.reserve(ckey.n));
@@ -1607,7 +1613,7 @@ sph_status Engine::capture_build_graph() {
   }
   launch_pdl(k_check_build, 1, 1, st, ok, err_all.p, t_n.p, cap_nodes, l_counts.p, cap_self, cap_pair, gb_last_q,
              prm.pair_cache ? (unsigned int)l_ptask.n : 0xffffffffu,
-             prm.pair_cache ? (unsigned int)l_stask.n : 0xffffffffu, big_count.p, cap_big, gstat.p); count_launch();
+             prm.pair_cache ? (unsigned int)l_stask.n : 0xffffffffu, big_count.p, gb_cap_big, gstat.p); count_launch();
   CKB(cudaStreamEndCapture(st, &g1));
   gb_build = launch_count() - c0;
   cudaGraphNode_t n1, n2, n3, n4;

@@ -231,6 +231,7 @@ class Engine {
   DBuf<float> sort_r;
   DBuf<unsigned int> sort_i;
   int cap_big = 0;
+  int gb_cap_big = 0;    // captured build: its capacity (0: captured without the global sort)
   DBuf<int> big_node, big_axis;
   DBuf<unsigned long long> big_count;   // segments << 40 | entries
   DBuf<unsigned int> big_off;
