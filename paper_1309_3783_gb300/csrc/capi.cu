@@ -83,7 +83,6 @@ void launch_task_offsets(Engine& E);
 void launch_unit_list(Engine& E);
 void launch_task_items(Engine& E);
 void launch_reduce(Engine& E);
-void launch_save_acc(Engine& E);
 void launch_kick(Engine& E);
 void launch_drift(Engine& E);
 void launch_set_h(Engine& E, int b, const float* src);
@@ -1032,7 +1031,6 @@ sph_status Engine::force() {
   {
     Scope sc(this, PH_REDUCE);
     launch_reduce(*this);
-    launch_save_acc(*this);
   }
   CK(cudaGetLastError());
   have_force = true;
@@ -1327,7 +1325,6 @@ sph_status Engine::capture_step_graph() {
   launch_live_tasks(*this, false);
   launch_force(*this);
   launch_reduce(*this);
-  launch_save_acc(*this);
   launch_kick(*this);
   CKG(cudaStreamEndCapture(st, &body));
   g_force = launch_count() - c1;
@@ -1727,7 +1724,6 @@ sph_status Engine::capture_build_graph() {
   };
   auto reduce = [&] {
     launch_reduce(*this);
-    launch_save_acc(*this);
   };
   sph_status ps;
   if (keep_prof) {

@@ -1897,38 +1897,53 @@ __global__ void k_unit_list(unsigned int ntcap, const unsigned int* __restrict__
   const unsigned int nt = ntile_dev ? min(ntcap, *ntile_dev) : ntcap;
   const int lane = threadIdx.x & 31;
   const unsigned int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (unsigned int t = warp; t < nt; t += nwarps) {
-    const int leaf = (int)TL.leaf[t];
-    const float4 lo = TL.lo[t], hi = TL.hi[t], cl = TL.cen[t];
-    const float H = lo.w * (float)box[T.box[leaf]].invL;
-    float est = 0.0f;
-    for (int A = leaf; A >= 0; A = T.parent[A]) {
-      const unsigned int n = (unsigned int)__popc(T.pmask[A]) + (A == leaf ? 1u : 0u);
-      const float e = ldexpf(1.0f, -T.level[A]);
-      for (unsigned int k = lane; k < n; k += 32) {
-        int B = A, dx = 0, dy = 0, dz = 0;
-        if (A != leaf || k > 0u) {
-          const uint2 pr = Lq.csr[T.pstart[A] + k - (A == leaf ? 1u : 0u)];
-          B = (int)pr.x;
-          axis_vec((int)pr.y, dx, dy, dz);
+  // a warp takes up to 16 adjacent clusters and their places in the list with one atomic
+  // (one per cluster on the one counter: 0.96 ms for 1.2M clusters), fewer where that
+  // would leave warps idle
+  const unsigned int run = min(16u, max(1u, nt / nwarps));
+  for (unsigned int t0 = warp * run; t0 < nt; t0 += nwarps * run) {
+    unsigned int mine = 0;       // lane j: the units of cluster t0 + j
+    for (unsigned int j = 0; j < run && t0 + j < nt; ++j) {
+      const unsigned int t = t0 + j;
+      const int leaf = (int)TL.leaf[t];
+      const float4 lo = TL.lo[t], hi = TL.hi[t], cl = TL.cen[t];
+      const float H = lo.w * (float)box[T.box[leaf]].invL;
+      float est = 0.0f;
+      for (int A = leaf; A >= 0; A = T.parent[A]) {
+        const unsigned int n = (unsigned int)__popc(T.pmask[A]) + (A == leaf ? 1u : 0u);
+        const float e = ldexpf(1.0f, -T.level[A]);
+        for (unsigned int k = lane; k < n; k += 32) {
+          int B = A, dx = 0, dy = 0, dz = 0;
+          if (A != leaf || k > 0u) {
+            const uint2 pr = Lq.csr[T.pstart[A] + k - (A == leaf ? 1u : 0u)];
+            B = (int)pr.x;
+            axis_vec((int)pr.y, dx, dy, dz);
+          }
+          const float4 cA = T.cen[A];
+          // the partner cell's centre in the frame of the own leaf; the part of each of
+          // its edges within H of the own box
+          const float bx = e * dx - (cl.x - cA.x), by = e * dy - (cl.y - cA.y), bz = e * dz - (cl.z - cA.z);
+          const float fx = fminf(hi.x + H, bx + 0.5f * e) - fmaxf(lo.x - H, bx - 0.5f * e);
+          const float fy = fminf(hi.y + H, by + 0.5f * e) - fmaxf(lo.y - H, by - 0.5f * e);
+          const float fz = fminf(hi.z + H, bz + 0.5f * e) - fmaxf(lo.z - H, bz - 0.5f * e);
+          const float ie = 1.0f / e;
+          est += fmaxf(fx, 0.0f) * ie * (fmaxf(fy, 0.0f) * ie) * (fmaxf(fz, 0.0f) * ie) * (float)T.count[B];
         }
-        const float4 cA = T.cen[A];
-        // the partner cell's centre in the frame of the own leaf; the part of each of
-        // its edges within H of the own box
-        const float bx = e * dx - (cl.x - cA.x), by = e * dy - (cl.y - cA.y), bz = e * dz - (cl.z - cA.z);
-        const float fx = fminf(hi.x + H, bx + 0.5f * e) - fmaxf(lo.x - H, bx - 0.5f * e);
-        const float fy = fminf(hi.y + H, by + 0.5f * e) - fmaxf(lo.y - H, by - 0.5f * e);
-        const float fz = fminf(hi.z + H, bz + 0.5f * e) - fmaxf(lo.z - H, bz - 0.5f * e);
-        const float ie = 1.0f / e;
-        est += fmaxf(fx, 0.0f) * ie * (fmaxf(fy, 0.0f) * ie) * (fmaxf(fz, 0.0f) * ie) * (float)T.count[B];
       }
+      est = warp_sum(est);
+      const unsigned int parts = (unsigned int)fminf(32.0f, fmaxf(1.0f, ceilf(est * (1.0f / UNIT_PARTNERS))));
+      if ((unsigned int)lane == j) mine = parts;
     }
-    est = warp_sum(est);
-    const unsigned int parts = (unsigned int)fminf(32.0f, fmaxf(1.0f, ceilf(est * (1.0f / UNIT_PARTNERS))));
+    const unsigned int total = __reduce_add_sync(0xffffffffu, mine);
     unsigned int at = 0;
-    if (lane == 0) at = atomicAdd(n_units, parts);
+    if (lane == 0) at = atomicAdd(n_units, total);
     at = __shfl_sync(0xffffffffu, at, 0);
-    if ((unsigned int)lane < parts && at + lane < cap) units[at + lane] = make_uint2(t, (unsigned int)lane | (parts << 16));
+    for (unsigned int j = 0; j < run && t0 + j < nt; ++j) {
+      const unsigned int parts = __shfl_sync(0xffffffffu, mine, (int)j);
+      if ((unsigned int)lane < parts && at + lane < cap)
+        units[at + lane] = make_uint2(t0 + j, (unsigned int)lane | (parts << 16));
+      at += parts;
+    }
   }
 }
 
@@ -2426,28 +2441,28 @@ __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ 
     hi.x = warp_max(hi.x); hi.y = warp_max(hi.y); hi.z = warp_max(hi.z);
     // only particles that iterate change H: the cluster's largest H grows to theirs
     hm = warp_max(hm);
-    if (lane != 0) continue;
-    if (hm > TL.lo[t].w) TL.lo[t].w = hm;
-    TL.active[t] = 1;
-    TL.changed[t] = 1;
+    if (lane == 0) {
+      if (hm > TL.lo[t].w) TL.lo[t].w = hm;
+      TL.active[t] = 1;
+      TL.changed[t] = 1;
+    }
+    if (lane >= 12) continue;
+    // a lane per bound: the lower and upper corners of the iterating particles' box, then
+    // of those that took a new h since the recording
+    const int k = lane % 3;
+    const bool up = (lane / 3) & 1;
     const float4 lc = TL.cen[t];
+    const float mine = up ? (k == 0 ? hi.x : (k == 1 ? hi.y : hi.z)) : (k == 0 ? lo.x : (k == 1 ? lo.y : lo.z));
+    const float lck = k == 0 ? lc.x : (k == 1 ? lc.y : lc.z);
+    unsigned int* arr = lane < 6 ? (up ? T.ahi : T.alo) : (up ? T.chi : T.clo);
     for (int id = (int)TL.leaf[t]; id >= 0; id = T.parent[id]) {
-      T.active[id] = 1;
-      T.changed[id] = 1;
-      const float4 cc = T.cen[id];
-      const float ox = lc.x - cc.x, oy = lc.y - cc.y, oz = lc.z - cc.z;   // exact
-      atomicMin(&T.alo[3 * id], float_key(lo.x + ox));
-      atomicMin(&T.alo[3 * id + 1], float_key(lo.y + oy));
-      atomicMin(&T.alo[3 * id + 2], float_key(lo.z + oz));
-      atomicMax(&T.ahi[3 * id], float_key(hi.x + ox));
-      atomicMax(&T.ahi[3 * id + 1], float_key(hi.y + oy));
-      atomicMax(&T.ahi[3 * id + 2], float_key(hi.z + oz));
-      atomicMin(&T.clo[3 * id], float_key(lo.x + ox));
-      atomicMin(&T.clo[3 * id + 1], float_key(lo.y + oy));
-      atomicMin(&T.clo[3 * id + 2], float_key(lo.z + oz));
-      atomicMax(&T.chi[3 * id], float_key(hi.x + ox));
-      atomicMax(&T.chi[3 * id + 1], float_key(hi.y + oy));
-      atomicMax(&T.chi[3 * id + 2], float_key(hi.z + oz));
+      if (lane == 0) {
+        T.active[id] = 1;
+        T.changed[id] = 1;
+      }
+      const float key_at = mine + (lck - reinterpret_cast<const float*>(&T.cen[id])[k]);   // the offset is exact
+      if (up) atomicMax(&arr[3 * id + k], float_key(key_at));
+      else atomicMin(&arr[3 * id + k], float_key(key_at));
     }
   }
 }
@@ -2617,7 +2632,8 @@ __global__ void k_set_drift(int nbox, BoxDesc* __restrict__ box, const unsigned 
 __global__ void __launch_bounds__(256) k_reduce(int nbox, const long long* __restrict__ boff,
                                                 const BoxDesc* __restrict__ box, const unsigned int* __restrict__ perm,
                                                 const float4* __restrict__ cen4, const float4* __restrict__ vel4,
-                                                const float4* __restrict__ facc, double* __restrict__ red) {
+                                                const float4* __restrict__ facc, float4* __restrict__ a_in,
+                                                double* __restrict__ red) {
   pdl_wait();
   __shared__ double part[8][8];
   for (int b = blockIdx.y; b < nbox; b += gridDim.y) {
@@ -2627,19 +2643,22 @@ __global__ void __launch_bounds__(256) k_reduce(int nbox, const long long* __res
     double val[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (long long p = p0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; p < p1;
          p += (long long)gridDim.x * blockDim.x) {
-      if ((long long)perm[p] - p0 >= nown) continue;   // a halo particle: summed by its owner
-      const double m = cen4[p].w;
-      const float4 vv = vel4[p];
+      const unsigned int i = perm[p];
       const float4 a = facc[p];
-      const double vx = vv.x, vy = vv.y, vz = vv.z;
-      val[0] += m * a.x;
-      val[1] += m * a.y;
-      val[2] += m * a.z;
-      val[3] += m * (vx * a.x + vy * a.y + vz * a.z + (double)a.w);
+      a_in[i] = a;
+      if ((long long)i - p0 >= nown) continue;   // a halo particle: summed by its owner
+      const float4 vv = vel4[p];
+      const double m = widen_any(cen4[p].w);
+      const double vx = widen_any(vv.x), vy = widen_any(vv.y), vz = widen_any(vv.z);
+      const double ax = widen_any(a.x), ay = widen_any(a.y), az = widen_any(a.z);
+      val[0] += m * ax;
+      val[1] += m * ay;
+      val[2] += m * az;
+      val[3] += m * (vx * ax + vy * ay + vz * az + widen_any(a.w));
       val[4] += m * vx;
       val[5] += m * vy;
       val[6] += m * vz;
-      val[7] += m * (0.5 * (vx * vx + vy * vy + vz * vz) + (double)vv.w);
+      val[7] += m * (0.5 * (vx * vx + vy * vy + vz * vz) + widen_any(vv.w));
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -2660,14 +2679,6 @@ __global__ void __launch_bounds__(256) k_reduce(int nbox, const long long* __res
 }
 
 // =========================================================================== time stepping
-// accelerations of the last force pass, kept in caller order for the next kick
-__global__ void k_save_acc(long long N, const unsigned int* __restrict__ perm, const float4* __restrict__ facc,
-                           float4* __restrict__ a_in) {
-  pdl_wait();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x)
-    a_in[perm[p]] = facc[p];
-}
-
 // caller-order (a, du/dt) into the saved accelerations: which = 0 sets a (n x 3), 1 sets du/dt
 __global__ void k_set_acc(long long off, long long n, int which, const float* __restrict__ src,
                           float4* __restrict__ a_in) {
@@ -3026,7 +3037,7 @@ void launch_reduce(Engine& E) {
   const int gx = (int)std::max<long long>(1, std::min<long long>((maxn + 255) / 256, std::max(E.nsm * 4 / E.nbox, std::min(E.nsm * 4, 65536 / E.nbox))));
   launch_pdl(k_reduce, dim3(gx, std::min(E.nbox, 65535)), 256, E.st, E.nbox, E.boff.p, E.box.p, E.perm.p, E.cen4.p,
              E.vel4.p, E.facc.p,
-                                                                 E.red.p); count_launch();
+                                                                 E.a_in.p, E.red.p); count_launch();
 }
 
 cudaError_t add_cond_set_node(cudaGraphNode_t* node, cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps,
@@ -3063,8 +3074,6 @@ void launch_iter_next(Engine& E, cudaGraphConditionalHandle iter, cudaGraphCondi
 void launch_set_drift(Engine& E) {
   launch_pdl(k_set_drift, 1, 256, E.st, E.nbox, E.box.p, E.dmax_bits.p); count_launch();
 }
-
-void launch_save_acc(Engine& E) { launch_pdl(k_save_acc, E.grid(E.N), 256, E.st, E.N, E.perm.p, E.facc.p, E.a_in.p); count_launch(); }
 
 void launch_kick(Engine& E) { launch_pdl(k_kick, E.grid(E.N), 256, E.st, E.N, E.bid.p, E.box.p, E.a_in.p, E.v.p, E.u.p); count_launch(); }
 

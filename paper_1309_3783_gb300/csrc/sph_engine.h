@@ -66,10 +66,11 @@ extern const char* const kPhaseNames[PH_COUNT];
 void exclusive_scan(const unsigned int* in, unsigned int* out, long long n, unsigned int* tile_sums,
                     unsigned int* total, cudaStream_t st, const unsigned int* n_dev = nullptr,
                     const int* gate = nullptr);
-// Up to this many particles one block does both scans of a gathered pass's packing (4096
-// entries of each per microsecond or so, against the 25 us of seven launches; clusters
-// are a sixteenth to a thirtieth of the particles in ordinary boxes).
-constexpr long long PACK_ONE = 1 << 20;
+// Up to this many particles one block does both scans of a gathered pass's packing (a
+// microsecond per 1000 clusters, 38 us for the 36k of a million particles, against the
+// 25 us of seven launches; clusters are a sixteenth to a thirtieth of the particles in
+// ordinary boxes).
+constexpr long long PACK_ONE = 1 << 19;
 void launch_pack_scan(struct Engine& E, long long nt, const unsigned int* ntd, const int* it_dev);
 long long radix_scratch_words(long long n);
 void radix_sort(unsigned long long* k0, unsigned int* v0, unsigned long long* k1, unsigned int* v1, long long n,

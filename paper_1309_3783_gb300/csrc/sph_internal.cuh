@@ -206,6 +206,15 @@ __device__ __forceinline__ double widen(float f) {
                                           ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
 
+// The FP64 value of any float (zeros, subnormals, infinities and NaN by the conversion).
+__device__ __forceinline__ double widen_any(float f) {
+  const unsigned int b = __float_as_uint(f), e = (b >> 23) & 0xffu;
+  if (e == 0u || e == 0xffu) return (double)f;
+  return __longlong_as_double((long long)(((unsigned long long)(b >> 31) << 63) |
+                                          ((unsigned long long)(e + 896u) << 52) |
+                                          ((unsigned long long)(b & 0x7fffffu) << 29)));
+}
+
 // ------------------------------------------------------------ warp helpers
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
