@@ -126,6 +126,33 @@ __global__ void k_check_build(cudaGraphConditionalHandle ok, const unsigned int*
   *status = held ? 1u : 0u;
 }
 
+// Thread w writes word w of the host's status (zero where there is no such counter yet).
+__global__ void k_read_status(HostStatus* out, const unsigned int* ea, const int* itv, const int* tn, const int* lc,
+                              const int* ntl, const unsigned long long* bcw, const unsigned int* gs,
+                              const unsigned int* flag, const unsigned int* rc, const unsigned int* g_n) {
+  pdl_wait();
+  const int w = threadIdx.x;
+  const unsigned int* src = nullptr;
+  if (w < 4) src = ea ? ea + w : nullptr;
+  else if (w < 8) src = itv ? reinterpret_cast<const unsigned int*>(itv) + w - 4 : nullptr;
+  else if (w < 16) src = tn ? reinterpret_cast<const unsigned int*>(tn) + w - 8 : nullptr;
+  else if (w < 24) src = lc ? reinterpret_cast<const unsigned int*>(lc) + w - 16 : nullptr;
+  else if (w == 24) src = ntl ? reinterpret_cast<const unsigned int*>(ntl) : nullptr;
+  else if (w < 27) src = bcw ? reinterpret_cast<const unsigned int*>(bcw) + w - 25 : nullptr;
+  else if (w == 27) src = gs;
+  else if (w == 28) src = flag;
+  else if (w == 29) src = rc;
+  else if (w == 30) src = g_n ? g_n + 1 : nullptr;
+  if (w < 31) reinterpret_cast<volatile unsigned int*>(out)[w] = src ? *src : 0u;
+}
+
+void launch_read_status(Engine& E) {
+  launch_pdl(k_read_status, 1, 32, E.st, E.hst, E.err_all.p, E.it_dev.p, E.t_n.p, E.l_counts.p,
+             E.dev_counters.p ? E.dev_counters.p + 4 : nullptr, E.big_count.p, E.gstat.p, E.reuse_flag.p, E.rec_ctr.p,
+             E.g_n.p);
+  count_launch();
+}
+
 // ============================================================== keys
 // floor(u 2^56) of u in [0, 1); 2^56 - 1 above and 0 below (invalid input, which the
 // ingest has flagged).  Exact for u >= 2^-4, else rounded down.

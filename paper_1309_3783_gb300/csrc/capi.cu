@@ -77,6 +77,7 @@ void launch_iter_next(Engine& E, cudaGraphConditionalHandle iter, cudaGraphCondi
 void launch_iter_step(Engine& E);
 void launch_set_drift(Engine& E);
 void launch_pass_setup(Engine& E, bool brackets, bool errors, int it);
+void launch_read_status(Engine& E);
 void launch_mark_active_cells(Engine& E);
 void launch_count_unconverged(Engine& E, int* out);
 void launch_task_offsets(Engine& E);
@@ -189,6 +190,8 @@ Engine::~Engine() {
   if (ev_fork) cudaEventDestroy(ev_fork);
   if (ev_join) cudaEventDestroy(ev_join);
   if (st_side) cudaStreamDestroy(st_side);
+  if (hst) cudaFreeHost(hst);
+  if (hbox_pin) cudaFreeHost(hbox_pin);
 }
 
 sph_status Engine::ensure_side_stream() {
@@ -203,6 +206,18 @@ sph_status Engine::ensure_side_stream() {
 cudaError_t Engine::sync_stream() {
   ++host_syncs;
   return cudaStreamSynchronize(st);
+}
+
+cudaError_t Engine::read_status() {
+  if (!hst) {
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&hst), sizeof(HostStatus), cudaHostAllocMapped);
+    if (e != cudaSuccess) {
+      hst = nullptr;
+      return e;
+    }
+  }
+  launch_read_status(*this);
+  return sync_stream();
 }
 
 int Engine::grid(long long work, int threads) const {
@@ -565,8 +580,16 @@ sph_status Engine::build_once(bool* retry) {
     launch_pdl(k_ingest, grid(N), 256, st, N, bid.p, box.p, x.p, v.p, m.p, u.p, h.p, prm.gamma_kernel, H_in.p); count_launch();
   }
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(hbox.data(), box.p, nbox * sizeof(BoxDesc), cudaMemcpyDeviceToHost, st));
+  if (hbox_pin_n < nbox) {
+    if (hbox_pin) cudaFreeHost(hbox_pin);
+    hbox_pin = nullptr;
+    hbox_pin_n = 0;
+    CK(cudaMallocHost(reinterpret_cast<void**>(&hbox_pin), (size_t)(nbox + nbox / 2) * sizeof(BoxDesc)));
+    hbox_pin_n = nbox + nbox / 2;
+  }
+  CK(cudaMemcpyAsync(hbox_pin, box.p, nbox * sizeof(BoxDesc), cudaMemcpyDeviceToHost, st));
   CK(sync_stream());
+  std::copy(hbox_pin, hbox_pin + nbox, hbox.begin());
   const int box_bits = ceil_log2(nbox);
   int dc = std::min(std::min(prm.max_depth, SPH_MAX_DEPTH), (64 - box_bits) / 3);
   int need = 0;
@@ -630,11 +653,11 @@ sph_status Engine::build_once(bool* retry) {
   // The tree's size is read before anything uses the tree: when it overflowed,
   // nodes past the last complete allocation were never written, and the build is
   // retried with more room before any kernel reads them.
+  CK(read_status());
   int tn[8];
   unsigned int ea[4];
-  CK(cudaMemcpyAsync(tn, t_n.p, sizeof(tn), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(ea, err_all.p, sizeof(ea), cudaMemcpyDeviceToHost, st));
-  CK(sync_stream());
+  std::copy(hst->tn, hst->tn + 8, tn);
+  std::copy(hst->ea, hst->ea + 4, ea);
   if (ea[0] & ERR_DEPTH) depth_hint = 0;     // the bound blocked a split: full depth
   if ((ea[0] & ERR_OVERFLOW) || tn[0] > cap_nodes) {
     sph_status s = ensure_tree_capacity(std::max(2 * cap_nodes, tn[0] + 1024));
@@ -720,14 +743,12 @@ sph_status Engine::build_once(bool* retry) {
   if (prm.pair_cache) launch_task_offsets(*this);
   prof_end(PH_AXIS_SORT, ev, l0);
   CK(cudaGetLastError());
+  CK(read_status());
   int lc[8];
-  unsigned long long bcw = 0;
-  CK(cudaMemcpyAsync(lc, l_counts.p, sizeof(lc), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&bcw, big_count.p, sizeof(bcw), cudaMemcpyDeviceToHost, st));
-  unsigned int ntl = 0;
-  CK(cudaMemcpyAsync(&ntl, dev_counters.p + 4, sizeof(ntl), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(ea, err_all.p, sizeof(ea), cudaMemcpyDeviceToHost, st));
-  CK(sync_stream());
+  std::copy(hst->lc, hst->lc + 8, lc);
+  std::copy(hst->ea, hst->ea + 4, ea);
+  const unsigned long long bcw = (unsigned long long)hst->bcw[0] | ((unsigned long long)hst->bcw[1] << 32);
+  const unsigned int ntl = hst->ntl;
   const int last_q = lc[2 + (rounds & 1)];
   if ((ea[0] & ERR_OVERFLOW) || lc[0] > cap_self || lc[1] > cap_pair || last_q != 0) {
     sph_status s = ensure_list_capacity(std::max(cap_self, lc[0]) * 2, std::max(cap_pair, lc[1]) * 2,
@@ -961,12 +982,11 @@ sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
       }
     }
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(itv, it_dev.p, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&ngath, g_n.p + 1, sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-    unsigned int rc = 0;
+    CK(read_status());
+    std::copy(hst->itv, hst->itv + 3, itv);
+    ngath = hst->ngath;
+    const unsigned int rc = hst->rc;
     const bool read_rec = rebuilds == 0 && it == 1 && rec_valid;
-    if (read_rec) CK(cudaMemcpyAsync(&rc, rec_ctr.p, sizeof(rc), cudaMemcpyDeviceToHost, st));
-    CK(sync_stream());
     if (read_rec) {
       rec_used = rc;
       rec_need = std::max<long long>(rec_need, rc);
@@ -1340,13 +1360,9 @@ sph_status Engine::step_graph() {
     if (s != SPH_OK) return s;
   }
   CK(cudaGraphLaunch(step_x, st));
-  unsigned int flag = 0, ea = 0, rc = 0;
-  int itv[2] = {0, 0};
-  CK(cudaMemcpyAsync(&flag, reuse_flag.p, sizeof(flag), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&ea, err_all.p, sizeof(ea), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(itv, it_dev.p, sizeof(itv), cudaMemcpyDeviceToHost, st));
-  if (R.pool) CK(cudaMemcpyAsync(&rc, rec_ctr.p, sizeof(rc), cudaMemcpyDeviceToHost, st));
-  CK(sync_stream());
+  CK(read_status());
+  const unsigned int flag = hst->flag, ea = hst->ea[0], rc = hst->rc;
+  const int itv[2] = {hst->itv[0], hst->itv[1]};
   if (R.pool && !flag) {
     rec_used = rc;
     rec_need = std::max<long long>(rec_need, rc);
@@ -1760,20 +1776,11 @@ sph_status Engine::build_step_graph() {
     if (s != SPH_OK) return s;
   }
   CK(cudaGraphLaunch(bstep_x, st));
-  unsigned int gs = 0, ea = 0;
-  int itv[2] = {0, 0}, tn[8], lc[8];
-  unsigned int ntl = 0;
-  unsigned long long bcw = 0;
-  CK(cudaMemcpyAsync(&gs, gstat.p, sizeof(gs), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&ea, err_all.p, sizeof(ea), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(itv, it_dev.p, sizeof(itv), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(tn, t_n.p, sizeof(tn), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(lc, l_counts.p, sizeof(lc), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&ntl, dev_counters.p + 4, sizeof(ntl), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&bcw, big_count.p, sizeof(bcw), cudaMemcpyDeviceToHost, st));
-  unsigned int rc = 0;
-  if (R.pool) CK(cudaMemcpyAsync(&rc, rec_ctr.p, sizeof(rc), cudaMemcpyDeviceToHost, st));
-  CK(sync_stream());
+  CK(read_status());
+  const unsigned int gs = hst->gs, ea = hst->ea[0], ntl = hst->ntl, rc = hst->rc;
+  const int itv[2] = {hst->itv[0], hst->itv[1]};
+  const int *tn = hst->tn, *lc = hst->lc;
+  const unsigned long long bcw = (unsigned long long)hst->bcw[0] | ((unsigned long long)hst->bcw[1] << 32);
   const bool held = gs == 1u;
   if (R.pool && held) {
     rec_used = rc;

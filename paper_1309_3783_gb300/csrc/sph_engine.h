@@ -76,6 +76,21 @@ long long radix_scratch_words(long long n);
 void radix_sort(unsigned long long* k0, unsigned int* v0, unsigned long long* k1, unsigned int* v1, long long n,
                 int bits, unsigned int* scratch, cudaStream_t st);
 
+// What the host reads where it waits for the stream: written by one kernel into mapped
+// page-locked memory.  (Copies to pageable memory return when they are done: seven of
+// them after a captured step were seven waits, 60 us.)
+struct HostStatus {
+  unsigned int ea[4];        // error bits
+  int itv[4];                // the h iteration: number, first active count, how it stopped
+  int tn[8];                 // tree counters
+  int lc[8];                 // list counters
+  unsigned int ntl;          // clusters
+  unsigned int bcw[2];       // cells for the global sort, and their entries (low, high half)
+  unsigned int gs, flag;     // a captured build held; a reuse test failed
+  unsigned int rc, ngath;    // pair records, gathered passes
+};
+static_assert(sizeof(HostStatus) == 31 * 4, "one word per thread of k_read_status");
+
 class Engine {
  public:
   Engine(const sph_params& prm, int device, cudaStream_t st);
@@ -259,6 +274,9 @@ class Engine {
   DBuf<unsigned int> n_units;
   bool unit_list = false;
   DBuf<int> dev_counters;         // [0] particles still active after a ghost pass
+  HostStatus* hst = nullptr;      // page-locked, mapped
+  BoxDesc* hbox_pin = nullptr;    // page-locked copy of the boxes, for the read after the ingest
+  int hbox_pin_n = 0;
   DBuf<unsigned char> staging;    // output staging (input order)
   DBuf<unsigned char> staging_many;   // one region per field of a multi-field read
 
@@ -331,6 +349,7 @@ class Engine {
   // helpers
   int grid(long long work, int threads = 256) const;
   cudaError_t sync_stream();
+  cudaError_t read_status();      // the device's counters into *hst, and waits for the stream
   sph_status cuda_fail(cudaError_t e, const char* where);
   sph_status fail(sph_status s, const std::string& msg);
   sph_status ensure_particle_capacity();
