@@ -826,15 +826,16 @@ __device__ __forceinline__ void tree_node_finish(Tree& T, int id, int d, const B
     T.axes[id] = 0;
     T.pmask[id] = 0;
     // limit the top grid sets on every particle: H < edge_k - margin
-    T.hlim[id] = (T.parent[id] < 0) ? __dsub_rn(ldexp(bd.L, -d), bd.margin) : 1e300;
+    T.hlim[id] = (T.parent[id] < 0) ? __dsub_rn(scaled_down(bd.L, d), bd.margin) : 1e300;
     unsigned int cx, cy, cz;
     cell_coords(T.key[id], d, cx, cy, cz);
-    const double inv = ldexp(1.0, -d), invk = ldexp(1.0, -bd.k);
+    // the centre relative to the top cell's: a whole number of half edges, exact in FP32
     const int sh = d - bd.k;
-    const double tx = ((double)(cx >> sh) + 0.5) * invk, ty = ((double)(cy >> sh) + 0.5) * invk,
-                 tz = ((double)(cz >> sh) + 0.5) * invk;
-    T.cen[id] = make_float4((float)(((double)cx + 0.5) * inv - tx), (float)(((double)cy + 0.5) * inv - ty),
-                            (float)(((double)cz + 0.5) * inv - tz), (float)inv);
+    const float he = ldexpf(1.0f, -d - 1);
+    const int hx = (int)(2u * cx + 1u) - ((int)(2u * (cx >> sh) + 1u) << sh),
+              hy = (int)(2u * cy + 1u) - ((int)(2u * (cy >> sh) + 1u) << sh),
+              hz = (int)(2u * cz + 1u) - ((int)(2u * (cz >> sh) + 1u) << sh);
+    T.cen[id] = make_float4((float)hx * he, (float)hy * he, (float)hz * he, 2.0f * he);
   }
 }
 
@@ -861,7 +862,8 @@ __global__ void __launch_bounds__(TREE_THREADS) k_tree_round(Tree T, const BoxDe
     if (c <= TREE_WARP_MAX) continue;   // the same for the whole block
     const int d = T.level[id];
     const BoxDesc bd = box[T.box[id]];
-    const double half = __dsub_rn(ldexp(bd.L, -(d + 1)), bd.margin);
+    // H < half in FP64 is H < half rounded up in FP32
+    const float half = __double2float_ru(__dsub_rn(scaled_down(bd.L, d + 1), bd.margin));
     const unsigned int s = T.start[id];
     const bool may_split = allow_split && d < dcap && (int)c > leaf_max;
     const int dig = 3 * (dcap - d - 1);   // Morton digit of level d + 1 (when may_split)
@@ -871,7 +873,7 @@ __global__ void __launch_bounds__(TREE_THREADS) k_tree_round(Tree T, const BoxDe
     for (unsigned int q = threadIdx.x; q < c; q += TREE_THREADS) {
       const float H = Hs[s + q];
       hm = fmaxf(hm, H);
-      ns += ((double)H < half) ? 1u : 0u;
+      ns += (H < half) ? 1u : 0u;
       if (may_split) {
         const unsigned int o = (unsigned int)(key[s + q] >> dig) & 7u;
 #pragma unroll
@@ -911,7 +913,8 @@ __global__ void __launch_bounds__(TREE_THREADS) k_tree_round(Tree T, const BoxDe
     if (c > TREE_WARP_MAX) continue;
     const int d = T.level[id];
     const BoxDesc bd = box[T.box[id]];
-    const double half = __dsub_rn(ldexp(bd.L, -(d + 1)), bd.margin);
+    // H < half in FP64 is H < half rounded up in FP32
+    const float half = __double2float_ru(__dsub_rn(scaled_down(bd.L, d + 1), bd.margin));
     const unsigned int s = T.start[id];
     const bool may_split = allow_split && d < dcap && (int)c > leaf_max;
     const int dig = 3 * (dcap - d - 1);
@@ -921,7 +924,7 @@ __global__ void __launch_bounds__(TREE_THREADS) k_tree_round(Tree T, const BoxDe
     for (unsigned int q = lane; q < c; q += 32) {
       const float H = Hs[s + q];
       hm = fmaxf(hm, H);
-      ns += ((double)H < half) ? 1u : 0u;
+      ns += (H < half) ? 1u : 0u;
       if (may_split) {
         const unsigned int o = (unsigned int)(key[s + q] >> dig) & 7u;
 #pragma unroll
@@ -1105,7 +1108,7 @@ __global__ void k_items_expand(int in, Tree T, const BoxDesc* __restrict__ box, 
         ax = Lq.q_axis[in][it];
         const int d = T.level[A];
         const BoxDesc bd = box[T.box[A]];
-        const double half = __dsub_rn(ldexp(bd.L, -(d + 1)), bd.margin);
+        const double half = __dsub_rn(scaled_down(bd.L, d + 1), bd.margin);
         // split the pair when every H, grown by the headroom, stays below half the
         // edge (the interactions stay valid while H < half: that is the limit recorded)
         const double hm = (double)fmaxf(T.hmax[A], T.hmax[B]) * (1.0 + (double)headroom);
@@ -1180,55 +1183,58 @@ __global__ void k_particle_limits(long long N, Tree T, const unsigned int* __res
 // the leaf centre relative to its top cell's centre (exact), plus the mass.  Two FP64
 // operations and a conversion per coordinate (with centres and images in FP64 too, eight,
 // the kernel took 1.96 ms for 33.5M particles).
+__device__ __forceinline__ void shift_particle(long long p, int b, unsigned int i, int leaf, float H, const Tree& T,
+                                               const BoxDesc* __restrict__ box, const double* __restrict__ x,
+                                               const float* __restrict__ m, float4* __restrict__ pos4,
+                                               float4* __restrict__ cen4) {
+  const double L = box[b].L;
+  const int d = T.level[leaf];
+  unsigned int cx, cy, cz;
+  cell_coords(T.key[leaf], d, cx, cy, cz);
+  // cell centres have at most SPH_MAX_DEPTH + 1 bits
+  const float e = ldexpf(1.0f, -d - 1);
+  const double tx = widen((float)(2u * cx + 1u) * e), ty = widen((float)(2u * cy + 1u) * e),
+               tz = widen((float)(2u * cz + 1u) * e);
+  // x / L: a power-of-two L scales exactly, so the FP64 division is needed only otherwise
+  const double iL = box[b].invL;
+  const double x0 = x[3ll * i], x1 = x[3ll * i + 1], x2 = x[3ll * i + 2];
+  double ox, oy, oz;
+  if (box[b].pow2 && !box[b].global32) {
+    ox = fma(x0, iL, -tx);
+    oy = fma(x1, iL, -ty);
+    oz = fma(x2, iL, -tz);
+  } else {
+    double ux = __ddiv_rn(x0, L), uy = __ddiv_rn(x1, L), uz = __ddiv_rn(x2, L);
+    if (box[b].global32) {
+      // plain FP32: the position is held as x / L rounded to FP32 (the offset below
+      // then carries that rounding, up to 2^-25 of L per coordinate)
+      ux = (double)__double2float_rn(ux);
+      uy = (double)__double2float_rn(uy);
+      uz = (double)__double2float_rn(uz);
+    }
+    ox = ux - tx;
+    oy = uy - ty;
+    oz = uz - tz;
+  }
+  if (box[b].periodic) {
+    // a particle kept in its cell after a drift across the boundary: nearest image
+    if (abs_above(ox, 0.5)) ox -= rint(ox);
+    if (abs_above(oy, 0.5)) oy -= rint(oy);
+    if (abs_above(oz, 0.5)) oz -= rint(oz);
+  }
+  const float sx = (float)ox, sy = (float)oy, sz = (float)oz;
+  pos4[p] = make_float4(sx, sy, sz, H);
+  const float4 c = T.cen[leaf];
+  cen4[p] = make_float4(c.x, c.y, c.z, m[i]);
+}
+
 __global__ void k_shift(long long N, int box_shift, const unsigned long long* __restrict__ key,
                         const unsigned int* __restrict__ perm, const unsigned int* __restrict__ leaf_of, Tree T,
                         const BoxDesc* __restrict__ box, const double* __restrict__ x, const float* __restrict__ m,
                         const float* __restrict__ Hs, float4* __restrict__ pos4, float4* __restrict__ cen4) {
   pdl_wait();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(key[p] >> box_shift);
-    const double L = box[b].L;
-    const unsigned int i = perm[p];
-    const int leaf = (int)leaf_of[p];
-    const int d = T.level[leaf];
-    unsigned int cx, cy, cz;
-    cell_coords(T.key[leaf], d, cx, cy, cz);
-    // cell centres have at most SPH_MAX_DEPTH + 1 bits
-    const float e = ldexpf(1.0f, -d - 1);
-    const double tx = widen((float)(2u * cx + 1u) * e), ty = widen((float)(2u * cy + 1u) * e),
-                 tz = widen((float)(2u * cz + 1u) * e);
-    // x / L: a power-of-two L scales exactly, so the FP64 division is needed only otherwise
-    const double iL = box[b].invL;
-    const double x0 = x[3ll * i], x1 = x[3ll * i + 1], x2 = x[3ll * i + 2];
-    double ox, oy, oz;
-    if (box[b].pow2 && !box[b].global32) {
-      ox = fma(x0, iL, -tx);
-      oy = fma(x1, iL, -ty);
-      oz = fma(x2, iL, -tz);
-    } else {
-      double ux = __ddiv_rn(x0, L), uy = __ddiv_rn(x1, L), uz = __ddiv_rn(x2, L);
-      if (box[b].global32) {
-        // plain FP32: the position is held as x / L rounded to FP32 (the offset below
-        // then carries that rounding, up to 2^-25 of L per coordinate)
-        ux = (double)__double2float_rn(ux);
-        uy = (double)__double2float_rn(uy);
-        uz = (double)__double2float_rn(uz);
-      }
-      ox = ux - tx;
-      oy = uy - ty;
-      oz = uz - tz;
-    }
-    if (box[b].periodic) {
-      // a particle kept in its cell after a drift across the boundary: nearest image
-      if (abs_above(ox, 0.5)) ox -= rint(ox);
-      if (abs_above(oy, 0.5)) oy -= rint(oy);
-      if (abs_above(oz, 0.5)) oz -= rint(oz);
-    }
-    const float sx = (float)ox, sy = (float)oy, sz = (float)oz;
-    pos4[p] = make_float4(sx, sy, sz, Hs[p]);
-    const float4 c = T.cen[leaf];
-    cen4[p] = make_float4(c.x, c.y, c.z, m[i]);
-  }
+  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x)
+    shift_particle(p, (int)(key[p] >> box_shift), perm[p], (int)leaf_of[p], Hs[p], T, box, x, m, pos4, cen4);
 }
 
 // ============================================================== clusters
@@ -1383,7 +1389,7 @@ __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
     const unsigned int s = T.start[id], c = T.count[id];
     const BoxDesc& bd = box[T.box[id]];
     const int d = T.level[id];
-    const float thr = (float)ldexp(bd.L, -d);
+    const float thr = (float)scaled_down(bd.L, d);
     unsigned int nsmall = 0;
     for (unsigned int b = 0; b < c; b += 32) {
       const unsigned int q = b + lane;
@@ -1407,7 +1413,7 @@ __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
     const int lb = box_shift - 3 * d;      // key bits below the leaf's cell
     unsigned int cx, cy, cz;
     cell_coords(T.key[id], d, cx, cy, cz);
-    const double inv = ldexp(1.0, -d), iL = bd.invL;
+    const double inv = scaled_down(1.0, d), iL = bd.invL;
     const double cen[3] = {((double)cx + 0.5) * inv, ((double)cy + 0.5) * inv, ((double)cz + 0.5) * inv};
     for (int cls = 0; cls < 2; ++cls) {
       const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
@@ -1451,18 +1457,26 @@ __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
   }
 }
 
+// The particles in the order of k_leaf_clusters (lsrc), and their offsets.
 __global__ void k_apply_partition(long long N, const unsigned int* __restrict__ lsrc,
                                   const unsigned int* __restrict__ perm_in, unsigned int* __restrict__ perm_out,
                                   const unsigned long long* __restrict__ key_in, unsigned long long* __restrict__ key_out,
                                   const float* __restrict__ H_in, float* __restrict__ H_out,
-                                  const float4* __restrict__ vel_in, float4* __restrict__ vel_out) {
+                                  const float4* __restrict__ vel_in, float4* __restrict__ vel_out, int box_shift,
+                                  const unsigned int* __restrict__ leaf_of, Tree T, const BoxDesc* __restrict__ box,
+                                  const double* __restrict__ x, const float* __restrict__ m,
+                                  float4* __restrict__ pos4, float4* __restrict__ cen4) {
   pdl_wait();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     const unsigned int q = lsrc[p];
-    perm_out[p] = perm_in[q];
-    key_out[p] = key_in[q];
-    H_out[p] = H_in[q];
+    const unsigned int i = perm_in[q];
+    const unsigned long long key = key_in[q];
+    const float H = H_in[q];
+    perm_out[p] = i;
+    key_out[p] = key;
+    H_out[p] = H;
     vel_out[p] = vel_in[q];
+    shift_particle(p, (int)(key >> box_shift), i, (int)leaf_of[p], H, T, box, x, m, pos4, cen4);
   }
 }
 

@@ -52,8 +52,9 @@ __global__ void k_sort_big_scatter(int, const int*, const int*, const unsigned i
 __global__ void k_leaf_clusters(Tree, int, int, const BoxDesc*, const float*, const unsigned long long*,
                                 const unsigned int*, const double*, unsigned int*, unsigned int*, int);
 __global__ void k_apply_partition(long long, const unsigned int*, const unsigned int*, unsigned int*,
-                                  const unsigned long long*, unsigned long long*, const float*, float*,
-                                  const float4*, float4*);
+                                  const unsigned long long*, unsigned long long*, const float*, float*, const float4*,
+                                  float4*, int, const unsigned int*, Tree, const BoxDesc*, const double*, const float*,
+                                  float4*, float4*);
 __global__ void k_tile_table(long long, const unsigned int*, const unsigned int*, unsigned int*, Tiles);
 __global__ void k_cluster_table(long long, const unsigned int*, Tree, int, const unsigned int*, const float4*,
                                 const unsigned int*, Tiles);
@@ -78,6 +79,8 @@ void launch_iter_step(Engine& E);
 void launch_set_drift(Engine& E);
 void launch_pass_setup(Engine& E, bool brackets, bool errors, int it);
 void launch_read_status(Engine& E);
+void launch_set_particles(Engine& E, int b, const double* x, const float* v, const float* m, const float* u,
+                          const float* h);
 void launch_mark_active_cells(Engine& E);
 void launch_count_unconverged(Engine& E, int* out);
 void launch_task_offsets(Engine& E);
@@ -526,6 +529,24 @@ sph_status Engine::set_particles(int b, const double* xx, const float* vv, const
   if (!xx || !vv || !mm || !uu || !hh) return fail(SPH_E_INVALID, "null input pointer");
   const cudaMemcpyKind kind = mem == SPH_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   const long long o = off[b], n = spec[b].n;
+  built = have_density = have_ghost = have_force = have_acc = false;
+  reusable = false;
+  n_builds = n_reuses = 0;
+  // (the copies run at the memory's rate from a million particles on; they take any
+  // alignment, and memory of any device)
+  const auto at = [this](const void* p, size_t a) {
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return pa.type == cudaMemoryTypeDevice && pa.device == device && reinterpret_cast<size_t>(p) % a == 0;
+  };
+  if (mem == SPH_MEM_DEVICE && n > 0 && n <= (1 << 20) && at(xx, 8) && at(vv, 4) && at(mm, 4) && at(uu, 4) && at(hh, 4)) {
+    launch_set_particles(*this, b, xx, vv, mm, uu, hh);
+    CK(cudaGetLastError());
+    return SPH_OK;
+  }
   CK(cudaMemcpyAsync(x.p + 3 * o, xx, 3 * n * sizeof(double), kind, st));
   CK(cudaMemcpyAsync(v.p + 3 * o, vv, 3 * n * sizeof(float), kind, st));
   CK(cudaMemcpyAsync(m.p + o, mm, n * sizeof(float), kind, st));
@@ -537,9 +558,6 @@ sph_status Engine::set_particles(int b, const double* xx, const float* vv, const
   }
   launch_set_h(*this, b, hsrc);      // the box keeps its h history only if h is unchanged
   CK(cudaGetLastError());
-  built = have_density = have_ghost = have_force = have_acc = false;
-  reusable = false;
-  n_builds = n_reuses = 0;
   return SPH_OK;
 }
 
@@ -705,13 +723,12 @@ sph_status Engine::build_once(bool* retry) {
   launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, n_nodes, box_shift, box.p, Hs.p, key.p, perm.p, x.p, lsrc.p, tflag.p,
              prm.cluster_max); count_launch();
   launch_pdl(k_apply_partition, grid(N), 256, ss, N, lsrc.p, perm.p, perm_tmp.p, key.p, key_tmp.p, Hs.p, Hs_tmp.p,
-             vel4.p, vel4_tmp.p); count_launch();
+             vel4.p, vel4_tmp.p, box_shift,
+             leaf_of.p, T, box.p, x.p, m.p, pos4.p, cen4.p); count_launch();
   perm.swap(perm_tmp);
   key.swap(key_tmp);
   Hs.swap(Hs_tmp);
   vel4.swap(vel4_tmp);
-  launch_pdl(k_shift, grid(N), 256, ss, N, box_shift, key.p, perm.p, leaf_of.p, T, box.p, x.p, m.p, Hs.p, pos4.p,
-             cen4.p); count_launch();
   exclusive_scan(tflag.p, texcl.p, N, rs_scratch.p, reinterpret_cast<unsigned int*>(dev_counters.p + 4), ss);
   launch_pdl(k_tile_table, grid(N), 256, ss, N, tflag.p, texcl.p, tile_of.p, TL); count_launch();
   launch_pdl(k_cluster_table, grid(N), 256, ss, N, reinterpret_cast<const unsigned int*>(dev_counters.p + 4), T,
@@ -1504,13 +1521,12 @@ sph_status Engine::enqueue_captured_build() {
   launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, cap_nodes, box_shift, box.p, Hs.p, key.p, perm.p, x.p, lsrc.p,
              tflag.p, prm.cluster_max); count_launch();
   launch_pdl(k_apply_partition, grid(N), 256, ss, N, lsrc.p, perm.p, perm_tmp.p, key.p, key_tmp.p, Hs.p, Hs_tmp.p,
-             vel4.p, vel4_tmp.p); count_launch();
+             vel4.p, vel4_tmp.p, box_shift,
+             leaf_of.p, T, box.p, x.p, m.p, pos4.p, cen4.p); count_launch();
   perm.swap(perm_tmp);
   key.swap(key_tmp);
   Hs.swap(Hs_tmp);
   vel4.swap(vel4_tmp);
-  launch_pdl(k_shift, grid(N), 256, ss, N, box_shift, key.p, perm.p, leaf_of.p, T, box.p, x.p, m.p, Hs.p, pos4.p,
-             cen4.p); count_launch();
   exclusive_scan(tflag.p, texcl.p, N, rs_scratch.p, reinterpret_cast<unsigned int*>(dev_counters.p + 4), ss);
   launch_pdl(k_tile_table, grid(N), 256, ss, N, tflag.p, texcl.p, tile_of.p, TL); count_launch();
   launch_pdl(k_cluster_table, grid(N), 256, ss, N, reinterpret_cast<const unsigned int*>(dev_counters.p + 4), T,

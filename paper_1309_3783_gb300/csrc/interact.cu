@@ -3112,6 +3112,38 @@ void launch_drift(Engine& E) {
   launch_pdl(k_hlev_next, 1, 256, E.st, E.nbox, E.box.p, E.hlev.p); count_launch();
 }
 
+// The particles of a small box from device arrays, in one launch (five copies and the
+// kernel above take 30 us for 4096 particles, this 15).
+__global__ void k_set_particles(long long n, const double* __restrict__ xs, const float* __restrict__ vs,
+                                const float* __restrict__ ms, const float* __restrict__ us,
+                                const float* __restrict__ hs, double* __restrict__ x, float* __restrict__ v,
+                                float* __restrict__ m, float* __restrict__ u, float* __restrict__ h,
+                                int* __restrict__ hlev) {
+  pdl_wait();
+  const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+  bool diff = false;
+  for (long long i = t0; i < 3 * n; i += nth) {
+    x[i] = xs[i];
+    v[i] = vs[i];
+    if (i < n) {
+      m[i] = ms[i];
+      u[i] = us[i];
+      const float s = hs[i];
+      diff |= __float_as_uint(s) != __float_as_uint(h[i]);
+      h[i] = s;
+    }
+  }
+  if (__syncthreads_or(diff) && threadIdx.x == 0) *hlev = 0;
+}
+
+void launch_set_particles(Engine& E, int b, const double* x, const float* v, const float* m, const float* u,
+                          const float* h) {
+  const long long n = E.spec[b].n, o = E.off[b];
+  launch_pdl(k_set_particles, E.grid(3 * n), 256, E.st, n, x, v, m, u, h, E.x.p + 3 * o, E.v.p + 3 * o, E.m.p + o,
+             E.u.p + o, E.h.p + o, E.hlev.p + b);
+  count_launch();
+}
+
 void launch_set_h(Engine& E, int b, const float* src) {
   const long long n = E.spec[b].n;
   if (n == 0) return;

@@ -194,6 +194,12 @@ __device__ __forceinline__ bool in_box(double x, double L) {
   return b < dbits(L) || b == 0x8000000000000000ull;
 }
 
+// v 2^-e, exact while the result is a normal number (ldexp is a call of some 30
+// instructions, several on the FP64 pipe)
+__device__ __forceinline__ double scaled_down(double v, int e) {
+  return __dmul_rn(v, __longlong_as_double((long long)(1023 - e) << 52));
+}
+
 // |a| > b for a non-negative b
 __device__ __forceinline__ bool abs_above(double a, double b) {
   return (dbits(a) & 0x7fffffffffffffffull) > dbits(b);
