@@ -368,20 +368,27 @@ __global__ void k_tile_boxes(long long ntile, Tiles TL, const float4* __restrict
 // ============================================================== radix sort
 // Stable LSD radix sort of (64-bit key, 32-bit value), 8-bit digits.  Each
 // pass: per-tile digit histograms, one exclusive scan of the digit-major
-// histogram table, then a stable scatter that ranks equal digits by
-// (round, warp, lane) order inside the tile.
+// histogram table, then a stable scatter.  A tile's warps take runs of it and rank
+// their keys among themselves, round by round, without waiting for one another; one
+// scan over the warps and digits then places every key in the tile, where the tile is
+// put in order in shared memory, so that equal digits leave in whole runs.  (Ranking
+// round by round over the whole block, with three barriers each, and writing every
+// key straight to its place took 15 us a pass for 10^5 keys and 0.24 to 0.56 ms for
+// 33.5M.)  Tiles of 4096, or of 1024 where that leaves multiprocessors without one.
 constexpr int RS_THREADS = 256;
-constexpr int RS_ITEMS = 8;
-constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+constexpr int RS_WARPS = RS_THREADS / 32;
+static int rs_items(long long n) { return n <= (1 << 18) ? 4 : 16; }
 
-__global__ void k_radix_hist(long long n, const unsigned long long* __restrict__ key, int shift,
-                             unsigned int* __restrict__ hist, int ntiles) {
+template <int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(long long n, const unsigned long long* __restrict__ key,
+                                                           int shift, unsigned int* __restrict__ hist, int ntiles) {
   pdl_wait();
   __shared__ unsigned int cnt[256];
   cnt[threadIdx.x] = 0;
   __syncthreads();
-  const long long base = (long long)blockIdx.x * RS_TILE;
-  for (int r = 0; r < RS_ITEMS; ++r) {
+  const long long base = (long long)blockIdx.x * (RS_THREADS * ITEMS);
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
     const long long i = base + r * RS_THREADS + threadIdx.x;
     if (i < n) atomicAdd(&cnt[(unsigned int)(key[i] >> shift) & 255u], 1u);
   }
@@ -389,43 +396,86 @@ __global__ void k_radix_hist(long long n, const unsigned long long* __restrict__
   hist[(long long)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
-__global__ void k_radix_scatter(long long n, const unsigned long long* __restrict__ kin,
-                                const unsigned int* __restrict__ vin, unsigned long long* __restrict__ kout,
-                                unsigned int* __restrict__ vout, int shift, const unsigned int* __restrict__ offs,
-                                int ntiles) {
+__device__ unsigned int block_exclusive_scan(unsigned int v, unsigned int* tmp, unsigned int& total);
+
+template <int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(long long n, const unsigned long long* __restrict__ kin,
+                                                              const unsigned int* __restrict__ vin,
+                                                              unsigned long long* __restrict__ kout,
+                                                              unsigned int* __restrict__ vout, int shift,
+                                                              const unsigned int* __restrict__ offs, int ntiles) {
   pdl_wait();
-  __shared__ unsigned int base[256];
-  __shared__ unsigned int wcnt[RS_THREADS / 32][256];
+  constexpr int TILE = RS_THREADS * ITEMS;
+  __shared__ unsigned long long sk[TILE];          // the tile's keys in order, then its values
+  __shared__ unsigned int wcnt[RS_WARPS][256];     // keys of a digit in the warps before
+  __shared__ unsigned int gbase[256];              // where the tile's run of a digit goes, less its place in the tile
+  __shared__ unsigned int tmp[32];
+  unsigned int* sv = reinterpret_cast<unsigned int*>(sk);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  base[tid] = offs[(long long)tid * ntiles + blockIdx.x];
-  for (int k = 0; k < RS_THREADS / 32; ++k) wcnt[k][tid] = 0;
+  const long long tile0 = (long long)blockIdx.x * TILE;
+  const int cnt = (int)min((long long)TILE, n - tile0);
+  const unsigned int goff = offs[(long long)tid * ntiles + blockIdx.x];
+  for (int k = 0; k < RS_WARPS; ++k) wcnt[k][tid] = 0;
+  unsigned long long key[ITEMS];
+  unsigned int val[ITEMS], at[ITEMS];
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const int i = (w * ITEMS + r) * 32 + lane;
+    key[r] = i < cnt ? kin[tile0 + i] : 0ull;
+    val[r] = i < cnt ? vin[tile0 + i] : 0u;
+  }
   __syncthreads();
-  const long long tile0 = (long long)blockIdx.x * RS_TILE;
   const unsigned int lt = (1u << lane) - 1u;
-  for (int r = 0; r < RS_ITEMS; ++r) {
-    const long long i = tile0 + r * RS_THREADS + tid;
-    const bool valid = i < n;
-    unsigned long long k = valid ? kin[i] : 0ull;
-    const unsigned int d = valid ? ((unsigned int)(k >> shift) & 255u) : 256u;
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const bool valid = (w * ITEMS + r) * 32 + lane < cnt;
+    const unsigned int d = valid ? ((unsigned int)(key[r] >> shift) & 255u) : 256u;
     const unsigned int peers = __match_any_sync(0xffffffffu, d);
-    const unsigned int lrank = __popc(peers & lt);
-    if (valid && lrank == 0) wcnt[w][d] = __popc(peers);
-    __syncthreads();
-    if (valid) {
-      unsigned int pre = 0;
-      for (int q = 0; q < w; ++q) pre += wcnt[q][d];
-      const unsigned int pos = base[d] + pre + lrank;
-      kout[pos] = k;
-      vout[pos] = vin[i];
+    const unsigned int before = valid ? wcnt[w][d] : 0u;
+    at[r] = before + __popc(peers & lt);
+    __syncwarp();
+    if (valid && (peers & lt) == 0u) wcnt[w][d] = before + __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  unsigned int sum = 0;
+  for (int k = 0; k < RS_WARPS; ++k) {
+    const unsigned int c = wcnt[k][tid];
+    wcnt[k][tid] = sum;
+    sum += c;
+  }
+  unsigned int total;
+  const unsigned int first = block_exclusive_scan(sum, tmp, total);
+  gbase[tid] = goff - first;
+  for (int k = 0; k < RS_WARPS; ++k) wcnt[k][tid] += first;
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    if ((w * ITEMS + r) * 32 + lane < cnt) {
+      at[r] += wcnt[w][(unsigned int)(key[r] >> shift) & 255u];
+      sk[at[r]] = key[r];
     }
-    __syncthreads();
-    unsigned int tot = 0;
-    for (int q = 0; q < RS_THREADS / 32; ++q) {
-      tot += wcnt[q][tid];
-      wcnt[q][tid] = 0;
+  }
+  __syncthreads();
+  unsigned int dst[ITEMS];
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const int i = r * RS_THREADS + tid;
+    if (i < cnt) {
+      const unsigned long long k = sk[i];
+      dst[r] = gbase[(unsigned int)(k >> shift) & 255u] + (unsigned int)i;
+      kout[dst[r]] = k;
     }
-    base[tid] += tot;
-    __syncthreads();
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r)
+    if ((w * ITEMS + r) * 32 + lane < cnt) sv[at[r]] = val[r];
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const int i = r * RS_THREADS + tid;
+    if (i < cnt) vout[dst[r]] = sv[i];
   }
 }
 
@@ -624,26 +674,37 @@ void launch_pack_scan(Engine& E, long long nt, const unsigned int* ntd, const in
 }
 
 long long radix_scratch_words(long long n) {
-  const long long ntiles = (n + RS_TILE - 1) / RS_TILE;
-  return 256 * ntiles + (256 * ntiles + SC_TILE - 1) / SC_TILE + 16;
+  // (tiles of 1024 and of 4096: the scratch of a size covers every smaller one too)
+  const long long small = (std::min<long long>(n, 1 << 18) + 1023) / 1024, large = (n + 4095) / 4096;
+  const long long ntiles = std::max(small, large);
+  const long long words = 256 * ntiles + (256 * ntiles + SC_TILE - 1) / SC_TILE + 16;
+  return std::max(words, (n + SC_TILE - 1) / SC_TILE + 16);
 }
 
-// Sorts (k0, v0) by the low `bits` bits of the key; the result lands in
-// (k0, v0) (using (k1, v1) as the other half of each pass).
-void radix_sort(unsigned long long* k0, unsigned int* v0, unsigned long long* k1, unsigned int* v1, long long n,
-                int bits, unsigned int* scratch, cudaStream_t st) {
-  if (n <= 1 || bits <= 0) return;
-  const long long ntiles = (n + RS_TILE - 1) / RS_TILE;
+int radix_passes(int bits) { return (bits + 7) / 8; }
+
+template <int ITEMS>
+static void radix_pass(long long n, int shift, const unsigned long long* ka, const unsigned int* va,
+                       unsigned long long* kb, unsigned int* vb, unsigned int* scratch, cudaStream_t st) {
+  const long long ntiles = (n + RS_THREADS * ITEMS - 1) / (RS_THREADS * ITEMS);
   unsigned int* hist = scratch;
-  unsigned int* sums = scratch + 256 * ntiles;
-  int passes = (bits + 7) / 8;
-  unsigned long long *ka = k0, *kb = k1;
-  unsigned int *va = v0, *vb = v1;
+  launch_pdl(k_radix_hist<ITEMS>, (unsigned)ntiles, RS_THREADS, st, n, ka, shift, hist, (int)ntiles); count_launch();
+  exclusive_scan(hist, hist, 256 * ntiles, scratch + 256 * ntiles, nullptr, st);
+  launch_pdl(k_radix_scatter<ITEMS>, (unsigned)ntiles, RS_THREADS, st, n, ka, va, kb, vb, shift, hist, (int)ntiles);
+  count_launch();
+}
+
+// Sorts (k0, v0), or with from_second what lies in (k1, v1), by the low `bits` bits of
+// the key; the result lands in (k0, v0), without a copy when the number of passes is odd
+// for an input in (k1, v1) and even otherwise.
+void radix_sort(unsigned long long* k0, unsigned int* v0, unsigned long long* k1, unsigned int* v1, long long n,
+                int bits, unsigned int* scratch, cudaStream_t st, bool from_second) {
+  unsigned long long *ka = from_second ? k1 : k0, *kb = from_second ? k0 : k1;
+  unsigned int *va = from_second ? v1 : v0, *vb = from_second ? v0 : v1;
+  const int passes = n > 1 ? radix_passes(std::max(bits, 0)) : 0;
   for (int p = 0; p < passes; ++p) {
-    const int shift = 8 * p;
-    launch_pdl(k_radix_hist, (unsigned)ntiles, RS_THREADS, st, n, ka, shift, hist, (int)ntiles); count_launch();
-    exclusive_scan(hist, hist, 256 * ntiles, sums, nullptr, st);
-    launch_pdl(k_radix_scatter, (unsigned)ntiles, RS_THREADS, st, n, ka, va, kb, vb, shift, hist, (int)ntiles); count_launch();
+    if (rs_items(n) == 4) radix_pass<4>(n, 8 * p, ka, va, kb, vb, scratch, st);
+    else radix_pass<16>(n, 8 * p, ka, va, kb, vb, scratch, st);
     std::swap(ka, kb);
     std::swap(va, vb);
   }

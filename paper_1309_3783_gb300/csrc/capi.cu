@@ -646,8 +646,10 @@ sph_status Engine::build_once(bool* retry) {
   // ---- keys and sort
   long long l0;
   int ev = prof_begin(PH_SORT, &l0);
-  launch_pdl(k_keys, grid(N), 256, st, N, dcap, bid.p, box.p, x.p, key.p, perm.p); count_launch();
-  radix_sort(key.p, perm.p, key_tmp.p, perm_tmp.p, N, key_bits, rs_scratch.p, st);
+  const bool odd = (radix_passes(key_bits) & 1) != 0;
+  launch_pdl(k_keys, grid(N), 256, st, N, dcap, bid.p, box.p, x.p, odd ? key_tmp.p : key.p, odd ? perm_tmp.p : perm.p);
+  count_launch();
+  radix_sort(key.p, perm.p, key_tmp.p, perm_tmp.p, N, key_bits, rs_scratch.p, st, odd);
   launch_pdl(k_gather_sorted, grid(N), 256, st, N, perm.p, H_in.p, v.p, u.p, bid.p, box.p, a_in.p, vpred, Hs.p,
                                            vel4.p); count_launch();
   prof_end(PH_SORT, ev, l0);
@@ -1483,8 +1485,10 @@ sph_status Engine::enqueue_captured_build() {
   launch_pdl(k_check_shape, 1, 256, st, nbox, box.p, dc, prm.split_headroom, err_all.p); count_launch();
   long long l0;
   int ev = prof_begin(PH_SORT, &l0);
-  launch_pdl(k_keys, grid(N), 256, st, N, dcap, bid.p, box.p, x.p, key.p, perm.p); count_launch();
-  radix_sort(key.p, perm.p, key_tmp.p, perm_tmp.p, N, key_bits, rs_scratch.p, st);
+  const bool odd = (radix_passes(key_bits) & 1) != 0;
+  launch_pdl(k_keys, grid(N), 256, st, N, dcap, bid.p, box.p, x.p, odd ? key_tmp.p : key.p, odd ? perm_tmp.p : perm.p);
+  count_launch();
+  radix_sort(key.p, perm.p, key_tmp.p, perm_tmp.p, N, key_bits, rs_scratch.p, st, odd);
   launch_pdl(k_gather_sorted, grid(N), 256, st, N, perm.p, H_in.p, v.p, u.p, bid.p, box.p, a_in.p, vpred, Hs.p,
              vel4.p); count_launch();
   prof_end(PH_SORT, ev, l0);

@@ -74,7 +74,8 @@ constexpr long long PACK_ONE = 1 << 19;
 void launch_pack_scan(struct Engine& E, long long nt, const unsigned int* ntd, const int* it_dev);
 long long radix_scratch_words(long long n);
 void radix_sort(unsigned long long* k0, unsigned int* v0, unsigned long long* k1, unsigned int* v1, long long n,
-                int bits, unsigned int* scratch, cudaStream_t st);
+                int bits, unsigned int* scratch, cudaStream_t st, bool from_second = false);
+int radix_passes(int bits);
 
 // What the host reads where it waits for the stream: written by one kernel into mapped
 // page-locked memory.  (Copies to pageable memory return when they are done: seven of
