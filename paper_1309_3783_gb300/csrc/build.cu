@@ -666,6 +666,7 @@ __global__ void __launch_bounds__(1024) k_pack_scan(long long ntcap, const unsig
     scan_store(nt + 1, v, base, run, make_uint4(c[0], c[1], c[2], c[3]));
     carry += total;
   }
+  if (threadIdx.x == 0) pk_tot[1] = carry;
 }
 
 void launch_pack_scan(Engine& E, long long nt, const unsigned int* ntd, const int* it_dev) {
@@ -886,6 +887,7 @@ __device__ __forceinline__ void tree_node_finish(Tree& T, int id, int d, const B
     T.nchild[id] = (sp && fits) ? nch : 0;
     T.axes[id] = 0;
     T.pmask[id] = 0;
+    T.rmask[id] = 0;
     // limit the top grid sets on every particle: H < edge_k - margin
     T.hlim[id] = (T.parent[id] < 0) ? __dsub_rn(scaled_down(bd.L, d), bd.margin) : 1e300;
     unsigned int cx, cy, cz;
@@ -1608,25 +1610,25 @@ __global__ void k_mark_axes(Lists Lq, int cap_pair, Tree T) {
     const unsigned int bit = 1u << Lq.pair_axis[i];
     const int A = Lq.pair_a[i];
     atomicOr(&T.axes[A], bit);
-    atomicOr(&T.axes[Lq.pair_b[i]], bit);
+    const int B = Lq.pair_b[i];
+    atomicOr(&T.axes[B], bit);
     atomicOr(&T.pmask[A], bit);
+    atomicOr(&T.rmask[B], bit);
   }
 }
 
-// The pairs by their first cell, and the number of (pair, cluster of the first cell)
-// tasks, which bounds the gathered passes' task list.
+// The pairs by cell: those of which it is the first, by axis, then those of which it is
+// the second.
 __global__ void k_pair_csr(Lists Lq, int cap_pair, Tree T) {
   pdl_wait();
   const int n = min(Lq.counts[1], cap_pair);
-  unsigned int tasks = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int A = Lq.pair_a[i];
-    const int ax = Lq.pair_axis[i];
-    Lq.csr[T.pstart[A] + (unsigned int)__popc(T.pmask[A] & ((1u << ax) - 1u))] = make_uint2((unsigned int)Lq.pair_b[i], (unsigned int)ax);
-    tasks += T.ntile[A];
+    const int A = Lq.pair_a[i], B = Lq.pair_b[i], ax = Lq.pair_axis[i];
+    const unsigned int below = (1u << ax) - 1u;
+    Lq.csr[T.pstart[A] + (unsigned int)__popc(T.pmask[A] & below)] = make_uint2((unsigned int)B, (unsigned int)ax);
+    Lq.csr[T.pstart[B] + (unsigned int)(__popc(T.pmask[B]) + __popc(T.rmask[B] & below))] =
+        make_uint2((unsigned int)A, (unsigned int)ax | 16u);
   }
-  tasks = __reduce_add_sync(0xffffffffu, tasks);
-  if ((threadIdx.x & 31) == 0 && tasks) atomicAdd(&Lq.counts[6], (int)tasks);
 }
 
 // Storage for the sorted lists: every (cell, needed axis) gets ntile entries.
@@ -1647,7 +1649,7 @@ __global__ void k_sort_alloc(Tree T, int nnodes, Lists Lq, int* __restrict__ big
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nnodes; id += gridDim.x * blockDim.x) {
     const unsigned int ax = T.axes[id];
     if (!ax) continue;
-    const unsigned int npr = (unsigned int)__popc(T.pmask[id]);
+    const unsigned int npr = (unsigned int)(__popc(T.pmask[id]) + __popc(T.rmask[id]));
     if (npr) T.pstart[id] = (unsigned int)atomicAdd(&Lq.counts[8], (int)npr);
     const unsigned int c = T.ntile[id];
     if (c <= 32u) {

@@ -431,6 +431,7 @@ sph_status Engine::ensure_tree_capacity(int nodes) {
   CK(t_axes.reserve(n));
   CK(t_sortbase.reserve(n));
   CK(t_pmask.reserve(n));
+  CK(t_rmask.reserve(n));
   CK(t_pstart.reserve(n));
   CK(t_key.reserve(n));
   CK(t_level.reserve(n));
@@ -467,6 +468,7 @@ sph_status Engine::ensure_tree_capacity(int nodes) {
   T.axes = t_axes.p;
   T.sortbase = t_sortbase.p;
   T.pmask = t_pmask.p;
+  T.rmask = t_rmask.p;
   T.pstart = t_pstart.p;
   T.active = t_active.p;
   T.changed = t_changed.p;
@@ -493,7 +495,7 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
     CK(l_pb.reserve(pairs));
     CK(l_pax.reserve(pairs));
     CK(l_ptoff.reserve(pairs + 1));
-    CK(l_csr.reserve(pairs));
+    CK(l_csr.reserve(2 * (size_t)pairs));
   }
   CK(scan_tmp.reserve((size_t)std::max(cap_pair, cap_self) / 2048 + 64));
   if (queue > cap_queue || !q_kind[0].p) {
@@ -794,7 +796,6 @@ sph_status Engine::build_once(bool* retry) {
   n_big_entries = bc[1];
   n_ptasks = lc[6];
   n_stasks = ntl;           // the self interactions are the leaves': one task per cluster
-  CK(g_live.reserve(std::max<size_t>((size_t)(n_ptasks + n_stasks), 1)));
   if (prm.pair_cache) {     // the passes list their tasks, for their pair records
     CK(l_ptask.reserve(std::max<size_t>((size_t)n_ptasks, 1)));
     CK(l_stask.reserve(std::max<size_t>((size_t)n_stasks, 1)));
@@ -1579,7 +1580,6 @@ sph_status Engine::capture_build_graph() {
   // capacities with room to grow: a count past one makes the build not hold, and
   // the host completes that step with a build of its own
   const size_t cp = (size_t)(n_ptasks + n_ptasks / 4 + 1024), cs = (size_t)(n_stasks + n_stasks / 4 + 1024);
-  CK(g_live.reserve(cp + cs));
   if (prm.pair_cache) {
     CK(l_ptask.reserve(cp));
     CK(l_stask.reserve(cs));

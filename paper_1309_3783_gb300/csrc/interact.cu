@@ -211,12 +211,6 @@ struct Counters {
   unsigned int cand = 0, pairs = 0, sides = 0, rechecks = 0;
 };
 
-// A later pass of the h iteration gathers (the symmetric tasks stand aside) when
-// its task builder chose to and its tasks fitted the buffer.
-__device__ __forceinline__ bool gather_on(const int* gflag, const unsigned int* g_n, unsigned int cap_g) {
-  return gflag[0] != 0 && *g_n <= cap_g;
-}
-
 template <bool COUNT>
 __device__ __forceinline__ void commit_counters(const Counters& C, unsigned long long* pc, int which) {
   if (!COUNT) return;
@@ -1263,7 +1257,10 @@ __device__ __forceinline__ unsigned int unit_first(const UnitShared& K, int it) 
 // box and, in a later pass (PART; iact: the own cluster holds iterating particles),
 // iterates itself or meets the own cluster's.  K.cell is -1 past the last group.
 // The cell edge sets the guard band (K.eb; it grows along the chain).
-template <bool PART>
+// GATHER (the own side only, of a packed cluster): the pairs of which the cell is the
+// second come too, the self interaction has all of the leaf's clusters, and only the own
+// reach counts.
+template <bool PART, bool GATHER>
 __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T, const uint2* __restrict__ csr,
                                                    bool iact) {
   const int lane = threadIdx.x & 31;
@@ -1271,7 +1268,8 @@ __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T,
   const unsigned int at = K.at, idx = K.idx;
   const int d = T.level[A];
   const bool leaf = T.child[A] < 0;
-  const unsigned int n = (unsigned int)__popc(T.pmask[A]) + (leaf ? 1u : 0u);     // a leaf's list starts with its self interaction
+  // a leaf's list starts with its self interaction
+  const unsigned int n = (unsigned int)__popc(T.pmask[A]) + (GATHER ? (unsigned int)__popc(T.rmask[A]) : 0u) + (leaf ? 1u : 0u);
   const unsigned int mine = at + lane;
   const bool valid = lane < GROUP && mine < n;
   bool live = false;
@@ -1284,8 +1282,14 @@ __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T,
       B = (int)pr.x;
       ax = (int)pr.y;
     }
+    const bool second = GATHER && (ax & 16) != 0;
     int dx, dy, dz;
-    axis_vec(ax, dx, dy, dz);
+    axis_vec(GATHER ? ax & 15 : ax, dx, dy, dz);
+    if (second) {
+      dx = -dx;
+      dy = -dy;
+      dz = -dz;
+    }
     const float3 off = self ? make_float3(0.f, 0.f, 0.f) : make_float3(e * dx, e * dy, e * dz);   // exact
     const float4 cA = T.cen[A], cB = T.cen[B], cl = K.cl;
     const float3 dl = make_float3(cl.x - cA.x, cl.y - cA.y, cl.z - cA.z);   // the leaf centre in A's frame, exact
@@ -1295,7 +1299,7 @@ __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T,
     const float slack = e * 1.52587890625e-05f + K.es + 1e-6f * fmaxf(HmB, T.hmax[A] * invL);   // 2^-16 e
     const unsigned int t0 = T.tile0[B], nt = T.ntile[B];
     unsigned int sb = SORT_NONE;
-    if (!self) {
+    if (!self && !second) {      // (the sorted lists run away from a pair's first cell)
       const unsigned int sbB = T.sortbase[B];
       if (sbB != SORT_NONE) sb = sbB + (unsigned int)__popc(T.axes[B] & ((1u << ax) - 1u)) * nt;
     }
@@ -1303,15 +1307,16 @@ __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T,
     const float offBp = e * (n2 == 1 ? 1.0f : (n2 == 2 ? 1.41421356237f : 1.73205080757f));
     // sort keys are the projections at the build; a cluster's projection has
     // since moved by at most the drift
-    const float win = offBp - K.drift - box_rhi(box_shift(bil, dl), axis_unit_f(ax));
+    const float win = offBp - K.drift - box_rhi(box_shift(bil, dl), axis_unit_f(GATHER ? ax & 15 : ax));
     K.gsh[lane] = make_float4((off.x - cB.x) - dl.x, (off.y - cB.y) - dl.y, (off.z - cB.z) - dl.z, slack);
-    K.gwin[lane] = make_float4(win, HmB, __uint_as_float(sb), __uint_as_float(self ? t0 + nt - (K.ti + 1u) : nt));
-    K.gtb[lane] = self ? K.ti + 1u : t0;
+    K.gwin[lane] = make_float4(win, GATHER ? 0.0f : HmB, __uint_as_float(sb),
+                               __uint_as_float(self && !GATHER ? t0 + nt - (K.ti + 1u) : nt));
+    K.gtb[lane] = self && !GATHER ? K.ti + 1u : t0;
     // the partner cell, widened by the drift of particles kept in it since the build
     const float h = 0.5f * e + K.drift;
     const float3 cb = make_float3(off.x - dl.x, off.y - dl.y, off.z - dl.z);
     live = self || box_near(bil, Box3{make_float3(cb.x - h, cb.y - h, cb.z - h), make_float3(cb.x + h, cb.y + h, cb.z + h)},
-                            fmaxf(clo.w, HmB) + slack);
+                            (GATHER ? clo.w : fmaxf(clo.w, HmB)) + slack);
     if (PART && live && !iact) {
       // only the partner cell's iterating particles need this cluster
       live = T.active[B] != 0;
@@ -1399,7 +1404,7 @@ __device__ __forceinline__ void unit_single(UnitShared& K, bool self, int item, 
 // uniform box has no such candidate and pays nothing.
 constexpr float FINE_H = 0.7f;
 
-template <bool PART>
+template <bool PART, bool GATHER>
 __device__ __forceinline__ unsigned int scan_clusters(UnitShared& K, float4* jlo, float4* jhi, const Tiles& TL,
                                                       const float* __restrict__ sort_r,
                                                       const unsigned int* __restrict__ sort_i, int it,
@@ -1419,7 +1424,7 @@ __device__ __forceinline__ unsigned int scan_clusters(UnitShared& K, float4* jlo
   if (e < nt) {
     const unsigned int t = sorted ? sort_i[sb + e] : K.gtb[it] + e;
     const float4 lo = TL.lo[t];
-    const float Hj = lo.w * invL;
+    const float Hj = GATHER ? 0.0f : lo.w * invL;      // (gathered: the own reach only)
     if (!sorted || sort_r[sb + e] + win.x <= fmaxf(Hi, Hj) + slack) {
       const float4 lc = TL.cen[t], hi = TL.hi[t];
       const float3 o = make_float3(lc.x + sh.x, lc.y + sh.y, lc.z + sh.z);
@@ -1433,7 +1438,7 @@ __device__ __forceinline__ unsigned int scan_clusters(UnitShared& K, float4* jlo
       if (pass) {
         K.co[lane] = make_float4(o.x, o.y, o.z, __uint_as_float(TL.start[t]));
         K.cn[lane] = (unsigned char)TL.n[t];
-        fine = Hj < FINE_H * Hi;
+        fine = (GATHER ? lo.w * invL : Hj) < FINE_H * Hi;
         if (fine) {
           jlo[lane] = make_float4(bj.lo.x, bj.lo.y, bj.lo.z, Hj);
           jhi[lane] = make_float4(bj.hi.x, bj.hi.y, bj.hi.z, 0.0f);
@@ -1464,13 +1469,13 @@ struct Walk {
 };
 
 // The next candidates (W.mask, non-zero) of the unit; false at its end.
-template <bool PART>
+template <bool PART, bool GATHER = false>
 __device__ __forceinline__ bool unit_next(UnitShared& K, Walk& W, float4* jlo, float4* jhi, const Lists& Lq,
                                           const Tree& T, const Tiles& TL, const float* __restrict__ sort_r,
                                           const unsigned int* __restrict__ sort_i, bool any, bool all, float3 ip, float iH) {
   while (!W.mask) {
     if (W.e0 < W.nt) {
-      W.mask = scan_clusters<PART>(K, jlo, jhi, TL, sort_r, sort_i, W.it, W.e0, W.nt, any, all, ip, iH);
+      W.mask = scan_clusters<PART, GATHER>(K, jlo, jhi, TL, sort_r, sort_i, W.it, W.e0, W.nt, any, all, ip, iH);
     } else if (W.live) {
       W.it = __ffs(W.live) - 1;
       W.live &= W.live - 1;
@@ -1478,7 +1483,7 @@ __device__ __forceinline__ bool unit_next(UnitShared& K, Walk& W, float4* jlo, f
       // with parts, every parts-th run of 32 clusters, from one that depends on the interaction
       W.e0 = 32u * unit_first(K, W.it);
     } else if (K.cell >= 0) {
-      W.live = unit_group<PART>(K, T, Lq.csr, any);
+      W.live = unit_group<PART, GATHER>(K, T, Lq.csr, any);
     } else {
       return false;
     }
@@ -1771,7 +1776,6 @@ __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_B
                                                          unsigned long long* pc,
                                                          unsigned int* __restrict__ task_ctr, int partial_host,
                                                          const int* __restrict__ it_dev, const int* __restrict__ gflag,
-                                                         const unsigned int* __restrict__ g_n, unsigned int cap_g,
                                                          unsigned int ntcap, const unsigned int* __restrict__ ntile_dev,
                                                          const uint2* __restrict__ units,
                                                          const unsigned int* __restrict__ n_units, unsigned int cap_units,
@@ -1780,7 +1784,7 @@ __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_B
   const int partial = it_dev ? (*it_dev > 1 ? 1 : 0) : partial_host;
   if ((partial != 0) != PART) return;
   if (it_dev && it_dev[2] != 0) return;                        // the iteration has stopped
-  if (PART && gflag && gather_on(gflag, g_n, cap_g)) return;   // the pass gathers
+  if (PART && gflag && gflag[0] != 0) return;                  // the pass gathers
   __shared__ DensShared SH[SPH_WARPS_PER_CTA];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   DensShared& S = SH[wl];
@@ -1958,8 +1962,7 @@ __global__ void k_unit_list(unsigned int ntcap, const unsigned int* __restrict__
 template <bool DENS>
 __global__ void k_live_tasks(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box, long long npt,
                              long long nst, int partial_host, const int* __restrict__ it_dev, int cap_p, int cap_s,
-                             const int* __restrict__ gflag, const unsigned int* __restrict__ g_n,
-                             unsigned int cap_g) {
+                             const int* __restrict__ gflag) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   if (it_dev && it_dev[2] != 0) return;    // the iteration has stopped: no tasks
@@ -1970,7 +1973,7 @@ __global__ void k_live_tasks(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restri
   }
   // later iterations keep only what still iterates (with a device counter: from iteration 2 on)
   const int partial = it_dev ? (*it_dev > 1 ? 1 : 0) : partial_host;
-  if (DENS && partial && gflag && gather_on(gflag, g_n, cap_g)) return;   // the pass gathers
+  if (DENS && partial && gflag && gflag[0] != 0) return;       // the pass gathers
   const long long ntask = npt + nst;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < ntask; b0 += stride) {
@@ -2054,15 +2057,22 @@ __global__ void k_pack_leaf(long long ntcap, const unsigned int* __restrict__ nt
   }
 }
 
-// The packed clusters (after the scan of k_pack_leaf's counts: pk0[t], the first
-// packed cluster of the leaf whose first cluster is t): the sorted indices of the
-// iterating particles by rank (idx), and per packed cluster its first rank and
-// its leaf's first cluster (info) and its size (pn).  One warp per cluster.
-__device__ __forceinline__ void pack_fill(long long nt, const Tree& T, const Tiles& TL,
-                                          const unsigned char* __restrict__ act,
-                                          const unsigned int* __restrict__ rank, const unsigned int* __restrict__ pk0,
-                                          unsigned int* __restrict__ idx, uint2* __restrict__ info,
-                                          unsigned char* __restrict__ pn) {
+// The packed clusters of a later pass, when it gathers (after the scan of k_pack_leaf's
+// counts: pk0[t], the first packed cluster of the leaf whose first cluster is t): the
+// sorted indices of the iterating particles by rank (idx), and per packed cluster its
+// first rank and its leaf's first cluster (info) and its size (pn).  The pass gathers
+// when it is a later one and at most an eighth of the particles iterate (gflag[0]).  One
+// warp per cluster.
+__global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ ntile_dev, const int* __restrict__ it_dev,
+                            long long N, Tree T, Tiles TL, const unsigned char* __restrict__ act,
+                            const unsigned int* __restrict__ rank, const unsigned int* __restrict__ pk0,
+                            const unsigned int* __restrict__ pk_tot, unsigned int* __restrict__ idx,
+                            uint2* __restrict__ info, unsigned char* __restrict__ pn, int* __restrict__ gflag) {
+  pdl_wait();
+  const bool on = later_pass(it_dev) && 8ull * pk_tot[0] <= (unsigned long long)N;
+  if (blockIdx.x == 0 && threadIdx.x == 0) gflag[0] = on ? 1 : 0;
+  if (!on) return;
+  const long long nt = ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap;
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -2081,69 +2091,6 @@ __device__ __forceinline__ void pack_fill(long long nt, const Tree& T, const Til
       info[pid] = make_uint2(r0 + k, t0);
       pn[pid] = (unsigned char)min(32u, na - k);
     }
-  }
-}
-
-// The packed clusters and the gathered tasks of a later pass, when it gathers:
-// (interaction, packed cluster), bit 31 of the interaction marking a self interaction
-// and bit 30 the direction of a pair (0: the packed clusters of A against B, 1: of B
-// against A).  The pass gathers when it is a later one, the caller allows it and at
-// most an eighth of the particles iterate (gflag[0]); the symmetric path runs instead
-// when the tasks exceed the buffer.  One thread per interaction, self interactions
-// first; warp-aggregated appends.
-__global__ void k_pack_tasks(Lists Lq, Tree T, Tiles TL, long long ntcap, const unsigned int* __restrict__ ntile_dev,
-                             const unsigned char* __restrict__ act, const unsigned int* __restrict__ rank,
-                             unsigned int* __restrict__ idx, uint2* __restrict__ info, unsigned char* __restrict__ pn,
-                             long long npair, long long nself, int cap_pair, int cap_self,
-                             const int* __restrict__ it_dev, long long N,
-                             const unsigned int* __restrict__ pk0, const unsigned int* __restrict__ pk_tot,
-                             uint2* __restrict__ tasks, unsigned int* __restrict__ g_n, unsigned int cap_g,
-                             int* __restrict__ gflag) {
-  pdl_wait();
-  const bool on = later_pass(it_dev) && 8ull * pk_tot[0] <= (unsigned long long)N;
-  if (blockIdx.x == 0 && threadIdx.x == 0) gflag[0] = on ? 1 : 0;
-  if (!on) return;
-  pack_fill(ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap, T, TL, act, rank, pk0, idx, info, pn);
-  if (npair < 0) {
-    npair = min(Lq.counts[1], cap_pair);
-    nself = min(Lq.counts[0], cap_self);
-  }
-  const int lane = threadIdx.x & 31;
-  const long long nitem = nself + npair;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < nitem; b0 += stride) {
-    const long long i = b0 + threadIdx.x;
-    unsigned int code = 0, a0 = 0, a1 = 0, c0 = 0, c1 = 0;
-    if (i < nself) {
-      const int A = Lq.self_a[i];
-      a0 = pk0[T.tile0[A]];
-      a1 = pk0[T.tile0[A] + T.ntile[A]];
-      code = (unsigned int)i | 0x80000000u;
-    } else if (i < nitem) {
-      const int j = (int)(i - nself);
-      const int A = Lq.pair_a[j], B = Lq.pair_b[j];
-      a0 = pk0[T.tile0[A]];
-      a1 = pk0[T.tile0[A] + T.ntile[A]];
-      c0 = pk0[T.tile0[B]];
-      c1 = pk0[T.tile0[B] + T.ntile[B]];
-      code = (unsigned int)j;
-    }
-    const unsigned int mine = (a1 - a0) + (c1 - c0);
-    unsigned int incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const unsigned int wtot = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned int base = 0;
-    if (lane == 31 && wtot) base = atomicAdd(g_n, wtot);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    unsigned int at = base + incl - mine;
-    for (unsigned int p = a0; p < a1; ++p, ++at)
-      if (at < cap_g) tasks[at] = make_uint2(code, p);
-    for (unsigned int p = c0; p < c1; ++p, ++at)
-      if (at < cap_g) tasks[at] = make_uint2(code | 0x40000000u, p);
   }
 }
 
@@ -2181,119 +2128,128 @@ __device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsi
   __syncwarp();
 }
 
-// One gathered task: packed cluster pid (of cell O) against the clusters of cell X.
-// The frame is the packed cluster's leaf centre; X's particles move into it by
-// the exact dyadic offset of the pair kernel's leaf frame (X's centre image minus
-// O's centre, taken in the same order), so each position is rounded once, at
-// most at the cells' scale, and the guard band holds as there.
+// One unit of a gathered pass: packed cluster pid, a part of its interactions: those of
+// every cell on its leaf's chain, in both directions of the pairs, walked as in
+// density_unit (a task per interaction set up, boxed and flushed a packed cluster 27
+// times, in batches mostly partly filled).  The frame is the leaf's centre, as there.
 template <bool KAHAN>
-__device__ __forceinline__ void gather_task(uint2 tk, const Lists& Lq, const Tree& T, const Tiles& TL,
-                                            const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
-                                            const float4* __restrict__ cen4, const unsigned int* __restrict__ perm,
-                                            const double* __restrict__ x, float4* dacc, unsigned int* dcnt, float4* dcomp,
+__device__ __forceinline__ void gather_unit(unsigned int pid, unsigned int part, unsigned int parts, const Lists& Lq,
+                                            const Tree& T, const Tiles& TL, const BoxDesc* __restrict__ box,
+                                            const float4* __restrict__ pos4, const float4* __restrict__ cen4,
+                                            const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
+                                            const unsigned int* __restrict__ perm, const double* __restrict__ x,
+                                            float4* dacc, unsigned int* dcnt, float4* dcomp,
                                             const uint2* __restrict__ pk_info, const unsigned char* __restrict__ pk_n,
                                             const unsigned int* __restrict__ pk_idx, DensShared& S) {
   const int lane = threadIdx.x & 31;
-  const bool self = (tk.x >> 31) != 0u, dir1 = ((tk.x >> 30) & 1u) != 0u;
-  const int item = (int)(tk.x & 0x3fffffffu);
-  int O, X, ax = 0;
-  if (self) {
-    O = X = Lq.self_a[item];
-  } else {
-    const int A = Lq.pair_a[item], B = Lq.pair_b[item];
-    ax = Lq.pair_axis[item];
-    O = dir1 ? B : A;
-    X = dir1 ? A : B;
-  }
-  // pair items join cells of one level: A's geometry serves both directions
-  const ItemGeom g = item_geom(T, box, self ? O : Lq.pair_a[item], ax);
-  const float3 offX = self ? make_float3(0.f, 0.f, 0.f)
-                           : (dir1 ? make_float3(-g.offB.x, -g.offB.y, -g.offB.z) : g.offB);
-  const uint2 info = pk_info[tk.y];
-  const unsigned int n = pk_n[tk.y];
-  const float4 cO = T.cen[O], cX = T.cen[X], cl = TL.cen[info.y];
-  const float3 shX = make_float3(offX.x - cX.x, offX.y - cX.y, offX.z - cX.z);
-  const float3 d = make_float3(cl.x - cO.x, cl.y - cO.y, cl.z - cO.z);
-  const float3 sh_part = make_float3(shX.x - d.x, shX.y - d.y, shX.z - d.z);
+  UnitShared& K = S.tk;
+  const uint2 info = pk_info[pid];
+  const unsigned int n = pk_n[pid];
+  unit_begin(K, info.y, T, TL, box, part, parts);
   const bool vi = (unsigned int)lane < n;
-  const DensI I = load_dens(vi, vi ? pk_idx[info.x + lane] : 0u, pos4, cen4, nullptr, g.invL);
-  __syncwarp();
+  const DensI I = load_dens(vi, vi ? pk_idx[info.x + lane] : 0u, pos4, cen4, nullptr, K.bhi.w);
   S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
   S.ig[lane] = I.g;
-  if (lane == 0) {
-    S.tk.box = T.box[O];
-    S.tk.eb = g.eb;
-  }
-  __syncwarp();
   // the packed particles' box and largest H: the own side reaches no further
   Box3 bo;
   bo.lo = make_float3(warp_min(vi ? I.p.x : 1e30f), warp_min(vi ? I.p.y : 1e30f), warp_min(vi ? I.p.z : 1e30f));
   bo.hi = make_float3(warp_max(vi ? I.p.x : -1e30f), warp_max(vi ? I.p.y : -1e30f), warp_max(vi ? I.p.z : -1e30f));
   const float Ho = warp_max(vi ? I.H : 0.0f);
-  const float slack = g.e * 1.52587890625e-05f + g.es + 1e-6f * fmaxf(T.hmax[O], T.hmax[X]) * g.invL;
-  const float reach = Ho + slack;
-  if (!self) {
-    // X's cell, widened by the drift since the build, in this frame
-    const float h = 0.5f * g.e + g.drift;
-    Box3 cx;
-    cx.lo = make_float3(cX.x + sh_part.x - h, cX.y + sh_part.y - h, cX.z + sh_part.z - h);
-    cx.hi = make_float3(cX.x + sh_part.x + h, cX.y + sh_part.y + h, cX.z + sh_part.z + h);
-    if (!box_near(bo, cx, reach)) return;
+  const float invL = K.bhi.w;
+  __syncwarp();
+  if (lane == 0) {
+    K.blo = K.clo = make_float4(bo.lo.x, bo.lo.y, bo.lo.z, Ho);
+    K.bhi = K.chi = make_float4(bo.hi.x, bo.hi.y, bo.hi.z, invL);
   }
+  __syncwarp();
   DensAcc<KAHAN> acc;
-  unsigned int cnt = 0, q = 0;
-  const unsigned int t0 = T.tile0[X], nt = T.ntile[X];
-  for (unsigned int b0 = 0; b0 < nt; b0 += 32) {
-    bool ok = false;
-    if (b0 + lane < nt) ok = box_near(bo, tile_box3(TL, T, t0 + b0 + lane, sh_part), reach);
-    unsigned int mask = __ballot_sync(0xffffffffu, ok);
-    while (mask) {
-      const int k = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const unsigned int tj = t0 + b0 + (unsigned int)k, gj = TL.start[tj] + lane;
-      const bool vj = (unsigned int)lane < TL.n[tj];
-      const float4 c = TL.cen[tj], r = vj ? pos4[gj] : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float3 pj = make_float3(r.x + (c.x + sh_part.x), r.y + (c.y + sh_part.y), r.z + (c.z + sh_part.z));
-      const bool pass = vj && near_box(pj, bo, reach);
-      const unsigned int bal = __ballot_sync(0xffffffffu, pass);
-      const unsigned int np = __popc(bal);
-      if (q + np > 32u) {
-        gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
-        q = 0;
-      }
-      if (pass) dens_put(S, (int)(q + __popc(bal & ((1u << lane) - 1u))), pj, r.w, gj, true);
-      q += np;
+  unsigned int cnt = 0, q = 0, done = 0xffffffffu;
+  S.is[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  Walk Wk;
+  bool own = false;      // the batch holds particles of the own leaf
+  int k = -1;
+  float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (;;) {
+    if (k < 0 && unit_next<false, true>(K, Wk, S.jlo, S.jhi, Lq, T, TL, sort_r, sort_i, true, true, I.p,
+                                        vi ? I.H : 0.0f)) {
+      k = __ffs(Wk.mask) - 1;
+      Wk.mask &= Wk.mask - 1;
+      if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
     }
+    const bool last = k < 0;
+    unsigned int bal = 0, gj = 0;
+    float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool pass = false;
+    if (!last) {
+      const float4 o = K.co[k];
+      const bool vj = (unsigned int)lane < K.cn[k];
+      gj = __float_as_uint(o.w) + lane;
+      pj = make_float4(nr.x + o.x, nr.y + o.y, nr.z + o.z, nr.w);
+      k = -1;
+      if (Wk.mask) {
+        k = __ffs(Wk.mask) - 1;
+        Wk.mask &= Wk.mask - 1;
+        if ((unsigned int)lane < K.cn[k]) nr = pos4[__float_as_uint(K.co[k].w) + lane];
+      }
+      pass = vj && near_box(make_float3(pj.x, pj.y, pj.z), bo, Ho + K.gsh[Wk.it].w);
+      bal = __ballot_sync(0xffffffffu, pass);
+    }
+    const unsigned int np = __popc(bal), rank = __popc(bal & ((1u << lane) - 1u));
+    if (last || q + np > 32u) {
+      const unsigned int room = last ? 0u : 32u - q;
+      if (pass && rank < room) dens_put(S, (int)(q + rank), make_float3(pj.x, pj.y, pj.z), pj.w, gj, true);
+      pass = pass && rank >= room;
+      q += room;
+      own = own || (room && Wk.it == K.selfit);
+      if (q) gather_batch<KAHAN>(I, S, q, own, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
+      q = 0u - room;
+      own = false;
+      const unsigned int now = K.gidx + (unsigned int)Wk.it;
+      if (!KAHAN && now != done) {      // (as in density_unit)
+        const float4 t = S.is[lane];
+        S.is[lane] = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
+        acc = DensAcc<KAHAN>();
+        done = now;
+      }
+    }
+    if (last) break;
+    if (pass) dens_put(S, (int)(q + rank), make_float3(pj.x, pj.y, pj.z), pj.w, gj, true);
+    own = own || Wk.it == K.selfit;
+    q += np;
   }
-  if (q) gather_batch<KAHAN>(I, S, q, self, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
+  if (!KAHAN) {
+    const float4 t = S.is[lane];
+    acc.s = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
+  }
   flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
 }
 
 #ifndef GATHER_BLOCKS
 #define GATHER_BLOCKS 8
 #endif
-// The gathered density pass (a later pass of the h iteration that gathers): the
-// tasks of k_pack_tasks, one per fetch; g_n[1] counts the passes that gathered.
-// Returns at once when the pass runs the symmetric tasks instead.
+// The gathered density pass (a later pass of the h iteration that gathers): units of the
+// packed clusters; g_n[1] counts the passes that gathered.  Returns at once when the pass
+// takes the clusters' units instead.
 template <bool KAHAN>
 __global__ void __launch_bounds__(SPH_THREADS, GATHER_BLOCKS) k_density_gather(
     Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box, const float4* __restrict__ pos4,
-    const float4* __restrict__ cen4, const unsigned int* __restrict__ perm, const double* __restrict__ x,
-    float4* dacc, unsigned int* dcnt, float4* dcomp, const uint2* __restrict__ tasks, unsigned int* __restrict__ g_n,
-    unsigned int cap_g, const int* __restrict__ gflag, const uint2* __restrict__ pk_info,
+    const float4* __restrict__ cen4, const float* __restrict__ sort_r, const unsigned int* __restrict__ sort_i,
+    const unsigned int* __restrict__ perm, const double* __restrict__ x, float4* dacc, unsigned int* dcnt,
+    float4* dcomp, unsigned int* __restrict__ g_n, const int* __restrict__ gflag, const uint2* __restrict__ pk_info,
     const unsigned char* __restrict__ pk_n, const unsigned int* __restrict__ pk_idx,
-    unsigned int* __restrict__ task_ctr) {
+    const unsigned int* __restrict__ pk_tot, unsigned int* __restrict__ task_ctr) {
   pdl_wait();
-  if (!gather_on(gflag, g_n, cap_g)) return;
+  if (gflag[0] == 0) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) g_n[1] += 1u;
   __shared__ DensShared SH[SPH_WARPS_PER_CTA];
   const int lane = threadIdx.x & 31;
   DensShared& S = SH[threadIdx.x >> 5];
-  const unsigned int ntask = *g_n;
+  const unsigned int npk = pk_tot[1], parts = unit_parts(npk), nunit = npk * parts;
   unsigned int t = 0;
   if (lane == 0) t = atomicAdd(task_ctr, 1u);
-  for (t = __shfl_sync(0xffffffffu, t, 0); t < ntask; t = __shfl_sync(0xffffffffu, t, 0)) {
-    gather_task<KAHAN>(tasks[t], Lq, T, TL, box, pos4, cen4, perm, x, dacc, dcnt, dcomp, pk_info, pk_n, pk_idx, S);
+  for (t = __shfl_sync(0xffffffffu, t, 0); t < nunit; t = __shfl_sync(0xffffffffu, t, 0)) {
+    gather_unit<KAHAN>(t / parts, t % parts, parts, Lq, T, TL, box, pos4, cen4, sort_r, sort_i, perm, x, dacc, dcnt,
+                       dcomp, pk_info, pk_n, pk_idx, S);
     if (lane == 0) t = atomicAdd(task_ctr, 1u);
   }
 }
@@ -2409,19 +2365,16 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
 // every cell the box of those particles in the cell's
 // frame.  One warp per cluster; the cluster's box of active particles is added
 // to every cell on its chain with ordered-key atomics.
-// Counts the particles still iterating per cluster (cnt[t], and cnt[ntile] = 0) and
-// clears the gathered task count for the packing that follows.
+// Counts the particles still iterating per cluster (cnt[t], and cnt[ntile] = 0) for the
+// packing that follows.
 __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ ntile_dev,
                               const unsigned char* __restrict__ act, const float4* __restrict__ pos4, Tree T, Tiles TL,
-                              unsigned int* __restrict__ cnt, unsigned int* __restrict__ g_n) {
+                              unsigned int* __restrict__ cnt) {
   pdl_wait();
   if (ntile_dev) ntile = min(ntile, (long long)*ntile_dev);   // a captured step: this build's clusters
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    cnt[ntile] = 0;
-    *g_n = 0;
-  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) cnt[ntile] = 0;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long t = warp; t < ntile; t += nwarps) {
     const unsigned int n = TL.n[t], s0 = TL.start[t];
@@ -2884,10 +2837,10 @@ void launch_live_tasks(Engine& E, bool dens, const int* it_dev) {
   const int grid = (int)std::min<long long>((n + 255) / 256, (long long)E.nsm * 16);
   if (dens)
     launch_pdl(k_live_tasks<true>, grid, 256, E.st, E.Lq, E.T, E.TL, E.box.p, npt, nst, E.partial_pass, it_dev,
-               cap_p, cap_s, it_dev ? E.gflag.p : nullptr, E.g_n.p, (unsigned int)E.g_live.n);
+               cap_p, cap_s, it_dev ? E.gflag.p : nullptr);
   else
     launch_pdl(k_live_tasks<false>, grid, 256, E.st, E.Lq, E.T, E.TL, E.box.p, npt, nst, 0, nullptr, cap_p, cap_s,
-               nullptr, nullptr, 0u);
+               nullptr);
   count_launch();
 }
 
@@ -2915,15 +2868,15 @@ void launch_density(Engine& E, const int* it_dev, int only) {
                                 : (rec ? k_density<false, false, false, true> : k_density<false, false, false, false>));
     launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st,
         E.Lq, E.T, E.TL, E.box.p, E.pos4.p, E.cen4.p, E.sort_r.p, E.sort_i.p, E.act.p, E.perm.p, E.x.p, E.dacc.p,
-        E.dcnt.p, E.dcomp.p, E.pc.p, E.task_ctr.p + part, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr, E.g_n.p,
-        (unsigned int)E.g_live.n, (unsigned int)(E.gcap ? E.N : E.n_tiles),
+        E.dcnt.p, E.dcomp.p, E.pc.p, E.task_ctr.p + part, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr,
+        (unsigned int)(E.gcap ? E.N : E.n_tiles),
         E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr,
         E.unit_list ? E.units.p : nullptr, E.n_units.p, (unsigned int)E.units.n, E.rec_for_force());
     count_launch();
   }
 }
 
-// The packing and the task list of a gathered later pass (a pass of the h
+// The packing of a gathered later pass (a pass of the h
 // iteration given by it_dev; the kernels decide on the device whether it gathers).
 void launch_gather_prep(Engine& E, const int* it_dev) {
   if (E.prm.h_gather == 0 || E.count_pairs) return;      // (gflag stays 0: no pass gathers)
@@ -2938,11 +2891,8 @@ void launch_gather_prep(Engine& E, const int* it_dev) {
     count_launch();
     exclusive_scan(E.pk_v.p, E.pk_v.p, nt + 1, E.pk_sums.p, E.pk_tot.p + 1, E.st, ntd, it_dev);
   }
-  const long long npair = E.gcap ? -1 : E.n_pairs, nself = E.gcap ? -1 : E.n_selfs;
-  const long long nitem = E.gcap ? (long long)E.cap_pair + E.cap_self : (long long)E.n_pairs + E.n_selfs;
-  launch_pdl(k_pack_tasks, E.grid(std::max<long long>(nitem, 32 * nt)), 256, E.st, E.Lq, E.T, E.TL, nt, ntd, E.act.p,
-             E.pk_cnt.p, E.pk_idx.p, E.pk_info.p, E.pk_n.p, npair, nself, E.cap_pair, E.cap_self, it_dev,
-             (long long)E.N, E.pk_v.p, E.pk_tot.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n, E.gflag.p);
+  launch_pdl(k_pack_fill, E.grid(32 * nt), 256, E.st, nt, ntd, it_dev, (long long)E.N, E.T, E.TL, E.act.p, E.pk_cnt.p,
+             E.pk_v.p, E.pk_tot.p, E.pk_idx.p, E.pk_info.p, E.pk_n.p, E.gflag.p);
   count_launch();
 }
 
@@ -2951,8 +2901,8 @@ void launch_density_gather(Engine& E) {
   const bool kahan = E.kahan();
   const auto k = kahan ? k_density_gather<true> : k_density_gather<false>;
   launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st, E.Lq, E.T, E.TL, E.box.p, E.pos4.p,
-             E.cen4.p, E.perm.p, E.x.p, E.dacc.p, E.dcnt.p, E.dcomp.p, E.g_live.p, E.g_n.p, (unsigned int)E.g_live.n,
-             E.gflag.p, E.pk_info.p, E.pk_n.p, E.pk_idx.p, E.task_ctr.p + 3);
+             E.cen4.p, E.sort_r.p, E.sort_i.p, E.perm.p, E.x.p, E.dacc.p, E.dcnt.p, E.dcomp.p, E.g_n.p, E.gflag.p,
+             E.pk_info.p, E.pk_n.p, E.pk_idx.p, E.pk_tot.p, E.task_ctr.p + 3);
   count_launch();
 }
 
@@ -3010,7 +2960,7 @@ void launch_mark_active_cells(Engine& E) {
   const long long nt = E.gcap ? E.N : E.n_tiles;
   launch_pdl(k_mark_active, E.grid(32 * nt), 256, E.st, nt,
              E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr, E.act.p, E.pos4.p, E.T,
-             E.TL, E.pk_cnt.p, E.g_n.p);
+             E.TL, E.pk_cnt.p);
   count_launch();
 }
 

@@ -197,7 +197,7 @@ class Engine {
 
   // cell tree
   int cap_nodes = 0;
-  DBuf<unsigned int> t_start, t_count, t_nsmall, t_axes, t_sortbase, t_pmask, t_pstart;
+  DBuf<unsigned int> t_start, t_count, t_nsmall, t_axes, t_sortbase, t_pmask, t_rmask, t_pstart;
   DBuf<unsigned long long> t_key;
   DBuf<int> t_level, t_box, t_child, t_nchild, t_parent, t_split, t_n;
   DBuf<float> t_hmax;
@@ -222,7 +222,7 @@ class Engine {
   // start, size), scan scratch and totals, the gathered tasks, their count and the
   // pass's choice
   DBuf<unsigned int> pk_cnt, pk_v, pk_idx, pk_sums, pk_tot, g_n;
-  DBuf<uint2> pk_info, g_live;
+  DBuf<uint2> pk_info;
   DBuf<unsigned char> pk_n;
   DBuf<int> gflag;
   long long n_ptasks = 0, n_stasks = 0;

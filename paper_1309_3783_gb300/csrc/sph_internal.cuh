@@ -269,6 +269,7 @@ struct Tree {
   unsigned int* sortbase;   // offset of the first sorted list of this cell
   unsigned int* pmask;      // bit a: a pair-interaction (A, B, a) with A this cell (one B per axis); the first of
                             //   them in Lists::csr, by axis
+  unsigned int* rmask;      // likewise with A its second cell; they follow there
   unsigned int* pstart;
   unsigned char* active;    // 1 when a particle inside still iterates h
   unsigned char* changed;   // 1 when a particle inside took a new h after the first density pass
@@ -324,7 +325,8 @@ struct Lists {
   int* q_a[2];
   int* q_b[2];
   int* q_axis[2];
-  uint2* csr;               // the pairs by their first cell: (B, axis)
+  uint2* csr;               // the pairs by cell: (partner, axis), where it is the first; then (partner,
+                            //   axis | 16), where it is the second
   unsigned int* p_toff;     // per pair: first task (i-tile) number, exclusive prefix
   unsigned int* s_toff;     // per self: first task number
   unsigned int* p_task;     // per pair task: its pair
