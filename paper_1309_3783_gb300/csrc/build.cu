@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(1024) k_pack_scan(long long ntcap, const unsig
   const long long nt = ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap;
   const unsigned int na = scan_in_block(nt + 1, cnt, cnt, tmp);
   if (threadIdx.x == 0) pk_tot[0] = na;
-  if (8ull * na > (unsigned long long)N) return;
+  if (GATHER_SHARE * na > (unsigned long long)N) return;
   __syncthreads();
   unsigned int carry = 0;
   for (long long b0 = 0; b0 <= nt; b0 += 4096) {

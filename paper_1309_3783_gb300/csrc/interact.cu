@@ -2061,7 +2061,7 @@ __global__ void k_pack_leaf(long long ntcap, const unsigned int* __restrict__ nt
 // counts: pk0[t], the first packed cluster of the leaf whose first cluster is t): the
 // sorted indices of the iterating particles by rank (idx), and per packed cluster its
 // first rank and its leaf's first cluster (info) and its size (pn).  The pass gathers
-// when it is a later one and at most an eighth of the particles iterate (gflag[0]).  One
+// when it is a later one and at most a third of the particles iterate (gflag[0]).  One
 // warp per cluster.
 __global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ ntile_dev, const int* __restrict__ it_dev,
                             long long N, Tree T, Tiles TL, const unsigned char* __restrict__ act,
@@ -2069,7 +2069,7 @@ __global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ nt
                             const unsigned int* __restrict__ pk_tot, unsigned int* __restrict__ idx,
                             uint2* __restrict__ info, unsigned char* __restrict__ pn, int* __restrict__ gflag) {
   pdl_wait();
-  const bool on = later_pass(it_dev) && 8ull * pk_tot[0] <= (unsigned long long)N;
+  const bool on = later_pass(it_dev) && GATHER_SHARE * pk_tot[0] <= (unsigned long long)N;
   if (blockIdx.x == 0 && threadIdx.x == 0) gflag[0] = on ? 1 : 0;
   if (!on) return;
   const long long nt = ntile_dev ? min(ntcap, (long long)*ntile_dev) : ntcap;

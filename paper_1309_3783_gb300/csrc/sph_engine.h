@@ -66,6 +66,11 @@ extern const char* const kPhaseNames[PH_COUNT];
 void exclusive_scan(const unsigned int* in, unsigned int* out, long long n, unsigned int* tile_sums,
                     unsigned int* total, cudaStream_t st, const unsigned int* n_dev = nullptr,
                     const int* gate = nullptr);
+// A later pass of the h iteration gathers when at most a third of the particles iterate
+// (packed clusters then halve the own side at least, and its partners' side is not
+// needed; passes of 977k Sod particles with a quarter iterating 0.25 -> 0.22 ms against an
+// eighth as the limit, 4.2M clustered h iteration 34.2 -> 33.9 ms; a half gains no more).
+constexpr unsigned long long GATHER_SHARE = 3;
 // Up to this many particles one block does both scans of a gathered pass's packing (a
 // microsecond per 1000 clusters, 38 us for the 36k of a million particles, against the
 // 25 us of seven launches; clusters are a sixteenth to a thirtieth of the particles in
@@ -219,8 +224,8 @@ class Engine {
   // gathered later passes of the h iteration: per cluster the particles still
   // iterating (scanned to ranks), per leaf start its packed clusters (scanned to
   // their first index), the packed clusters (indices by rank, first rank and leaf
-  // start, size), scan scratch and totals, the gathered tasks, their count and the
-  // pass's choice
+  // start, size), scan scratch and totals, the number of gathered passes (g_n[1]) and
+  // the pass's choice
   DBuf<unsigned int> pk_cnt, pk_v, pk_idx, pk_sums, pk_tot, g_n;
   DBuf<uint2> pk_info;
   DBuf<unsigned char> pk_n;
