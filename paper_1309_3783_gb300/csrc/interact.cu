@@ -21,15 +21,9 @@ constexpr float BAND_REL = 7.62939453125e-06f;  // 2^-17: guard band of the FP32
 struct ItemGeom {
   float e;          // cell edge (units of L)
   float3 offB;      // centre of B minus centre of A (units of L), exact: e * db
-  float offBp;      // projection of offB on the axis: e |db|
   float invL;
-  float eb;         // length scale of the position rounding: the cell edge, or 1 (L) for
-                    //   plain FP32 positions; the guard band is 2^-17 H (eb + H)
   float es;         // absolute rounding of plain FP32 positions added to the culling slack
-  float L32;        // L in FP32
   float drift;      // largest displacement since the decomposition was built (units of L)
-  double L, halfL;
-  int periodic;
 };
 
 __device__ __forceinline__ ItemGeom item_geom(const Tree& T, const BoxDesc* box, int A, int ax) {
@@ -40,27 +34,11 @@ __device__ __forceinline__ ItemGeom item_geom(const Tree& T, const BoxDesc* box,
   int dx, dy, dz;
   axis_vec(ax, dx, dy, dz);
   g.offB = make_float3(g.e * dx, g.e * dy, g.e * dz);
-  const int n2 = dx * dx + dy * dy + dz * dz;
-  g.offBp = g.e * (n2 == 1 ? 1.0f : (n2 == 2 ? 1.41421356237f : 1.73205080757f));
   g.invL = (float)bd.invL;
-  g.eb = bd.global32 ? 1.0f : g.e;
   g.es = bd.global32 ? 9.5367431640625e-07f : 0.0f;   // 2^-20 L: the 2^-25 rounding of both positions
-  g.L32 = (float)bd.L;
   g.drift = bd.drift_u;
-  g.L = bd.L;
-  g.halfL = 0.5 * bd.L;
-  g.periodic = bd.periodic;
   return g;
 }
-
-// The FP64 data of a box that the exact decisions need, passed by value (an
-// argument passed by reference to out-of-line code would live in local memory).
-struct BoxExact {
-  double L, halfL;
-  int periodic;
-};
-
-__device__ __forceinline__ BoxExact box_exact(const ItemGeom& g) { return BoxExact{g.L, g.halfL, g.periodic}; }
 
 // Units of work are handed out from a counter in device memory (zeroed before every
 // launch): their cost varies by orders of magnitude, so a static split leaves most
@@ -68,9 +46,9 @@ __device__ __forceinline__ BoxExact box_exact(const ItemGeom& g) { return BoxExa
 
 // blocks per SM of the recording first density pass (5, with a few registers
 // spilled for the record state, measured faster than 4 blocks without spills), of
-// the plain first pass (see k_density) and of the later passes (5: with 5 % of the
-// particles iterating, a later pass cost 26 % of a full pass unbounded at 3 blocks,
-// 21 % at 5, 25 % at 7)
+// the plain first pass (see k_density), of the later passes (4.2M clustered h iteration:
+// density phase 34.0 ms at 5, 33.6 at 6, 32.5 at 7, 33.1 at 8) and of the gathered ones
+// (32.4 ms at 8, 32.2 at 7, 32.3 at 6)
 #ifndef REC_BLOCKS
 #define REC_BLOCKS 5
 #endif
@@ -78,7 +56,7 @@ __device__ __forceinline__ BoxExact box_exact(const ItemGeom& g) { return BoxExa
 #define DENS_BLOCKS 7
 #endif
 #ifndef PART_BLOCKS
-#define PART_BLOCKS 5
+#define PART_BLOCKS 7
 #endif
 
 // Exact decision r_ij < H (physical H) from the caller's FP64 positions.
@@ -88,17 +66,6 @@ __device__ __noinline__ bool exact_less(int gi, int gj, float Hphys, const unsig
   const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
   const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
   return canonical_less(canonical_r2(xi, xj, L, halfL, periodic), Hphys);
-}
-
-// FP32 test with guard band; inside the band the FP64 decision is taken.
-__device__ __forceinline__ bool decide(float r2, float H2, float band, int gi, int gj, float Hphys,
-                                       const unsigned int* perm, const double* x, const ItemGeom& g,
-                                       unsigned int& rechecks) {
-  const float dl = r2 - H2;
-  if (dl < -band) return true;
-  if (dl > band) return false;
-  ++rechecks;
-  return exact_less(gi, gj, Hphys, perm, x, g.L, g.halfL, g.periodic);
 }
 
 // =========================================================================== density
@@ -1135,15 +1102,11 @@ __device__ __forceinline__ ActiveBox active_box(const DensI& I, const Box3& bi, 
   return a;
 }
 
-// Pair-interaction setup shared by the density and force kernels.
+// What the task lists of the pair records (params.pair_cache) need of a pair-interaction.
 struct PairSetup {
   int A, B;
   ItemGeom g;
-  float3 shA, shB;        // particle frame offsets: leaf frame -> A's frame (B includes e db)
-  float3 tshA, tshB;      // cluster box offsets (the leaf centre is added per cluster)
-  float3 u;
-  unsigned int sb, ntj;   // B's sorted cluster list (sb = SORT_NONE: B's clusters in their own order)
-  unsigned int tb0;       // B's first cluster
+  float3 tshA;            // cluster box offset of A's clusters (the leaf centre is added per cluster)
   float HmB, slack;
   Box3 cellB;             // B's cell in A's frame
 };
@@ -1152,18 +1115,9 @@ __device__ __forceinline__ PairSetup pair_setup(const Lists& Lq, const Tree& T, 
   PairSetup P;
   P.A = Lq.pair_a[item];
   P.B = Lq.pair_b[item];
-  const int ax = Lq.pair_axis[item];
-  P.g = item_geom(T, box, P.A, ax);
-  const float4 cA = T.cen[P.A], cB = T.cen[P.B];
-  P.shA = make_float3(-cA.x, -cA.y, -cA.z);
-  P.shB = make_float3(P.g.offB.x - cB.x, P.g.offB.y - cB.y, P.g.offB.z - cB.z);
-  P.tshA = P.shA;
-  P.tshB = P.shB;
-  P.u = axis_unit_f(ax);
-  P.ntj = T.ntile[P.B];
-  P.tb0 = T.tile0[P.B];
-  const unsigned int sbB = T.sortbase[P.B];
-  P.sb = sbB == SORT_NONE ? SORT_NONE : sbB + (unsigned int)__popc(T.axes[P.B] & ((1u << ax) - 1u)) * P.ntj;
+  P.g = item_geom(T, box, P.A, Lq.pair_axis[item]);
+  const float4 cA = T.cen[P.A];
+  P.tshA = make_float3(-cA.x, -cA.y, -cA.z);
   P.HmB = T.hmax[P.B] * P.g.invL;
   P.slack = P.g.e * 1.52587890625e-05f + P.g.es + 1e-6f * fmaxf(P.HmB, T.hmax[P.A] * P.g.invL);   // 2^-16 e
   // B's cell, widened by the drift of particles kept in it since the build
@@ -1171,27 +1125,6 @@ __device__ __forceinline__ PairSetup pair_setup(const Lists& Lq, const Tree& T, 
   P.cellB.lo = make_float3(P.g.offB.x - h, P.g.offB.y - h, P.g.offB.z - h);
   P.cellB.hi = make_float3(P.g.offB.x + h, P.g.offB.y + h, P.g.offB.z + h);
   return P;
-}
-
-// The frame of a pair task's particle arithmetic: the centre of the own cluster's
-// leaf.  A pair of large cells that cannot split (one particle of large H in it
-// is enough) still holds particles of small H; in A's frame their positions
-// would be rounded at A's scale, in their leaf's frame at the leaf's.  The own
-// offsets are used as stored (sh_own = -leaf centre cancels their leaf centre
-// exactly), B's particles move by the exact dyadic offset sh_part, so each
-// position is rounded once, at most at A's scale: the guard band stays valid.
-// d: the leaf centre in A's frame (exact), for moving boxes between the frames.
-struct LeafFrame {
-  float3 sh_own, sh_part, d;
-};
-
-__device__ __forceinline__ LeafFrame leaf_frame(const Tiles& TL, const Tree& T, unsigned int ti, const PairSetup& P) {
-  const float4 cl = TL.cen[ti], ca = T.cen[P.A];
-  LeafFrame F;
-  F.sh_own = make_float3(-cl.x, -cl.y, -cl.z);
-  F.d = make_float3(cl.x - ca.x, cl.y - ca.y, cl.z - ca.z);
-  F.sh_part = make_float3(P.shB.x - F.d.x, P.shB.y - F.d.y, P.shB.z - F.d.z);
-  return F;
 }
 
 // ------------------------------------------------------------- units of work
@@ -1204,6 +1137,13 @@ __device__ __forceinline__ LeafFrame leaf_frame(const Tiles& TL, const Tree& T, 
 // partners per own particle and task in a uniform box), and most batches were
 // partly filled.  Where a box has few clusters, a unit is split into parts (every
 // parts-th interaction), so that every warp has several.
+//
+// The frame of a unit's particle arithmetic is the centre of the own cluster's leaf.  A
+// pair of large cells that cannot split (one particle of large H in it is enough) still
+// holds particles of small H; in the cells' frame their positions would be rounded at
+// the cells' scale, in their leaf's frame at the leaf's.  Own offsets are used as stored,
+// the partners' move by an exact dyadic offset, so each position is rounded once, at most
+// at the cells' scale, and the guard band stays valid.
 // (One unit per warp in the smallest boxes, two where a cluster per warp would leave a
 // partial wave: lattices of 25^3 and 30^3 lose 10 % with twice the parts, of 36^3, 42^3
 // and a 40k Plummer box gain 10-40 %; three or five times the warps lose 5-30 % there.)
@@ -1754,15 +1694,15 @@ __device__ __forceinline__ void force_replay_task(bool self, int item, unsigned 
   if (vi) flush_force((int)(own0 + lane), S.iacc[lane], S.ivs[lane], facc, fvsig);
 }
 
-// Density interactions of one pass: the live pair and self tasks in one queue.
+// Density interactions of one pass: one queue of units (REC: of the listed tasks).
 // PART: a later pass of the h iteration (particles still iterating), where the own
 // side culls against the box of the cluster's iterating particles; the first pass
 // (every particle) has its own instance without that code.  Both are launched in
 // a captured step, and the one that does not match the iteration returns.
 // The first pass (PART = false) runs 7 blocks of 128 threads per SM (at most 73
-// registers, a few spilled): the pass waits mostly on partner loads, and more warps
-// in flight hide more of them (33.5M: 62.8 ms at 5 blocks, 61.5 at 6, 60.5 at 7,
-// 61.7 at 8, where the spills grow).
+// registers, a few spilled): issue slots bound the pass, and more warps in flight fill
+// them until the spills grow (density phase of the 33.5M step 36.4 ms at 6 blocks, 33.9 at
+// 7, 34.7 at 8, 38.9 at 10).
 template <bool COUNT, bool PART, bool KAHAN, bool REC>
 __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_BLOCKS : DENS_BLOCKS)) k_density(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box,
                                                          const float4* __restrict__ pos4,
@@ -2225,7 +2165,7 @@ __device__ __forceinline__ void gather_unit(unsigned int pid, unsigned int part,
 }
 
 #ifndef GATHER_BLOCKS
-#define GATHER_BLOCKS 8
+#define GATHER_BLOCKS 7
 #endif
 // The gathered density pass (a later pass of the h iteration that gathers): units of the
 // packed clusters; g_n[1] counts the passes that gathered.  Returns at once when the pass

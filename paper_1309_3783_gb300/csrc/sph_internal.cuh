@@ -337,7 +337,3 @@ struct Lists {
                             // [5] sort entries, [6] pair tasks, [7] self tasks, [8] entries of csr
 };
 
-// Per-box counters kept by the pair kernels when counting is on.
-struct PairCounters {
-  unsigned long long dens_pairs, dens_sides, dens_cand, force_pairs, force_cand, rechecks;
-};
