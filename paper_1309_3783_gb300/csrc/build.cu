@@ -1431,28 +1431,170 @@ __device__ __forceinline__ void divide_node(const NodeShared& S, int n, int cmax
 // its first particle a, the next node is the largest that starts at a and fits: its
 // bit b* is the smallest of the highest bits in which key[a] differs from key[a - 1]
 // (the node must start at a) and from key[a + 4 cmax] (it must end before).  One
-// warp per leaf.
+// warp per leaf; a leaf of more than CLUSTER_BLOCK particles, and of four times a warp's
+// share of all, takes a block, each warp a part of the walk (a warp alone with the 45
+// nodes of a 4800-particle leaf took longer than all the others of a 4.2M box together:
+// that phase of its build 1.18 -> 0.90 ms.  In larger boxes the leaf is no longer than
+// the rest, and the blocks' barriers cost 0.5 of 4.5 ms at 33.5M).
 constexpr int CLUSTER_WARPS = 4;
+constexpr unsigned int CLUSTER_BLOCK = 1024;
+
+// What the walk of one leaf needs.
+struct LeafWalk {
+  const unsigned long long* key;
+  const unsigned int* perm;
+  const double* x;
+  unsigned int *lsrc, *flag;
+  double iL, cen[3];
+  int lb, cmax;             // key bits below the leaf's cell; cluster size
+};
+
+__device__ __forceinline__ LeafWalk leaf_walk(const Tree& T, int id, const BoxDesc& bd, int box_shift,
+                                              const unsigned long long* key, const unsigned int* perm, const double* x,
+                                              unsigned int* lsrc, unsigned int* flag, int cmax) {
+  const int d = T.level[id];
+  unsigned int cx, cy, cz;
+  cell_coords(T.key[id], d, cx, cy, cz);
+  const double inv = scaled_down(1.0, d);
+  LeafWalk W{key, perm, x, lsrc, flag, bd.invL, {((double)cx + 0.5) * inv, ((double)cy + 0.5) * inv, ((double)cz + 0.5) * inv},
+             box_shift - 3 * d, cmax};
+  return W;
+}
+
+// The nodes of the class [beg, end) that start in [a, stop) (a: the start of a node).
+__device__ __forceinline__ void walk_nodes(NodeShared& S, const LeafWalk& W, unsigned int a, unsigned int stop,
+                                           unsigned int beg, unsigned int end) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int cap = 4u * (unsigned int)W.cmax;
+  while (a < stop) {
+    const unsigned long long ka = W.key[W.lsrc[a]];
+    int bs = W.lb;
+    if (a > beg) bs = min(bs, high_bit(W.key[W.lsrc[a - 1]] ^ ka));
+    if (a + cap < end) bs = min(bs, high_bit(ka ^ W.key[W.lsrc[a + cap]]));
+    unsigned int n = min(cap, end - a);   // equal keys (bs < 0): no node starts here, take a chunk
+    if (bs >= 0) {
+      unsigned int m = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned int q = 32u * i + lane;
+        m += __popc(__ballot_sync(0xffffffffu, q < n && ((W.key[W.lsrc[a + q]] ^ ka) >> bs) == 0ull));
+      }
+      n = m;      // (the node's particles are adjacent)
+    }
+    n = min(n, stop - a);                 // (only a chunk that runs on past equal keys could reach the next walk's)
+    if (n <= (unsigned int)W.cmax) {
+      if ((unsigned int)lane < n) W.flag[a + lane] = lane == 0 ? 1u : 0u;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned int q = 32u * i + lane;
+        if (q >= n) break;
+        const unsigned int src = W.lsrc[a + q];
+        const long long p = W.perm[src];
+        S.src[q] = src;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) S.x[k][q] = (float)(W.x[3 * p + k] * W.iL - W.cen[k]);
+      }
+      __syncwarp();
+      if (n <= 64u) divide_node<2>(S, (int)n, W.cmax, W.lsrc + a, W.flag + a);
+      else divide_node<4>(S, (int)n, W.cmax, W.lsrc + a, W.flag + a);
+      __syncwarp();
+    }
+    a += n;
+  }
+}
+
+// A node start in the cap particles from p on (beg < p; end if there is none to be
+// told).  The two neighbours whose keys differ in the highest bit among the cap + 2
+// particles around belong to different nodes: a node of both would reach beyond a bit no
+// neighbours here differ in, so hold them all, which are too many.
+__device__ __forceinline__ unsigned int node_start(const LeafWalk& W, unsigned int p, unsigned int end) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int cap = 4u * (unsigned int)W.cmax;
+  if (p + cap >= end) return end;
+  int hb = -1;
+  unsigned int at = end;
+  for (unsigned int q = p + lane; q <= p + cap; q += 32) {
+    const int b = high_bit(W.key[W.lsrc[q - 1]] ^ W.key[W.lsrc[q]]);
+    if (b > hb) {
+      hb = b;
+      at = q;
+    }
+  }
+  const int top = __reduce_max_sync(0xffffffffu, hb);
+  if (top < 0) return end;      // one key throughout: chunks of it count from its first particle
+  return __reduce_min_sync(0xffffffffu, hb == top ? at : 0xffffffffu);
+}
 
 __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
     Tree T, int nnodes, int box_shift, const BoxDesc* __restrict__ box, const float* __restrict__ Hs,
     const unsigned long long* __restrict__ key, const unsigned int* __restrict__ perm, const double* __restrict__ x,
-    unsigned int* lsrc, unsigned int* __restrict__ flag, int cmax) {
+    unsigned int* lsrc, unsigned int* flag, int cmax, long long N) {
   pdl_wait();
+  const unsigned int big = max(CLUSTER_BLOCK, (unsigned int)(4 * N / (gridDim.x * CLUSTER_WARPS)));
   __shared__ NodeShared SH[CLUSTER_WARPS];
+  __shared__ unsigned int s_small[CLUSTER_WARPS], s_start[2][CLUSTER_WARPS];
   nnodes = min(nnodes, T.n_nodes[0]);
-  const int lane = threadIdx.x & 31;
-  NodeShared& S = SH[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  NodeShared& S = SH[w];
+  const unsigned int lt = (1u << lane) - 1u;
+  // large leaves: one block each
+  for (int id = blockIdx.x; id < nnodes; id += gridDim.x) {
+    const unsigned int c = T.count[id];
+    if (c <= big || T.child[id] >= 0) continue;      // the same for the whole block
+    const unsigned int s = T.start[id];
+    const BoxDesc& bd = box[T.box[id]];
+    const float thr = (float)scaled_down(bd.L, T.level[id]);
+    const unsigned int per = ((c + CLUSTER_WARPS - 1) / CLUSTER_WARPS + 31u) & ~31u;
+    const unsigned int w0 = min(c, w * per), w1 = min(c, w0 + per);
+    unsigned int ns = 0;
+    for (unsigned int b = w0; b < w1; b += 32) {
+      const unsigned int q = b + lane;
+      ns += __popc(__ballot_sync(0xffffffffu, q < w1 && !(Hs[s + q] > thr)));
+    }
+    if (lane == 0) s_small[w] = ns;
+    __syncthreads();
+    unsigned int nsmall = 0, os = 0;
+    for (int k = 0; k < CLUSTER_WARPS; ++k) {
+      if (k < w) os += s_small[k];
+      nsmall += s_small[k];
+    }
+    unsigned int ol = nsmall + (w0 - os);      // w0 particles come before this warp's, os of them small
+    for (unsigned int b = w0; b < w1; b += 32) {
+      const unsigned int q = b + lane;
+      const bool valid = q < w1;
+      const bool large = valid && Hs[s + q] > thr;
+      const unsigned int bs = __ballot_sync(0xffffffffu, valid && !large);
+      const unsigned int bl = __ballot_sync(0xffffffffu, large);
+      if (valid) lsrc[s + (large ? ol + __popc(bl & lt) : os + __popc(bs & lt))] = s + q;
+      os += __popc(bs);
+      ol += __popc(bl);
+    }
+    __syncthreads();
+    const LeafWalk W = leaf_walk(T, id, bd, box_shift, key, perm, x, lsrc, flag, cmax);
+    for (int cls = 0; cls < 2; ++cls) {
+      const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
+      const unsigned int from = w == 0 ? beg : node_start(W, beg + (unsigned int)(((unsigned long long)(end - beg) * w) / CLUSTER_WARPS), end);
+      if (lane == 0) s_start[cls][w] = from;
+    }
+    __syncthreads();      // (the walks reorder what the starts were read from)
+    for (int cls = 0; cls < 2; ++cls) {
+      const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
+      const unsigned int from = s_start[cls][w];
+      unsigned int stop = end;
+      for (int k = CLUSTER_WARPS - 1; k > w; --k) stop = min(stop, s_start[cls][k]);
+      walk_nodes(S, W, from, stop, beg, end);
+    }
+    __syncthreads();
+  }
+  // the other leaves: one warp each
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  const unsigned int lt = (1u << lane) - 1u;
-  const unsigned int cap = 4u * (unsigned int)cmax;
   for (int id = warp; id < nnodes; id += nwarps) {
-    if (T.child[id] >= 0) continue;
     const unsigned int s = T.start[id], c = T.count[id];
+    if (c > big || T.child[id] >= 0) continue;
     const BoxDesc& bd = box[T.box[id]];
-    const int d = T.level[id];
-    const float thr = (float)scaled_down(bd.L, d);
+    const float thr = (float)scaled_down(bd.L, T.level[id]);
     unsigned int nsmall = 0;
     for (unsigned int b = 0; b < c; b += 32) {
       const unsigned int q = b + lane;
@@ -1473,50 +1615,9 @@ __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
       ol += __popc(bl);
     }
     __syncwarp();
-    const int lb = box_shift - 3 * d;      // key bits below the leaf's cell
-    unsigned int cx, cy, cz;
-    cell_coords(T.key[id], d, cx, cy, cz);
-    const double inv = scaled_down(1.0, d), iL = bd.invL;
-    const double cen[3] = {((double)cx + 0.5) * inv, ((double)cy + 0.5) * inv, ((double)cz + 0.5) * inv};
-    for (int cls = 0; cls < 2; ++cls) {
-      const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
-      unsigned int a = beg;
-      while (a < end) {
-        const unsigned long long ka = key[lsrc[a]];
-        int bs = lb;
-        if (a > beg) bs = min(bs, high_bit(key[lsrc[a - 1]] ^ ka));
-        if (a + cap < end) bs = min(bs, high_bit(ka ^ key[lsrc[a + cap]]));
-        unsigned int n = min(cap, end - a);   // equal keys (bs < 0): no node starts here, take a chunk
-        if (bs >= 0) {
-          unsigned int m = 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const unsigned int q = 32u * i + lane;
-            m += __popc(__ballot_sync(0xffffffffu, q < n && ((key[lsrc[a + q]] ^ ka) >> bs) == 0ull));
-          }
-          n = m;      // (the node's particles are adjacent)
-        }
-        if (n <= (unsigned int)cmax) {
-          if ((unsigned int)lane < n) flag[a + lane] = lane == 0 ? 1u : 0u;
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const unsigned int q = 32u * i + lane;
-            if (q >= n) break;
-            const unsigned int src = lsrc[a + q];
-            const long long p = perm[src];
-            S.src[q] = src;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) S.x[k][q] = (float)(x[3 * p + k] * iL - cen[k]);
-          }
-          __syncwarp();
-          if (n <= 64u) divide_node<2>(S, (int)n, cmax, lsrc + a, flag + a);
-          else divide_node<4>(S, (int)n, cmax, lsrc + a, flag + a);
-          __syncwarp();
-        }
-        a += n;
-      }
-    }
+    const LeafWalk W = leaf_walk(T, id, bd, box_shift, key, perm, x, lsrc, flag, cmax);
+    walk_nodes(S, W, s, s + nsmall, s, s + nsmall);
+    walk_nodes(S, W, s + nsmall, s + c, s + nsmall, s + c);
   }
 }
 

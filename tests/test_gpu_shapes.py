@@ -76,17 +76,20 @@ def _check_passes(api, box, leaf, cmax):
 # and from 4256 clusters on the list of units.
 @pytest.mark.parametrize("n,leaf,cmax,clump", [(33, 400, 32, 0.0), (131, 400, 32, 0.0), (1025, 31, 24, 0.1),
                                                (1500, 130, 16, 0.3), (4097, 4800, 32, 0.4), (30000, 400, 32, 0.2),
-                                               (60001, 48, 24, 0.1), (130003, 400, 32, 0.2)])
+                                               (60001, 48, 24, 0.1), (130003, 400, 32, 0.2),
+                                               (20000, 4800, 32, 0.6), (20000, 1100, 16, 0.6), (9000, 4800, 32, -1.0)])
 def test_clusters_and_units(api, n, leaf, cmax, clump):
     side = int(np.ceil(n ** (1 / 3)))
     box = inputs.lattice_box(side, jitter=0.3, seed=n, v_sigma=0.3, periodic=n != 1500)
     box = box.subset(np.arange(box.n - n, box.n))
     rng = np.random.default_rng(n)
-    k = int(clump * n)
+    k = int(max(clump, 0.0) * n)
     if k:      # a clump ten times as dense as its surroundings, h to match
         r = 0.5 * (k / n / 10) ** (1 / 3)
         box.x[:k] = np.mod(np.array([0.4, 0.55, 0.6]) + rng.uniform(-r, r, (k, 3)), box.L)
         box.h[:k] *= np.float32(10 ** (-1 / 3))
+    if clump < 0:      # points shared by more particles than a node takes: their keys are equal
+        box.x[: n // 3] = box.x[rng.integers(0, 12, n // 3) + n // 2]
     box.h = np.minimum(box.h * rng.uniform(0.8, 1.2, n), 0.24 * box.L / 1.8258).astype(np.float32)
     _check_passes(api, box, leaf, cmax)
 
