@@ -725,18 +725,12 @@ __global__ void k_gather_sorted(long long N, const unsigned int* __restrict__ pe
                                 const BoxDesc* __restrict__ box, const float4* __restrict__ a_in, int vpred,
                                 float* __restrict__ Hs, float4* __restrict__ vel4) {
   pdl_wait();
-  int lb = -1;             // (FP64 once per box)
-  float hdt = 0.0f;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
     const unsigned int i = perm[p];
     Hs[p] = H_in[i];
     float4 w = make_float4(v[3ll * i], v[3ll * i + 1], v[3ll * i + 2], u[i]);
     if (vpred) {
-      const int b = bid[i];
-      if (b != lb) {
-        hdt = (float)(0.5 * box[b].dt);
-        lb = b;
-      }
+      const float hdt = (float)(0.5 * box[bid[i]].dt);
       if (hdt != 0.0f) {
         const float4 a = a_in[i];
         w.x += a.x * hdt;

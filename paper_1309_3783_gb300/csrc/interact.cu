@@ -2597,14 +2597,8 @@ void launch_set_acc(Engine& E, long long off, long long n, int which, const floa
 __global__ void k_kick(long long N, const int* __restrict__ bid, const BoxDesc* __restrict__ box,
                        const float4* __restrict__ a_in, float* __restrict__ v, float* __restrict__ u) {
   pdl_wait();
-  int lb = -1;             // (FP64 once per box)
-  float hdt = 0.0f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const int b = bid[i];
-    if (b != lb) {
-      hdt = (float)(0.5 * box[b].dt);
-      lb = b;
-    }
+    const float hdt = (float)(0.5 * box[bid[i]].dt);      // (kept from round to round it held the loads up: 0.26 -> 0.54 ms)
     if (hdt == 0.0f) continue;
     const float4 a = a_in[i];
     v[3 * i] += a.x * hdt;
