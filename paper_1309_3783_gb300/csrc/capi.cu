@@ -336,6 +336,7 @@ sph_status Engine::relayout(const std::vector<BoxSpec>& boxes, const std::vector
   h.swap(rl_h);
   hhist.swap(rl_hh);
   a_in.swap(rl_a);
+  acc_edited = true;
   return SPH_OK;
 }
 
@@ -1075,6 +1076,7 @@ sph_status Engine::force() {
   CK(cudaGetLastError());
   have_force = true;
   have_acc = true;
+  acc_edited = false;
   have_fcount = count_pairs;
   return SPH_OK;
 }
@@ -1405,6 +1407,7 @@ sph_status Engine::step_graph() {
   ++n_reuses;
   built = true;
   have_density = have_ghost = have_force = have_acc = true;
+  acc_edited = false;
   rec_valid = R.pool != nullptr;
   last_iters = itv[0];
   last_rebuilds = 0;
@@ -1848,6 +1851,7 @@ sph_status Engine::build_step_graph() {
     }
   }
   have_density = have_ghost = have_force = have_acc = true;
+  acc_edited = false;
   last_iters = itv[0];
   last_rebuilds = 0;
   last_gathered = 0;
@@ -2075,6 +2079,7 @@ sph_status Engine::set_field(int b, int field, const void* src, long long n, int
     dsrc = reinterpret_cast<const float*>(staging.p);
   }
   if (!have_acc) CK(cudaMemsetAsync(a_in.p + o, 0, nb * sizeof(float4), st));
+  acc_edited = true;
   launch_set_acc(*this, o, nb, field == SPH_FIELD_A ? 0 : 1, dsrc);
   CK(cudaGetLastError());
   have_acc = true;

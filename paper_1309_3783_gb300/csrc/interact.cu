@@ -3034,7 +3034,28 @@ void launch_set_h(Engine& E, int b, const float* src) {
   launch_pdl(k_set_h, E.grid(n), 256, E.st, n, src, E.h.p + E.off[b], E.hlev.p + b); count_launch();
 }
 
+// The accelerations and du/dt of the last force pass from their copy in caller order,
+// which needs no scatter (1.28 and 0.57 ms for 33.5M particles through the permutation).
+__global__ void k_get_acc(long long off, long long n, int field, const float4* __restrict__ a_in, float* __restrict__ out) {
+  pdl_wait();
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
+    const float4 a = a_in[off + q];
+    if (field == SPH_FIELD_DUDT) {
+      out[q] = a.w;
+    } else {
+      out[3 * q] = a.x;
+      out[3 * q + 1] = a.y;
+      out[3 * q + 2] = a.z;
+    }
+  }
+}
+
 void launch_get_field(Engine& E, long long off, long long n, int field, void* out) {
+  if ((field == SPH_FIELD_A || field == SPH_FIELD_DUDT) && !E.acc_edited) {
+    launch_pdl(k_get_acc, E.grid(n), 256, E.st, off, n, field, E.a_in.p, reinterpret_cast<float*>(out));
+    count_launch();
+    return;
+  }
   launch_pdl(k_get_field, E.grid(n), 256, E.st, off, n, field, E.perm.p, E.Hs.p, E.cen4.p, E.vel4.p, E.dacc.p, E.dcnt.p,
                                            E.ghost4.p, E.facc.p, E.fvsig.p, E.fcnt.p, E.h.p, E.prm.gamma_gas, out);
   count_launch();

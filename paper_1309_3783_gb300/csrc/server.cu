@@ -119,6 +119,7 @@ static sph_status apply_layout(sph_server* s) {
   // starting forces of new boxes come from their first (dt = 0) tick; the kick of
   // every box reads a_in, so the engine never recomputes forces on its own
   E.have_acc = true;
+  E.acc_edited = true;
   s->layout = s->resident;
   return SPH_OK;
 }

@@ -329,6 +329,7 @@ class Engine {
   long long steps_in_layout = 0;  // steps since the boxes were last laid out (a capture pays off after a few)
   long long last_unconverged = 0;
   bool built = false, have_density = false, have_ghost = false, have_force = false, have_acc = false;
+  bool acc_edited = false;        // a_in is no longer the last force pass's (set by the caller, moved to a new layout)
   bool have_fcount = false;       // the last force pass counted pairs (fcnt is filled)
 
   // profiling: CUDA events around each phase on the engine's stream
