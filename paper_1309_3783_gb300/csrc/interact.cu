@@ -44,13 +44,13 @@ __device__ __forceinline__ ItemGeom item_geom(const Tree& T, const BoxDesc* box,
 // launch): their cost varies by orders of magnitude, so a static split leaves most
 // SMs idle behind the longest ones.
 
-// blocks per SM of the recording first density pass (5, with a few registers
-// spilled for the record state, measured faster than 4 blocks without spills), of
+// blocks per SM of the recording first density pass (4.2M clustered 10.2 ms at 5, 9.9 at
+// 6, 9.2 at 7), of
 // the plain first pass (see k_density), of the later passes (4.2M clustered h iteration:
 // density phase 34.0 ms at 5, 33.6 at 6, 32.5 at 7, 33.1 at 8) and of the gathered ones
 // (32.4 ms at 8, 32.2 at 7, 32.3 at 6)
 #ifndef REC_BLOCKS
-#define REC_BLOCKS 5
+#define REC_BLOCKS 7
 #endif
 #ifndef DENS_BLOCKS
 #define DENS_BLOCKS 7
@@ -634,19 +634,19 @@ __device__ __forceinline__ void dens_row(const DensI& I, float ilo, const DensSh
 }
 
 // The masks as exact decisions (counting and recording passes, which need them
-// before the sweeps): both decisions of a slot inside either band, in FP64.
-__device__ __noinline__ void resolve_masks(const DensShared& S, float ilo, float jlo, unsigned int& mI,
-                                           unsigned int& mJ, unsigned int& rc, const unsigned int* perm,
-                                           const double* x, const float4* pos4, const BoxDesc* box) {
+// before the sweeps): both decisions of a pair inside either band, in FP64.  Each lane
+// walks its own candidates; S.m holds the slots' lower bounds.
+__device__ __noinline__ void resolve_masks(const DensShared& S, float ilo, unsigned int& mI, unsigned int& mJ,
+                                           unsigned int& rc, const unsigned int* perm, const double* x,
+                                           const float4* pos4, const BoxDesc* box) {
   const int lane = threadIdx.x & 31;
-  const BoxDesc& bd = box[S.tk.box];
   const float4 P = S.ip[lane];
-  for (int s = 0; s < 32; ++s) {
-    const float lo = __shfl_sync(0xffffffffu, jlo, s);     // the slot's lane holds its lower bound
+  for (unsigned int m = mI | mJ; m; m &= m - 1) {
+    const int s = __ffs(m) - 1;
     const unsigned int bit = 1u << s;
-    if (!((mI | mJ) & bit)) continue;
     const float r2 = pair_r2(P.x - S.x[s], P.y - S.y[s], P.z - S.z[s]);
-    if (((mI & bit) && r2 >= ilo) || ((mJ & bit) && r2 >= lo)) {
+    if (((mI & bit) && r2 >= ilo) || ((mJ & bit) && r2 >= S.m[s])) {
+      const BoxDesc& bd = box[S.tk.box];
       rc += 2;
       const int gi = S.ig[lane];
       mI = exact_less(gi, S.g[s], pos4[gi].w, perm, x, bd.L, 0.5 * bd.L, bd.periodic) ? (mI | bit) : (mI & ~bit);
@@ -698,7 +698,12 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   mI &= allow;
   mJ &= allow;
   unsigned int rc = 0;
-  if (COUNT || (REC && !PART)) resolve_masks(S, ilo, jlo, mI, mJ, rc, perm, x, pos4, box);
+  if (COUNT || (REC && !PART)) {
+    S.m[lane] = jlo;
+    __syncwarp();
+    resolve_masks(S, ilo, mI, mJ, rc, perm, x, pos4, box);
+    __syncwarp();
+  }
   // the pairs for the force pass: each unordered pair once (inside one cluster,
   // the partners above the lane)
   if (REC && !PART) rec_batch(R, W, S, jvalid, (mI | mJ) & (own_only ? upper_mask(lane) : 0xffffffffu));
@@ -1665,8 +1670,8 @@ __device__ __forceinline__ bool changed_out_of_reach(bool self, int item, unsign
   return !box_near(bi, cb, reach);
 }
 
-// A force task replayed from the records of the first density pass: the frames
-// of the particle arithmetic are those of force_pair_task / force_self_task, the
+// A force task replayed from the records of the first density pass: the frame
+// of the particle arithmetic is that of the units, the
 // batches follow the recording warp's chain of chunks.  Valid while no particle of
 // the own cluster or of the partner cell (the own cell for a self task) has taken
 // a new h since the recording: the recorded pairs are then the pairs at the
@@ -1677,14 +1682,27 @@ __device__ __forceinline__ void force_replay_task(bool self, int item, unsigned 
     const float4* __restrict__ cen4, const float4* __restrict__ vel4, const float4* __restrict__ ghost4,
     const ForceArgs& A, float4* facc, float* fvsig, ForceShared& S, Counters* C) {
   const int lane = threadIdx.x & 31;
-  unit_begin(S.tk, ti, T, TL, box, 0u, 1u);
-  unit_single(S.tk, self, item, Lq, T);
+  // of a unit's constants only what the batches read, and the partners' frame
+  const int A0 = self ? Lq.self_a[item] : Lq.pair_a[item], B0 = self ? A0 : Lq.pair_b[item];
+  const int bx = T.box[A0];
+  const float e = ldexpf(1.0f, -T.level[A0]);
+  int dx = 0, dy = 0, dz = 0;
+  if (!self) axis_vec(Lq.pair_axis[item], dx, dy, dz);
+  const float4 cA = T.cen[A0], cB = T.cen[B0], cl = TL.cen[ti];
+  const float3 sh = make_float3((e * dx - cB.x) - (cl.x - cA.x), (e * dy - cB.y) - (cl.y - cA.y),
+                                (e * dz - cB.z) - (cl.z - cA.z));
+  __syncwarp();
+  if (lane == 0) {
+    S.tk.box = bx;
+    S.tk.L32 = (float)box[bx].L;
+    S.tk.bhi.w = (float)box[bx].invL;
+    S.tk.eb = box[bx].global32 ? 1.0f : e;
+  }
+  __syncwarp();
   const unsigned int own0 = TL.start[ti];
   const bool vi = (unsigned int)lane < TL.n[ti];
   if (lane == 0) S.own0 = own0;
   force_stage_own(S, lane, vi, own0 + lane, A.pos4, cen4, vel4, ghost4);
-  const float4 sh4 = S.tk.gsh[0];
-  const float3 sh = make_float3(sh4.x, sh4.y, sh4.z);
   unsigned int b = rec.x;
   for (unsigned int k = 0; k < rec.y; ++k, ++b) {
     if (k > 0 && b % REC_CHUNK == 0u) b = R.next[b / REC_CHUNK - 1u] * REC_CHUNK;   // the chunk is full: next one
