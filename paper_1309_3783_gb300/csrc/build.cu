@@ -66,7 +66,25 @@ __global__ void k_ingest(long long N, const int* __restrict__ bid, BoxDesc* box,
       if (mn != 0xffffffffu) atomicMin(reinterpret_cast<unsigned int*>(&box[b].Hmin), mn);
     }
   }
-  if (rb >= 0 && (threadIdx.x & 31) == 0) {
+  // the block's warps mostly hold one box: one atomic for all of them (one per warp of a
+  // million-particle box, 19,000 on one address, took half of the kernel)
+  __shared__ int s_b[32];
+  __shared__ unsigned int s_mx[32], s_mn[32];
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    s_b[w] = rb;
+    s_mx[w] = rmx;
+    s_mn[w] = rmn;
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && rb >= 0) {
+    for (int k = 0; k < w; ++k)
+      if (s_b[k] == rb) return;            // an earlier warp of this box adds it
+    for (int k = w + 1; k < nw; ++k)
+      if (s_b[k] == rb) {
+        rmx = max(rmx, s_mx[k]);
+        rmn = min(rmn, s_mn[k]);
+      }
     if (rmx) atomicMax(reinterpret_cast<unsigned int*>(&box[rb].Hmax), rmx);
     if (rmn != 0xffffffffu) atomicMin(reinterpret_cast<unsigned int*>(&box[rb].Hmin), rmn);
   }
@@ -283,7 +301,22 @@ __global__ void k_displacement(long long N, const int* __restrict__ bid, const B
       atomicMax(&dmax[b], dbits(sqrt(__longlong_as_double((long long)bits))));
     }
   }
-  if (rb >= 0 && (threadIdx.x & 31) == 0) atomicMax(&dmax[rb], dbits(sqrt(__longlong_as_double((long long)rbits))));
+  // one atomic per block and box, as in k_ingest
+  __shared__ int s_b[32];
+  __shared__ unsigned long long s_bits[32];
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    s_b[w] = rb;
+    s_bits[w] = rbits;
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && rb >= 0) {
+    for (int k = 0; k < w; ++k)
+      if (s_b[k] == rb) return;
+    for (int k = w + 1; k < nw; ++k)
+      if (s_b[k] == rb) rbits = s_bits[k] > rbits ? s_bits[k] : rbits;
+    atomicMax(&dmax[rb], dbits(sqrt(__longlong_as_double((long long)rbits))));
+  }
 }
 
 // The smallest H limit along a cell's chain (limits order like their bits as signed
