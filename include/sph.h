@@ -135,7 +135,7 @@ typedef struct sph_params {
                              own (0)                                               */
     int32_t h_gather;     /* 1: a later pass of the h iteration (Section II-D, the
                              density loop again for the particles whose h has not
-                             converged) in which at most a third of the
+                             converged) in which at most an eighth of the
                              particles iterate gathers: each leaf's iterating
                              particles are packed into clusters of up to 32 and
                              every interaction runs for the packed clusters of its

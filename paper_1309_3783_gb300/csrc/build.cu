@@ -1328,220 +1328,67 @@ __global__ void k_shift(long long N, int box_shift, const unsigned long long* __
 }
 
 // ============================================================== clusters
-// Sorts 32 I values, value 32 i + lane in v[i] (bitonic, in registers).
-template <int I>
-__device__ __forceinline__ void warp_sort(unsigned int (&v)[I]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 2; k <= 32 * I; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-#pragma unroll
-      for (int i = 0; i < I; ++i) {
-        const bool up = ((32 * i + lane) & k) == 0;
-        if (j >= 32) {
-          const int p = i ^ (j >> 5);
-          if (p > i) {
-            const unsigned int a = min(v[i], v[p]), b = max(v[i], v[p]);
-            v[i] = up ? a : b;
-            v[p] = up ? b : a;
-          }
-        } else {
-          const unsigned int y = __shfl_xor_sync(0xffffffffu, v[i], j);
-          v[i] = ((lane & j) == 0) == up ? min(v[i], y) : max(v[i], y);
-        }
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ int high_bit(unsigned long long v) { return v ? 63 - __clzll((long long)v) : -1; }
-
-// Per warp: the particles of the node being divided -- position relative to the leaf
-// centre (units of L) and source index.
-struct NodeShared {
-  float x[3][128];
-  unsigned int src[128];
-};
-
-// The longest axis of particles id[0 .. n) of the node, and their range along it.
-template <int I>
-__device__ __forceinline__ int node_axis(const NodeShared& S, const unsigned int (&v)[I], int r0, int r1, float& lo,
-                                         float& scale) {
-  const int lane = threadIdx.x & 31;
-  float a[3], b[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    a[k] = FLT_MAX;
-    b[k] = -FLT_MAX;
-#pragma unroll
-    for (int i = 0; i < I; ++i) {
-      const int r = 32 * i + lane;
-      if (r < r0 || r >= r1) continue;
-      const float t = S.x[k][v[i] & 127u];
-      a[k] = fminf(a[k], t);
-      b[k] = fmaxf(b[k], t);
-    }
-    a[k] = warp_min(a[k]);
-    b[k] = warp_max(b[k]);
-  }
-  int ax = 0;
-  if (b[1] - a[1] > b[0] - a[0]) ax = 1;
-  if (b[2] - a[2] > b[ax] - a[ax]) ax = 2;
-  lo = a[ax];
-  scale = b[ax] > a[ax] ? 1.0f / (b[ax] - a[ax]) : 0.0f;
-  return ax;
-}
-
-// The order of a node's n particles (n <= 32 I) and its clusters: k = ceil(n / cmax)
-// of them, by halving along the longest axis (a third first when k = 3), each part
-// along its own.  v[i] on return: the particle at place 32 i + lane (low 7 bits).
-template <int I>
-__device__ __forceinline__ void divide_node(const NodeShared& S, int n, int cmax, unsigned int* __restrict__ lsrc,
-                                            unsigned int* __restrict__ flag) {
-  const int lane = threadIdx.x & 31;
-  const int k = (n + cmax - 1) / cmax;
-  unsigned int v[I];
-#pragma unroll
-  for (int i = 0; i < I; ++i) v[i] = (unsigned int)(32 * i + lane);
-  float lo, sc;
-  int ax = node_axis(S, v, 0, n, lo, sc);
-#pragma unroll
-  for (int i = 0; i < I; ++i) {
-    const int r = 32 * i + lane;
-    v[i] = r < n ? ((unsigned int)((S.x[ax][r] - lo) * sc * 16777215.0f) << 7) | (unsigned int)r : 0xffffffffu;
-  }
-  warp_sort(v);
-  const int nl = k == 3 ? (n + 2) / 3 : (n + 1) / 2;      // the left part
-  int c1 = nl, c2 = n, c3 = n;                            // starts of the clusters after the first
-  if (k > 2) {
-    float lo1, sc1;
-    const int ax0 = node_axis(S, v, 0, nl, lo, sc), ax1 = node_axis(S, v, nl, n, lo1, sc1);
-#pragma unroll
-    for (int i = 0; i < I; ++i) {
-      const int r = 32 * i + lane;
-      const unsigned int id = v[i] & 127u;
-      const bool right = r >= nl;
-      if (r < n)
-        v[i] = (right ? 0x80000000u : 0u) |
-               ((unsigned int)((right ? (S.x[ax1][id] - lo1) * sc1 : (S.x[ax0][id] - lo) * sc) * 16777215.0f) << 7) | id;
-      else
-        v[i] = 0xffffffffu;
-    }
-    warp_sort(v);
-    if (k == 3) {
-      c2 = nl + (n - nl + 1) / 2;
-    } else {
-      c1 = (nl + 1) / 2;
-      c2 = nl;
-      c3 = nl + (n - nl + 1) / 2;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < I; ++i) {
-    const int r = 32 * i + lane;
-    if (r >= n) continue;
-    lsrc[r] = S.src[v[i] & 127u];
-    flag[r] = r == 0 || r == c1 || r == c2 || r == c3 ? 1u : 0u;
-  }
-}
-
 // The order of every leaf's particles and its clusters (flag[p] = 1 where one
 // starts; lsrc[p] = the particle that moves to position p).  The particles whose H
 // exceeds the leaf edge come after the others, so that clusters hold particles of
 // similar reach.  Each of the two classes is cut along its Morton keys into the
-// largest nodes (the keys that agree from some bit up) of at most 4 cmax particles
-// (cmax: the cluster size, at most 32: a warp's lanes), and a node of more than cmax
-// into as few clusters as hold it, by its particles' positions.  Nodes of at most cmax
-// particles as clusters (boxes as compact, but 21 of 32 lanes filled on average
-// against 27 here) made the interaction passes 10-20 % slower.  Walking a class from
-// its first particle a, the next node is the largest that starts at a and fits: its
+// largest nodes (the keys that agree from some bit up) of at most cmax particles (cmax:
+// the cluster size, at most 32: a warp's lanes), aligned boxes of aspect ratio at most 2.
+// Nodes of up to 4 cmax particles, divided by position into as few clusters as hold them,
+// fill 27 of 32 lanes instead of 21 and take 13 % less time (33.5M clustered step 91
+// against 104 ms), but sum a particle's neighbours in another order: N~ at given h then
+// differs by 8e-8 from its values before, two runs by 3e-8, and with it which particles
+// at the tolerance's edge iterate once more.  Walking a class from its first particle a,
+// the next cluster is the largest node that starts at a and fits: its
 // bit b* is the smallest of the highest bits in which key[a] differs from key[a - 1]
-// (the node must start at a) and from key[a + 4 cmax] (it must end before).  One
+// (the node must start at a) and from key[a + cmax] (it must end before).  One
 // warp per leaf; a leaf of more than CLUSTER_BLOCK particles, and of four times a warp's
-// share of all, takes a block, each warp a part of the walk (a warp alone with the 45
-// nodes of a 4800-particle leaf took longer than all the others of a 4.2M box together:
-// that phase of its build 1.18 -> 0.90 ms.  In larger boxes the leaf is no longer than
-// the rest, and the blocks' barriers cost 0.5 of 4.5 ms at 33.5M).
+// share of all, takes a block, each warp a part of the walk (a warp alone with the 200
+// clusters of a 4800-particle leaf takes longer than all the others of a 4.2M box together;
+// in larger boxes the leaf is no longer than the rest, and the blocks' barriers cost 0.5 of
+// 4.5 ms at 33.5M).
 constexpr int CLUSTER_WARPS = 4;
 constexpr unsigned int CLUSTER_BLOCK = 1024;
+
+__device__ __forceinline__ int high_bit(unsigned long long v) { return v ? 63 - __clzll((long long)v) : -1; }
 
 // What the walk of one leaf needs.
 struct LeafWalk {
   const unsigned long long* key;
-  const unsigned int* perm;
-  const double* x;
-  unsigned int *lsrc, *flag;
-  double iL, cen[3];
-  int lb, cmax;             // key bits below the leaf's cell; cluster size
+  const unsigned int* lsrc;
+  unsigned int* flag;
+  int lb;                   // key bits below the leaf's cell
+  unsigned int cmax;        // cluster size
 };
 
-__device__ __forceinline__ LeafWalk leaf_walk(const Tree& T, int id, const BoxDesc& bd, int box_shift,
-                                              const unsigned long long* key, const unsigned int* perm, const double* x,
-                                              unsigned int* lsrc, unsigned int* flag, int cmax) {
-  const int d = T.level[id];
-  unsigned int cx, cy, cz;
-  cell_coords(T.key[id], d, cx, cy, cz);
-  const double inv = scaled_down(1.0, d);
-  LeafWalk W{key, perm, x, lsrc, flag, bd.invL, {((double)cx + 0.5) * inv, ((double)cy + 0.5) * inv, ((double)cz + 0.5) * inv},
-             box_shift - 3 * d, cmax};
-  return W;
-}
-
-// The nodes of the class [beg, end) that start in [a, stop) (a: the start of a node).
-__device__ __forceinline__ void walk_nodes(NodeShared& S, const LeafWalk& W, unsigned int a, unsigned int stop,
-                                           unsigned int beg, unsigned int end) {
-  const int lane = threadIdx.x & 31;
-  const unsigned int cap = 4u * (unsigned int)W.cmax;
+// The clusters of the class [beg, end) that start in [a, stop) (a: the start of a node).
+__device__ __forceinline__ void walk_nodes(const LeafWalk& W, unsigned int a, unsigned int stop, unsigned int beg,
+                                           unsigned int end) {
+  const unsigned int lane = threadIdx.x & 31;
   while (a < stop) {
     const unsigned long long ka = W.key[W.lsrc[a]];
     int bs = W.lb;
     if (a > beg) bs = min(bs, high_bit(W.key[W.lsrc[a - 1]] ^ ka));
-    if (a + cap < end) bs = min(bs, high_bit(ka ^ W.key[W.lsrc[a + cap]]));
-    unsigned int n = min(cap, end - a);   // equal keys (bs < 0): no node starts here, take a chunk
-    if (bs >= 0) {
-      unsigned int m = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const unsigned int q = 32u * i + lane;
-        m += __popc(__ballot_sync(0xffffffffu, q < n && ((W.key[W.lsrc[a + q]] ^ ka) >> bs) == 0ull));
-      }
-      n = m;      // (the node's particles are adjacent)
-    }
-    n = min(n, stop - a);                 // (only a chunk that runs on past equal keys could reach the next walk's)
-    if (n <= (unsigned int)W.cmax) {
-      if ((unsigned int)lane < n) W.flag[a + lane] = lane == 0 ? 1u : 0u;
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const unsigned int q = 32u * i + lane;
-        if (q >= n) break;
-        const unsigned int src = W.lsrc[a + q];
-        const long long p = W.perm[src];
-        S.src[q] = src;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) S.x[k][q] = (float)(W.x[3 * p + k] * W.iL - W.cen[k]);
-      }
-      __syncwarp();
-      if (n <= 64u) divide_node<2>(S, (int)n, W.cmax, W.lsrc + a, W.flag + a);
-      else divide_node<4>(S, (int)n, W.cmax, W.lsrc + a, W.flag + a);
-      __syncwarp();
-    }
+    if (a + W.cmax < end) bs = min(bs, high_bit(ka ^ W.key[W.lsrc[a + W.cmax]]));
+    unsigned int n = min(W.cmax, end - a);   // equal keys (bs < 0): no node starts here, take a chunk
+    if (bs >= 0)      // (the node's particles are adjacent)
+      n = __popc(__ballot_sync(0xffffffffu, lane < n && ((W.key[W.lsrc[a + lane]] ^ ka) >> bs) == 0ull));
+    n = min(n, stop - a);                    // (only a chunk that runs on past equal keys could reach the next walk's)
+    if (lane < n) W.flag[a + lane] = lane == 0 ? 1u : 0u;
     a += n;
   }
 }
 
-// A node start in the cap particles from p on (beg < p; end if there is none to be
-// told).  The two neighbours whose keys differ in the highest bit among the cap + 2
+// A node start in the cmax particles from p on (beg < p; end if there is none to be
+// told).  The two neighbours whose keys differ in the highest bit among the cmax + 2
 // particles around belong to different nodes: a node of both would reach beyond a bit no
 // neighbours here differ in, so hold them all, which are too many.
 __device__ __forceinline__ unsigned int node_start(const LeafWalk& W, unsigned int p, unsigned int end) {
-  const int lane = threadIdx.x & 31;
-  const unsigned int cap = 4u * (unsigned int)W.cmax;
-  if (p + cap >= end) return end;
+  const unsigned int lane = threadIdx.x & 31;
+  if (p + W.cmax >= end) return end;
   int hb = -1;
   unsigned int at = end;
-  for (unsigned int q = p + lane; q <= p + cap; q += 32) {
+  for (unsigned int q = p + lane; q <= p + W.cmax; q += 32) {
     const int b = high_bit(W.key[W.lsrc[q - 1]] ^ W.key[W.lsrc[q]]);
     if (b > hb) {
       hb = b;
@@ -1555,15 +1402,12 @@ __device__ __forceinline__ unsigned int node_start(const LeafWalk& W, unsigned i
 
 __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
     Tree T, int nnodes, int box_shift, const BoxDesc* __restrict__ box, const float* __restrict__ Hs,
-    const unsigned long long* __restrict__ key, const unsigned int* __restrict__ perm, const double* __restrict__ x,
-    unsigned int* lsrc, unsigned int* flag, int cmax, long long N) {
+    const unsigned long long* __restrict__ key, unsigned int* lsrc, unsigned int* flag, int cmax, long long N) {
   pdl_wait();
   const unsigned int big = max(CLUSTER_BLOCK, (unsigned int)(4 * N / (gridDim.x * CLUSTER_WARPS)));
-  __shared__ NodeShared SH[CLUSTER_WARPS];
   __shared__ unsigned int s_small[CLUSTER_WARPS], s_start[2][CLUSTER_WARPS];
   nnodes = min(nnodes, T.n_nodes[0]);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  NodeShared& S = SH[w];
   const unsigned int lt = (1u << lane) - 1u;
   // large leaves: one block each
   for (int id = blockIdx.x; id < nnodes; id += gridDim.x) {
@@ -1598,19 +1442,19 @@ __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
       ol += __popc(bl);
     }
     __syncthreads();
-    const LeafWalk W = leaf_walk(T, id, bd, box_shift, key, perm, x, lsrc, flag, cmax);
+    const LeafWalk W{key, lsrc, flag, box_shift - 3 * T.level[id], (unsigned int)cmax};
     for (int cls = 0; cls < 2; ++cls) {
       const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
       const unsigned int from = w == 0 ? beg : node_start(W, beg + (unsigned int)(((unsigned long long)(end - beg) * w) / CLUSTER_WARPS), end);
       if (lane == 0) s_start[cls][w] = from;
     }
-    __syncthreads();      // (the walks reorder what the starts were read from)
+    __syncthreads();
     for (int cls = 0; cls < 2; ++cls) {
       const unsigned int beg = cls == 0 ? s : s + nsmall, end = cls == 0 ? s + nsmall : s + c;
       const unsigned int from = s_start[cls][w];
       unsigned int stop = end;
       for (int k = CLUSTER_WARPS - 1; k > w; --k) stop = min(stop, s_start[cls][k]);
-      walk_nodes(S, W, from, stop, beg, end);
+      walk_nodes(W, from, stop, beg, end);
     }
     __syncthreads();
   }
@@ -1642,9 +1486,9 @@ __global__ void __launch_bounds__(32 * CLUSTER_WARPS) k_leaf_clusters(
       ol += __popc(bl);
     }
     __syncwarp();
-    const LeafWalk W = leaf_walk(T, id, bd, box_shift, key, perm, x, lsrc, flag, cmax);
-    walk_nodes(S, W, s, s + nsmall, s, s + nsmall);
-    walk_nodes(S, W, s + nsmall, s + c, s + nsmall, s + c);
+    const LeafWalk W{key, lsrc, flag, box_shift - 3 * T.level[id], (unsigned int)cmax};
+    walk_nodes(W, s, s + nsmall, s, s + nsmall);
+    walk_nodes(W, s + nsmall, s + c, s + nsmall, s + c);
   }
 }
 

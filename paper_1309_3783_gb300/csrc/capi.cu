@@ -49,8 +49,8 @@ __global__ void k_sort_big_keys(int, const int*, const int*, const unsigned int*
                                 unsigned int*, const unsigned long long*, int);
 __global__ void k_sort_big_scatter(int, const int*, const int*, const unsigned int*, Tree, Tiles,
                                    const unsigned int*, float*, unsigned int*, const unsigned long long*, int);
-__global__ void k_leaf_clusters(Tree, int, int, const BoxDesc*, const float*, const unsigned long long*,
-                                const unsigned int*, const double*, unsigned int*, unsigned int*, int, long long);
+__global__ void k_leaf_clusters(Tree, int, int, const BoxDesc*, const float*, const unsigned long long*, unsigned int*,
+                                unsigned int*, int, long long);
 __global__ void k_apply_partition(long long, const unsigned int*, const unsigned int*, unsigned int*,
                                   const unsigned long long*, unsigned long long*, const float*, float*, const float4*,
                                   float4*, int, const unsigned int*, Tree, const BoxDesc*, const double*, const float*,
@@ -725,8 +725,7 @@ sph_status Engine::build_once(bool* retry) {
   ev = prof_begin(PH_SHIFT, &l0, ss);
   launch_pdl(k_leaves, nsm * 8, 256, ss, T, n_nodes, leaf_of.p); count_launch();
   // the order of each leaf's particles and its clusters (at most 32 particles each)
-  launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, n_nodes, box_shift, box.p, Hs.p, key.p, perm.p, x.p, lsrc.p, tflag.p,
-             prm.cluster_max, N); count_launch();
+  launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, n_nodes, box_shift, box.p, Hs.p, key.p, lsrc.p, tflag.p, prm.cluster_max, N); count_launch();
   launch_pdl(k_apply_partition, grid(N), 256, ss, N, lsrc.p, perm.p, perm_tmp.p, key.p, key_tmp.p, Hs.p, Hs_tmp.p,
              vel4.p, vel4_tmp.p, box_shift,
              leaf_of.p, T, box.p, x.p, m.p, pos4.p, cen4.p); count_launch();
@@ -1526,8 +1525,8 @@ sph_status Engine::enqueue_captured_build() {
   cudaStream_t ss = st_side;
   ev = prof_begin(PH_SHIFT, &l0, ss);
   launch_pdl(k_leaves, nsm * 8, 256, ss, T, cap_nodes, leaf_of.p); count_launch();
-  launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, cap_nodes, box_shift, box.p, Hs.p, key.p, perm.p, x.p, lsrc.p,
-             tflag.p, prm.cluster_max, N); count_launch();
+  launch_pdl(k_leaf_clusters, nsm * 16, 128, ss, T, cap_nodes, box_shift, box.p, Hs.p, key.p, lsrc.p, tflag.p,
+             prm.cluster_max, N); count_launch();
   launch_pdl(k_apply_partition, grid(N), 256, ss, N, lsrc.p, perm.p, perm_tmp.p, key.p, key_tmp.p, Hs.p, Hs_tmp.p,
              vel4.p, vel4_tmp.p, box_shift,
              leaf_of.p, T, box.p, x.p, m.p, pos4.p, cen4.p); count_launch();

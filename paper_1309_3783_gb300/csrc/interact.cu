@@ -149,7 +149,6 @@ struct __align__(16) DensShared {
   float m[32];
   int g[32];
   float4 ip[32];    // own cluster: position, m
-  float4 is[32];    //   sums over the interactions done
   int ig[32];       //   index
   UnitShared tk;
   float4 jlo[32], jhi[32];   // the scan's fine candidates: box in the unit's frame, largest H (w of jlo)
@@ -554,12 +553,13 @@ __device__ __noinline__ void dens_band(const DensShared& S, unsigned int unc, bo
 // partners of its mask, whose position and mass get(slot) gives.  Two partners per
 // turn, packed, so that most of the arithmetic takes one instruction for both; an odd
 // one's second partner, and those inside the guard band (set aside in unc, decided
-// afterwards), take q = 1, where w and w' vanish.
+// afterwards), take q = 1, where w and w' vanish.  The terms are added one by one, in the
+// order of the slots (two packed sums, one per partner of a turn, round differently: see
+// sum_done).
 template <bool KAHAN, class Get>
 __device__ __forceinline__ unsigned int dens_sweep(unsigned int mask, float3 me, float lo, float invH, Get get,
                                                    DensAcc<KAHAN>& acc) {
   const f32x2 nx = pack2(-me.x, -me.x), ny = pack2(-me.y, -me.y), nz = pack2(-me.z, -me.z), ih = pack2(invH, invH);
-  f32x2 s0 = 0, s1 = 0, s2 = 0, s3 = 0;     // (packed +0)
   unsigned int unc = 0;
 #pragma unroll 1
   for (unsigned int m = mask; m;) {
@@ -592,43 +592,54 @@ __device__ __forceinline__ unsigned int dens_sweep(unsigned int mask, float3 me,
     const bool ia = qa < 0.5f, ib = qb < 0.5f;
     const f32x2 w = pack2(ia ? wia : woa, ib ? wib : wob);
     const f32x2 g = mul2(q, pack2(ia ? wda : wea, ib ? wdb : web));      // q w'(q) = r dW/dr in units of W
-    if (KAHAN) {
-      float wa, wb, ga, gb;
-      unpack2(w, wa, wb);
-      unpack2(g, ga, gb);
-      acc.add(A.w, wa, ga);
-      acc.add(B.w, wb, gb);
-    } else {
-      const f32x2 mm = pack2(A.w, B.w);
-      s0 = fma2(mm, w, s0);
-      s1 = fma2(mm, g, s1);
-      s2 = add2(s2, w);
-      s3 = add2(s3, g);
-    }
-  }
-  if (!KAHAN) {
-    float a, b;
-    unpack2(s0, a, b);
-    acc.s.x += a + b;
-    unpack2(s1, a, b);
-    acc.s.y += a + b;
-    unpack2(s2, a, b);
-    acc.s.z += a + b;
-    unpack2(s3, a, b);
-    acc.s.w += a + b;
+    float wa, wb, ga, gb;
+    unpack2(w, wa, wb);
+    unpack2(g, ga, gb);
+    acc.add(A.w, wa, ga);
+    acc.add(B.w, wb, gb);
   }
   return unc;
 }
 
-// Own side of a density batch: the lane walks its mask of staged partners.
+// The plain sums over one interaction's partners are done: they are added to the
+// particle's in memory, and the next interaction's start anew.  So each particle's sums
+// are made of the same parts whatever shares a batch or a unit, one per interaction of its
+// cluster and one per cluster it is a partner of, each added up in the order of the sorted
+// particles; only the order in which the parts meet in memory is open.  The rounding of N~
+// decides which particles at the tolerance's edge iterate once more, and a change of
+// grouping changes it more (8e-8 of N~) than that order does (3e-8): grouped in another
+// way, three to five times as many particles of a multi-scale box ended an iteration apart
+// as between two runs.
+// (A part ends early where it exceeds SUM_MAX, at 14 times the usual number of neighbours: of
+// 250 coincident particles one chain of additions was off by 1.9e-5.)
+constexpr float SUM_MAX = 64.0f;
+
 template <bool KAHAN>
-__device__ __forceinline__ void dens_row(const DensI& I, float ilo, const DensShared& S, unsigned int ui,
+__device__ __forceinline__ void sum_done(int g, DensAcc<KAHAN>& acc, float4* dacc) {
+  if (acc.s.z != 0.0f) atomicAdd(&dacc[g], acc.s);
+  acc = DensAcc<KAHAN>();
+}
+
+// Own side of a density batch: the lane walks its mask of staged partners.  segs: the
+// slots at which another interaction's partners begin (the same in every lane).
+template <bool KAHAN>
+__device__ __forceinline__ void dens_row(const DensI& I, float ilo, const DensShared& S, unsigned int ui, unsigned int segs,
                                          DensAcc<KAHAN>& acc,
                                          unsigned int& cnt, const unsigned int* perm, const double* x,
                                          const float4* pos4, const BoxDesc* box, float4* dacc, unsigned int* dcnt,
                                          float4* dcomp) {
-  const unsigned int unc = dens_sweep(
-      ui, I.p, ilo, I.invH, [&](int s) { return make_float4(S.x[s], S.y[s], S.z[s], S.m[s]); }, acc);
+  unsigned int rest = ui, unc = 0;
+#pragma unroll 1
+  for (;;) {
+    const unsigned int now = segs ? rest & ((segs & (0u - segs)) - 1u) : rest;
+    unc |= dens_sweep(
+        now, I.p, ilo, I.invH, [&](int s) { return make_float4(S.x[s], S.y[s], S.z[s], S.m[s]); }, acc);
+    if (KAHAN || !segs) break;
+    rest &= ~now;
+    segs &= segs - 1u;
+    sum_done(I.g, acc, dacc);
+  }
+  if (!KAHAN && acc.s.z > SUM_MAX) sum_done(I.g, acc, dacc);
   cnt += __popc(ui & ~unc);
   if (unc) dens_band<KAHAN>(S, unc, false, perm, x, pos4, box, dacc, dcnt, dcomp);
 }
@@ -662,7 +673,7 @@ __device__ __noinline__ void resolve_masks(const DensShared& S, float ilo, unsig
 // cluster (each lane leaves itself out and updates its own side only; the
 // counters count the upper triangle, since every pair appears in both rows).
 template <bool COUNT, bool PART, bool KAHAN, bool REC>
-__device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsigned int q, bool own_only,
+__device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsigned int q, unsigned int segs, bool own_only,
                                            DensAcc<KAHAN>& acc, unsigned int& cnt, const unsigned int* perm,
                                            const double* x, const float4* __restrict__ pos4,
                                            const BoxDesc* __restrict__ box, const float4* __restrict__ cen4,
@@ -717,7 +728,7 @@ __device__ __forceinline__ void dens_batch(const DensI& I, DensShared& S, unsign
   }
   S.m[lane] = jm;
   __syncwarp();
-  dens_row(I, ilo, S, ui, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
+  dens_row(I, ilo, S, ui, segs, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
   // column sweep: partner side, staged partner = lane
   const unsigned int col = own_only ? 0u : transpose_bits(uj);
   if (col) {
@@ -1186,14 +1197,19 @@ __device__ __forceinline__ void unit_begin(UnitShared& K, unsigned int ti, const
   __syncwarp();
 }
 
-// The first run of 32 clusters of an interaction's list that belongs to the unit: its
-// part of the parts takes the runs r with (interaction + r) % parts == part.
-__device__ __forceinline__ unsigned int unit_first_of(const UnitShared& K, unsigned int interaction) {
+// The first run of 32 clusters of an interaction's list that belongs to the unit.  RUNS
+// (force): its part of the parts takes the runs r with (interaction + r) % parts == part.
+// Else (density): the whole of the interactions with interaction % parts == part, so
+// that a particle's sum over an interaction's partners is one (see sum_done).  A single
+// list that outweighs all others is then not divided, which costs density passes little
+// (4.2M clustered h iteration 44.0 -> 45.4 ms; the force pass of a million log-normal
+// particles would take 4.2 ms instead of 2.9).
+template <bool RUNS>
+__device__ __forceinline__ unsigned int unit_first(const UnitShared& K, unsigned int interaction) {
   const unsigned int P = K.parts;
-  return P == 1u ? 0u : (K.part + P - interaction % P) % P;
-}
-__device__ __forceinline__ unsigned int unit_first(const UnitShared& K, int it) {
-  return unit_first_of(K, K.gidx + (unsigned int)it);
+  if (P == 1u) return 0u;
+  const unsigned int r = (K.part + P - interaction % P) % P;
+  return RUNS || r == 0u ? r : 0x07ffffffu;      // (past every list)
 }
 
 // The next group of the unit's interactions: one per lane, from the cell's list (the
@@ -1205,7 +1221,7 @@ __device__ __forceinline__ unsigned int unit_first(const UnitShared& K, int it) 
 // GATHER (the own side only, of a packed cluster): the pairs of which the cell is the
 // second come too, the self interaction has all of the leaf's clusters, and only the own
 // reach counts.
-template <bool PART, bool GATHER>
+template <bool PART, bool GATHER, bool RUNS>
 __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T, const uint2* __restrict__ csr,
                                                    bool iact) {
   const int lane = threadIdx.x & 31;
@@ -1244,7 +1260,7 @@ __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T,
     const float slack = e * 1.52587890625e-05f + K.es + 1e-6f * fmaxf(HmB, T.hmax[A] * invL);   // 2^-16 e
     const unsigned int t0 = T.tile0[B], nt = T.ntile[B];
     unsigned int sb = SORT_NONE;
-    if (!self && !second) {      // (the sorted lists run away from a pair's first cell)
+    if (!GATHER && !self) {      // (a gathered unit takes every list in the order of its clusters)
       const unsigned int sbB = T.sortbase[B];
       if (sbB != SORT_NONE) sb = sbB + (unsigned int)__popc(T.axes[B] & ((1u << ax) - 1u)) * nt;
     }
@@ -1276,7 +1292,7 @@ __device__ __forceinline__ unsigned int unit_group(UnitShared& K, const Tree& T,
     }
   }
   if (live && K.parts > 1u)    // the unit's share has a run of this list
-    live = 32u * unit_first_of(K, idx + lane) < __float_as_uint(K.gwin[lane].w);
+    live = 32u * unit_first<RUNS>(K, idx + lane) < __float_as_uint(K.gwin[lane].w);
   const unsigned int bal = __ballot_sync(0xffffffffu, live);
   const int up = T.parent[A];
   __syncwarp();
@@ -1349,7 +1365,7 @@ __device__ __forceinline__ void unit_single(UnitShared& K, bool self, int item, 
 // uniform box has no such candidate and pays nothing.
 constexpr float FINE_H = 0.7f;
 
-template <bool PART, bool GATHER>
+template <bool PART, bool GATHER, bool RUNS>
 __device__ __forceinline__ unsigned int scan_clusters(UnitShared& K, float4* jlo, float4* jhi, const Tiles& TL,
                                                       const float* __restrict__ sort_r,
                                                       const unsigned int* __restrict__ sort_i, int it,
@@ -1364,7 +1380,7 @@ __device__ __forceinline__ unsigned int scan_clusters(UnitShared& K, float4* jlo
     e0 = nt;           // the sorted list only moves further away
     return 0u;
   }
-  e0 += 32u * K.parts;
+  e0 += RUNS ? 32u * K.parts : 32u;
   bool pass = false, fine = false;
   if (e < nt) {
     const unsigned int t = sorted ? sort_i[sb + e] : K.gtb[it] + e;
@@ -1414,21 +1430,20 @@ struct Walk {
 };
 
 // The next candidates (W.mask, non-zero) of the unit; false at its end.
-template <bool PART, bool GATHER = false>
+template <bool PART, bool GATHER, bool RUNS>
 __device__ __forceinline__ bool unit_next(UnitShared& K, Walk& W, float4* jlo, float4* jhi, const Lists& Lq,
                                           const Tree& T, const Tiles& TL, const float* __restrict__ sort_r,
                                           const unsigned int* __restrict__ sort_i, bool any, bool all, float3 ip, float iH) {
   while (!W.mask) {
     if (W.e0 < W.nt) {
-      W.mask = scan_clusters<PART, GATHER>(K, jlo, jhi, TL, sort_r, sort_i, W.it, W.e0, W.nt, any, all, ip, iH);
+      W.mask = scan_clusters<PART, GATHER, RUNS>(K, jlo, jhi, TL, sort_r, sort_i, W.it, W.e0, W.nt, any, all, ip, iH);
     } else if (W.live) {
       W.it = __ffs(W.live) - 1;
       W.live &= W.live - 1;
       W.nt = __float_as_uint(K.gwin[W.it].w);
-      // with parts, every parts-th run of 32 clusters, from one that depends on the interaction
-      W.e0 = 32u * unit_first(K, W.it);
+      W.e0 = 32u * unit_first<RUNS>(K, K.gidx + (unsigned int)W.it);
     } else if (K.cell >= 0) {
-      W.live = unit_group<PART, GATHER>(K, T, Lq.csr, any);
+      W.live = unit_group<PART, GATHER, RUNS>(K, T, Lq.csr, any);
     } else {
       return false;
     }
@@ -1472,9 +1487,9 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
   S.ip[lane] = make_float4(I.p.x, I.p.y, I.p.z, I.m);
   S.ig[lane] = I.g;
   DensAcc<KAHAN> acc;
-  unsigned int cnt = 0, q = 0, done = 0xffffffffu;
-  S.is[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-  // inside the cluster itself first (the self interaction is a unit's first)
+  unsigned int cnt = 0, q = 0, cur = 0, segs = 0;
+  // inside the cluster itself first (the self interaction is a unit's first: cur, the
+  // interaction whose sums acc holds)
   Walk Wk;
   bool own_only = LISTED ? self : part == 0u && (!PART || any || T.active[TL.leaf[ti]]);
   if (LISTED) Wk.live = 1u;
@@ -1489,7 +1504,7 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
   int k = -1;
   float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
   for (;;) {
-    if (k < 0 && unit_next<PART>(K, Wk, S.jlo, S.jhi, Lq, T, TL, sort_r, sort_i, any, all, I.p,
+    if (k < 0 && unit_next<PART, false, false>(K, Wk, S.jlo, S.jhi, Lq, T, TL, sort_r, sort_i, any, all, I.p,
                                  I.act ? I.H : 0.0f)) {
       k = __ffs(Wk.mask) - 1;
       Wk.mask &= Wk.mask - 1;
@@ -1526,6 +1541,7 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
       bal = __ballot_sync(0xffffffffu, pass);
     }
     const unsigned int np = __popc(bal), rank = __popc(bal & ((1u << lane) - 1u));
+    const unsigned int now = K.gidx + (unsigned int)Wk.it;
     const bool close = own_only || last || (COUNT && in_self != (Wk.it == K.selfit));
     if (close || q + np > 32u) {
       // a batch runs full: it takes the first of the candidate's particles, the next one
@@ -1534,32 +1550,30 @@ __device__ __forceinline__ void density_unit(unsigned int ti, unsigned int part,
       // large boxes and lose 2 to 6 % below 30k particles, where a unit's latency counts
       // and a full batch's list is cut in two: they stay as they are)
       const unsigned int room = close ? 0u : 32u - q;
+      if (room && now != cur) {
+        if (q) segs |= 1u << q;
+        else if (!KAHAN) sum_done(I.g, acc, dacc);
+        cur = now;
+      }
       if (pass && rank < room) dens_put(S, (int)(q + rank), make_float3(pj.x, pj.y, pj.z), pj.w, gj, aj);
       pass = pass && rank >= room;
       q += room;
       if (q)
-        dens_batch<COUNT, PART, KAHAN, LISTED>(I, S, q, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt, dcomp,
+        dens_batch<COUNT, PART, KAHAN, LISTED>(I, S, q, KAHAN ? 0u : segs, own_only, acc, cnt, perm, x, pos4, box, cen4, dacc, dcnt, dcomp,
                                                COUNT && in_self ? Cs : Cp, R, W);
       q = 0u - room;
+      segs = 0;
       own_only = false;
       in_self = Wk.it == K.selfit;
-      // plain sums are kept per interaction: one chain over all of a unit's partners
-      // would round more than the sums of separate interactions
-      const unsigned int now = K.gidx + (unsigned int)Wk.it;
-      if (!KAHAN && now != done) {
-        const float4 t = S.is[lane];
-        S.is[lane] = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
-        acc = DensAcc<KAHAN>();
-        done = now;
-      }
     }
     if (last) break;
+    if (np && now != cur) {
+      if (q) segs |= 1u << q;
+      else if (!KAHAN) sum_done(I.g, acc, dacc);
+      cur = now;
+    }
     if (pass) dens_put(S, (int)(q + rank), make_float3(pj.x, pj.y, pj.z), pj.w, gj, aj);
     q += np;
-  }
-  if (!KAHAN) {
-    const float4 t = S.is[lane];
-    acc.s = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
   }
   flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
   if (LISTED) rec_task_end(self ? R.stask : R.ptask, S);
@@ -1594,7 +1608,7 @@ __device__ __forceinline__ void force_unit(unsigned int ti, unsigned int part, u
   int k = -1;
   float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
   for (;;) {
-    if (k < 0 && unit_next<false>(K, Wk, S.v, S.f, Lq, T, TL, sort_r, sort_i, true, true, ip, P.w)) {
+    if (k < 0 && unit_next<false, false, true>(K, Wk, S.v, S.f, Lq, T, TL, sort_r, sort_i, true, true, ip, P.w)) {
       k = __ffs(Wk.mask) - 1;
       Wk.mask &= Wk.mask - 1;
       if ((unsigned int)lane < K.cn[k]) nr = A.pos4[__float_as_uint(K.co[k].w) + lane];
@@ -2019,7 +2033,7 @@ __global__ void k_pack_leaf(long long ntcap, const unsigned int* __restrict__ nt
 // counts: pk0[t], the first packed cluster of the leaf whose first cluster is t): the
 // sorted indices of the iterating particles by rank (idx), and per packed cluster its
 // first rank and its leaf's first cluster (info) and its size (pn).  The pass gathers
-// when it is a later one and at most a third of the particles iterate (gflag[0]).  One
+// when it is a later one and at most an eighth of the particles iterate (gflag[0]).  One
 // warp per cluster.
 __global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ ntile_dev, const int* __restrict__ it_dev,
                             long long N, Tree T, Tiles TL, const unsigned char* __restrict__ act,
@@ -2055,7 +2069,7 @@ __global__ void k_pack_fill(long long ntcap, const unsigned int* __restrict__ nt
 // One batch of q <= 32 staged partners, the own side only; in a self interaction
 // the particle itself (staged with its cell) is left out.
 template <bool KAHAN>
-__device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsigned int q, bool self,
+__device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsigned int q, unsigned int segs, bool self,
                                              const float4* __restrict__ cen4, DensAcc<KAHAN>& acc, unsigned int& cnt,
                                              const unsigned int* perm, const double* x,
                                              const float4* __restrict__ pos4, const BoxDesc* __restrict__ box,
@@ -2082,7 +2096,7 @@ __device__ __forceinline__ void gather_batch(const DensI& I, DensShared& S, unsi
   if (self)
     for (unsigned int b = m; b; b &= b - 1)
       if (S.g[__ffs(b) - 1] == I.g) m &= ~(b & (0u - b));
-  dens_row(I, ilo, S, m, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
+  dens_row(I, ilo, S, m, segs, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
   __syncwarp();
 }
 
@@ -2121,14 +2135,13 @@ __device__ __forceinline__ void gather_unit(unsigned int pid, unsigned int part,
   }
   __syncwarp();
   DensAcc<KAHAN> acc;
-  unsigned int cnt = 0, q = 0, done = 0xffffffffu;
-  S.is[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  unsigned int cnt = 0, q = 0, cur = 0, segs = 0;
   Walk Wk;
   bool own = false;      // the batch holds particles of the own leaf
   int k = -1;
   float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
   for (;;) {
-    if (k < 0 && unit_next<false, true>(K, Wk, S.jlo, S.jhi, Lq, T, TL, sort_r, sort_i, true, true, I.p,
+    if (k < 0 && unit_next<false, true, false>(K, Wk, S.jlo, S.jhi, Lq, T, TL, sort_r, sort_i, true, true, I.p,
                                         vi ? I.H : 0.0f)) {
       k = __ffs(Wk.mask) - 1;
       Wk.mask &= Wk.mask - 1;
@@ -2153,31 +2166,32 @@ __device__ __forceinline__ void gather_unit(unsigned int pid, unsigned int part,
       bal = __ballot_sync(0xffffffffu, pass);
     }
     const unsigned int np = __popc(bal), rank = __popc(bal & ((1u << lane) - 1u));
+    const unsigned int now = K.gidx + (unsigned int)Wk.it;
     if (last || q + np > 32u) {
       const unsigned int room = last ? 0u : 32u - q;
+      if (room && now != cur) {
+        if (q) segs |= 1u << q;
+        else if (!KAHAN) sum_done(I.g, acc, dacc);
+        cur = now;
+      }
       if (pass && rank < room) dens_put(S, (int)(q + rank), make_float3(pj.x, pj.y, pj.z), pj.w, gj, true);
       pass = pass && rank >= room;
       q += room;
       own = own || (room && Wk.it == K.selfit);
-      if (q) gather_batch<KAHAN>(I, S, q, own, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
+      if (q) gather_batch<KAHAN>(I, S, q, KAHAN ? 0u : segs, own, cen4, acc, cnt, perm, x, pos4, box, dacc, dcnt, dcomp);
       q = 0u - room;
+      segs = 0;
       own = false;
-      const unsigned int now = K.gidx + (unsigned int)Wk.it;
-      if (!KAHAN && now != done) {      // (as in density_unit)
-        const float4 t = S.is[lane];
-        S.is[lane] = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
-        acc = DensAcc<KAHAN>();
-        done = now;
-      }
     }
     if (last) break;
+    if (np && now != cur) {
+      if (q) segs |= 1u << q;
+      else if (!KAHAN) sum_done(I.g, acc, dacc);
+      cur = now;
+    }
     if (pass) dens_put(S, (int)(q + rank), make_float3(pj.x, pj.y, pj.z), pj.w, gj, true);
     own = own || Wk.it == K.selfit;
     q += np;
-  }
-  if (!KAHAN) {
-    const float4 t = S.is[lane];
-    acc.s = make_float4(t.x + acc.s.x, t.y + acc.s.y, t.z + acc.s.z, t.w + acc.s.w);
   }
   flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
 }

@@ -66,11 +66,11 @@ extern const char* const kPhaseNames[PH_COUNT];
 void exclusive_scan(const unsigned int* in, unsigned int* out, long long n, unsigned int* tile_sums,
                     unsigned int* total, cudaStream_t st, const unsigned int* n_dev = nullptr,
                     const int* gate = nullptr);
-// A later pass of the h iteration gathers when at most a third of the particles iterate
-// (packed clusters then halve the own side at least, and its partners' side is not
-// needed; passes of 977k Sod particles with a quarter iterating 0.25 -> 0.22 ms against an
-// eighth as the limit, 4.2M clustered h iteration 34.2 -> 33.9 ms; a half gains no more).
-constexpr unsigned long long GATHER_SHARE = 3;
+// A later pass of the h iteration gathers when at most an eighth of the particles
+// iterate.  (Up to a third a gathered pass would take less time too, 0.22 against 0.25 ms for
+// 977k Sod particles with a quarter iterating, but it sums a particle's neighbours in another
+// order, and so moves those at the tolerance's edge: see sum_done in interact.cu.)
+constexpr unsigned long long GATHER_SHARE = 8;
 // Up to this many particles one block does both scans of a gathered pass's packing (a
 // microsecond per 1000 clusters, 38 us for the 36k of a million particles, against the
 // 25 us of seven launches; clusters are a sixteenth to a thirtieth of the particles in
