@@ -1538,9 +1538,10 @@ __global__ void k_cluster_table(long long N, const unsigned int* __restrict__ nt
   nnodes = min(nnodes, T.n_nodes[0]);
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nnodes; id += gridDim.x * blockDim.x) {
     const unsigned int s = T.start[id], c = T.count[id];
-    const unsigned int t0 = tile_of[s];
+    // (an empty node: see alloc_nodes; a captured build gets here before its check)
+    const unsigned int t0 = c ? tile_of[s] : 0u;
     T.tile0[id] = t0;
-    T.ntile[id] = tile_of[s + c - 1] - t0 + 1u;
+    T.ntile[id] = c ? tile_of[s + c - 1] - t0 + 1u : 0u;
   }
   const int lane = threadIdx.x & 31;
   const unsigned int warp = (unsigned int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
