@@ -417,9 +417,10 @@ typedef struct sph_server sph_server;
 
 /* A server keeps many boxes resident on the device and advances all admitted
  * boxes by one step per tick with one batched pipeline (one launch per kernel
- * for all boxes).  Boxes are admitted while their device footprint fits in
- * budget_bytes (0 = 80 % of free device memory) and at most max_boxes are
- * resident; the rest wait in submission order. */
+ * for all boxes).  Boxes are admitted while their device footprint, taken as 520
+ * bytes per particle (560 to 635 are held), fits in budget_bytes (0 = 80 % of free
+ * device memory) and at most max_boxes are resident; the rest wait in submission
+ * order. */
 sph_status sph_server_create(sph_ctx* ctx, int64_t budget_bytes, int32_t max_boxes, sph_server** out);
 
 /* Queue a box of n particles (host arrays as in sph_box_set) to advance

@@ -242,7 +242,8 @@ sph_status Engine::fail(sph_status s, const std::string& msg) {
 }
 
 size_t Engine::footprint_bytes() const {
-  // device bytes per particle of the resident state plus the lists (estimate)
+  // device bytes per particle of the resident state plus the lists: the estimate that the
+  // server's admission uses (560 to 635 are held)
   return (size_t)N * 520 + 4096;
 }
 
@@ -488,25 +489,20 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
   if (selfs > cap_self || !l_self.p) {
     cap_self = selfs;
     CK(l_self.reserve(selfs));
-    CK(l_stoff.reserve(selfs + 1));
+    if (prm.pair_cache) CK(l_stoff.reserve(selfs + 1));
   }
   if (pairs > cap_pair || !l_pa.p) {
     cap_pair = pairs;
     CK(l_pa.reserve(pairs));
     CK(l_pb.reserve(pairs));
     CK(l_pax.reserve(pairs));
-    CK(l_ptoff.reserve(pairs + 1));
-    CK(l_csr.reserve(2 * (size_t)pairs));
+    if (prm.pair_cache) CK(l_ptoff.reserve(pairs + 1));
   }
-  CK(scan_tmp.reserve((size_t)std::max(cap_pair, cap_self) / 2048 + 64));
-  if (queue > cap_queue || !q_kind[0].p) {
+  if (prm.pair_cache) CK(scan_tmp.reserve((size_t)std::max(cap_pair, cap_self) / 2048 + 64));
+  queue = std::max(queue, cap_pair);
+  if (queue > cap_queue || !q_mem[0].p) {
     cap_queue = queue;
-    for (int k = 0; k < 2; ++k) {
-      CK(q_kind[k].reserve(queue));
-      CK(q_a[k].reserve(queue));
-      CK(q_b[k].reserve(queue));
-      CK(q_ax[k].reserve(queue));
-    }
+    for (int k = 0; k < 2; ++k) CK(q_mem[k].reserve(4 * (size_t)queue));
   }
   CK(l_counts.reserve(12));
   Lq.self_a = l_self.p;
@@ -514,13 +510,15 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
   Lq.pair_b = l_pb.p;
   Lq.pair_axis = l_pax.p;
   for (int k = 0; k < 2; ++k) {
-    Lq.q_kind[k] = q_kind[k].p;
-    Lq.q_a[k] = q_a[k].p;
-    Lq.q_b[k] = q_b[k].p;
-    Lq.q_axis[k] = q_ax[k].p;
+    Lq.q_kind[k] = q_mem[k].p;
+    Lq.q_a[k] = q_mem[k].p + (size_t)cap_queue;
+    Lq.q_b[k] = q_mem[k].p + 2 * (size_t)cap_queue;
+    Lq.q_axis[k] = q_mem[k].p + 3 * (size_t)cap_queue;
   }
   Lq.p_toff = l_ptoff.p;
-  Lq.csr = l_csr.p;
+  // the pairs by cell are written when the expansion is done, into one of its queues
+  // (two 8-byte entries a pair; 32 bytes a particle less than storage of their own)
+  Lq.csr = reinterpret_cast<uint2*>(q_mem[0].p);
   Lq.s_toff = l_stoff.p;
   Lq.counts = l_counts.p;
   return SPH_OK;

@@ -76,6 +76,10 @@ struct sph_server {
   std::string err;
 };
 
+// What admission takes a particle to need, by which callers have chosen their budgets.  (A
+// box of 262,144 and more holds 560 to 590 bytes per particle after its first passes and 610
+// to 635 once steps are captured, so a budget near the device's free memory is too large
+// by that share.)
 static const long long kBytesPerParticle = 520;
 
 static sph_status srv_fail(sph_server* s, sph_status st, const std::string& m) {

@@ -218,7 +218,6 @@ class Engine {
   // interaction lists
   int cap_self = 0, cap_pair = 0, cap_queue = 0;
   DBuf<int> l_self, l_pa, l_pb, l_pax, l_counts;
-  DBuf<uint2> l_csr;
   DBuf<unsigned int> l_ptoff, l_stoff, scan_tmp, l_ptask, l_stask, l_nlive;
   DBuf<uint2> l_plive;
   // gathered later passes of the h iteration: per cluster the particles still
@@ -232,7 +231,7 @@ class Engine {
   DBuf<int> gflag;
   long long n_ptasks = 0, n_stasks = 0;
   int partial_pass = 0;           // 1 while the density passes cover only particles still iterating h
-  DBuf<int> q_kind[2], q_a[2], q_b[2], q_ax[2];
+  DBuf<int> q_mem[2];             // the expansion queues: kind, a, b, axis one after another
   Lists Lq{};
 
   // the pairs of the first density pass of an h iteration, kept for the force pass
