@@ -128,11 +128,10 @@ typedef struct sph_params {
                              per batch, about one batch per particle (the pool
                              starts at 1.5 and grows to what a recording took;
                              tasks a full pool could not keep cull again).  The pair
-                             set is the same.  Recorded passes run a task per
-                             interaction and cluster; on GB300 the two passes
-                             together then take 1.1 to 1.8 times as long as
-                             without records; 0: the force pass culls on its
-                             own (0)                                               */
+                             set is the same.  Only passes with pair counting
+                             (sph_box_count_pairs) keep records: on GB300 the
+                             others take less time without (recorded, 1.2 to 1.7
+                             times as long); 0: the force pass culls on its own (0) */
     int32_t h_gather;     /* 1: a later pass of the h iteration (Section II-D, the
                              density loop again for the particles whose h has not
                              converged) in which at most an eighth of the

@@ -129,17 +129,16 @@ __global__ void k_check_shape(int nbox, const BoxDesc* __restrict__ box, int dc,
 
 // The end of a captured build: it held when no check failed and every count fits
 // its capacity (tree nodes, selfs, pairs, the empty last expansion queue, the
-// task tables, the global sort's segments); the IF node of the passes follows.
+// global sort's segments); the IF node of the passes follows.
 __global__ void k_check_build(cudaGraphConditionalHandle ok, const unsigned int* __restrict__ err_all,
                               const int* __restrict__ t_n, int cap_nodes, const int* __restrict__ counts, int cap_self,
-                              int cap_pair, int last_q, unsigned int cap_ptask, unsigned int cap_stask,
+                              int cap_pair, int last_q,
                               const unsigned long long* __restrict__ big_count, int cap_big,
                               unsigned int* __restrict__ status) {
   pdl_wait();
   const unsigned int bad = ERR_BAD_INPUT | ERR_H_TOO_LARGE | ERR_OVERFLOW | ERR_DEPTH | ERR_SHAPE;
   const bool held = (*err_all & bad) == 0u && t_n[0] <= cap_nodes && counts[0] <= cap_self && counts[1] <= cap_pair &&
-                    counts[last_q] == 0 && (unsigned int)counts[6] <= cap_ptask &&
-                    (unsigned int)counts[7] <= cap_stask && (long long)(*big_count >> 40) <= (long long)cap_big;
+                    counts[last_q] == 0 && (long long)(*big_count >> 40) <= (long long)cap_big;
   cudaGraphSetConditional(ok, held ? 1u : 0u);
   *status = held ? 1u : 0u;
 }

@@ -61,9 +61,9 @@ __global__ void k_cluster_table(long long, const unsigned int*, Tree, int, const
 __global__ void k_box_reset(int, BoxDesc*);
 __global__ void k_check_shape(int, const BoxDesc*, int, float, unsigned int*);
 __global__ void k_check_build(cudaGraphConditionalHandle, const unsigned int*, const int*, int, const int*, int, int, int,
-                              unsigned int, unsigned int, const unsigned long long*, int, unsigned int*);
+                              const unsigned long long*, int, unsigned int*);
 // launchers of interact.cu
-void launch_live_tasks(Engine& E, bool dens, const int* it_dev = nullptr);
+void launch_live_tasks(Engine& E);
 void launch_density(Engine& E, const int* it_dev = nullptr, int only = -1);
 void launch_gather_prep(Engine& E, const int* it_dev);
 void launch_density_gather(Engine& E);
@@ -759,7 +759,8 @@ sph_status Engine::build_once(bool* retry) {
   launch_pdl(k_sort_alloc, grid(n_nodes), 256, st, T, n_nodes, Lq, big_node.p, big_axis.p, big_off.p, big_count.p,
              cap_big, mid_seg.p, mid_count.p, 0xffffffffu, 0xffffffffu, err_all.p); count_launch();
   launch_pdl(k_pair_csr, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
-  if (prm.pair_cache) launch_task_offsets(*this);
+  const bool tasks = recording();
+  if (tasks) launch_task_offsets(*this);
   prof_end(PH_AXIS_SORT, ev, l0);
   CK(cudaGetLastError());
   CK(read_status());
@@ -794,7 +795,7 @@ sph_status Engine::build_once(bool* retry) {
   n_big_entries = bc[1];
   n_ptasks = lc[6];
   n_stasks = ntl;           // the self interactions are the leaves': one task per cluster
-  if (prm.pair_cache) {     // the passes list their tasks, for their pair records
+  if (tasks) {              // the passes list their tasks, for their pair records
     CK(l_ptask.reserve(std::max<size_t>((size_t)n_ptasks, 1)));
     CK(l_stask.reserve(std::max<size_t>((size_t)n_stasks, 1)));
     CK(l_plive.reserve(std::max<size_t>((size_t)(n_ptasks + n_stasks), 1)));
@@ -809,7 +810,8 @@ sph_status Engine::build_once(bool* retry) {
   unit_list = n_tiles >= nsm * 28 && n_tiles < (long long)nsm * 28 * 512;
   if (unit_list) CK(units.reserve((size_t)n_tiles * 2 + 65536));
   launch_unit_list(*this);
-  if (prm.pair_cache) launch_task_items(*this);
+  if (tasks) launch_task_items(*this);
+  tasks_listed = tasks;
   CK(sort_r.reserve(std::max<long long>(n_entries, 1)));
   CK(sort_i.reserve(std::max<long long>(n_entries, 1)));
   ev = prof_begin(PH_AXIS_SORT, &l0);
@@ -850,25 +852,21 @@ sph_status Engine::build_once(bool* retry) {
 // The pool holds the last recordings' need with a quarter to spare, and at least
 // 1.5 batches per particle (clustered boxes take about one).  A recording that
 // runs out keeps the tasks it completed; the others take the full force path.
-// A larger pool moves the buffers, so the captured steps are captured again.
 sph_status Engine::rec_prepare() {
-  if (!prm.pair_cache) return SPH_OK;
+  if (!recording()) return SPH_OK;
   if (rec_unread && rec_ctr.p) {
     // the last recording's need was not read back with a synchronisation of its own
     unsigned int rc = 0;
     CK(cudaMemcpyAsync(&rc, rec_ctr.p, sizeof(rc), cudaMemcpyDeviceToHost, st));
     CK(sync_stream());
-    rec_used = rc;
     rec_need = std::max<long long>(rec_need, rc);
   }
   rec_unread = false;
   long long want = std::max<long long>(rec_need + rec_need / 4, (N + N / 2) / REC_CHUNK) + 64;
   want = std::min<long long>(want, (long long)(REC_NONE / REC_CHUNK) - 1);
-  bool moved = false;
   if ((size_t)want > rec_next.n || !rec_pool.p) {
     rec_pool.release();
     rec_next.release();
-    moved = true;
     if (rec_pool.reserve((size_t)want * REC_CHUNK * 64) != cudaSuccess ||
         rec_next.reserve((size_t)want) != cudaSuccess) {
       // no room for the records: the force pass culls on its own
@@ -876,13 +874,11 @@ sph_status Engine::rec_prepare() {
       rec_pool.release();
       rec_next.release();
       R = PairRec{};
-      if (!gcap) graph_ready = bgraph_ready = false;
       return SPH_OK;
     }
   }
   CK(rec_ctr.reserve(1));
   const size_t np = std::max<size_t>(l_ptask.n, 1), ns = std::max<size_t>(l_stask.n, 1);
-  if (np > rec_pt.n || ns > rec_st.n) moved = true;
   CK(rec_pt.reserve(np));
   CK(rec_st.reserve(ns));
   R.pool = rec_pool.p;
@@ -891,18 +887,13 @@ sph_status Engine::rec_prepare() {
   R.ptask = rec_pt.p;
   R.stask = rec_st.p;
   R.cap = (unsigned int)(rec_next.n);
-  if (moved && !gcap) {
-    graph_ready = false;
-    bgraph_ready = false;
-  }
   return SPH_OK;
 }
 
 void Engine::rec_enqueue_reset() {
   rec_valid = false;
-  if (!prm.pair_cache || !rec_pool.p) return;
-  const size_t np = gcap ? rec_pt.n : (size_t)n_ptasks, ns = gcap ? rec_st.n : (size_t)n_stasks;
-  const size_t nn = gcap ? (size_t)cap_nodes : (size_t)n_nodes, nt = gcap ? (size_t)N : (size_t)n_tiles;
+  if (!recording() || !rec_pool.p) return;
+  const size_t np = (size_t)n_ptasks, ns = (size_t)n_stasks, nn = (size_t)n_nodes, nt = (size_t)n_tiles;
   cudaMemsetAsync(rec_ctr.p, 0, sizeof(unsigned int), st);
   if (np) cudaMemsetAsync(rec_pt.p, 0xff, np * sizeof(uint2), st);
   if (ns) cudaMemsetAsync(rec_st.p, 0xff, ns * sizeof(uint2), st);
@@ -919,7 +910,7 @@ void Engine::rec_enqueue_reset() {
 sph_status Engine::density_pass() {
   {
     Scope sc(this, PH_DENSITY_TASKS);
-    launch_live_tasks(*this, true);
+    launch_live_tasks(*this);
   }
   {
     Scope sc(this, PH_DENSITY);
@@ -930,17 +921,25 @@ sph_status Engine::density_pass() {
 }
 
 sph_status Engine::density() {
-  if (!built) {
-    sph_status s = build();
+  sph_status s = ensure_built();
+  if (s != SPH_OK) return s;
+  for (;;) {
+    if (count_pairs) CK(cudaMemsetAsync(pc.p, 0, 16 * sizeof(unsigned long long), st));
+    launch_pass_setup(*this, false, false, 0);
+    const unsigned int held = R.cap;
+    s = rec_prepare();
     if (s != SPH_OK) return s;
+    rec_enqueue_reset();
+    s = density_pass();
+    if (s != SPH_OK) return s;
+    if (!rec_valid || R.cap <= held) break;
+    // a new pool: once more where it was too small
+    unsigned int rc = 0;
+    CK(cudaMemcpyAsync(&rc, rec_ctr.p, sizeof(rc), cudaMemcpyDeviceToHost, st));
+    CK(sync_stream());
+    if (rc <= R.cap) break;
+    rec_need = std::max<long long>(rec_need, rc);
   }
-  if (count_pairs) CK(cudaMemsetAsync(pc.p, 0, 16 * sizeof(unsigned long long), st));
-  launch_pass_setup(*this, false, false, 0);
-  sph_status s = rec_prepare();
-  if (s != SPH_OK) return s;
-  rec_enqueue_reset();
-  s = density_pass();
-  if (s != SPH_OK) return s;
   {
     Scope sc(this, PH_GHOST);
     launch_ghost(*this, 0, 1);
@@ -955,14 +954,12 @@ sph_status Engine::density() {
 }
 
 sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
-  if (!built) {
-    sph_status s = build();
-    if (s != SPH_OK) return s;
-  }
+  sph_status s = ensure_built();
+  if (s != SPH_OK) return s;
   if (count_pairs) CK(cudaMemsetAsync(pc.p, 0, 16 * sizeof(unsigned long long), st));
   CK(it_dev.reserve(4));
   launch_pass_setup(*this, true, true, 1);
-  sph_status s = rec_prepare();
+  s = rec_prepare();
   if (s != SPH_OK) return s;
   rec_enqueue_reset();
   // Iterations run in batches launched without a host round trip: the iteration
@@ -984,7 +981,7 @@ sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
           launch_gather_prep(*this, it_dev.p);
         }
         fresh = false;
-        launch_live_tasks(*this, true, it_dev.p);
+        if (it + k == 1) launch_live_tasks(*this);      // (only a first pass records)
       }
       {
         // iteration it + k unless the iteration stopped earlier in the batch (its
@@ -1006,7 +1003,6 @@ sph_status Engine::h_update(long long* n_unconverged, int* iterations) {
     const unsigned int rc = hst->rc;
     const bool read_rec = rebuilds == 0 && it == 1 && rec_valid;
     if (read_rec) {
-      rec_used = rc;
       rec_need = std::max<long long>(rec_need, rc);
       rec_unread = false;
     }
@@ -1060,7 +1056,7 @@ sph_status Engine::force() {
   if (count_pairs) CK(cudaMemsetAsync(fcnt.p, 0, N * sizeof(unsigned int), st));
   {
     Scope sc(this, PH_FORCE_TASKS);
-    launch_live_tasks(*this, false);
+    launch_live_tasks(*this);
   }
   {
     Scope sc(this, PH_FORCE);
@@ -1277,10 +1273,6 @@ void Engine::drop_step_graph() {
 
 sph_status Engine::capture_step_graph() {
   drop_step_graph();
-  {
-    const sph_status rs = rec_prepare();
-    if (rs != SPH_OK) return rs;
-  }
   CK(dmax_bits.reserve(nbox));
   CK(reuse_flag.reserve(1));
   CK(it_dev.reserve(4));
@@ -1326,7 +1318,6 @@ sph_status Engine::capture_step_graph() {
   launch_pdl(k_leaf_hmax, nsm * 8, 256, st, T, n_nodes, Hs.p); count_launch();
   launch_pdl(k_tile_boxes, grid(32 * n_tiles), 256, st, n_tiles, TL, pos4.p); count_launch();
   launch_pass_setup(*this, true, true, 0);
-  rec_enqueue_reset();
   launch_iter_start(*this, iter);
   CKG(cudaStreamEndCapture(st, &body));
   g_keep = launch_count() - c1;
@@ -1341,7 +1332,6 @@ sph_status Engine::capture_step_graph() {
   c1 = launch_count();
   CKG(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
   launch_gather_prep(*this, it_dev.p);
-  launch_live_tasks(*this, true, it_dev.p);
   launch_density(*this, it_dev.p);
   launch_density_gather(*this);
   launch_ghost(*this, 1, 0, it_dev.p);
@@ -1361,7 +1351,6 @@ sph_status Engine::capture_step_graph() {
   CKG(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
   CKG(cudaMemsetAsync(facc.p, 0, N * sizeof(float4), st));
   CKG(cudaMemsetAsync(fvsig.p, 0, N * sizeof(float), st));
-  launch_live_tasks(*this, false);
   launch_force(*this);
   launch_reduce(*this);
   launch_kick(*this);
@@ -1380,13 +1369,8 @@ sph_status Engine::step_graph() {
   }
   CK(cudaGraphLaunch(step_x, st));
   CK(read_status());
-  const unsigned int flag = hst->flag, ea = hst->ea[0], rc = hst->rc;
+  const unsigned int flag = hst->flag, ea = hst->ea[0];
   const int itv[2] = {hst->itv[0], hst->itv[1]};
-  if (R.pool && !flag) {
-    rec_used = rc;
-    rec_need = std::max<long long>(rec_need, rc);
-    rec_unread = false;
-  }
   const bool rebuild = flag != 0 || (ea & ERR_REBUILD) != 0u;
   count_launches(g_pre + (flag ? 0 : g_keep + (long long)itv[0] * g_iter + (rebuild ? 0 : g_force)));
   if (rebuild) {
@@ -1405,7 +1389,7 @@ sph_status Engine::step_graph() {
   built = true;
   have_density = have_ghost = have_force = have_acc = true;
   acc_edited = false;
-  rec_valid = R.pool != nullptr;
+  rec_valid = false;
   last_iters = itv[0];
   last_rebuilds = 0;
   last_gathered = 0;
@@ -1550,10 +1534,6 @@ sph_status Engine::enqueue_captured_build() {
   count_launch();
   launch_pdl(k_pair_csr, nsm * 8, 256, st, Lq, cap_pair, T); count_launch();
   launch_unit_list(*this);
-  if (prm.pair_cache) {
-    launch_task_offsets(*this);
-    launch_task_items(*this);
-  }
   if (prm.sort_merge)
     launch_pdl(k_sort_merge, nsm * 8, 256, st, mid_seg.p, mid_count.p, T, TL, sort_r.p, sort_i.p);
   else
@@ -1579,17 +1559,6 @@ sph_status Engine::capture_build_graph() {
   drop_build_graph();
   // capacities with room to grow: a count past one makes the build not hold, and
   // the host completes that step with a build of its own
-  const size_t cp = (size_t)(n_ptasks + n_ptasks / 4 + 1024), cs = (size_t)(n_stasks + n_stasks / 4 + 1024);
-  if (prm.pair_cache) {
-    CK(l_ptask.reserve(cp));
-    CK(l_stask.reserve(cs));
-    CK(l_plive.reserve(cp + cs));
-  }
-  CK(l_nlive.reserve(1));
-  Lq.p_task = l_ptask.p;
-  Lq.s_task = l_stask.p;
-  Lq.p_live = l_plive.p;
-  Lq.n_live = l_nlive.p;
   CK(sort_r.reserve((size_t)(n_entries + n_entries / 4 + 4096)));
   CK(sort_i.reserve(sort_r.n));
   // a box without cells of many clusters is captured without their sort (20 launches,
@@ -1610,8 +1579,6 @@ sph_status Engine::capture_build_graph() {
   CK(it_dev.reserve(4));
   {
     sph_status s = ensure_side_stream();
-    if (s != SPH_OK) return s;
-    s = rec_prepare();
     if (s != SPH_OK) return s;
   }
   if (prof) {
@@ -1645,8 +1612,7 @@ sph_status Engine::capture_build_graph() {
     if (s != SPH_OK) return s;
   }
   launch_pdl(k_check_build, 1, 1, st, ok, err_all.p, t_n.p, cap_nodes, l_counts.p, cap_self, cap_pair, gb_last_q,
-             prm.pair_cache ? (unsigned int)l_ptask.n : 0xffffffffu,
-             prm.pair_cache ? (unsigned int)l_stask.n : 0xffffffffu, big_count.p, gb_cap_big, gstat.p); count_launch();
+             big_count.p, gb_cap_big, gstat.p); count_launch();
   CKB(cudaStreamEndCapture(st, &g1));
   gb_build = launch_count() - c0;
   cudaGraphNode_t n1, n2, n3, n4;
@@ -1663,7 +1629,6 @@ sph_status Engine::capture_build_graph() {
   long long c1 = launch_count();
   CKB(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
   launch_pass_setup(*this, true, true, 0);
-  rec_enqueue_reset();
   launch_iter_start(*this, iter);
   CKB(cudaStreamEndCapture(st, &body));
   gb_setup = launch_count() - c1;
@@ -1689,7 +1654,6 @@ sph_status Engine::capture_build_graph() {
   prof_into_graph = false;
   CKB(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode));
   launch_gather_prep(*this, it_dev.p);
-  launch_live_tasks(*this, true, it_dev.p);
   launch_density(*this, it_dev.p);
   launch_density_gather(*this);
   launch_ghost(*this, 1, 0, it_dev.p);
@@ -1756,7 +1720,6 @@ sph_status Engine::capture_build_graph() {
   auto force_tasks = [&] {
     cudaMemsetAsync(facc.p, 0, N * sizeof(float4), st);
     cudaMemsetAsync(fvsig.p, 0, N * sizeof(float), st);
-    launch_live_tasks(*this, false);
   };
   auto reduce = [&] {
     launch_reduce(*this);
@@ -1797,16 +1760,11 @@ sph_status Engine::build_step_graph() {
   }
   CK(cudaGraphLaunch(bstep_x, st));
   CK(read_status());
-  const unsigned int gs = hst->gs, ea = hst->ea[0], ntl = hst->ntl, rc = hst->rc;
+  const unsigned int gs = hst->gs, ea = hst->ea[0], ntl = hst->ntl;
   const int itv[2] = {hst->itv[0], hst->itv[1]};
   const int *tn = hst->tn, *lc = hst->lc;
   const unsigned long long bcw = (unsigned long long)hst->bcw[0] | ((unsigned long long)hst->bcw[1] << 32);
   const bool held = gs == 1u;
-  if (R.pool && held) {
-    rec_used = rc;
-    rec_need = std::max<long long>(rec_need, rc);
-    rec_unread = false;
-  }
   const bool rebuild = !held || (ea & ERR_REBUILD) != 0u;
   count_launches(gb_build + (held ? gb_setup + (long long)itv[0] * gb_iter + (rebuild ? 0 : gb_force) : 0));
   if (held) {
@@ -1820,8 +1778,7 @@ sph_status Engine::build_step_graph() {
     n_pairs = lc[1];
     n_segments = lc[4];
     n_entries = (unsigned int)lc[5];
-    n_ptasks = lc[6];
-    n_stasks = ntl;
+    tasks_listed = false;
     n_tiles = ntl;
     n_big = (int)(bcw >> 40);
     n_big_entries = (long long)(bcw & ((1ull << 40) - 1ull));
@@ -1837,7 +1794,7 @@ sph_status Engine::build_step_graph() {
     return step_rest_after_build();
   }
   ++steps_graph;
-  rec_valid = R.pool != nullptr;
+  rec_valid = false;
   if (bgraph_prof) {
     for (const GProfRec& r : gprof_recs) {
       float t = 0.0f;

@@ -44,11 +44,10 @@ __device__ __forceinline__ ItemGeom item_geom(const Tree& T, const BoxDesc* box,
 // launch): their cost varies by orders of magnitude, so a static split leaves most
 // SMs idle behind the longest ones.
 
-// blocks per SM of the recording first density pass (4.2M clustered 10.2 ms at 5, 9.9 at
-// 6, 9.2 at 7), of
-// the plain first pass (see k_density), of the later passes (4.2M clustered h iteration:
-// density phase 34.0 ms at 5, 33.6 at 6, 32.5 at 7, 33.1 at 8) and of the gathered ones
-// (32.4 ms at 8, 32.2 at 7, 32.3 at 6)
+// Blocks per SM of the recording first density pass (4.2M clustered 10.2 ms at 5, 9.9 at 6,
+// 9.2 at 7), of the plain first pass (see k_density) and of the later passes (4.2M clustered
+// h iteration, density phase: 34.0 ms at 5, 33.6 at 6, 32.5 at 7, 33.1 at 8); for the
+// gathered ones see GATHER_BLOCKS.
 #ifndef REC_BLOCKS
 #define REC_BLOCKS 7
 #endif
@@ -1923,29 +1922,15 @@ __global__ void k_unit_list(unsigned int ntcap, const unsigned int* __restrict__
   }
 }
 
-// Tasks of one pass that have work, as (interaction, cluster); bit 31 of the
-// interaction marks a self task.  Pair tasks: in a density pass those whose
-// cluster or partner cell still iterates h, and in every pass those whose
-// cluster lies within reach of the partner cell (the test the sweep would
-// start with).  Self tasks: in a density pass those whose cell still iterates
-// h.  Self tasks come first: the costliest tasks are then taken early and the
-// short pair tasks fill the end of the pass.  One thread per task;
-// warp-aggregated appends.
-template <bool DENS>
+// Tasks of a recording first density pass, or of the force pass that replays it, as
+// (interaction, cluster); bit 31 of the interaction marks a self task.  Pair tasks: those
+// whose cluster lies within reach of the partner cell (the test the sweep would start
+// with).  Self tasks come first: the costliest tasks are then taken early and the short
+// pair tasks fill the end of the pass.  One thread per task; warp-aggregated appends.
 __global__ void k_live_tasks(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box, long long npt,
-                             long long nst, int partial_host, const int* __restrict__ it_dev, int cap_p, int cap_s,
-                             const int* __restrict__ gflag) {
+                             long long nst) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
-  if (it_dev && it_dev[2] != 0) return;    // the iteration has stopped: no tasks
-  if (npt < 0) {
-    // a captured step: the task counts of this build, from the device
-    npt = min(Lq.counts[6], cap_p);
-    nst = min(Lq.counts[7], cap_s);
-  }
-  // later iterations keep only what still iterates (with a device counter: from iteration 2 on)
-  const int partial = it_dev ? (*it_dev > 1 ? 1 : 0) : partial_host;
-  if (DENS && partial && gflag && gflag[0] != 0) return;       // the pass gathers
   const long long ntask = npt + nst;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < ntask; b0 += stride) {
@@ -1958,31 +1943,16 @@ __global__ void k_live_tasks(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restri
       const int A = Lq.self_a[item];
       ti = T.tile0[A] + (ts - Lq.s_toff[item]);
       rec = (unsigned int)item | 0x80000000u;
-      live = !DENS || T.active[A];
+      live = true;
     } else if (t < ntask) {
       const unsigned int tp = (unsigned int)(t - nst);
       const int item = (int)Lq.p_task[tp];
-      const int A0 = Lq.pair_a[item], B0 = Lq.pair_b[item];
+      const int A0 = Lq.pair_a[item];
       ti = T.tile0[A0] + (tp - Lq.p_toff[item]);
       rec = (unsigned int)item;
-      const bool iact = !DENS || partial == 0 || TL.active[ti];
-      live = iact || T.active[B0];
-      if (live) {
-        const PairSetup P = pair_setup(Lq, T, box, item);
-        const Box3 bi = tile_box3(TL, T, ti, P.tshA);
-        const float Hi = TL.lo[ti].w * P.g.invL;
-        live = box_near(bi, P.cellB, fmaxf(Hi, P.HmB) + P.slack);
-        if (live && !iact) {
-          // only B's active particles need this cluster: their box, in A's frame,
-          // must lie within B's largest H
-          Box3 ba;
-          ba.lo = make_float3(key_float(T.alo[3 * B0]) + P.g.offB.x, key_float(T.alo[3 * B0 + 1]) + P.g.offB.y,
-                              key_float(T.alo[3 * B0 + 2]) + P.g.offB.z);
-          ba.hi = make_float3(key_float(T.ahi[3 * B0]) + P.g.offB.x, key_float(T.ahi[3 * B0 + 1]) + P.g.offB.y,
-                              key_float(T.ahi[3 * B0 + 2]) + P.g.offB.z);
-          live = box_near(bi, ba, P.HmB + P.slack);
-        }
-      }
+      const PairSetup P = pair_setup(Lq, T, box, item);
+      const Box3 bi = tile_box3(TL, T, ti, P.tshA);
+      live = box_near(bi, P.cellB, fmaxf(TL.lo[ti].w * P.g.invL, P.HmB) + P.slack);
     }
     const unsigned int bal = __ballot_sync(0xffffffffu, live);
     unsigned int at = 0;
@@ -2196,6 +2166,7 @@ __device__ __forceinline__ void gather_unit(unsigned int pid, unsigned int part,
   flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
 }
 
+// (4.2M clustered h iteration, density phase: 32.4 ms at 8, 32.2 at 7, 32.3 at 6)
 #ifndef GATHER_BLOCKS
 #define GATHER_BLOCKS 7
 #endif
@@ -2331,17 +2302,16 @@ __global__ void k_ghost(long long N, int mode, int it_host, const int* __restric
   }
 }
 
-// Mark every cell that holds a particle still iterating h (and its ancestors).
-// After an h iteration: the clusters and cells that still hold a particle
-// iterating h (a cluster's largest H follows the H its particles took), and for
-// every cell the box of those particles in the cell's
-// frame.  One warp per cluster; the cluster's box of active particles is added
-// to every cell on its chain with ordered-key atomics.
-// Counts the particles still iterating per cluster (cnt[t], and cnt[ntile] = 0) for the
-// packing that follows.
+// After an h iteration: marks the clusters and cells that still hold a particle iterating
+// h (a cluster's largest H follows the H its particles took), with the box of those
+// particles in each cell's frame.  One warp per cluster; the cluster's box of active
+// particles is added to every cell on its chain with ordered-key atomics.  With pair
+// records (rec) also the clusters and cells that changed since the recording, and the
+// boxes of the particles that did.  Counts the particles still iterating per cluster
+// (cnt[t], and cnt[ntile] = 0) for the packing that follows.
 __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ ntile_dev,
                               const unsigned char* __restrict__ act, const float4* __restrict__ pos4, Tree T, Tiles TL,
-                              unsigned int* __restrict__ cnt) {
+                              unsigned int* __restrict__ cnt, int rec) {
   pdl_wait();
   if (ntile_dev) ntile = min(ntile, (long long)*ntile_dev);   // a captured step: this build's clusters
   const int lane = threadIdx.x & 31;
@@ -2369,9 +2339,9 @@ __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ 
     if (lane == 0) {
       if (hm > TL.lo[t].w) TL.lo[t].w = hm;
       TL.active[t] = 1;
-      TL.changed[t] = 1;
+      if (rec) TL.changed[t] = 1;
     }
-    if (lane >= 12) continue;
+    if (lane >= (rec ? 12 : 6)) continue;
     // a lane per bound: the lower and upper corners of the iterating particles' box, then
     // of those that took a new h since the recording
     const int k = lane % 3;
@@ -2383,7 +2353,7 @@ __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ 
     for (int id = (int)TL.leaf[t]; id >= 0; id = T.parent[id]) {
       if (lane == 0) {
         T.active[id] = 1;
-        T.changed[id] = 1;
+        if (rec) T.changed[id] = 1;
       }
       const float key_at = mine + (lck - reinterpret_cast<const float*>(&T.cen[id])[k]);   // the offset is exact
       if (up) atomicMax(&arr[3 * id + k], float_key(key_at));
@@ -2392,7 +2362,6 @@ __global__ void k_mark_active(long long ntile, const unsigned int* __restrict__ 
   }
 }
 
-// clusters of the i cell per interaction: the prefix of these numbers the tasks
 // Tasks: one per (interaction, cluster of its first cell).  Counts per
 // interaction over the whole list capacity (zero past the list), so that the
 // prefix and the task totals are ready before the host reads the list sizes.
@@ -2406,15 +2375,9 @@ __global__ void k_task_tiles(Lists Lq, Tree T, int cap_pair, int cap_self) {
 }
 
 // task -> interaction tables (one warp per interaction)
-// npair < 0: the list sizes come from the device (a captured step); the tables
-// hold cap_p pair tasks and cap_s self tasks, and nothing is written past them.
-__global__ void k_task_items(Lists Lq, Tree T, int npair, int nself, int cap_pair, int cap_self, unsigned int cap_p,
-                             unsigned int cap_s) {
+// The tables hold cap_p pair tasks and cap_s self tasks, and nothing is written past them.
+__global__ void k_task_items(Lists Lq, Tree T, int npair, int nself, unsigned int cap_p, unsigned int cap_s) {
   pdl_wait();
-  if (npair < 0) {
-    npair = min(Lq.counts[1], cap_pair);
-    nself = min(Lq.counts[0], cap_self);
-  }
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -2775,10 +2738,10 @@ __global__ void k_get_field(long long off, long long n, int field, const unsigne
 // may run in several host threads)
 static int resident_ctas(const void* fn) {
   static std::mutex mu;
-  static const void* fns[24] = {nullptr};   // the 12 density, 2 gathered density and 4 force instances
-  static int val[24] = {0};
+  static const void* fns[16] = {nullptr};   // the 10 density, 2 gathered density and 3 force instances
+  static int val[16] = {0};
   std::lock_guard<std::mutex> lock(mu);
-  for (int k = 0; k < 24; ++k) {
+  for (int k = 0; k < 16; ++k) {
     if (fns[k] == fn) return val[k];
     if (!fns[k]) {
       int nb = 0;
@@ -2791,22 +2754,13 @@ static int resident_ctas(const void* fn) {
   return 4;
 }
 
-void launch_live_tasks(Engine& E, bool dens, const int* it_dev) {
+void launch_live_tasks(Engine& E) {
   if (!E.rec_for_force().pool) return;     // the passes walk their clusters' interactions (with pair records they list their tasks)
   cudaMemsetAsync(E.Lq.n_live, 0, sizeof(unsigned int), E.st);
-  // a captured rebuild step sizes the launch by the task capacity and the kernel
-  // reads the counts of the build from the device
-  const int cap_p = (int)E.l_ptask.n, cap_s = (int)E.l_stask.n;
-  const long long npt = E.gcap ? -1 : E.n_ptasks, nst = E.gcap ? -1 : E.n_stasks;
-  const long long n = E.gcap ? (long long)cap_p + cap_s : E.n_ptasks + E.n_stasks;
+  const long long n = E.n_ptasks + E.n_stasks;
   if (n == 0) return;
-  const int grid = (int)std::min<long long>((n + 255) / 256, (long long)E.nsm * 16);
-  if (dens)
-    launch_pdl(k_live_tasks<true>, grid, 256, E.st, E.Lq, E.T, E.TL, E.box.p, npt, nst, E.partial_pass, it_dev,
-               cap_p, cap_s, it_dev ? E.gflag.p : nullptr);
-  else
-    launch_pdl(k_live_tasks<false>, grid, 256, E.st, E.Lq, E.T, E.TL, E.box.p, npt, nst, 0, nullptr, cap_p, cap_s,
-               nullptr);
+  launch_pdl(k_live_tasks, (int)std::min<long long>((n + 255) / 256, (long long)E.nsm * 16), 256, E.st, E.Lq, E.T, E.TL,
+             E.box.p, E.n_ptasks, E.n_stasks);
   count_launch();
 }
 
@@ -2820,18 +2774,16 @@ void launch_density(Engine& E, const int* it_dev, int only) {
     if (it_dev && only >= 0 && part != only) continue;
     const bool kahan = E.kahan();
     // the first pass records its pairs for the force pass when the records are on
-    const bool rec = part == 0 && E.rec_valid;
+    const bool rec = part == 0 && E.rec_for_force().pool != nullptr;
     decltype(&k_density<false, false, false, false>) k;
     if (kahan)
       k = E.count_pairs ? (part ? k_density<true, true, true, false>
                                 : (rec ? k_density<true, false, true, true> : k_density<true, false, true, false>))
-                        : (part ? k_density<false, true, true, false>
-                                : (rec ? k_density<false, false, true, true> : k_density<false, false, true, false>));
+                        : (part ? k_density<false, true, true, false> : k_density<false, false, true, false>);
     else
       k = E.count_pairs ? (part ? k_density<true, true, false, false>
                                 : (rec ? k_density<true, false, false, true> : k_density<true, false, false, false>))
-                        : (part ? k_density<false, true, false, false>
-                                : (rec ? k_density<false, false, false, true> : k_density<false, false, false, false>));
+                        : (part ? k_density<false, true, false, false> : k_density<false, false, false, false>);
     launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st,
         E.Lq, E.T, E.TL, E.box.p, E.pos4.p, E.cen4.p, E.sort_r.p, E.sort_i.p, E.act.p, E.perm.p, E.x.p, E.dacc.p,
         E.dcnt.p, E.dcomp.p, E.pc.p, E.task_ctr.p + part, E.partial_pass, it_dev, it_dev ? E.gflag.p : nullptr,
@@ -2874,8 +2826,7 @@ void launch_density_gather(Engine& E) {
 
 void launch_force(Engine& E) {
   const bool rec = E.rec_for_force().pool != nullptr;
-  const auto k = E.count_pairs ? (rec ? k_force<true, true> : k_force<true, false>)
-                               : (rec ? k_force<false, true> : k_force<false, false>);
+  const auto k = E.count_pairs ? (rec ? k_force<true, true> : k_force<true, false>) : k_force<false, false>;
   cudaMemsetAsync(E.task_ctr.p + 2, 0, sizeof(unsigned int), E.st);
   launch_pdl(k, E.nsm * resident_ctas((const void*)k), SPH_THREADS, E.st,
       E.Lq, E.T, E.TL, E.box.p, E.pos4.p, E.cen4.p, E.vel4.p, E.ghost4.p, E.sort_r.p, E.sort_i.p, E.perm.p, E.x.p,
@@ -2926,7 +2877,7 @@ void launch_mark_active_cells(Engine& E) {
   const long long nt = E.gcap ? E.N : E.n_tiles;
   launch_pdl(k_mark_active, E.grid(32 * nt), 256, E.st, nt,
              E.gcap ? reinterpret_cast<const unsigned int*>(E.dev_counters.p + 4) : nullptr, E.act.p, E.pos4.p, E.T,
-             E.TL, E.pk_cnt.p);
+             E.TL, E.pk_cnt.p, E.rec_for_force().pool ? 1 : 0);
   count_launch();
 }
 
@@ -2939,8 +2890,7 @@ void launch_task_offsets(Engine& E) {
 }
 
 void launch_task_items(Engine& E) {
-  launch_pdl(k_task_items, E.nsm * 8, 256, E.st, E.Lq, E.T, E.gcap ? -1 : E.n_pairs, E.gcap ? -1 : E.n_selfs,
-             E.cap_pair, E.cap_self, (unsigned int)E.l_ptask.n, (unsigned int)E.l_stask.n);
+  launch_pdl(k_task_items, E.nsm * 8, 256, E.st, E.Lq, E.T, E.n_pairs, E.n_selfs, (unsigned int)E.l_ptask.n, (unsigned int)E.l_stask.n);
   count_launch();
 }
 

@@ -235,18 +235,25 @@ class Engine {
   Lists Lq{};
 
   // the pairs of the first density pass of an h iteration, kept for the force pass
-  // (params.pair_cache): pool of batches in chunks, chunk links, chunk counter,
-  // per-task records
+  // (params.pair_cache, while pairs are counted): pool of batches in chunks, chunk links,
+  // chunk counter, per-task records
   DBuf<unsigned int> rec_pool, rec_next, rec_ctr;
   DBuf<uint2> rec_pt, rec_st;
   PairRec R{};
   bool rec_valid = false;         // the records hold for the next force pass
   long long rec_need = 0;         // chunks the last recordings took (the pool grows to this)
-  long long rec_used = 0;         // chunks the last recording read back took
   bool rec_unread = false;        // the last recording's chunk count was not read back yet
   sph_status rec_prepare();       // pool and record arrays sized for the next recording
   void rec_enqueue_reset();       // a recording starts with the next full density pass
-  PairRec rec_for_force() const { return rec_valid ? R : PairRec{}; }
+  // Recorded passes run a task per interaction and cluster, which takes 1.2 to 2.3 times as
+  // long as the units of the others with all of a force pass's culling saved (density and
+  // force at the same h, ms, with and without: 1M lattice 2.46 / 1.41, 262k Plummer 0.85 /
+  // 0.63, 1M log-normal 7.5 / 6.2, 4.2M clustered 28.2 / 20.1; the lattice took 2.02 when
+  // both kinds of pass ran such tasks).  So only passes that count pairs record.
+  bool recording() const { return prm.pair_cache != 0 && count_pairs; }
+  bool tasks_listed = false;      // the build's tasks are in their tables
+  sph_status ensure_built() { return built && (!recording() || tasks_listed) ? SPH_OK : build(); }
+  PairRec rec_for_force() const { return rec_valid && recording() ? R : PairRec{}; }
 
   // sorted projections
   DBuf<float> sort_r;
