@@ -21,15 +21,16 @@ def _run(api, box, graphs, steps, dt, **prm):
     ctx = api.sph_ctx_create(p, 0)
     try:
         b = api.box_from(ctx, box)
-        trace = []
-        for _ in range(steps):
-            b.step(dt)
-            trace.append(b.stats())
-        out = {f: b.get(f) for f in ("x", "h", "rho", "a", "count")}
-        b.close()
+        try:
+            trace = []
+            for _ in range(steps):
+                b.step(dt)
+                trace.append(b.stats())
+            return {f: b.get(f) for f in ("x", "h", "rho", "a", "count")}, trace
+        finally:
+            b.close()
     finally:
         api.sph_ctx_destroy(ctx)
-    return out, trace
 
 
 def _same_run(got, ref, L):
@@ -70,3 +71,57 @@ def test_node_overflow_in_a_captured_build(api):
     assert trace[at - 1]["graph_steps"] > 0 and trace[at]["graph_steps"] == trace[at - 1]["graph_steps"]
     assert trace[-1]["graph_steps"] > trace[at]["graph_steps"]
     _same_run(got, ref, box.L)
+
+
+def test_first_cell_of_many_clusters_in_a_captured_step(api):
+    """Steps captured while no cell needs the global sort (more than 2048 clusters) leave it
+    out; when one grows past that, the host completes the step, and the next capture sorts."""
+    # a block over two top cells of edge 1/2, 23 of its 50 planes in the first, that drifts
+    # along -x by a plane a step: the first holds 26 planes, 2032 clusters, after the third
+    # step and 2110 after the fourth.  A particle far from the block keeps the top cells
+    # that large.
+    side = 50
+    box = inputs.lattice_box(side, jitter=0.2, seed=1, v_sigma=0.0, periodic=False)
+    box.x = np.array([0.5 - 23 * 0.0084, 0.06, 0.06]) + box.x / box.L * 0.42
+    box.L = 1.0
+    box.x[-1] = [0.76, 0.64, 0.64]
+    box.v = np.tile(np.array([-1.0, 0.0, 0.0], np.float32), (box.n, 1))
+    box.v[-1] = 0.0
+    box.u = np.full(box.n, 1e-6, np.float32)
+    box.h = np.full(box.n, 1.2348 * 0.42 / side, np.float32)
+    box.h[-1] = 0.18
+    prm = {"leaf_max": 200000, "h_tol": 1e-5}
+    got, trace = _run(api, box, 1, 7, 0.0084, **prm)
+    ref, _ = _run(api, box, 0, 7, 0.0084, **prm)
+    graphs = [t["graph_steps"] for t in trace]
+    print("[graphs]", graphs, [t["top_level"] for t in trace], [t["n_sorted_entries"] for t in trace])
+    assert {t["top_level"] for t in trace} == {1}
+    assert graphs == [0, 0, 1, 1, 2, 3, 4]
+    _same_run(got, ref, box.L)
+
+
+@pytest.mark.parametrize("field", ["a", "dudt"])
+def test_forces_read_after_they_were_set(api, field):
+    """set_field replaces the saved accelerations that the next kick takes; what get returns
+    stays the last force pass's."""
+    box = inputs.lattice_box(16, jitter=0.2, seed=8)
+    ctx = api.sph_ctx_create(api.sph_params_default(), 0)
+    try:
+        b = api.box_from(ctx, box)
+        try:
+            b.step(0.0)
+            before = {k: b.get(k) for k in ("a", "dudt")}
+            new = np.random.default_rng(1).normal(size=before[field].shape).astype(np.float32)
+            b.set_field(field, new)
+            for k in before:
+                assert np.array_equal(b.get(k), before[k])
+            v = b.get("v")
+            dt = 1e-5
+            b.step(dt)
+            kick = {"a": before["a"], field: new}["a"]       # the opening kick takes what was set
+            second = b.get("a")
+            np.testing.assert_allclose(b.get("v"), v + 0.5 * dt * (kick + second), rtol=1e-5, atol=1e-7)
+        finally:
+            b.close()
+    finally:
+        api.sph_ctx_destroy(ctx)
