@@ -45,9 +45,9 @@ __device__ __forceinline__ ItemGeom item_geom(const Tree& T, const BoxDesc* box,
 // SMs idle behind the longest ones.
 
 // Blocks per SM of the recording first density pass (4.2M clustered 10.2 ms at 5, 9.9 at 6,
-// 9.2 at 7), of the plain first pass (see k_density) and of the later passes (4.2M clustered
-// h iteration, density phase: 34.0 ms at 5, 33.6 at 6, 32.5 at 7, 33.1 at 8); for the
-// gathered ones see GATHER_BLOCKS.
+// 9.2 at 7), of the plain first pass (see k_density) and of the later passes; the
+// gathered ones have GATHER_BLOCKS.  (4.2M clustered h iteration, all three at once: density
+// phase 39.4 ms at 6, 38.8 at 7, 40.6 at 8.)
 #ifndef REC_BLOCKS
 #define REC_BLOCKS 7
 #endif
@@ -1732,8 +1732,8 @@ __device__ __forceinline__ void force_replay_task(bool self, int item, unsigned 
 // a captured step, and the one that does not match the iteration returns.
 // The first pass (PART = false) runs 7 blocks of 128 threads per SM (at most 73
 // registers, a few spilled): issue slots bound the pass, and more warps in flight fill
-// them until the spills grow (density phase of the 33.5M step 36.4 ms at 6 blocks, 33.9 at
-// 7, 34.7 at 8, 38.9 at 10).
+// them until the spills grow (density phase of the 33.5M step 42.0 ms at 6 blocks, 41.1 at
+// 7, 41.5 at 8).
 template <bool COUNT, bool PART, bool KAHAN, bool REC>
 __global__ void __launch_bounds__(SPH_THREADS, PART ? PART_BLOCKS : (REC ? REC_BLOCKS : DENS_BLOCKS)) k_density(Lists Lq, Tree T, Tiles TL, const BoxDesc* __restrict__ box,
                                                          const float4* __restrict__ pos4,
@@ -2166,7 +2166,6 @@ __device__ __forceinline__ void gather_unit(unsigned int pid, unsigned int part,
   flush_dens(I.g, acc, cnt, dacc, dcnt, dcomp);
 }
 
-// (4.2M clustered h iteration, density phase: 32.4 ms at 8, 32.2 at 7, 32.3 at 6)
 #ifndef GATHER_BLOCKS
 #define GATHER_BLOCKS 7
 #endif
