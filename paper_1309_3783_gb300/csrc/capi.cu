@@ -500,7 +500,7 @@ sph_status Engine::ensure_list_capacity(int selfs, int pairs, int queue) {
   }
   if (prm.pair_cache) CK(scan_tmp.reserve((size_t)std::max(cap_pair, cap_self) / 2048 + 64));
   queue = std::max(queue, cap_pair);
-  if (queue > cap_queue || !q_mem[0].p) {
+  if (queue > cap_queue || !q_mem[0].p || !q_mem[1].p) {
     cap_queue = queue;
     for (int k = 0; k < 2; ++k) CK(q_mem[k].reserve(4 * (size_t)queue));
   }
